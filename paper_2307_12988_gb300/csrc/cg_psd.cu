@@ -6,15 +6,12 @@
 // PSD: Welch's method -- segments of M = 2L samples advanced by L, segment
 // mean removed, periodic Hann window, |rfft|^2 averaged over the complete
 // segments, one-sided density (factor 2 except at DC and M/2) / (fs sum w^2).
-// psd_welch_kernel<L>: one segment per block pass, L/16 threads; the
-// segment's L packed complex values z_n = x_2n + i x_2n+1 stay in shared
-// memory (one pad per 16 values against bank conflicts) through in-place
-// Stockham stages of radix 16 (and one smaller radix), each thread holding
-// 16 values in registers between a stage's read and write, twiddles of all
-// but a final small-radix stage from a shared table; the real-FFT split X_k = E_k + W_M^k O_k gives |X_k|^2 for
-// k = 0..L, which each thread accumulates in FP64 registers over all the
-// segments its block takes; per-block partials are summed and scaled by
-// psd_reduce_kernel.
+// psd_welch_kernel<L>: one segment per group of L/32 threads; the segment's L
+// packed complex values z_n = x_2n + i x_2n+1 are transformed in place in
+// shared memory (radix 16, and one smaller radix); the real-FFT split
+// X_k = E_k + W_M^k O_k gives |X_k|^2 for k = 0..L, which the threads add up
+// over all their segments as FP32 pairs; the groups' rows are summed and
+// scaled by psd_reduce_kernel.
 //
 // Resonance: S(f) = A f0^4 / ((f0^2 - f^2)^2 + (f f0 / Q)^2) + B fitted to
 // ln S over the bins of a band by Levenberg-Marquardt in FP64 (one block:
@@ -30,200 +27,423 @@
 
 #include "cg_fft.cuh"
 #include "cg_internal.h"
+#include "cg_stage.cuh"
+
+namespace cg {
+constexpr int kWelchThreads = 512;   // threads of a block of the Welch kernel
+}
 
 struct cg_psd_s {
     int device = 0;
     int L = 0;                 // complex transform length (M / 2)
-    int grid = 0;              // blocks of the Welch kernel
+    int grid = 0;              // blocks of the Welch kernel at most
+    int groups = 0;            // segments a block transforms at a time
     size_t smem = 0;
     double sum_w2 = 0.0;       // sum of the squared window
-    float* win = nullptr;      // [M]
-    float2* twL = nullptr;     // [L] W_L^m
-    float2* twM = nullptr;     // [L + 1] W_M^k
-    double* part = nullptr;    // [grid][L + 1] per-block sums of |X_k|^2
+    float* win = nullptr;      // [M / 2 + 1] the window's first half (it is symmetric)
+    float2* tw = nullptr;      // the kernel's twiddles (WelchTables)
+    int2* pair0 = nullptr;     // [L / 32] buffer places of the last pair of each thread
+    int* bin = nullptr;        // [L + 1] PSD bin of each slot of a row of part
+    float2* part = nullptr;    // [grid * groups][L + 1] sums of |X_k|^2 as FP32 pairs
 };
 
 namespace cg {
 
 namespace {
 
+// The transform of one segment: L = 16 * 16 * R3 * R4 complex points, by a
+// group of L / 32 threads (each 32 points).
+template <int L>
+struct Welch {
+    static constexpr int NT = L / 32;                   // threads of a group
+    static constexpr int G = kWelchThreads / NT;        // groups of a block
+    static constexpr int R3 = L == 2048 ? 8 : 16;
+    static constexpr int R4 = L / (256 * R3);           // 1, 1, 2, 4
+    static constexpr int B = L / 16;                    // points of one first-digit block
+    static constexpr int M = 2 * L;
+    // twiddle tables, float2 entries, in the order the threads read them
+    static constexpr int kT2 = 0;                       // [15][16]      W_256^(r k1)
+    static constexpr int kT3 = kT2 + 15 * 16;           // [R3 - 1][256] W_(256 R3)^(r (k1 + 16 k2)), k1 slowest
+    static constexpr int kT4 = kT3 + (R3 - 1) * 256;    // [R4 - 1][L / R4] W_L^(r k), by position
+    static constexpr int kSplit = kT4 + (R4 - 1) * (L / R4);   // [16][NT] W_M^k of a thread's 16 bin pairs
+    static constexpr int kHalf = kSplit + L / 2;        // W_M^(L / 2)
+    static constexpr int kTables = kHalf + 1;
+    // shared memory: the groups' points, the tables of stages 2 and 3, half
+    // the window, warp sums, the extra bin's sum of each group
+    static constexpr int kSmemZ = G * L * 8;
+    static constexpr int kSmemT = kSmemZ + (15 * 16 + (R3 - 1) * 256) * 8;
+    static constexpr int kSmemW = kSmemT + (M / 2 + 4) * 4;
+    static constexpr int kSmem = kSmemW + G * (2 * NT / 32) * 4 + G * 8;
+};
+
 struct PsdArgs {
     const float* x;
     int64_t stride;            // elements between consecutive samples
     int64_t K;                 // segments
+    int vec2;                  // sample pairs are 8-byte aligned and contiguous
     const float* win;
-    const float2* twL;
-    const float2* twM;
-    double* part;
+    const float2* tw;
+    const int2* pair0;
+    float2* part;
 };
 
-// position of complex value i in the exchange buffer: one pad per 16 values,
-// so the first stage's 16-value-stride writes fall on distinct banks
-__device__ __forceinline__ int zp(int i) { return i + (i >> 4); }
-
-// twiddles: W_L^(q s) for q < min(L, 4096), s = max(1, L / 4096), in shared
-// memory (every stage but a last one of radix < 16 at L > 4096 indexes a
-// multiple of s); that last stage reads the full table from global memory
-template <int L>
-struct TwShared {
-    static constexpr int kStride = L > 4096 ? L / 4096 : 1;
-    static constexpr int kSize = L > 4096 ? 4096 : L;
-};
-
-template <int R>
-struct StageShape {
-    static constexpr int kPerThread = 16 / R;   // butterflies per thread
-};
-
-// one in-place Stockham stage of radix R over the L values in z
-// twiddle source of a stage: 0 the global table, 1 the shared W_L^(q s)
-// table, 2 the shared W_256^q table (the Ns = 16 stage: consecutive frames
-// read consecutive entries instead of entries 16 apart)
-template <int L, int R, int kTw>
-__device__ __forceinline__ void stage_inplace(float2* z, int Ns, const float2* __restrict__ ts,
-                                              const float2* __restrict__ t256, const float2* __restrict__ twL)
+// Shared-memory place of point p: its low four bits XORed with the next four.
+// Every stage's accesses of a half warp then fall on distinct banks (the
+// strides of the stages are 2 NT, L / 256, R4 and 1).  The map is linear over
+// XOR, so a butterfly computes the address of its first point and reaches the
+// others (p ^ d with d disjoint from p, known at compile time) by an XOR with
+// a constant and the instruction's immediate offset.
+__host__ __device__ constexpr int zsw(int p) { return p ^ ((p >> 4) & 15); }
+__device__ __forceinline__ uint32_t zat(uint32_t a, int d)
 {
-    constexpr int NT = L / 16, per = L / R, NB = StageShape<R>::kPerThread;
-    const int t = threadIdx.x;
-    float2 a[NB][R];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        const int j = t + NT * b;
-#pragma unroll
-        for (int r = 0; r < R; ++r) a[b][r] = z[zp(j + r * per)];
-    }
-    __syncthreads();
-    const int twstep = L / (Ns * R);
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        const int j = t + NT * b;
-        const int k = j & (Ns - 1);
-        if (Ns > 1) {
-#pragma unroll
-            for (int r = 1; r < R; ++r) {
-                const int m = r * k * twstep;
-                const float2 w = kTw == 2   ? t256[r * k]
-                                 : kTw == 1 ? ts[m / TwShared<L>::kStride]
-                                            : __ldg(&twL[m]);
-                a[b][r] = cmul(a[b][r], w);
-            }
-        }
-        Dft<R>::run(a[b]);
-        const int idx = (j - k) * R + k;
-#pragma unroll
-        for (int r = 0; r < R; ++r) z[zp(idx + r * Ns)] = a[b][r];
-    }
-    __syncthreads();
+    return (a ^ static_cast<uint32_t>((zsw(d) & 15) << 3)) + static_cast<uint32_t>((d & ~15) << 3);
+}
+__device__ __forceinline__ float2 zld(uint32_t a)
+{
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void zst(uint32_t a, float2 v)
+{
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};\n" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
 }
 
-template <int L>
-__global__ void __launch_bounds__(L / 16) psd_welch_kernel(PsdArgs a)
+template <int NT>
+__device__ __forceinline__ void group_sync(int g)
 {
-    constexpr int NT = L / 16, M = 2 * L;
-    extern __shared__ __align__(16) float2 z[];   // [L + L/16] (padded), then the twiddle table
-    float2* ts = z + L + L / 16;                  // [TwShared<L>::kSize]
-    float2* t256 = ts + TwShared<L>::kSize;       // [256] W_256^q
-    __shared__ double red[NT / 32];
-    const int t = threadIdx.x;
-    for (int i = t; i < TwShared<L>::kSize; i += NT) ts[i] = a.twL[i * TwShared<L>::kStride];
-    for (int i = t; i < 256; i += NT) t256[i] = a.twL[i * (L / 256)];
-    // FP64 sums of |X_k|^2 in registers; at L = 16384 (1024 threads, 64
-    // registers each) in the block's own L2-resident row of part instead
-    constexpr bool kRowAcc = L == 16384;
-    double* row = a.part + static_cast<int64_t>(blockIdx.x) * (L + 1);
-    double acc[kRowAcc ? 1 : 17];
-#pragma unroll
-    for (int j = 0; j < (kRowAcc ? 1 : 17); ++j) acc[j] = 0.0;
-    if constexpr (kRowAcc) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) row[t + NT * j] = 0.0;
-        if (t == 0) row[L] = 0.0;
-    }
-    for (int64_t s = blockIdx.x; s < a.K; s += gridDim.x) {
+    asm volatile("bar.sync %0, %1;\n" ::"r"(g + 1), "n"(NT) : "memory");
+}
+
+// s + e = a + b exactly (Knuth's two-sum)
+__device__ __forceinline__ float two_sum(float a, float b, float& e)
+{
+    const float s = a + b, bb = s - a;
+    e = (a - (s - bb)) + (b - bb);
+    return s;
+}
+
+// Sums of |X_k|^2 as unevaluated FP32 pairs (hi, lo).  An FP64 sum costs a
+// conversion and an addition at 2 lanes per cycle and SM (16,384 bins: 16,000
+// cycles of a segment's 61,000); the pair costs 7 FP32 operations at 128 lanes
+// per cycle.  The lost part of each addition is exact; lo, kept below an ulp
+// of hi by a normalisation every eighth segment, rounds it 2^-24 below that.
+__device__ __forceinline__ void pair_add(float2& a, float b)
+{
+    float e;
+    a.x = two_sum(a.x, b, e);
+    a.y += e;
+}
+// an infinite or undefined sum stays what it is
+__device__ __forceinline__ void pair_norm(float2& a)
+{
+    const float h = a.x + a.y;
+    const bool fin = fabsf(a.x) < INFINITY;
+    a = make_float2(fin ? h : a.x, fin ? a.y - (h - a.x) : 0.f);
+}
+__device__ __forceinline__ void pair_add2(float2& a, float2 b)
+{
+    pair_add(a, b.x);
+    a.y += b.y;
+    pair_norm(a);
+}
+
+// Welch sums.  One segment per group of NT threads, its L packed complex
+// values z_n = x_2n + i x_2n+1 in shared memory.  The transform runs in place
+// (digit-reversed result): the points of a butterfly go back where they were
+// read, so a thread needs no barrier between its reads and its writes, and
+// after the first stage (stride L / 16) all remaining butterflies of a warp
+// stay inside the warp's own 1,024 points -- two block barriers per
+// transform instead of eight, and 16 live values per thread.  That leaves the
+// registers for the sums of |X_k|^2: the thread that holds bins k and L - k
+// (one split, two bins from the same two points and twiddle) adds them up over
+// all its segments.
+//
+// What bounds it: shared-memory traffic (1.3 MB per 32,768-sample segment,
+// 10,000 cycles) and the transform's FP32 work.  Before, the sums lived in
+// L2 as FP64 rows and every table but one was read from L2 (0.75 MB per
+// segment), the sums and the mean ran in FP64 on every thread, and each stage
+// took two barriers of 1,024 threads.  Ten minutes of centres (36,620
+// segments of 32,768): 7.99 -> 3.11 ms (27,000 cycles a segment; the shared
+// memory is busy for 54 % of them).
+template <int L>
+__global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
+{
+    using W = Welch<L>;
+    constexpr int NT = W::NT, R3 = W::R3, R4 = W::R4, B = W::B, M = W::M, G = W::G;
+    extern __shared__ __align__(1024) unsigned char psm[];
+    const int g = threadIdx.x / NT, t = threadIdx.x % NT, w = t >> 5, lane = t & 31;
+    const uint32_t z = static_cast<uint32_t>(__cvta_generic_to_shared(psm)) + g * L * 8;
+    float2* const ts = reinterpret_cast<float2*>(psm + W::kSmemZ);
+    const float2* const t2 = ts + W::kT2;
+    const float2* const t3 = ts + W::kT3;
+    float* const win = reinterpret_cast<float*>(psm + W::kSmemT);
+    float* const red = reinterpret_cast<float*>(psm + W::kSmemW) + g * (2 * NT / 32);
+    float2* const half = reinterpret_cast<float2*>(psm + W::kSmemW + G * (2 * NT / 32) * 4) + g;
+    const int64_t slot = static_cast<int64_t>(g) * gridDim.x + blockIdx.x;   // this group's first segment
+    const int64_t nslot = static_cast<int64_t>(G) * gridDim.x;
+    const uint32_t zt = z + 8 * zsw(t);             // point t, and NT - 1 - t
+    const uint32_t zr = z + 8 * zsw(NT - 1 - t);
+
+    auto stage_x = [&](int64_t s) {   // the thread's own 32 points of segment s, asynchronously
         const float* x = a.x + s * static_cast<int64_t>(L) * a.stride;
-        float2 v[16];
-        float sum = 0.0f;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int64_t n = t + NT * j;
-            v[j] = make_float2(__ldg(x + 2 * n * a.stride), __ldg(x + (2 * n + 1) * a.stride));
-            sum += v[j].x + v[j].y;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        if ((t & 31) == 0) red[t >> 5] = sum;
-        __syncthreads();
-        double tot = 0.0;
-#pragma unroll 1
-        for (int w = 0; w < NT / 32; ++w) tot += red[w];
-        const float mean = static_cast<float>(tot / M);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int n = t + NT * j;
-            z[zp(n)] = make_float2((v[j].x - mean) * __ldg(a.win + 2 * n), (v[j].y - mean) * __ldg(a.win + 2 * n + 1));
-        }
-        __syncthreads();
-        // L = 16^3 * Rl (Rl = 2, 4) or 16^2 * 8
-        stage_inplace<L, 16, 1>(z, 1, ts, t256, a.twL);
-        stage_inplace<L, 16, 2>(z, 16, ts, t256, a.twL);
-        if constexpr (L == 2048) {
-            stage_inplace<L, 8, 1>(z, 256, ts, t256, a.twL);
+        if (a.vec2) {
+            x += 2 * t;
+#pragma unroll 8
+            for (int i = 0; i < 32; ++i)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(zat(zt, NT * i)), "l"(x + 2 * NT * i) : "memory");
         } else {
-            stage_inplace<L, 16, 1>(z, 256, ts, t256, a.twL);
-            if constexpr (L == 8192) stage_inplace<L, 2, 0>(z, 4096, ts, t256, a.twL);
-            if constexpr (L == 16384) stage_inplace<L, 4, 0>(z, 4096, ts, t256, a.twL);
-        }
-        // real-FFT split at every bin k = 0..L
-#pragma unroll
-        for (int j = 0; j < 17; ++j) {
-            const int k = t + NT * j;
-            if (j < 16 || t == 0) {
-                const int kk = (j == 16) ? L : k;
-                const float2 Zb = z[zp(kk & (L - 1))];
-                const float2 Zr = z[zp((L - kk) & (L - 1))];
-                const float2 E = make_float2(0.5f * (Zb.x + Zr.x), 0.5f * (Zb.y - Zr.y));
-                const float2 Dd = make_float2(0.5f * (Zb.x - Zr.x), 0.5f * (Zb.y + Zr.y));
-                const float2 O = make_float2(Dd.y, -Dd.x);
-                const float2 X = cadd(E, cmul(__ldg(&a.twM[kk]), O));
-                const double P = static_cast<double>(fmaf(X.x, X.x, X.y * X.y));
-                if constexpr (kRowAcc)
-                    row[kk] += P;
-                else
-                    acc[j] += P;
+            x += 2 * t * a.stride;
+#pragma unroll 4
+            for (int i = 0; i < 32; ++i) {
+                const float* p = x + 2 * NT * i * a.stride;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(zat(zt, NT * i)), "l"(p) : "memory");
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(zat(zt, NT * i) + 4), "l"(p + a.stride) : "memory");
             }
         }
-        __syncthreads();
-    }
-    if constexpr (!kRowAcc) {
+        cp_async_commit();
+    };
+    if (slot < a.K) stage_x(slot);
+    for (int i = threadIdx.x; i < W::kT4; i += kWelchThreads) ts[i] = a.tw[i];
+    for (int i = threadIdx.x; i <= M / 2; i += kWelchThreads) win[i] = a.win[i];
+    if (t == 0) *half = make_float2(0.f, 0.f);
+    const int2 p15 = a.pair0[t];
+    float2 acc[16][2];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) row[t + NT * j] = acc[j];
-        if (t == 0) row[L] = acc[16];
+    for (int i = 0; i < 16; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
+    __syncthreads();
+
+    int since = 0;   // segments since the sums were normalised
+    for (int64_t s = slot; s < a.K; s += nslot) {
+        // the next segment into L2 meanwhile
+        if (s + nslot < a.K && a.stride <= 4) {
+            const char* nx = reinterpret_cast<const char*>(a.x + (s + nslot) * static_cast<int64_t>(L) * a.stride);
+            for (int64_t i = t; i < M * a.stride / 32; i += NT) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(nx + 128 * i));
+        }
+        cp_async_wait_all();   // own points only: no barrier
+        // ---- segment mean: FP32 sums of 32 samples per first-stage column ----
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            float sum = 0.0f;
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const float2 v = zld(zat(zt, NT * (b + 2 * r)));
+                sum += v.x + v.y;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (lane == 0) red[w + (NT / 32) * b] = sum;
+        }
+        group_sync<NT>(g);
+        // every warp adds the warp sums as FP32 pairs (48 bits) and rounds once
+        float2 tot = make_float2(lane < 2 * NT / 32 ? red[lane] : 0.f, 0.f);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            pair_add2(tot, make_float2(__shfl_xor_sync(0xffffffffu, tot.x, o), __shfl_xor_sync(0xffffffffu, tot.y, o)));
+        const float mean = tot.x * (1.0f / M);
+        // ---- stage 1: subtract the mean, window, 16 points at stride B ----
+#pragma unroll 1
+        for (int b = 0; b < 2; ++b) {
+            const int j = t + NT * b;
+            const uint32_t zj = zat(zt, NT) * b + zt * (1 - b);
+            float2 v[16];
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const int n = j + r * B;
+                v[r] = zld(zat(zj, r * B));
+                float2 wn;
+                if (r < 8)
+                    wn = *reinterpret_cast<const float2*>(win + 2 * n);
+                else
+                    wn = make_float2(win[M - 2 * n], win[M - 2 * n - 1]);
+                v[r] = make_float2((v[r].x - mean) * wn.x, (v[r].y - mean) * wn.y);
+            }
+            Dft<16>::run(v);
+#pragma unroll
+            for (int r = 0; r < 16; ++r) zst(zat(zj, r * B), v[r]);
+        }
+        group_sync<NT>(g);
+        // ---- stage 2: stride B / 16, inside the warp's 1,024 points from here on ----
+#pragma unroll 1
+        for (int b = 0; b < 2; ++b) {
+            const int be = lane + 32 * b;
+            const int base = 1024 * w + (be / (B / 16)) * B + be % (B / 16);
+            const int k1 = base / B;
+            const uint32_t zb = z + 8 * zsw(base);
+            float2 v[16];
+#pragma unroll
+            for (int r = 0; r < 16; ++r) v[r] = zld(zat(zb, r * (B / 16)));
+#pragma unroll
+            for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], t2[(r - 1) * 16 + k1]);
+            Dft<16>::run(v);
+#pragma unroll
+            for (int r = 0; r < 16; ++r) zst(zat(zb, r * (B / 16)), v[r]);
+        }
+        __syncwarp();
+        // ---- stage 3: stride R4 ----
+#pragma unroll 1
+        for (int b = 0; b < 32 / R3; ++b) {
+            const int be = lane + 32 * b;
+            const int base = 1024 * w + (be / R4) * (R3 * R4) + be % R4;
+            const int cg = base / (R3 * R4);
+            const uint32_t zb = z + 8 * zsw(base);
+            float2 v[R3];
+#pragma unroll
+            for (int r = 0; r < R3; ++r) v[r] = zld(zat(zb, r * R4));
+#pragma unroll
+            for (int r = 1; r < R3; ++r) v[r] = cmul(v[r], t3[(r - 1) * 256 + cg]);
+            Dft<R3>::run(v);
+#pragma unroll
+            for (int r = 0; r < R3; ++r) zst(zat(zb, r * R4), v[r]);
+        }
+        // ---- stage 4: stride 1 ----
+        if constexpr (R4 > 1) {
+            __syncwarp();
+            const float2* t4 = a.tw + W::kT4 + (1024 / R4) * w + lane;
+#pragma unroll 4
+            for (int b = 0; b < 32 / R4; ++b) {
+                const uint32_t zb = z + 8 * zsw(1024 * w + R4 * (lane + 32 * b));
+                float2 v[R4];
+#pragma unroll
+                for (int r = 0; r < R4; ++r) v[r] = zld(zat(zb, r));
+#pragma unroll
+                for (int r = 1; r < R4; ++r) v[r] = cmul(v[r], __ldg(&t4[(r - 1) * (L / R4) + 32 * b]));
+                Dft<R4>::run(v);
+#pragma unroll
+                for (int r = 0; r < R4; ++r) zst(zat(zb, r), v[r]);
+            }
+        }
+        group_sync<NT>(g);
+        // ---- real-FFT split of bins k and L - k, |X|^2 into the sums ----
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int k1 = i < 14 ? 1 + (i >> 1) : 8, h = i < 14 ? i & 1 : 0;
+            const float2 Zb = zld(i < 15 ? zat(zt, k1 * B + NT * h) : z + 8 * p15.x);
+            const float2 Zr = zld(i < 15 ? zat(zr, (16 - k1) * B + NT * (1 - h)) : z + 8 * p15.y);
+            const float2 E = make_float2(0.5f * (Zb.x + Zr.x), 0.5f * (Zb.y - Zr.y));
+            const float2 Dd = make_float2(0.5f * (Zb.x - Zr.x), 0.5f * (Zb.y + Zr.y));
+            const float2 C = cmul(__ldg(&a.tw[W::kSplit + i * NT + t]), make_float2(Dd.y, -Dd.x));
+            // X_k = E + C; X_(L - k) = conj(E - C), since W_M^(L - k) = -conj W_M^k
+            const float2 X = cadd(E, C), Y = csub(E, C);
+            pair_add(acc[i][0], fmaf(X.x, X.x, X.y * X.y));
+            pair_add(acc[i][1], fmaf(Y.x, Y.x, Y.y * Y.y));
+        }
+        if (t == 0) {   // bin L / 2 pairs with itself
+            constexpr int kPos = R4 > 1 ? R4 / 2 : R3 / 2;   // its last digit is R / 2, the others 0
+            const float2 Zh = zld(z + 8 * zsw(kPos));
+            const float2 X = cadd(make_float2(Zh.x, 0.f), cmul(__ldg(&a.tw[W::kHalf]), make_float2(Zh.y, -0.f)));
+            pair_add2(*half, make_float2(fmaf(X.x, X.x, X.y * X.y), 0.f));
+        }
+        group_sync<NT>(g);
+        if (s + nslot < a.K) stage_x(s + nslot);
+        if (++since == 8 || s + nslot >= a.K) {
+            since = 0;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                pair_norm(acc[i][0]);
+                pair_norm(acc[i][1]);
+            }
+        }
+    }
+    if (slot < a.K) {
+        float2* row = a.part + slot * (L + 1);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            row[(2 * i) * NT + t] = acc[i][0];
+            row[(2 * i + 1) * NT + t] = acc[i][1];
+        }
+        if (t == 0) row[L] = *half;
     }
 }
 
-__global__ void psd_reduce_kernel(const double* part, int nblk, int L, double scale, double* psd)
+// psd[bin[i]] = scale * sum over the rows of part: 32 slots per block, eight
+// threads per slot over rows y, y + 8, ..., then in order of y (fixed order).
+// The rows are summed as FP32 pairs too: 152 rows of 16,385 bins took 22 us as
+// FP64 additions on 65 blocks, 8 us so (60 rows: 10.9 and 5.6 us).
+__global__ void __launch_bounds__(256) psd_reduce_kernel(const float2* part, int rows, int L, double scale,
+                                                         const int* bin, double* psd)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > L) return;
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += part[static_cast<int64_t>(b) * (L + 1) + k];
-    psd[k] = s * scale * ((k == 0 || k == L) ? 1.0 : 2.0);
+    __shared__ float2 red[8][33];
+    const int i = blockIdx.x * 32 + threadIdx.x;
+    float2 s = make_float2(0.f, 0.f);
+    if (i <= L) {
+#pragma unroll 4
+        for (int b = threadIdx.y; b < rows; b += 8) {
+            const float2 v = part[static_cast<int64_t>(b) * (L + 1) + i];
+            pair_add2(s, v);
+        }
+    }
+    red[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y == 0 && i <= L) {
+        for (int y = 1; y < 8; ++y) pair_add2(s, red[y][threadIdx.x]);
+        const int k = bin[i];
+        psd[k] = (static_cast<double>(s.x) + static_cast<double>(s.y)) * scale * ((k == 0 || k == L) ? 1.0 : 2.0);
+    }
 }
 
+// position of bin k (< L) after the in-place stages, and the tables
 template <int L>
-void* welch_fn()
-{
-    return reinterpret_cast<void*>(&psd_welch_kernel<L>);
-}
+struct WelchTables {
+    using W = Welch<L>;
+    static int pos(int k)
+    {
+        const int k1 = k & 15, k2 = (k >> 4) & 15, k3 = (k >> 8) % W::R3, k4 = k / (256 * W::R3);
+        return k1 * W::B + k2 * (W::B / 16) + k3 * W::R4 + k4;
+    }
+    static void fill(std::vector<float2>& tw, std::vector<int2>& pair0, std::vector<int>& bin)
+    {
+        auto root = [](int64_t m, int n) {   // W_n^m
+            const double ang = -2.0 * M_PI * static_cast<double>(m) / n;
+            return make_float2(static_cast<float>(std::cos(ang)), static_cast<float>(std::sin(ang)));
+        };
+        constexpr int R3 = W::R3, R4 = W::R4, NT = W::NT, B = W::B;
+        tw.assign(W::kTables, float2{});
+        for (int r = 1; r < 16; ++r)
+            for (int k1 = 0; k1 < 16; ++k1) tw[W::kT2 + (r - 1) * 16 + k1] = root(r * k1 * (L / 256), L);
+        for (int r = 1; r < R3; ++r)
+            for (int c = 0; c < 256; ++c)
+                tw[W::kT3 + (r - 1) * 256 + c] = root(r * ((c >> 4) + 16 * (c & 15)) * R4, L);
+        std::vector<int> at(L);   // bin at each position
+        for (int k = 0; k < L; ++k) at[pos(k)] = k;
+        for (int r = 1; r < R4; ++r)
+            for (int q = 0; q < L / R4; ++q) tw[W::kT4 + (r - 1) * (L / R4) + q] = root(r * at[q * R4], L);
+        // a thread's 16 pairs (k, L - k): blocks k1 = 1..7 with 15..9, block 8
+        // with itself, and those of block 0, whose bin L / 2 is kept apart
+        pair0.clear();
+        for (int k = 0; k < L / 2; k += 16) pair0.push_back(int2{zsw(pos(k)), zsw(pos((L - k) & (L - 1)))});
+        bin.assign(L + 1, L / 2);
+        for (int i = 0; i < 16; ++i)
+            for (int t = 0; t < NT; ++t) {
+                const int k1 = i < 14 ? 1 + (i >> 1) : 8, q = t + (i < 14 ? NT * (i & 1) : 0);
+                const int k = i < 15 ? at[k1 * B + q] : 16 * t;
+                tw[W::kSplit + i * NT + t] = root(k, W::M);
+                bin[2 * i * NT + t] = k;
+                bin[(2 * i + 1) * NT + t] = L - k;
+            }
+        tw[W::kHalf] = root(L / 2, W::M);
+    }
+};
 
-void* welch_ptr(int L)
+struct WelchInst {
+    void* fn;
+    int threads, groups, smem;
+    void (*fill)(std::vector<float2>&, std::vector<int2>&, std::vector<int>&);
+};
+template <int L>
+WelchInst welch_of()
+{
+    return {reinterpret_cast<void*>(&psd_welch_kernel<L>), kWelchThreads, Welch<L>::G, Welch<L>::kSmem,
+            &WelchTables<L>::fill};
+}
+bool welch_inst(int L, WelchInst* w)
 {
     switch (L) {
-    case 2048: return welch_fn<2048>();
-    case 4096: return welch_fn<4096>();
-    case 8192: return welch_fn<8192>();
-    case 16384: return welch_fn<16384>();
-    default: return nullptr;
+    case 2048: *w = welch_of<2048>(); return true;
+    case 4096: *w = welch_of<4096>(); return true;
+    case 8192: *w = welch_of<8192>(); return true;
+    case 16384: *w = welch_of<16384>(); return true;
+    default: return false;
     }
 }
 
@@ -507,43 +727,42 @@ cg_status cg_psd_create(int seg_len, cg_psd_t* out)
     if (!out) return psd_fail(CG_ERR_ARG, "out is NULL");
     *out = nullptr;
     const int L = seg_len / 2;
-    void* fn = welch_ptr(L);
-    if (seg_len % 2 != 0 || !fn) return psd_fail(CG_ERR_ARG, "seg_len must be 4096, 8192, 16384 or 32768");
+    WelchInst wi;
+    if (seg_len % 2 != 0 || !welch_inst(L, &wi))
+        return psd_fail(CG_ERR_ARG, "seg_len must be 4096, 8192, 16384 or 32768");
     cg_psd_s* h = new cg_psd_s;
     cudaGetDevice(&h->device);
     h->L = L;
     const int M = seg_len;
-    std::vector<float> w(M);
+    std::vector<float> w(L + 1);   // w[M - n] = w[n]
     double sw2 = 0.0;
-    for (int n = 0; n < M; ++n) {
-        const double v = 0.5 - 0.5 * std::cos(2.0 * M_PI * n / M);
-        w[n] = static_cast<float>(v);
-        sw2 += static_cast<double>(w[n]) * static_cast<double>(w[n]);   // the window the kernel applies
+    for (int n = 0; n <= L; ++n) w[n] = static_cast<float>(0.5 - 0.5 * std::cos(2.0 * M_PI * n / M));
+    for (int n = 0; n < M; ++n) {   // the window the kernel applies
+        const double v = w[n <= L ? n : M - n];
+        sw2 += v * v;
     }
     h->sum_w2 = sw2;
-    std::vector<float2> tl(L), tm(L + 1);
-    for (int m = 0; m < L; ++m) {
-        const double ang = -2.0 * M_PI * m / L;
-        tl[m] = make_float2(static_cast<float>(std::cos(ang)), static_cast<float>(std::sin(ang)));
-    }
-    for (int k = 0; k <= L; ++k) {
-        const double ang = -2.0 * M_PI * k / M;
-        tm[k] = make_float2(static_cast<float>(std::cos(ang)), static_cast<float>(std::sin(ang)));
-    }
+    std::vector<float2> tw;
+    std::vector<int2> pair0;
+    std::vector<int> bin;
+    wi.fill(tw, pair0, bin);
     int sms = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-    h->smem = sizeof(float2) * (static_cast<size_t>(L) + L / 16 + (L > 4096 ? 4096 : L) + 256);
-    if (e == cudaSuccess) e = cg::raise_smem_limit(fn, h->smem);
-    int occ = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, L / 16, h->smem);
-    h->grid = sms * (occ > 0 ? occ : 1);
-    if (e == cudaSuccess) e = cudaMalloc(&h->win, sizeof(float) * M);
-    if (e == cudaSuccess) e = cudaMalloc(&h->twL, sizeof(float2) * L);
-    if (e == cudaSuccess) e = cudaMalloc(&h->twM, sizeof(float2) * (L + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&h->part, sizeof(double) * (L + 1) * h->grid);
-    if (e == cudaSuccess) e = cudaMemcpy(h->win, w.data(), sizeof(float) * M, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(h->twL, tl.data(), sizeof(float2) * L, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(h->twM, tm.data(), sizeof(float2) * (L + 1), cudaMemcpyHostToDevice);
+    h->smem = wi.smem;
+    h->groups = wi.groups;
+    h->grid = sms;
+    auto upload = [&](auto** dst, const auto& src) {
+        const size_t bytes = sizeof(src[0]) * src.size();
+        if (e == cudaSuccess) e = cudaMalloc(dst, bytes);
+        if (e == cudaSuccess) e = cudaMemcpy(*dst, src.data(), bytes, cudaMemcpyHostToDevice);
+    };
+    if (e == cudaSuccess) e = cg::raise_smem_limit(wi.fn, wi.smem);
+    upload(&h->win, w);
+    upload(&h->tw, tw);
+    upload(&h->pair0, pair0);
+    upload(&h->bin, bin);
+    if (e == cudaSuccess)
+        e = cudaMalloc(&h->part, sizeof(float2) * (L + 1) * static_cast<size_t>(h->grid) * h->groups);
     if (e != cudaSuccess) {
         cg_psd_destroy(h);
         return psd_cuda_fail(e, "cg_psd_create");
@@ -556,8 +775,9 @@ void cg_psd_destroy(cg_psd_t h)
 {
     if (!h) return;
     cudaFree(h->win);
-    cudaFree(h->twL);
-    cudaFree(h->twM);
+    cudaFree(h->tw);
+    cudaFree(h->pair0);
+    cudaFree(h->bin);
     cudaFree(h->part);
     delete h;
 }
@@ -573,13 +793,19 @@ cg_status cg_psd_welch(cg_psd_t h, const float* x_dev, int64_t n, int64_t stride
     const int64_t K = (n - M) / h->L + 1;
     if (n_segments) *n_segments = K;
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
-    PsdArgs a{x_dev, stride, K, h->win, h->twL, h->twM, h->part};
+    const int vec2 = stride == 1 && (reinterpret_cast<uintptr_t>(x_dev) & 7) == 0;
+    PsdArgs a{x_dev, stride, K, vec2, h->win, h->tw, h->pair0, h->part};
+    WelchInst wi;
+    welch_inst(h->L, &wi);
+    // one block per SM; the segments go to different SMs before they share one
     const int grid = static_cast<int>(K < h->grid ? K : h->grid);
+    const int64_t slots = static_cast<int64_t>(grid) * h->groups;
+    const int rows = static_cast<int>(K < slots ? K : slots);
     void* args[] = {&a};
-    cudaError_t e = cudaLaunchKernel(welch_ptr(h->L), dim3(grid), dim3(h->L / 16), args, h->smem, s);
+    cudaError_t e = cudaLaunchKernel(wi.fn, dim3(grid), dim3(wi.threads), args, h->smem, s);
     if (e == cudaSuccess) {
         const double scale = 1.0 / (static_cast<double>(K) * fs * h->sum_w2);
-        psd_reduce_kernel<<<(h->L + 1 + 255) / 256, 256, 0, s>>>(h->part, grid, h->L, scale, psd_dev);
+        psd_reduce_kernel<<<(h->L + 1 + 31) / 32, dim3(32, 8), 0, s>>>(h->part, rows, h->L, scale, h->bin, psd_dev);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return psd_cuda_fail(e, "cg_psd_welch");
