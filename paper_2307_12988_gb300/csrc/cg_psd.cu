@@ -14,8 +14,8 @@
 // scaled by psd_reduce_kernel.
 //
 // Resonance: S(f) = A f0^4 / ((f0^2 - f^2)^2 + (f f0 / Q)^2) + B fitted to
-// ln S over the bins of a band by Levenberg-Marquardt in FP64 (one block:
-// per-point sums reduced in shared memory, the 4x4 solve on one thread);
+// ln S over the bins of a band by Levenberg-Marquardt in FP64 (one cluster of
+// eight blocks shares the per-point work, each takes the 4x4 solve);
 // initial values from the band (largest bin, smallest bin, half-height
 // width); standard errors from diag(H^-1) chi^2 / (n - 4).
 #include <cmath>
@@ -450,7 +450,11 @@ bool welch_inst(int L, WelchInst* w)
 // ---------------------------------------------------------------------------
 // resonance fit
 // ---------------------------------------------------------------------------
-constexpr int kResThreads = 256;
+constexpr int kResThreads = 256;   // threads of a block
+constexpr int kResWarps = kResThreads / 32;
+constexpr int kResBlocks = 8;      // blocks of the cluster
+constexpr int kResRow = 32 * kResBlocks;     // points of a row: 32 per block
+constexpr int kResLogRows = 64;    // rows whose ln S is kept (16,384 bins)
 
 struct ResArgs {
     const double* psd;
@@ -461,237 +465,422 @@ struct ResArgs {
     double* out;               // [12]
 };
 
-// per-point sums: 10 of J^T J (upper), 4 of J^T r, chi^2, bad-point count
-struct ResSums {
-    double v[16];
-};
-
-__device__ __forceinline__ void res_point(double f, double S, const double (&p)[4], ResSums& s)
+// 1/v and 1/sqrt(v): the hardware's FP64 seed (about 20 bits) and two Newton
+// steps, each doubling the correct bits (the second ends at FP64's rounding)
+__device__ __forceinline__ double rcp_newton(double v)
 {
-    const double f0 = p[0], Q = p[1], A = p[2], B = p[3];
-    const double u = f0 * f0 - f * f;
-    const double c = f * f0 / Q;
-    const double D = u * u + c * c;
-    const double f04 = f0 * f0 * f0 * f0;
-    const double g = f04 / D;
-    const double m = A * g + B;
-    if (!(m > 0.0) || !(m < INFINITY)) {
-        s.v[15] += 1.0;
-        return;
-    }
-    const double dD0 = 4.0 * f0 * u + 2.0 * f * f * f0 / (Q * Q);
-    const double dDQ = -2.0 * c * c / Q;
-    const double im = 1.0 / m;
-    double J[4];
-    J[0] = A * (4.0 * f0 * f0 * f0 / D - f04 * dD0 / (D * D)) * im;
-    J[1] = -A * f04 * dDQ / (D * D) * im;
-    J[2] = g * im;
-    J[3] = im;
-    const double r = log(S) - log(m);
-    int q = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = i; j < 4; ++j) s.v[q++] += J[i] * J[j];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) s.v[10 + i] += J[i] * r;
-    s.v[14] += r * r;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
+    r = fma(r, fma(-v, r, 1.0), r);
+    return fma(r, fma(-v, r, 1.0), r);
+}
+__device__ __forceinline__ double rsqrt_newton(double v)
+{
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
+    r = fma(0.5 * r, fma(-v * r, r, 1.0), r);
+    return fma(0.5 * r, fma(-v * r, r, 1.0), r);
 }
 
-// (H + lambda diag H) d = g, Jacobi-scaled Cholesky; false if not positive definite
-__device__ bool res_solve(const double* Hu, const double* g, double lambda, double* d)
+// ln m for positive finite m by table (P. T. P. Tang, ACM TOMS 16, 1990):
+// m = 2^e z, c near 1/z from the top seven bits of z, ln m = e ln 2 - ln c +
+// ln(1 + eps) with eps = z c - 1, |eps| < 2^-7.  tab[i] = (c, -ln c).
+__device__ __forceinline__ double log_table(double m, const double2* tab)
 {
-    double H[4][4];
-    int q = 0;
-    for (int i = 0; i < 4; ++i)
-        for (int j = i; j < 4; ++j) H[i][j] = H[j][i] = Hu[q++];
-    double s[4];
-    for (int i = 0; i < 4; ++i) {
-        if (!(H[i][i] > 0.0) || !(H[i][i] < INFINITY)) return false;
-        s[i] = 1.0 / sqrt(H[i][i]);
+    const int hi = __double2hiint(m);
+    if (hi < 0x00100000) return log(m);   // subnormal
+    const double2 t = tab[(hi >> 13) & 127];
+    const double z = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(m));
+    const double eps = fma(z, t.x, -1.0);
+    double q = fma(eps, -1.0 / 8.0, 1.0 / 7.0);
+    q = fma(q, eps, -1.0 / 6.0);
+    q = fma(q, eps, 1.0 / 5.0);
+    q = fma(q, eps, -1.0 / 4.0);
+    q = fma(q, eps, 1.0 / 3.0);
+    q = fma(q, eps, -1.0 / 2.0);
+    // the exponent as a double without the FP64 pipe's conversion: 2^52 + 2^31 + e minus 2^52 + 2^31
+    const double e = __hiloint2double(0x43300000, static_cast<int>(0x80000000u + ((hi >> 20) - 1023))) -
+                     __hiloint2double(0x43300000, static_cast<int>(0x80000000u));
+    return fma(e, 0.6931471805599453094, t.y) + fma(q, eps * eps, eps);
+}
+
+// the point's contribution: the four derivatives of ln m and the residual
+// (all zero, and bad set, where the model is not positive and finite)
+struct ResPoint {
+    double v[5];
+    bool bad;
+};
+
+// per-step constants of the model, taken once per step
+enum { kRf02, kRf04, kRh2, kRhq, kRA, kRB, kRif0, kRf0, kRA4, kRAq, kResConst };
+
+// m = A g + B, g = f0^4 / D, D = u^2 + f^2 h^2, u = f0^2 - f^2, h = f0 / Q:
+//   dm/df0 = 4 A g (1/f0 - f0 (u + f^2 / (2 Q^2)) / D),  dm/dQ = 2 A g f^2 h^2 / (Q D).
+// About 35 FP64 operations (two reciprocals, a logarithm): FP64 issues a warp
+// instruction in tens of cycles here, so their number is what a step costs.
+__device__ __forceinline__ ResPoint res_point(double f2, double logS, const double* q, const double2* tab)
+{
+    ResPoint o{};
+    const double u = q[kRf02] - f2;
+    const double w = f2 * q[kRh2];
+    const double iD = rcp_newton(fma(u, u, w));
+    const double g = q[kRf04] * iD;
+    const double m = fma(q[kRA], g, q[kRB]);
+    const int hi = __double2hiint(m);
+    if (!(hi >= 0 && hi < 0x7ff00000) || m == 0.0) {   // not positive and finite
+        o.bad = true;
+        return o;
     }
-    double Mx[4][4], Lc[4][4] = {};
-    for (int i = 0; i < 4; ++i)
-        for (int j = 0; j < 4; ++j) Mx[i][j] = (i == j) ? 1.0 + lambda : H[i][j] * s[i] * s[j];
+    const double im = rcp_newton(m);
+    const double s = g * im;
+    const double t = fma(f2, q[kRhq], u) * iD;
+    o.v[0] = q[kRA4] * s * fma(-q[kRf0], t, q[kRif0]);
+    o.v[1] = q[kRAq] * s * (w * iD);
+    o.v[2] = s;
+    o.v[3] = im;
+    o.v[4] = logS - log_table(m, tab);
+    return o;
+}
+
+// (H + lambda diag H) d = g by one warp, lane r = lane % 4 holding row r of H
+// and g[r]: Jacobi scaling, then Gauss-Jordan elimination down the diagonal
+// (the scaled matrix is symmetric positive definite: no pivoting), rows in
+// parallel.  d: this lane's component; false if not positive definite.
+__device__ __forceinline__ bool res_solve(const double (&H)[4], double g, double lambda, double& d)
+{
+    const int r = threadIdx.x & 3;
+    const double dg = r == 0 ? H[0] : r == 1 ? H[1] : r == 2 ? H[2] : H[3];
+    if (!__all_sync(0xffffffffu, dg > 0.0 && dg < INFINITY)) return false;
+    const double s = rsqrt_newton(dg);
+    double M[4];
+#pragma unroll
     for (int j = 0; j < 4; ++j) {
-        double v = Mx[j][j];
-        for (int k = 0; k < j; ++k) v -= Lc[j][k] * Lc[j][k];
+        const double sj = __shfl_sync(0xffffffffu, s, j);
+        M[j] = j == r ? 1.0 + lambda : H[j] * s * sj;
+    }
+    double b = g * s, mine = 0.0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const double v = __shfl_sync(0xffffffffu, M[c], c);
         if (!(v > 0.0)) return false;
-        Lc[j][j] = sqrt(v);
-        for (int i = j + 1; i < 4; ++i) {
-            double w = Mx[i][j];
-            for (int k = 0; k < j; ++k) w -= Lc[i][k] * Lc[j][k];
-            Lc[i][j] = w / Lc[j][j];
-        }
+        const double inv = rcp_newton(v);
+        const double f = r == c ? 0.0 : M[c] * inv;
+        mine = r == c ? inv : mine;
+#pragma unroll
+        for (int j = c + 1; j < 4; ++j) M[j] = fma(-f, __shfl_sync(0xffffffffu, M[j], c), M[j]);
+        b = fma(-f, __shfl_sync(0xffffffffu, b, c), b);
     }
-    double zz[4], u[4];
-    for (int i = 0; i < 4; ++i) {
-        double v = g[i] * s[i];
-        for (int k = 0; k < i; ++k) v -= Lc[i][k] * zz[k];
-        zz[i] = v / Lc[i][i];
-    }
-    for (int i = 3; i >= 0; --i) {
-        double v = zz[i];
-        for (int k = i + 1; k < 4; ++k) v -= Lc[k][i] * u[k];
-        u[i] = v / Lc[i][i];
-    }
-    for (int i = 0; i < 4; ++i) d[i] = u[i] * s[i];
+    d = b * mine * s;
     return true;
 }
 
-// diag(H^-1) by Gauss-Jordan on the 4x4 matrix; false if singular
-__device__ bool res_inv_diag(const double* Hu, double* dg)
+// diag(H^-1) by Gauss-Jordan with row pivoting on the 4x4 matrix (in
+// registers: rows are swapped by selects); false if singular
+__device__ __forceinline__ bool res_inv_diag(const double* Hu, double (&dg)[4])
 {
     double A[4][8];
     int q = 0;
+#pragma unroll
     for (int i = 0; i < 4; ++i)
+#pragma unroll
         for (int j = i; j < 4; ++j) A[i][j] = A[j][i] = Hu[q++];
+#pragma unroll
     for (int i = 0; i < 4; ++i)
+#pragma unroll
         for (int j = 0; j < 4; ++j) A[i][4 + j] = (i == j) ? 1.0 : 0.0;
+#pragma unroll
     for (int c = 0; c < 4; ++c) {
         int piv = c;
+        double best = fabs(A[c][c]);
+#pragma unroll
         for (int r = c + 1; r < 4; ++r)
-            if (fabs(A[r][c]) > fabs(A[piv][c])) piv = r;
-        if (!(fabs(A[piv][c]) > 0.0)) return false;
-        for (int j = 0; j < 8; ++j) {
-            const double tmp = A[c][j];
-            A[c][j] = A[piv][j];
-            A[piv][j] = tmp;
-        }
+            if (fabs(A[r][c]) > best) {
+                best = fabs(A[r][c]);
+                piv = r;
+            }
+        if (!(best > 0.0)) return false;
+#pragma unroll
+        for (int r = c + 1; r < 4; ++r)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const double x = A[c][j], y = A[r][j];
+                A[c][j] = piv == r ? y : x;
+                A[r][j] = piv == r ? x : y;
+            }
         const double ip = 1.0 / A[c][c];
+#pragma unroll
         for (int j = 0; j < 8; ++j) A[c][j] *= ip;
+#pragma unroll
         for (int r = 0; r < 4; ++r)
             if (r != c) {
                 const double fct = A[r][c];
+#pragma unroll
                 for (int j = 0; j < 8; ++j) A[r][j] -= fct * A[c][j];
             }
     }
+#pragma unroll
     for (int i = 0; i < 4; ++i) dg[i] = A[i][4 + i];
     return true;
 }
 
-__global__ void __launch_bounds__(kResThreads) resonance_fit_kernel(ResArgs a)
+// The fit by one cluster of eight blocks.  What bounds it is FP64 (2 lanes a
+// cycle per SM, a division or a logarithm tens of operations): on one block a
+// step of a 393-bin band took 30 us.  Row c of the band (points 256 c ..) is
+// split into 32 points per block; a block's warps evaluate its rows in
+// parallel, then each warp adds two of the 16 sums (10 of J^T J, 4 of J^T r,
+// chi^2, bad points) over the rows in order, lane by lane, and reduces the
+// lanes; every block receives all blocks' sums through distributed shared
+// memory, adds them in block order and takes the same step, so one cluster
+// barrier per step is all that the blocks exchange.  ln S is taken once.  The
+// fit of a 393-bin band: 330 us on one block, 137 on the cluster, 101 with
+// the solve in registers and two divisions per point, 71 with Newton
+// reciprocals, the table logarithm and the solve over four lanes.
+__global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads)
+    resonance_fit_kernel(ResArgs a)
 {
-    __shared__ double red[kResThreads / 32][16];
-    __shared__ ResSums tot;
+    __shared__ double red[2][kResBlocks][16];       // sums of every block, by parity of the step
+    __shared__ double tot[16];
+    __shared__ double pts[2][kResWarps][6][32];     // a round's points, double-buffered
+    __shared__ double logs[kResLogRows][32];
+    __shared__ double2 tab[128];                    // (c, -ln c) of log_table
+    __shared__ double con[kResConst];               // constants of the step
+    __shared__ double s_v[2][kResWarps];
+    __shared__ int s_i[2][kResWarps];
     __shared__ double sp[4];        // parameters at which the sums are taken
     __shared__ int s_ctl;           // 0 continue, 1 stop
-    const int t = threadIdx.x;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    unsigned rank;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     const double* S = a.psd + a.k0;
-    // sums over the band at sp -> tot (all threads take part)
-    auto sums = [&]() {
-        ResSums s;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) s.v[i] = 0.0;
-        const double p[4] = {sp[0], sp[1], sp[2], sp[3]};
-        for (int i = t; i < a.np; i += kResThreads) res_point((a.k0 + i) * a.df, S[i], p, s);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            double v = s.v[i];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if ((t & 31) == 0) red[t >> 5][i] = v;
+    const int rows = (a.np + kResRow - 1) / kResRow;
+    for (int c = warp; c < rows && c < kResLogRows; c += kResWarps) {
+        const int i = c * kResRow + static_cast<int>(rank) * 32 + lane;
+        if (i < a.np) logs[c][lane] = log(S[i]);   // read back by this thread only
+    }
+    if (t < 128) {
+        const double c = static_cast<double>(1.0f / (1.0f + (t + 0.5f) * (1.0f / 128.0f)));
+        tab[t] = make_double2(c, -log(c));
+    }
+    // the two sums of this warp: pairs (i, j) of J^T J row by row, then J^T r, r r and the bad points
+    const int q0 = 2 * warp;
+    auto pair_of = [](int q, int& i, int& j) {
+        if (q < 10) {
+            i = q < 4 ? 0 : q < 7 ? 1 : q < 9 ? 2 : 3;
+            j = q - (i == 0 ? 0 : i == 1 ? 3 : i == 2 ? 5 : 6);
+        } else {
+            i = q < 14 ? q - 10 : 4;
+            j = 4;
         }
-        __syncthreads();
+    };
+    int i0, j0, i1, j1;
+    pair_of(q0, i0, j0);
+    pair_of(q0 + 1, i1, j1);
+    int parity = 0;
+    // constants of the model at sp, by one warp: lane 0 has 1/f0, lane 1 1/Q
+    auto constants = [&]() {
+        const double inv = rcp_newton(sp[lane & 1]);
+        const double if0 = __shfl_sync(0xffffffffu, inv, 0), iQ = __shfl_sync(0xffffffffu, inv, 1);
+        const double f0 = sp[0], A = sp[2], f02 = f0 * f0, h = f0 * iQ;
+        if (lane == 0) {
+            con[kRf02] = f02;
+            con[kRf04] = f02 * f02;
+            con[kRh2] = h * h;
+            con[kRhq] = 0.5 * iQ * iQ;
+            con[kRA] = A;
+            con[kRB] = sp[3];
+            con[kRif0] = if0;
+            con[kRf0] = f0;
+            con[kRA4] = 4.0 * A;
+            con[kRAq] = 2.0 * A * iQ;
+        }
+        __syncwarp();
+    };
+    // sums over the band at sp -> tot (all threads of the cluster take part)
+    auto sums = [&]() {
+        double sa = 0.0, sb = 0.0;
+        int buf = 0;
+        for (int c0 = 0; c0 < rows; c0 += kResWarps, buf ^= 1) {
+            const int c = c0 + warp;
+            const int i = c * kResRow + static_cast<int>(rank) * 32 + lane;
+            ResPoint o{};
+            if (i < a.np) {
+                const double f = (a.k0 + i) * a.df;
+                o = res_point(f * f, c < kResLogRows ? logs[c][lane] : log(S[i]), con, tab);
+            }
+#pragma unroll
+            for (int q = 0; q < 5; ++q) pts[buf][warp][q][lane] = o.v[q];
+            pts[buf][warp][5][lane] = o.bad ? 1.0 : 0.0;
+            __syncthreads();
+            const int nr = rows - c0 < kResWarps ? rows - c0 : kResWarps;
+            for (int k = 0; k < nr; ++k) {   // (points beyond the band add zeros)
+                sa = fma(pts[buf][k][i0][lane], pts[buf][k][j0][lane], sa);
+                sb = warp == kResWarps - 1 ? sb + pts[buf][k][5][lane]
+                                           : fma(pts[buf][k][i1][lane], pts[buf][k][j1][lane], sb);
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sa += __shfl_xor_sync(0xffffffffu, sa, o);
+            sb += __shfl_xor_sync(0xffffffffu, sb, o);
+        }
+        if (lane < kResBlocks) {   // lane b hands this block's two sums to block b
+            const uint32_t own = static_cast<uint32_t>(__cvta_generic_to_shared(&red[parity][rank][q0]));
+            uint32_t there;
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(own), "r"(lane));
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there), "d"(sa) : "memory");
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there + 8), "d"(sb) : "memory");
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
         if (t < 16) {
             double v = 0.0;
-            for (int w = 0; w < kResThreads / 32; ++w) v += red[w][t];
-            tot.v[t] = v;
+            for (int w = 0; w < kResBlocks; ++w) v += red[parity][w][t];
+            tot[t] = v;
         }
+        parity ^= 1;
         __syncthreads();
     };
-    // initial values (one thread, a pass over the band)
-    if (t == 0) {
+    // initial values: the largest bin (the first of equals), the smallest
+    // value, and the ends of the run above half height around the largest
+    {
+        double vmax = S[0], vmin = S[0];
         int kp = 0;
-        double B = S[0];
-        for (int i = 1; i < a.np; ++i) {
-            if (S[i] > S[kp]) kp = i;
-            if (S[i] < B) B = S[i];
+        for (int i = t; i < a.np; i += kResThreads) {
+            const double v = S[i];
+            if (v > vmax) {
+                vmax = v;
+                kp = i;
+            }
+            if (v < vmin) vmin = v;
         }
-        const double h = S[kp] - B, half = B + 0.5 * h;
-        int lo = kp, hi = kp;
-        while (lo > 0 && S[lo - 1] > half) --lo;
-        while (hi < a.np - 1 && S[hi + 1] > half) ++hi;
-        const double fl = (lo == 0) ? (a.k0 + lo) * a.df
-                                    : (a.k0 + lo - 1) * a.df + (half - S[lo - 1]) / (S[lo] - S[lo - 1]) * a.df;
-        const double fh = (hi == a.np - 1) ? (a.k0 + hi) * a.df
-                                           : (a.k0 + hi) * a.df + (S[hi] - half) / (S[hi] - S[hi + 1]) * a.df;
-        const double width = fmax(fh - fl, a.df);
-        const double f0 = (a.k0 + kp) * a.df;
-        const double Q = f0 / width;
-        sp[0] = f0;
-        sp[1] = Q;
-        sp[2] = h / (Q * Q);
-        sp[3] = B;
-        s_ctl = 0;
+        auto merge = [&](double om, int ok, double on) {
+            if (om > vmax || (om == vmax && ok < kp)) {
+                vmax = om;
+                kp = ok;
+            }
+            if (on < vmin) vmin = on;
+        };
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double om = __shfl_xor_sync(0xffffffffu, vmax, o), on = __shfl_xor_sync(0xffffffffu, vmin, o);
+            merge(om, __shfl_xor_sync(0xffffffffu, kp, o), on);
+        }
+        if (lane == 0) {
+            s_v[0][warp] = vmax;
+            s_v[1][warp] = vmin;
+            s_i[0][warp] = kp;
+        }
+        __syncthreads();
+        for (int w = 0; w < kResWarps; ++w) merge(s_v[0][w], s_i[0][w], s_v[1][w]);
+        const double B = vmin, h = vmax - B, half = B + 0.5 * h;
+        int lo = -1, hi = a.np;   // the last bin below kp and the first above it that are not above half
+        for (int i = t; i < a.np; i += kResThreads)
+            if (!(S[i] > half)) {
+                if (i < kp) lo = i;
+                if (i > kp && i < hi) hi = i;
+            }
+        lo = __reduce_max_sync(0xffffffffu, lo);
+        hi = __reduce_min_sync(0xffffffffu, hi);
+        __syncthreads();
+        if (lane == 0) {
+            s_i[0][warp] = lo;
+            s_i[1][warp] = hi;
+        }
+        __syncthreads();
+        if (t == 0) {
+            for (int w = 1; w < kResWarps; ++w) {
+                lo = s_i[0][w] > lo ? s_i[0][w] : lo;
+                hi = s_i[1][w] < hi ? s_i[1][w] : hi;
+            }
+            ++lo;
+            --hi;
+            const double fl = (lo == 0) ? (a.k0 + lo) * a.df
+                                        : (a.k0 + lo - 1) * a.df + (half - S[lo - 1]) / (S[lo] - S[lo - 1]) * a.df;
+            const double fh = (hi == a.np - 1) ? (a.k0 + hi) * a.df
+                                               : (a.k0 + hi) * a.df + (S[hi] - half) / (S[hi] - S[hi + 1]) * a.df;
+            const double width = fmax(fh - fl, a.df);
+            const double f0 = (a.k0 + kp) * a.df;
+            const double Q = f0 / width;
+            sp[0] = f0;
+            sp[1] = Q;
+            sp[2] = h / (Q * Q);
+            sp[3] = B;
+            s_ctl = 0;
+        }
+        __syncthreads();
     }
+    if (warp == 0) constants();
     __syncthreads();
-    double p[4], chi2 = 0.0, lambda = a.lambda0, Hc[10], gc[4];
-    int it = 0, st = 1;
     sums();
-    if (t == 0) {
-        for (int i = 0; i < 4; ++i) p[i] = sp[i];
-        chi2 = (tot.v[15] > 0.0) ? INFINITY : tot.v[14];
-        for (int i = 0; i < 10; ++i) Hc[i] = tot.v[i];
-        for (int i = 0; i < 4; ++i) gc[i] = tot.v[10 + i];
-        if (!(chi2 < INFINITY)) {
-            st = 3;
-            s_ctl = 1;
-        }
+    // warp 0 of each block takes the LM decisions, lane r = lane % 4 holding
+    // parameter r, its row of H and its gradient; every block comes to the same
+    const int r = lane & 3;
+    const int h0 = r, h1 = r == 0 ? 1 : 3 + r, h2 = r == 0 ? 2 : r == 1 ? 5 : 5 + r, h3 = r == 0 ? 3 : r == 1 ? 6 : 6 + r;
+    double p = sp[r], chi2 = (tot[15] > 0.0) ? INFINITY : tot[14], lambda = a.lambda0;
+    double H[4] = {tot[h0], tot[h1], tot[h2], tot[h3]}, gr = tot[10 + r];
+    int it = 0, st = 1;
+    bool stop = false;
+    if (!(chi2 < INFINITY)) {
+        st = 3;
+        stop = true;
     }
-    __syncthreads();
     while (true) {
-        // thread 0 proposes a trial point
-        if (t == 0 && s_ctl == 0) {
-            if (it >= a.max_iter) {
-                s_ctl = 1;
-            } else {
-                ++it;
-                double d[4];
-                if (!res_solve(Hc, gc, lambda, d)) {
-                    st = 2;
-                    s_ctl = 1;
+        if (warp == 0) {
+            // the next trial point
+            if (!stop) {
+                if (it >= a.max_iter) {
+                    stop = true;
                 } else {
-                    for (int i = 0; i < 4; ++i) sp[i] = p[i] + d[i];
+                    ++it;
+                    double d;
+                    if (!res_solve(H, gr, lambda, d)) {
+                        st = 2;
+                        stop = true;
+                    } else {
+                        if (lane < 4) sp[r] = p + d;
+                        __syncwarp();
+                        constants();
+                    }
                 }
             }
+            if (lane == 0) s_ctl = stop ? 1 : 0;
         }
         __syncthreads();
         if (s_ctl) break;
         sums();
-        if (t == 0) {
-            const double c2 = (tot.v[15] > 0.0) ? INFINITY : tot.v[14];
-            if (!(c2 < INFINITY)) {
-                lambda *= 10.0;
-            } else if (fabs(c2 - chi2) <= a.tol * chi2) {
-                if (c2 <= chi2) {
-                    for (int i = 0; i < 4; ++i) p[i] = sp[i];
-                    chi2 = c2;
-                }
-                st = 0;
-                s_ctl = 1;
-            } else if (c2 < chi2) {
-                for (int i = 0; i < 4; ++i) p[i] = sp[i];
+        if (warp == 0) {
+            const double c2 = (tot[15] > 0.0) ? INFINITY : tot[14];
+            const bool settled = (c2 < INFINITY) && fabs(c2 - chi2) <= a.tol * chi2;
+            const bool better = (c2 < INFINITY) && (settled ? c2 <= chi2 : c2 < chi2);
+            if (better) {
+                p = sp[r];
                 chi2 = c2;
-                for (int i = 0; i < 10; ++i) Hc[i] = tot.v[i];
-                for (int i = 0; i < 4; ++i) gc[i] = tot.v[10 + i];
-                lambda *= 0.1;
+                H[0] = tot[h0];
+                H[1] = tot[h1];
+                H[2] = tot[h2];
+                H[3] = tot[h3];
+                gr = tot[10 + r];
+            }
+            if (settled) {
+                st = 0;
+                stop = true;
             } else {
-                lambda *= 10.0;
+                lambda *= better ? 0.1 : 10.0;
             }
         }
-        __syncthreads();
     }
     // standard errors from the sums at the result
-    if (t == 0)
-        for (int i = 0; i < 4; ++i) sp[i] = p[i];
+    if (warp == 0) {
+        if (lane < 4) sp[r] = p;
+        __syncwarp();
+        constants();
+    }
     __syncthreads();
     sums();
-    if (t == 0) {
+    if (t == 0 && rank == 0) {
         double dg[4] = {NAN, NAN, NAN, NAN};
-        const bool inv = a.np > 4 && res_inv_diag(tot.v, dg);
+        const bool inv = a.np > 4 && res_inv_diag(tot, dg);
         for (int i = 0; i < 4; ++i) {
-            a.out[i] = p[i];
+            a.out[i] = sp[i];
             a.out[4 + i] = inv ? sqrt(dg[i] * chi2 / (a.np - 4)) : NAN;
         }
         a.out[8] = chi2;
@@ -825,7 +1014,8 @@ cg_status cg_resonance_fit(const double* psd_dev, int n_bins, double df, double 
     if (k1 - k0 + 1 < 8) return psd_fail(CG_ERR_ARG, "the band holds fewer than 8 bins");
     ResArgs a{psd_dev, k0, k1 - k0 + 1, df, max_iter, tol, 1e-3, out_dev};
     void* args[] = {&a};
-    cudaError_t e = cudaLaunchKernel(reinterpret_cast<void*>(&resonance_fit_kernel), dim3(1), dim3(kResThreads),
+    cudaError_t e = cudaLaunchKernel(reinterpret_cast<void*>(&resonance_fit_kernel), dim3(kResBlocks),
+                                     dim3(kResThreads),
                                      args, 0, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return psd_cuda_fail(e, "cg_resonance_fit");
     return CG_OK;
