@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(128) init_kernel(InitArgs a)
         }
     };
     uint32_t phase = 0u, pending = 0u;   // bit b: buffer b's parity / a copy in flight
-    int64_t task = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + warp;
+    int64_t task = static_cast<int64_t>(warp) * gridDim.x + blockIdx.x;   // (few tasks spread over the SMs)
     if (task * 32 < n && bulk_ok(task)) {
         issue(task, 0);
         pending |= 1u;
@@ -890,8 +890,7 @@ cudaError_t launch_init(const cg_plan_s* p, const float* y, const float* amps, i
     a.bulk = (p->T & 1) ? 1 : 0;
     a.err = p->d.err;
     const int64_t tasks = (n + 31) / 32;
-    const int64_t blocks = (tasks + 3) / 4;
-    const int grid = static_cast<int>(blocks < p->grid_init ? blocks : p->grid_init);
+    const int grid = static_cast<int>(tasks < p->grid_init ? tasks : p->grid_init);
     void* args[] = {&a};
     return cudaLaunchKernel(init_ptr(p->init_npad, p->n_outer), dim3(grid), dim3(128), args, p->init_smem, s);
 }

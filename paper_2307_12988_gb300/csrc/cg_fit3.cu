@@ -40,6 +40,7 @@
 // centre column being -2 A jc' / g; 9 sums (jc' jc', jc' F, jc', F F, F,
 // jc' r, F r, r, r r).  Its starting centre is the given one (the median
 // filter's) or the lowest tooth of the frame (first on ties) moved by q g.
+#include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -128,10 +129,8 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
         }
         tab[i] = make_float4(v[0], v[1], v[2], v[3]);
     }
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < nwarps * S::kSlots; ++i) tc::mbar_init(&bars_all[i], 1);
-        tc::fence_mbar_init();
-    }
+    for (int i = lane; i < S::kSlots; i += 32) tc::mbar_init(&bars[i], 1);
+    tc::fence_mbar_init();
     __syncthreads();
 
     // the last pair of a lane may hold teeth beyond T: their terms are zeroed
@@ -149,7 +148,11 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
         const int64_t c = *a.list_n;
         n = c < n ? c : n;
     }
-    int64_t next = 0, end = 0;   // the warp's current task [next, end)
+    // the warp's current task [next, end): its first one by its place (warp w
+    // of block b takes task b + w gridDim.x, so few tasks spread over the SMs),
+    // the others from the counter
+    bool first = true;
+    int64_t next = 0, end = 0;
     int64_t f = -1, fr = -1;     // task index and row of the frame being fit
     int64_t fn = -1, frn = -1;   // the group's next frame (its copy in flight)
     float pn[4] = {0.f, 1.f, 0.f, 0.f};   // its starting point, loaded when claimed
@@ -237,9 +240,15 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
         unsigned need = __ballot_sync(kFull, gl == 0 && fn < 0);
         while (need != 0 && next < n) {
             if (next >= end) {
-                unsigned long long t = 0;
-                if (lane == 0) t = atomicAdd(a.counter, 1ULL);
-                t = __shfl_sync(kFull, t, 0);
+                unsigned long long t = static_cast<unsigned>(warp) * gridDim.x + blockIdx.x;
+                if (!first) {
+                    t = static_cast<unsigned>(nwarps) * gridDim.x;
+                    if (t * a.task < static_cast<unsigned long long>(n)) {   // (else no task is left to claim)
+                        if (lane == 0) t += atomicAdd(a.counter, 1ULL);
+                        t = __shfl_sync(kFull, t, 0);
+                    }
+                }
+                first = false;
                 next = static_cast<int64_t>(t) * a.task;
                 if (next >= n) {
                     next = end = n;
@@ -656,13 +665,21 @@ cudaError_t launch_fit3(const cg_plan_s* p, Fit2Args a, cudaStream_t s)
 {
     const Fit3Inst* fi = fit3_find(p->T, p->opts.model, p->solve_f64 ? 1 : 0);
     if (!fi || !p->fit3_ok) return cudaErrorInvalidValue;
+    // frames per task: two per lane group; with few frames as few as give each
+    // warp scheduler (four per SM) a task of its own, since a warp's time is
+    // its longest frame's and does not depend on how many groups are busy
+    // (200 frames of 99 teeth: 28 us on one block of 32-frame tasks, 11 us so;
+    // 9,973 of 21 teeth: 22 and 10 us)
     const int gpw = 32 / fi->G;   // groups per warp
-    a.task = 2 * gpw;
+    const int64_t schedulers = 4 * static_cast<int64_t>(p->num_sms);
+    a.task = static_cast<int>(std::min<int64_t>(2 * gpw, (a.n + schedulers - 1) / schedulers));
     const int64_t tasks = (a.n + a.task - 1) / a.task;
-    const int64_t blocks = (tasks + p->fit3_warps - 1) / p->fit3_warps;
-    const int grid = static_cast<int>(blocks < p->grid_fit3 ? blocks : p->grid_fit3);
-    cudaError_t e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
+    const int grid = static_cast<int>(tasks < p->grid_fit3 ? tasks : p->grid_fit3);
+    // tasks beyond one per warp are claimed from the counter
+    if (tasks > static_cast<int64_t>(grid) * p->fit3_warps) {
+        cudaError_t e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s);
+        if (e != cudaSuccess) return e;
+    }
     void* args[] = {&a};
     return cudaLaunchKernel(fi->fn(), dim3(grid), dim3(32 * p->fit3_warps), args, p->fit3_smem, s);
 }
