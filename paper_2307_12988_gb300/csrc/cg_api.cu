@@ -136,7 +136,7 @@ void free_plan(cg_plan_s* p)
     free_tables(p->d);
     if (p->s_read) cudaStreamDestroy(p->s_read);
     if (p->s_fit) cudaStreamDestroy(p->s_fit);
-    for (cudaEvent_t e : {p->ev_fork, p->ev_read, p->ev_join_r, p->ev_join_f})
+    for (cudaEvent_t e : {p->ev_fork, p->ev_read, p->ev_join_r, p->ev_join_f, p->ev_fit})
         if (e) cudaEventDestroy(e);
     for (const auto& t : p->timed) {
         cudaEventDestroy(t.a);
@@ -299,7 +299,7 @@ cudaError_t setup_fit_kernels(cg_plan_s* p)
     p->ppl_exact = exact;
     if ((e = cudaStreamCreateWithFlags(&p->s_read, cudaStreamNonBlocking)) != cudaSuccess) return e;
     if ((e = cudaStreamCreateWithFlags(&p->s_fit, cudaStreamNonBlocking)) != cudaSuccess) return e;
-    for (cudaEvent_t* ev : {&p->ev_fork, &p->ev_read, &p->ev_join_r, &p->ev_join_f})
+    for (cudaEvent_t* ev : {&p->ev_fork, &p->ev_read, &p->ev_join_r, &p->ev_join_f, &p->ev_fit})
         if ((e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess) return e;
     p->G2 = G;
     p->PPL = ppl;
@@ -358,6 +358,35 @@ cudaError_t timed(cg_plan_s* p, int stage, cudaStream_t s, F&& launch)
     p->timed.push_back({stage, ev[0], ev[1]});
     return e;
 }
+
+// The fits of a plan's calls share its task counter and fallback list, so they
+// run one after another whatever streams the calls are on: begin() makes the
+// stream wait for the fit of a call on another stream, end() marks this one's
+// end.  (Captured calls are ordered by their graph alone.)
+struct FitOrder {
+    cg_plan_s* p;
+    cudaStream_t s;
+    unsigned long long id = 0;
+    bool captured = false;
+    cudaError_t begin()
+    {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        cudaError_t e = cudaStreamIsCapturing(s, &st);
+        if (e != cudaSuccess) return e;
+        captured = st != cudaStreamCaptureStatusNone;
+        if (captured) return cudaSuccess;
+        if ((e = cudaStreamGetId(s, &id)) != cudaSuccess) return e;
+        return p->fit_recorded && p->fit_stream_id != id ? cudaStreamWaitEvent(s, p->ev_fit, 0) : cudaSuccess;
+    }
+    cudaError_t end()
+    {
+        if (captured) return cudaSuccess;
+        const cudaError_t e = cudaEventRecord(p->ev_fit, s);
+        p->fit_recorded = p->fit_recorded || e == cudaSuccess;
+        p->fit_stream_id = id;
+        return e;
+    }
+};
 
 }  // namespace
 
@@ -791,14 +820,24 @@ static cg_status process_impl(cg_plan_t p, const void* frames, int sbytes, int64
                 return cuda_fail(e, "fallback count");
             p->d.fb_cap = cmax;
         }
-        // fork onto the plan's two streams; chunk c is read out (and its
-        // initial guess made) on s_read while chunk c-1 is fitted on s_fit; the
-        // guess goes to params and its flag to status, where the fit reads them
-        e = cudaEventRecord(p->ev_fork, s);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(p->s_read, p->ev_fork, 0);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(p->s_fit, p->ev_fork, 0);
         // the median filter runs over the call's whole time x tooth image
         const int64_t chunk = median ? n : p->chunk;
+        // One chunk: the kernels follow one another on the caller's stream
+        // (forking onto two streams and joining them again cost cross-stream
+        // waits on the GPU and nine calls on the host, 8 to 12 us a call).
+        // Several: fork onto the plan's two streams; chunk c
+        // is read out (and its initial guess made) on s_read while chunk c-1
+        // is fitted on s_fit.  The guess goes to params and its flag to
+        // status, where the fit reads them.
+        const bool fork = n > chunk;
+        const cudaStream_t sr = fork ? p->s_read : s, sf = fork ? p->s_fit : s;
+        e = cudaSuccess;
+        if (fork) {
+            e = cudaEventRecord(p->ev_fork, s);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(sr, p->ev_fork, 0);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(sf, p->ev_fork, 0);
+        }
+        FitOrder order{p, sf};
         for (int64_t c0 = 0; c0 < n && e == cudaSuccess; c0 += chunk) {
             const int64_t m = (n - c0) < chunk ? (n - c0) : chunk;
             const int64_t T = p->T;
@@ -810,25 +849,28 @@ static cg_status process_impl(cg_plan_t p, const void* frames, int sbytes, int64
             float* rc = rss ? rss + c0 : nullptr;
             int16_t* ic = iters ? iters + c0 : nullptr;
             int16_t* sc = status ? status + c0 : nullptr;
-            e = timed(p, CG_STAGE_READOUT, p->s_read, [&] {
+            e = timed(p, CG_STAGE_READOUT, sr, [&] {
                 if (sbytes == 1)
-                    return cg::launch_fast_readout_i8(p, reinterpret_cast<const int8_t*>(fb), m, ac, yc, p->s_read);
-                return gemm   ? cg::launch_gemm_readout(p, fc, m, ac, yc, p->s_read)
-                       : fold ? cg::launch_fold_readout(p, fc, m, ac, yc, p->s_read)
-                       : fast ? cg::launch_fast_readout(p, fc, m, ac, yc, p->s_read)
-                       : pow2 ? cg::launch_pow2_readout(p, fc, m, ac, yc, p->s_read)
-                              : cg::launch_readout(p, fc, m, ac, yc, p->s_read);
+                    return cg::launch_fast_readout_i8(p, reinterpret_cast<const int8_t*>(fb), m, ac, yc, sr);
+                return gemm   ? cg::launch_gemm_readout(p, fc, m, ac, yc, sr)
+                       : fold ? cg::launch_fold_readout(p, fc, m, ac, yc, sr)
+                       : fast ? cg::launch_fast_readout(p, fc, m, ac, yc, sr)
+                       : pow2 ? cg::launch_pow2_readout(p, fc, m, ac, yc, sr)
+                              : cg::launch_readout(p, fc, m, ac, yc, sr);
             });
             if (e == cudaSuccess && mlp)
-                e = timed(p, CG_STAGE_MLP, p->s_read, [&] { return cg::launch_mlp(p, yc, ac, m, pc, sc, p->s_read); });
+                e = timed(p, CG_STAGE_MLP, sr, [&] { return cg::launch_mlp(p, yc, ac, m, pc, sc, sr); });
             else if (e == cudaSuccess && !fano)
-                e = timed(p, CG_STAGE_INIT, p->s_read,
-                          [&] { return cg::launch_init(p, yc, ac, m, pc, sc, p->s_read, nullptr, nullptr); });
+                e = timed(p, CG_STAGE_INIT, sr,
+                          [&] { return cg::launch_init(p, yc, ac, m, pc, sc, sr, nullptr, nullptr); });
             if (e == cudaSuccess && median)   // the centre of the guess from the filtered image
-                e = timed(p, CG_STAGE_MEDIAN, p->s_read,
-                          [&] { return cg::launch_median(p, yc, ac, m, pc, p->s_read); });
-            if (e == cudaSuccess) e = cudaEventRecord(p->ev_read, p->s_read);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(p->s_fit, p->ev_read, 0);
+                e = timed(p, CG_STAGE_MEDIAN, sr,
+                          [&] { return cg::launch_median(p, yc, ac, m, pc, sr); });
+            if (fork) {
+                if (e == cudaSuccess) e = cudaEventRecord(p->ev_read, sr);
+                if (e == cudaSuccess) e = cudaStreamWaitEvent(sf, p->ev_read, 0);
+            }
+            if (e == cudaSuccess && c0 == 0) e = order.begin();
             if (e == cudaSuccess && mlp) {
                 // polish steps from the learned guess; frames that do not
                 // converge are listed and refit by the full LM from the moment
@@ -837,14 +879,14 @@ static cg_status process_impl(cg_plan_t p, const void* frames, int sbytes, int64
                 pol.max_iter = p->opts.polish_iter < p->opts.max_iter ? p->opts.polish_iter : p->opts.max_iter;
                 pol.fb_list = p->d.fb_list;
                 pol.fb_count = p->d.fb_count;
-                e = cudaMemsetAsync(p->d.fb_count, 0, sizeof(int), p->s_fit);
+                e = cudaMemsetAsync(p->d.fb_count, 0, sizeof(int), sf);
                 if (e == cudaSuccess)
-                    e = timed(p, CG_STAGE_FIT, p->s_fit, [&] {
-                        return cg::launch_fit2(p, yc, ac, m, pc, sc, pc, rc, ic, sc, p->s_fit, pol);
+                    e = timed(p, CG_STAGE_FIT, sf, [&] {
+                        return cg::launch_fit2(p, yc, ac, m, pc, sc, pc, rc, ic, sc, sf, pol);
                     });
                 if (e == cudaSuccess)
-                    e = timed(p, CG_STAGE_FALLBACK, p->s_fit, [&] {
-                        return cg::launch_init(p, yc, ac, m, pc, sc, p->s_fit, p->d.fb_list, p->d.fb_count);
+                    e = timed(p, CG_STAGE_FALLBACK, sf, [&] {
+                        return cg::launch_init(p, yc, ac, m, pc, sc, sf, p->d.fb_list, p->d.fb_count);
                     });
                 cg::FitLaunch fb;
                 fb.list = p->d.fb_list;
@@ -852,21 +894,24 @@ static cg_status process_impl(cg_plan_t p, const void* frames, int sbytes, int64
                 fb.iters_base = pol.max_iter;
                 fb.status_or = CG_FIT_FALLBACK;
                 if (e == cudaSuccess)
-                    e = timed(p, CG_STAGE_FALLBACK, p->s_fit, [&] {
-                        return cg::launch_fit2(p, yc, ac, m, pc, sc, pc, rc, ic, sc, p->s_fit, fb);
+                    e = timed(p, CG_STAGE_FALLBACK, sf, [&] {
+                        return cg::launch_fit2(p, yc, ac, m, pc, sc, pc, rc, ic, sc, sf, fb);
                     });
             } else if (e == cudaSuccess) {
                 // the Fano fit reads a given centre only from the median filter
                 const float* p0 = (fano && !median) ? nullptr : pc;
                 const int16_t* fl = fano ? nullptr : sc;
-                e = timed(p, CG_STAGE_FIT, p->s_fit,
-                          [&] { return cg::launch_fit2(p, yc, ac, m, p0, fl, pc, rc, ic, sc, p->s_fit); });
+                e = timed(p, CG_STAGE_FIT, sf,
+                          [&] { return cg::launch_fit2(p, yc, ac, m, p0, fl, pc, rc, ic, sc, sf); });
             }
         }
-        if (e == cudaSuccess) e = cudaEventRecord(p->ev_join_r, p->s_read);
-        if (e == cudaSuccess) e = cudaEventRecord(p->ev_join_f, p->s_fit);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->ev_join_r, 0);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->ev_join_f, 0);
+        if (e == cudaSuccess) e = order.end();
+        if (fork) {
+            if (e == cudaSuccess) e = cudaEventRecord(p->ev_join_r, sr);
+            if (e == cudaSuccess) e = cudaEventRecord(p->ev_join_f, sf);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->ev_join_r, 0);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->ev_join_f, 0);
+        }
     } else if (path == CG_PATH_FUSED) {
         e = timed(p, CG_STAGE_FUSED, s,
                   [&] { return cg::launch_fused(p, frames16, n, amps, y, params, rss, iters, status, s); });
@@ -941,6 +986,10 @@ cg_status cg_fit(cg_plan_t p, const float* y, int64_t n, const float* p0, float*
     cudaError_t e = cudaSuccess;
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     const bool fano = p->opts.model == CG_MODEL_FANO;
+    FitOrder order{p, s};
+    const bool ordered = (p->opts.init == CG_INIT_MEDIAN && !p0) || fano;
+    if (ordered) e = order.begin();
+    if (e != cudaSuccess) return cuda_fail(e, "cg_fit launch");
     if (p->opts.init == CG_INIT_MEDIAN && !p0) {
         // guess in params (Lorentzian: moments, then the filtered centre), then the fit from it
         if (!fano) e = cg::launch_init(p, y, nullptr, n, params, status, s, nullptr, nullptr);
@@ -952,6 +1001,7 @@ cg_status cg_fit(cg_plan_t p, const float* y, int64_t n, const float* p0, float*
     } else {
         e = cg::launch_fit(p, y, nullptr, n, p0, params, rss, iters, status, s);
     }
+    if (e == cudaSuccess && ordered) e = order.end();
     if (e != cudaSuccess) return cuda_fail(e, "cg_fit launch");
     return CG_OK;
 }

@@ -277,6 +277,11 @@ struct cg_plan_s {
     cg::FastArgs fa{};
     cudaStream_t s_read = nullptr, s_fit = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_read = nullptr, ev_join_r = nullptr, ev_join_f = nullptr;
+    // end of the last call's fit and the stream (its unique id) it ran on: the
+    // fits of a plan share its task counter and fallback list
+    cudaEvent_t ev_fit = nullptr;
+    unsigned long long fit_stream_id = 0;
+    bool fit_recorded = false;
     // learned initial guess
     bool mlp_ok = false;
     CUtensorMap mlp_map{};
