@@ -111,6 +111,8 @@ void free_tables(cg::DevTables& d)
     cudaFree(d.tw_M);
     cudaFree(d.tw_n1);
     cudaFree(d.tw_b);
+    cudaFree(d.gen_tw);
+    cudaFree(d.gen_pos);
     cudaFree(d.zidx);
     cudaFree(d.inv_ref);
     cudaFree(d.u);
@@ -637,6 +639,11 @@ cg_status cg_plan(cg_plan_t* out, double fs, int N, int T, const double* tooth_f
         delete p;
         return cuda_fail(e, "kernel configuration");
     }
+    if ((e = cg::setup_general(p, zidx)) != cudaSuccess) {
+        free_tables(p->d);
+        delete p;
+        return cuda_fail(e, "general readout set-up");
+    }
     p->d.ref_part_rows = p->grid_readout;
     if ((e = cudaMalloc(&p->d.ref_part, sizeof(double) * static_cast<size_t>(p->d.ref_part_rows) * T)) != cudaSuccess ||
         (e = cudaMalloc(&p->d.ref_out, sizeof(double) * T)) != cudaSuccess) {
@@ -856,7 +863,7 @@ static cg_status process_impl(cg_plan_t p, const void* frames, int sbytes, int64
                        : fold ? cg::launch_fold_readout(p, fc, m, ac, yc, sr)
                        : fast ? cg::launch_fast_readout(p, fc, m, ac, yc, sr)
                        : pow2 ? cg::launch_pow2_readout(p, fc, m, ac, yc, sr)
-                              : cg::launch_readout(p, fc, m, ac, yc, sr);
+                              : cg::launch_general_readout(p, fc, m, ac, yc, sr);
             });
             if (e == cudaSuccess && mlp)
                 e = timed(p, CG_STAGE_MLP, sr, [&] { return cg::launch_mlp(p, yc, ac, m, pc, sc, sr); });
@@ -916,7 +923,7 @@ static cg_status process_impl(cg_plan_t p, const void* frames, int sbytes, int64
         e = timed(p, CG_STAGE_FUSED, s,
                   [&] { return cg::launch_fused(p, frames16, n, amps, y, params, rss, iters, status, s); });
     } else {
-        e = timed(p, CG_STAGE_READOUT, s, [&] { return cg::launch_readout(p, frames16, n, amps, y, s); });
+        e = timed(p, CG_STAGE_READOUT, s, [&] { return cg::launch_general_readout(p, frames16, n, amps, y, s); });
         // without y_dev the fit reads the magnitudes and applies the reference itself
         if (e == cudaSuccess)
             e = timed(p, CG_STAGE_FIT, s,
@@ -971,7 +978,7 @@ cg_status cg_readout(cg_plan_t p, const int16_t* frames, int64_t n, float* amps,
     else if (p->pow2_ok && (p->opts.path == CG_PATH_AUTO || p->opts.path == CG_PATH_PIPELINE) && aligned4)
         e = cg::launch_pow2_readout(p, frames, n, amps, y, s);
     else
-        e = cg::launch_readout(p, frames, n, amps, y, s);
+        e = cg::launch_general_readout(p, frames, n, amps, y, s);
     if (e != cudaSuccess) return cuda_fail(e, "cg_readout launch");
     return CG_OK;
 }

@@ -43,6 +43,37 @@ struct ReadoutArgs {
     int sm_raw, sm_a, sm_b, sm_y, sm_acc, sm_total;
 };
 
+// One pass of the general readout: radices ra and rb (1: ra alone) over
+// blocks of s * ra * rb points.
+struct GenPass {
+    int ra, rb;
+    int per;                 // butterflies per frame, L / (ra rb)
+    int s;                   // points between rb's inputs (innermost stride)
+    int ns;                  // product of the earlier radices (= blocks)
+    int off_a, off_b;        // their twiddles
+    uint32_t magic_per, magic_s;   // for dividing by per and by s
+};
+
+// Arguments of the general readout (cg_general.cu).
+struct GenArgs {
+    const int16_t* frames;
+    int64_t n_frames;
+    int N, T, L, M, kind, F;
+    int pad, zstride;        // one pad per 16 points; points per frame in shared memory
+    int npass;
+    GenPass pass[kMaxStages];
+    uint32_t magic_l, magic_t;
+    const float2* tw;        // [L] twiddles of the passes
+    const float2* tw_n1;     // [L] W_N^(r n1)   (coset)
+    const float2* tw_M;      // [M] W_M^(r n2)   (coset)
+    const float2* tw_b;      // [T] W_N^(b_k)    (full)
+    const int2* pos;         // [T] places of Z_b and Z_(L - b)
+    const float* inv_ref;    // [T]
+    float* amps;             // [n][T] or null
+    float* y;                // [n][T] or null
+    int sm_n1, sm_b, sm_pos, sm_iref, sm_raw, sm_z, sm_total;
+};
+
 // Arguments of the fast readout (comb geometries, N = 10 P Q).
 struct FastArgs {
     const void* frames;      // int16 or int8 samples (the kernel's instantiation)
@@ -203,6 +234,8 @@ struct DevTables {
     float2* tw_M = nullptr;
     float2* tw_n1 = nullptr;
     float2* tw_b = nullptr;
+    float2* gen_tw = nullptr;     // general readout: twiddles by pass, tooth positions
+    int2* gen_pos = nullptr;
     int* zidx = nullptr;
     float* inv_ref = nullptr;
     float* u = nullptr;
@@ -240,6 +273,8 @@ struct cg_plan_s {
     cg::DevTables d;
     int grid_readout = 0, grid_fused = 0, grid_fit = 0;
     cg::ReadoutArgs ra{};
+    cg::GenArgs ga_gen{};    // general readout
+    int grid_general = 0;
     // throughput path (fast readout + register-resident LM over chunks)
     bool fit_ok = false;     // init + fit kernels of the throughput path configured
     bool fast_ok = false;    // geometry admits the fast readout
@@ -303,8 +338,10 @@ namespace cg {
 
 // launchers (cg_kernels.cu)
 cudaError_t configure_kernels(cg_plan_s* p);
-cudaError_t launch_readout(const cg_plan_s* p, const int16_t* frames, int64_t n, float* amps,
-                           float* y, cudaStream_t s);
+// general readout (cg_general.cu)
+cudaError_t setup_general(cg_plan_s* p, const std::vector<int>& zidx);
+cudaError_t launch_general_readout(const cg_plan_s* p, const int16_t* frames, int64_t n, float* amps,
+                                   float* y, cudaStream_t s);
 cudaError_t launch_fused(const cg_plan_s* p, const int16_t* frames, int64_t n, float* amps,
                          float* y, float* params, float* rss, int16_t* iters, int16_t* status,
                          cudaStream_t s);

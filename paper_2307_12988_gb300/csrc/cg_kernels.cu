@@ -146,7 +146,7 @@ __device__ __forceinline__ float tooth_amp(const ReadoutArgs& a, const unsigned 
 }
 
 // ---------------------------------------------------------------------------
-// readout kernel: MODE 0 = amps/y to global, MODE 1 = fused LM fit,
+// readout kernel: MODE 1 = amps/y to global and fused LM fit,
 // MODE 2 = reference accumulation (per-block FP64 partial sums)
 // ---------------------------------------------------------------------------
 template <int MODE, int G>
@@ -269,10 +269,6 @@ static void* readout_fn() { return reinterpret_cast<void*>(&readout_kernel<MODE,
 static void* readout_ptr(int mode, int G)
 {
     switch (mode * 100 + G) {
-    case 4: return readout_fn<0, 4>();
-    case 8: return readout_fn<0, 8>();
-    case 16: return readout_fn<0, 16>();
-    case 32: return readout_fn<0, 32>();
     case 104: return readout_fn<1, 4>();
     case 108: return readout_fn<1, 8>();
     case 116: return readout_fn<1, 16>();
@@ -309,14 +305,14 @@ cudaError_t configure_kernels(cg_plan_s* p)
 {
     cudaError_t e;
     const int G = p->G;
-    for (int mode = 0; mode < 3; ++mode) {
+    for (int mode = 1; mode < 3; ++mode) {
         void* fn = readout_ptr(mode, G);
         if (!fn) return cudaErrorInvalidValue;
         e = raise_smem_limit(fn, p->ra.sm_total);
         if (e != cudaSuccess) return e;
     }
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, readout_ptr(0, G), kThreads, p->ra.sm_total);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, readout_ptr(2, G), kThreads, p->ra.sm_total);
     if (e != cudaSuccess) return e;
     p->grid_readout = p->num_sms * (occ > 0 ? occ : 1);
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, readout_ptr(1, G), kThreads, p->ra.sm_total);
@@ -336,20 +332,6 @@ static int grid_for(int64_t n_frames, int F, int cap)
 {
     const int64_t nb = (n_frames + F - 1) / F;
     return static_cast<int>(nb < cap ? nb : cap);
-}
-
-cudaError_t launch_readout(const cg_plan_s* p, const int16_t* frames, int64_t n, float* amps,
-                           float* y, cudaStream_t s)
-{
-    ReadoutArgs a = p->ra;
-    a.frames = frames;
-    a.n_frames = n;
-    a.amps = amps;
-    a.y = y;
-    FitArgs fa = make_fit_args(p);
-    const int grid = grid_for(n, a.F, p->grid_readout);
-    void* args[] = {&a, &fa};
-    return cudaLaunchKernel(readout_ptr(0, p->G), dim3(grid), dim3(kThreads), args, a.sm_total, s);
 }
 
 cudaError_t launch_fused(const cg_plan_s* p, const int16_t* frames, int64_t n, float* amps,
