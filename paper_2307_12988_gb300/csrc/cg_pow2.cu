@@ -9,169 +9,169 @@
 //   pass 1  n = n1 + (L/16) n2:  DFT16 over n2 -> k2, twiddle W_L^{n1 k2};
 //   pass 2  n1 = m1 + R3 m2:     DFT16 over m2 -> j,  twiddle W_{L/16}^{m1 j};
 //   pass 3                        DFT_R3 over m1 -> j',
-// so that Z[k2 + 16 j + 256 j'] = sum_n z_n W_L^{n k}.  Between passes the
-// values go through a padded shared buffer (row stride 17 R3 complex values,
-// conflict-free for every access pattern above); the last pass writes Z at
-// position k + k / 16.  The real-FFT split X_b = E + W_N^b O is evaluated only
-// at the teeth.  Samples of the next batch stream in with cp.async while the
-// current batch is transformed.
+// so that Z[k2 + 16 j + 256 j'] = sum_n z_n W_L^{n k}.  The passes work in
+// place: a thread writes its results where it read its points, so after pass 1
+// the points of a warp's butterflies are its own (k2 blocks of L / 16) and
+// passes 2 and 3 need no barrier but the warp's.  The real-FFT split
+// X_b = E + W_N^b O is evaluated only at the teeth.  The samples go straight
+// from global memory to the registers of pass 1, one frame ahead.
+//
+// What bounds it: the shared-memory pipe (68 % busy: 870 wavefronts of 128
+// bytes a 4,096-sample frame) and instruction issue (55 %).  So the twiddles
+// of pass 1, which a thread needs unchanged in every frame, live in its
+// registers, and so do the next frame's samples: 128 registers, 512 threads an
+// SM.  30,000 frames of 4,096 samples, 201 teeth: 163 us with samples staged
+// and three barriered exchanges through shared memory, 150 in place at 768
+// threads with the twiddles in shared memory, 123 so.
 #include <cstdint>
 #include <cuda_runtime.h>
 
 #include "cg_fft.cuh"
 #include "cg_internal.h"
-#include "cg_stage.cuh"
 
 namespace cg {
 
 namespace {
 
-constexpr int kPow2Threads = 256;
-
 template <int L>
 struct Pow2Plan {
     static constexpr int TPF = L / 16;             // threads per frame
-    static constexpr int FPB = kPow2Threads / TPF;  // frames per block pass
+    static constexpr int NTH = TPF > 128 ? TPF : 128;   // threads per block
+    static constexpr int FPB = NTH / TPF;          // frames in flight per block
     static constexpr int R3 = L / 256;
-    static constexpr int RS = 17 * R3;             // exchange row stride (complex values)
-    static constexpr int BUF = 16 * RS;            // = L + L / 16
-    static constexpr int PP = 256 / TPF;           // pass-3 (k2, j) pairs per thread
+    static constexpr int PP = 16 / R3;             // pass-3 butterflies per thread
     static constexpr int N = 2 * L;
 };
 
-__device__ __forceinline__ int zpos(int k) { return k + (k >> 4); }
+// Place of point p: its low four bits XORed with the next four, which puts the
+// points of every access of a half warp on distinct banks (strides 1, R3 and
+// L / 16).  Linear over XOR: p ^ d with d disjoint from p is reached from the
+// address of p by a constant XOR and a constant offset.
+__host__ __device__ constexpr int zsw(int p) { return p ^ ((p >> 4) & 15); }
+__device__ __forceinline__ uint32_t zat(uint32_t a, int d)
+{
+    return (a ^ static_cast<uint32_t>((zsw(d) & 15) << 3)) + static_cast<uint32_t>((d & ~15) << 3);
+}
+__device__ __forceinline__ float2 zld(uint32_t a)
+{
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void zst(uint32_t a, float2 v)
+{
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};\n" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
 
 template <int L>
-__global__ void __launch_bounds__(kPow2Threads) pow2_readout_kernel(ReadoutArgs a)
+__global__ void __launch_bounds__(Pow2Plan<L>::NTH, 512 / Pow2Plan<L>::NTH) pow2_readout_kernel(ReadoutArgs a)
 {
     using P = Pow2Plan<L>;
-    constexpr int TPF = P::TPF, FPB = P::FPB, R3 = P::R3, RS = P::RS, BUF = P::BUF, PP = P::PP, N = P::N;
-    extern __shared__ __align__(16) unsigned char sm[];
+    constexpr int TPF = P::TPF, FPB = P::FPB, R3 = P::R3, PP = P::PP, N = P::N;
+    extern __shared__ __align__(1024) unsigned char sm[];
     const int T = a.T;
+    float2* Z = reinterpret_cast<float2*>(sm);                         // [FPB][L]
     // pass twiddles laid out so a warp reads consecutive entries:
     // tw1[k2][n1] = W_L^{n1 k2}, tw2[j][m1] = W_{L/16}^{m1 j}
-    float2* tw1 = reinterpret_cast<float2*>(sm);                       // [16][L/16]
-    float2* tw2 = tw1 + L;                                             // [16][R3]
+    float2* tw2 = Z + FPB * L;                                         // [16][R3]
     float2* twb = tw2 + 16 * R3;                                       // [T] W_N^{b_k}
-    int* bins = reinterpret_cast<int*>(twb + T);                       // [T]
-    float* iref = reinterpret_cast<float*>(bins + T);                  // [T]
-    float2* S = reinterpret_cast<float2*>(sm + a.sm_a);                // [FPB][BUF]
-    int16_t* raw0 = reinterpret_cast<int16_t*>(sm + a.sm_raw);         // [2][FPB N + 16]
-    constexpr int kRawStride = FPB * N + 16;
-    for (int i = threadIdx.x; i < L; i += blockDim.x) {
-        const int k2 = i / TPF, n1 = i - k2 * TPF;
-        tw1[i] = a.tw_L[n1 * k2];
-    }
-    for (int i = threadIdx.x; i < 16 * R3; i += blockDim.x) {
+    int2* pos = reinterpret_cast<int2*>(twb + T);                      // [T] places of Z_b and Z_(L - b)
+    float* iref = reinterpret_cast<float*>(pos + T);                   // [T]
+    const int fs = threadIdx.x / TPF;      // frame slot
+    const int lt = threadIdx.x % TPF;      // thread within the frame
+    const int lane = threadIdx.x & 31;
+    const int64_t step = static_cast<int64_t>(gridDim.x) * FPB;
+    int64_t f = static_cast<int64_t>(blockIdx.x) * FPB + fs;
+    uint32_t next[16];                     // the next frame's samples, two a word
+    auto fetch = [&](int64_t fr) {
+        const uint32_t* rw = reinterpret_cast<const uint32_t*>(a.frames + fr * N) + lt;
+#pragma unroll
+        for (int n2 = 0; n2 < 16; ++n2) next[n2] = __ldcs(rw + TPF * n2);
+    };
+    if (f < a.n_frames) fetch(f);
+    float2 tw1[16];                        // W_L^{n1 k2} of the thread's n1 = lt
+#pragma unroll
+    for (int k2 = 1; k2 < 16; ++k2) tw1[k2] = a.tw_L[lt * k2];
+    for (int i = threadIdx.x; i < 16 * R3; i += P::NTH) {
         const int j = i / R3, m1 = i - j * R3;
         tw2[i] = a.tw_L[16 * m1 * j];
     }
-    for (int i = threadIdx.x; i < T; i += blockDim.x) {
+    // place of Z_k: k = k2 + 16 j + 256 j' lies at point k2 L/16 + R3 j + j'
+    auto place = [](int k) { return zsw((k & 15) * TPF + ((k >> 4) & 15) * R3 + (k >> 8)); };
+    for (int i = threadIdx.x; i < T; i += P::NTH) {
+        const int b = a.zidx[i];
         twb[i] = a.tw_b[i];
-        bins[i] = a.zidx[i];
+        pos[i] = make_int2(place(b == L ? 0 : b), place(b == 0 ? 0 : L - b));
         iref[i] = a.inv_ref[i];
     }
-    const int fs = threadIdx.x / TPF;      // frame slot
-    const int lt = threadIdx.x % TPF;      // thread within the frame
-    float2* Sf = S + fs * BUF;
-    const int64_t nb = (a.n_frames + FPB - 1) / FPB;
-    int64_t b = blockIdx.x;
-    int buf = 0;
-    int off_cur = 0;   // element offset of the current batch inside its buffer
-    if (b < nb) {
-        const int nf0 = static_cast<int>((a.n_frames - b * FPB) < FPB ? (a.n_frames - b * FPB) : FPB);
-        off_cur = stage_async(a.frames, b * FPB * static_cast<int64_t>(N), static_cast<int64_t>(nf0) * N, raw0);
-    }
-    for (; b < nb; b += gridDim.x, buf ^= 1) {
-        const int64_t f0 = b * FPB;
-        const int nf = static_cast<int>((a.n_frames - f0) < FPB ? (a.n_frames - f0) : FPB);
-        // the next batch streams into the other buffer (a possibly empty group)
-        const int64_t bn = b + gridDim.x;
-        int off_next = 0;
-        if (bn < nb) {
-            const int nfn = static_cast<int>((a.n_frames - bn * FPB) < FPB ? (a.n_frames - bn * FPB) : FPB);
-            off_next = stage_async(a.frames, bn * FPB * static_cast<int64_t>(N), static_cast<int64_t>(nfn) * N,
-                                   raw0 + (buf ^ 1) * kRawStride);
-        } else {
-            cp_async_commit();
-        }
-        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-        __syncthreads();
-        const bool live = fs < nf;
+    __syncthreads();
+    const float2* Zf = Z + fs * L;
+    const uint32_t z = static_cast<uint32_t>(__cvta_generic_to_shared(Zf));
+    const uint32_t z1 = z + 8 * zsw(lt);                                  // pass 1: points lt + TPF n2
+    const uint32_t z2 = z + 8 * zsw((lt / R3) * TPF + lt % R3);           // pass 2: (k2, m1), points R3 m2 on
+    // pass 3: butterflies (k2, j) of the warp's own k2 blocks, 16 a block
+    const int k2w = (lt >> 5) * (32 / R3);
+    auto group_sync = [&] {
+        asm volatile("bar.sync %0, %1;\n" ::"r"(fs + 1), "n"(TPF) : "memory");
+    };
+    for (; f < a.n_frames; f += step) {
         // ---- pass 1: DFT16 over n2, twiddle W_L^{n1 k2} ----
         {
-            float2 z[16];
-            const uint32_t* rw = reinterpret_cast<const uint32_t*>(raw0 + buf * kRawStride + off_cur + fs * N);
+            float2 v[16];
 #pragma unroll
-            for (int n2 = 0; n2 < 16; ++n2) {
-                const uint32_t w = live ? rw[lt + TPF * n2] : 0u;
-                z[n2] = make_float2(static_cast<float>(static_cast<short>(w & 0xffffu)),
-                                    static_cast<float>(static_cast<short>(w >> 16)));
-            }
-            Dft<16>::run(z);
+            for (int n2 = 0; n2 < 16; ++n2)
+                v[n2] = make_float2(static_cast<float>(static_cast<short>(next[n2] & 0xffffu)),
+                                    static_cast<float>(static_cast<short>(next[n2] >> 16)));
+            if (f + step < a.n_frames) fetch(f + step);
+            Dft<16>::run(v);
 #pragma unroll
-            for (int k2 = 1; k2 < 16; ++k2) z[k2] = cmul(z[k2], tw1[k2 * TPF + lt]);
+            for (int k2 = 1; k2 < 16; ++k2) v[k2] = cmul(v[k2], tw1[k2]);
 #pragma unroll
-            for (int k2 = 0; k2 < 16; ++k2) Sf[k2 * RS + lt] = z[k2];
+            for (int k2 = 0; k2 < 16; ++k2) zst(zat(z1, k2 * TPF), v[k2]);
         }
-        __syncthreads();
+        group_sync();
         // ---- pass 2: DFT16 over m2, twiddle W_{L/16}^{m1 j} ----
         {
-            const int k2 = lt / R3, m1 = lt % R3;
-            float2 z[16];
+            float2 v[16];
 #pragma unroll
-            for (int m2 = 0; m2 < 16; ++m2) z[m2] = Sf[k2 * RS + m1 + R3 * m2];
-            Dft<16>::run(z);
+            for (int m2 = 0; m2 < 16; ++m2) v[m2] = zld(zat(z2, R3 * m2));
+            Dft<16>::run(v);
 #pragma unroll
-            for (int j = 1; j < 16; ++j) z[j] = cmul(z[j], tw2[j * R3 + m1]);
-            __syncthreads();
+            for (int j = 1; j < 16; ++j) v[j] = cmul(v[j], tw2[j * R3 + lt % R3]);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) Sf[k2 * RS + 17 * m1 + j] = z[j];
+            for (int j = 0; j < 16; ++j) zst(zat(z2, R3 * j), v[j]);
         }
-        __syncthreads();
-        // ---- pass 3: DFT_R3 over m1; Z[k2 + 16 j + 256 j'] at zpos ----
-        {
-            const int j = lt & 15;
-            float2 v[PP][R3];
+        __syncwarp();
+        // ---- pass 3: DFT_R3 over m1 ----
 #pragma unroll
-            for (int p = 0; p < PP; ++p) {
-                const int k2 = (lt >> 4) + (TPF / 16) * p;
+        for (int i = 0; i < PP; ++i) {
+            const int q = lane + 32 * i;
+            const uint32_t z3 = z + 8 * zsw((k2w + (q >> 4)) * TPF + R3 * (q & 15));
+            float2 v[R3];
 #pragma unroll
-                for (int m1 = 0; m1 < R3; ++m1) v[p][m1] = Sf[k2 * RS + 17 * m1 + j];
-            }
-            __syncthreads();
+            for (int m1 = 0; m1 < R3; ++m1) v[m1] = zld(zat(z3, m1));
+            Dft<R3>::run(v);
 #pragma unroll
-            for (int p = 0; p < PP; ++p) {
-                const int k2 = (lt >> 4) + (TPF / 16) * p;
-                Dft<R3>::run(v[p]);
-#pragma unroll
-                for (int jj = 0; jj < R3; ++jj) Sf[zpos(k2 + 16 * j + 256 * jj)] = v[p][jj];
-            }
+            for (int m1 = 0; m1 < R3; ++m1) zst(zat(z3, m1), v[m1]);
         }
-        __syncthreads();
+        group_sync();
         // ---- teeth: real-FFT split at the tooth bins, coalesced outputs ----
-        for (int item = threadIdx.x; item < nf * T; item += blockDim.x) {
-            const int f = item / T;
-            const int k = item - f * T;
-            const float2* Z = S + f * BUF;
-            const int bb = bins[k];
-            const int i1 = (bb == L) ? 0 : bb;
-            const int i2 = (bb == 0) ? 0 : L - bb;
-            const float2 Zb = Z[zpos(i1)];
-            const float2 Zr = Z[zpos(i2)];
+        const int64_t row = f * T;
+        for (int k = lt; k < T; k += TPF) {
+            const int2 p = pos[k];
+            const float2 Zb = Zf[p.x];
+            const float2 Zr = Zf[p.y];
             // E = (Zb + conj Zr) / 2, O = (Zb - conj Zr) / (2 i), X_b = E + W_N^b O
             const float2 E = make_float2(0.5f * (Zb.x + Zr.x), 0.5f * (Zb.y - Zr.y));
             const float2 Dd = make_float2(0.5f * (Zb.x - Zr.x), 0.5f * (Zb.y + Zr.y));
             const float2 O = make_float2(Dd.y, -Dd.x);
             const float2 X = cadd(E, cmul(twb[k], O));
             const float amp = cabs_approx(X);
-            const int64_t o = (f0 + f) * T + k;
-            if (a.amps) a.amps[o] = amp;
-            if (a.y) a.y[o] = __fmul_rn(amp, iref[k]);
+            if (a.amps) a.amps[row + k] = amp;
+            if (a.y) a.y[row + k] = __fmul_rn(amp, iref[k]);
         }
-        off_cur = off_next;
+        group_sync();   // the teeth are read before the next frame's points land
     }
-    cp_async_wait_all();
 }
 
 template <int L>
@@ -190,13 +190,14 @@ void* pow2_ptr(int L)
     }
 }
 
-int pow2_fpb(int L) { return kPow2Threads / (L / 16); }
+int pow2_threads(int L) { return L / 16 > 128 ? L / 16 : 128; }
+int pow2_fpb(int L) { return pow2_threads(L) / (L / 16); }
 
 }  // namespace
 
 // Chooses the power-of-two readout for full real transforms with L = N / 2 in
-// {1024, 2048, 4096}: shared-memory layout (twiddles and tooth tables, two
-// sample buffers, the exchange buffers) and the grid; leaves pow2_ok false
+// {1024, 2048, 4096}: shared memory (the frames' points, twiddles and tooth
+// tables) and the grid; leaves pow2_ok false
 // otherwise.
 cudaError_t setup_pow2(cg_plan_s* p)
 {
@@ -206,20 +207,13 @@ cudaError_t setup_pow2(cg_plan_s* p)
     void* fn = pow2_ptr(L);
     if (!fn) return cudaSuccess;
     const int fpb = pow2_fpb(L);
-    const int N = 2 * L;
     ReadoutArgs& r = p->pa;
     r = p->ra;
-    int off = 8 * L + 8 * 16 * (L / 256) + 8 * T + 4 * T + 4 * T;
-    off = (off + 15) & ~15;
-    r.sm_a = off;
-    off += fpb * (L + L / 16) * 8;
-    r.sm_raw = off;
-    off += 2 * (fpb * N + 16) * 2;
-    r.sm_total = (off + 15) & ~15;
+    r.sm_total = 8 * (fpb * L + 16 * (L / 256) + 2 * T) + 4 * T;
     cudaError_t e;
     if ((e = raise_smem_limit(fn, r.sm_total)) != cudaSuccess) return e;
     int occ = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kPow2Threads, r.sm_total)) != cudaSuccess)
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, pow2_threads(L), r.sm_total)) != cudaSuccess)
         return e;
     if (occ < 1) return cudaSuccess;
     p->grid_pow2 = p->num_sms * occ;
@@ -239,7 +233,7 @@ cudaError_t launch_pow2_readout(const cg_plan_s* p, const int16_t* frames, int64
     const int64_t nb = (n + fpb - 1) / fpb;
     const int grid = static_cast<int>(nb < p->grid_pow2 ? nb : p->grid_pow2);
     void* args[] = {&r};
-    return cudaLaunchKernel(pow2_ptr(p->L), dim3(grid), dim3(kPow2Threads), args, r.sm_total, s);
+    return cudaLaunchKernel(pow2_ptr(p->L), dim3(grid), dim3(pow2_threads(p->L)), args, r.sm_total, s);
 }
 
 }  // namespace cg
