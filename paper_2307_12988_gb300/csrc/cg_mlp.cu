@@ -18,47 +18,13 @@
 #include <cuda_runtime.h>
 
 #include "cg_internal.h"
+#include "cg_mlp.h"
 #include "cg_tc.cuh"
-
-struct cg_mlp_s {
-    int device = 0;
-    int n_in = 0, H = 0, n_out = 0, max_batch = 0;
-    int64_t np = 0;
-    int64_t step = 0;                 // Adam steps taken
-    float* theta = nullptr;           // [np] parameters
-    float* grad = nullptr;            // [np]
-    float* m = nullptr;               // [np] Adam first moment
-    float* v = nullptr;               // [np] Adam second moment
-    // activations and gradients of one batch
-    float *xb = nullptr, *tb = nullptr;          // gathered batch [max_batch][n_in / n_out]
-    float *z1 = nullptr, *a1 = nullptr, *z2 = nullptr, *a2 = nullptr, *out = nullptr;
-    float *g_out = nullptr, *g_z2 = nullptr, *g_z1 = nullptr;
-    float* part = nullptr;            // [kLossBlocks] loss partial sums
-    float* loss = nullptr;            // [1]
-    float* ws = nullptr;              // K-split partial sums of the weight gradients
-    int* err = nullptr;               // [1] set by a matrix-product block whose bounded wait ran out
-    std::vector<float> in_mean, in_scale, out_mean, out_scale;
-};
 
 namespace cg {
 namespace {
 
-constexpr int kLossBlocks = 256;
-constexpr float kGeluK = 0.7978845608028654f;   // sqrt(2 / pi)
-constexpr float kGeluC = 0.044715f;
-
 enum { kEpiNone = 0, kEpiBias = 1, kEpiBiasGelu = 2, kEpiGeluGrad = 3 };
-
-__device__ __forceinline__ float gelu_f(float z)
-{
-    const float t = tanhf(kGeluK * fmaf(kGeluC * z * z, z, z));
-    return 0.5f * z * (1.0f + t);
-}
-__device__ __forceinline__ float gelu_grad_f(float z)
-{
-    const float t = tanhf(kGeluK * fmaf(kGeluC * z * z, z, z));
-    return 0.5f * (1.0f + t) + 0.5f * z * (1.0f - t * t) * kGeluK * fmaf(3.0f * kGeluC, z * z, 1.0f);
-}
 
 // ---------------------------------------------------------------------------
 // C[m][n] = epilogue(sum_k opA(m,k) opB(k,n)) on the tensor cores.
@@ -86,14 +52,11 @@ __device__ __forceinline__ float gelu_grad_f(float z)
 // Epilogue: kEpiBias C = acc + bias[n]; kEpiBiasGelu C = z = acc + bias[n],
 // C2 = gelu(z); kEpiGeluGrad C = acc * gelu'(aux[m][n]).
 // ---------------------------------------------------------------------------
-constexpr int kGM = 128;            // rows per tile (MMA M)
-constexpr int kGK = 32;             // K elements per block (one 128-byte swizzle row of FP32)
 constexpr int kGN = 128;            // columns per tile at most (MMA N)
 constexpr int kGStages = 3;
 constexpr int kGWorkerWarps = 8;    // copy / split / epilogue warps
 constexpr int kGProducers = 32 * kGWorkerWarps;
 constexpr int kGThreads = kGProducers + 32;   // + the MMA warp
-constexpr int kGMaxSplit = 8;       // K ranges of one output tile at most
 constexpr uint32_t kGPolls = 1u << 22;
 constexpr int kGTile = kGM * kGK * 4;            // 16 KiB: one (hi or lo) tile of A or of B
 constexpr int kGStage = 4 * kGTile;              // A hi, A lo, B hi, B lo
@@ -129,15 +92,6 @@ __device__ __forceinline__ bool producers_any(bool flag)
     return r != 0;
 }
 __device__ __forceinline__ void producers_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(kGProducers) : "memory"); }
-
-// FP32 -> TF32, round to nearest (ties away), as a 32-bit pattern with the
-// low 13 mantissa bits zero
-__device__ __forceinline__ float tf32_rn(float x)
-{
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;\n" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
-}
 
 // cp.async of rows [row0, row0 + nrows) x K elements [k0, k0 + 32) of an
 // operand into the K-major 128-byte-swizzled tile `dst` (element (r, k) at
@@ -450,21 +404,6 @@ __global__ void __launch_bounds__(256) loss_final_kernel(const float* __restrict
     }
 }
 
-__global__ void adam_kernel(float* __restrict__ theta, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, int64_t np, float lr, float b1, float b2, float eps, float bc1,
-                            float bc2)
-{
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < np;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const float gi = g[i];
-        const float mi = fmaf(b1, m[i], (1.0f - b1) * gi);
-        const float vi = fmaf(b2, v[i], (1.0f - b2) * gi * gi);
-        m[i] = mi;
-        v[i] = vi;
-        theta[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
-    }
-}
-
 // dst[r][:] = src[idx[r]][:] for r < rows (an index outside [0, n_src) gives a zero row)
 __global__ void gather_rows_kernel(const float* __restrict__ src, int64_t n_src, const int32_t* __restrict__ idx,
                                    int rows, int width, float* __restrict__ dst)
@@ -490,39 +429,9 @@ cudaError_t sgemm(int M, int N, int K, const float* A, int lda, const float* B, 
     void* fn = reinterpret_cast<void*>(&tgemm_kernel<TA, TB, EPI>);
     cudaError_t e = raise_smem_limit(fn, kGSmem);
     if (e != cudaSuccess) return e;
-    // Tile width bn (128, 64, 32 or 16 columns) and K ranges: the pair with
-    // the least modelled time, waves x (a fixed cost + per K block the A tile
-    // and a bn-row B tile + the epilogue of bn columns), in units of one
-    // 128-row operand tile; K ranges of 4 blocks at least and only for
-    // products without an epilogue.  These products are small, so filling
-    // the SMs matters more than re-reading A once per column tile from L2.
-    static int n_sm = 0;
-    if (n_sm == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sm < 1)
-            n_sm = 1;
-    }
+    const SplitRule sr = split_rule(M, N, K, EPI == kEpiNone && ws && ldc == N);
+    const int bn = sr.bn, kb_per = sr.kb_per, splits = sr.splits;
     const int tiles_m = (M + kGM - 1) / kGM;
-    const int nkb = (K + kGK - 1) / kGK;
-    const int max_split = (EPI == kEpiNone && ws && ldc == N) ? std::min(kGMaxSplit, std::max(1, nkb / 4)) : 1;
-    int bn = kGN, kb_per = nkb, splits = 1;
-    double best = 0.0;
-    for (int w = kGN; w >= 16; w >>= 1) {
-        for (int sp = 1; sp <= max_split; ++sp) {
-            const int per = (nkb + sp - 1) / sp;
-            const int sp_eff = (nkb + per - 1) / per;
-            const int64_t ctas = static_cast<int64_t>(tiles_m) * ((N + w - 1) / w) * sp_eff;
-            const double waves = static_cast<double>((ctas + n_sm - 1) / n_sm);
-            const double tm = waves * (3.0 + per * (1.0 + w / 128.0) + 2.0 * w / 128.0) + (sp_eff > 1 ? 1.0 : 0.0);
-            if (best == 0.0 || tm < best) {
-                best = tm;
-                bn = w;
-                kb_per = per;
-                splits = sp_eff;
-            }
-        }
-    }
     const int tiles_n = (N + bn - 1) / bn;
     dim3 grid(tiles_n, tiles_m, splits);
     tgemm_kernel<TA, TB, EPI><<<grid, kGThreads, kGSmem, s>>>(M, N, K, bn, kb_per, A, lda, B, ldb, C, ldc, bias,
@@ -533,21 +442,6 @@ cudaError_t sgemm(int M, int N, int K, const float* A, int lda, const float* B, 
         split_sum_kernel<<<blocks, 256, 0, s>>>(ws, splits, mn, C);
     }
     return cudaGetLastError();
-}
-
-struct Offsets {
-    int64_t W1, b1, W2, b2, W3, b3;
-};
-Offsets offsets(const cg_mlp_s* m)
-{
-    Offsets o;
-    o.W1 = 0;
-    o.b1 = o.W1 + static_cast<int64_t>(m->H) * m->n_in;
-    o.W2 = o.b1 + m->H;
-    o.b2 = o.W2 + static_cast<int64_t>(m->H) * m->H;
-    o.W3 = o.b2 + m->H;
-    o.b3 = o.W3 + static_cast<int64_t>(m->n_out) * m->H;
-    return o;
 }
 
 // forward of rows x [n][n_in] (n <= max_batch) into the object's activations
@@ -602,14 +496,13 @@ cudaError_t backward_batch(cg_mlp_s* m, const float* x, const float* t, int n, f
     return cudaGetLastError();
 }
 
-cudaError_t adam(cg_mlp_s* m, float lr, float b1, float b2, float eps, cudaStream_t s)
+// the next Adam step's constants (counts the step)
+AdamStep next_adam(cg_mlp_s* m, float lr, float b1, float b2, float eps)
 {
     m->step += 1;
     const float bc1 = static_cast<float>(1.0 - std::pow(static_cast<double>(b1), static_cast<double>(m->step)));
     const float bc2 = static_cast<float>(1.0 - std::pow(static_cast<double>(b2), static_cast<double>(m->step)));
-    const int blocks = static_cast<int>(std::min<int64_t>((m->np + 255) / 256, 1024));
-    adam_kernel<<<blocks, 256, 0, s>>>(m->theta, m->grad, m->m, m->v, m->np, lr, b1, b2, eps, bc1, bc2);
-    return cudaGetLastError();
+    return {lr, b1, b2, eps, bc1, bc2};
 }
 
 uint64_t splitmix64(uint64_t z)
@@ -639,6 +532,7 @@ void free_mlp(cg_mlp_s* m)
                      m->g_z2, m->g_z1, m->part, m->loss, m->ws})
         if (q) cudaFree(q);
     if (m->err) cudaFree(m->err);
+    train_destroy(m);
     delete m;
 }
 
@@ -660,6 +554,43 @@ cg_status take_err(cg_mlp_s* m, const char* what)
 }
 
 }  // namespace
+
+// The tile width bn (128, 64, 32 or 16 columns) and K ranges with the least
+// modelled time, waves x (a fixed cost + per K block the A tile and a bn-row B
+// tile + the epilogue of bn columns), in units of one 128-row operand tile; K
+// ranges of 4 blocks at least and only for products without an epilogue.
+// These products are small, so filling the SMs matters more than re-reading A
+// once per column tile from L2.
+SplitRule split_rule(int M, int N, int K, bool can_split)
+{
+    static int n_sm = 0;
+    if (n_sm == 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sm < 1)
+            n_sm = 1;
+    }
+    const int tiles_m = (M + kGM - 1) / kGM;
+    const int nkb = (K + kGK - 1) / kGK;
+    const int max_split = can_split ? std::min(kGMaxSplit, std::max(1, nkb / 4)) : 1;
+    SplitRule r{kGN, nkb, 1};
+    double best = 0.0;
+    for (int w = kGN; w >= 16; w >>= 1) {
+        for (int sp = 1; sp <= max_split; ++sp) {
+            const int per = (nkb + sp - 1) / sp;
+            const int sp_eff = (nkb + per - 1) / per;
+            const int64_t ctas = static_cast<int64_t>(tiles_m) * ((N + w - 1) / w) * sp_eff;
+            const double waves = static_cast<double>((ctas + n_sm - 1) / n_sm);
+            const double tm = waves * (3.0 + per * (1.0 + w / 128.0) + 2.0 * w / 128.0) + (sp_eff > 1 ? 1.0 : 0.0);
+            if (best == 0.0 || tm < best) {
+                best = tm;
+                r = {w, per, sp_eff};
+            }
+        }
+    }
+    return r;
+}
+
 }  // namespace cg
 
 using namespace cg;
@@ -732,6 +663,8 @@ cg_status cg_mlp_create(cg_mlp_t* out, int n_in, int n_hidden, int n_out, int ma
     if (e == cudaSuccess) e = cudaMemset(m->v, 0, sizeof(float) * m->np);
     if (e == cudaSuccess) e = cudaMemset(m->grad, 0, sizeof(float) * m->np);
     if (e == cudaSuccess) e = cudaMemset(m->err, 0, sizeof(int));
+    if (e == cudaSuccess) e = train_create(m);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) {
         free_mlp(m);
         return cuda_fail_m(e, "cg_mlp_create");
@@ -764,6 +697,8 @@ cg_status cg_mlp_set_params(cg_mlp_t m, const float* host, int64_t count)
     if (e == cudaSuccess) e = cudaMemcpy(m->theta, host, sizeof(float) * count, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(m->m, 0, sizeof(float) * m->np);
     if (e == cudaSuccess) e = cudaMemset(m->v, 0, sizeof(float) * m->np);
+    if (e == cudaSuccess) e = train_refresh(m, nullptr);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     m->step = 0;
     return e == cudaSuccess ? CG_OK : cuda_fail_m(e, "cg_mlp_set_params");
 }
@@ -790,7 +725,14 @@ cg_status cg_mlp_backward(cg_mlp_t m, const float* x, const float* t, int64_t n,
     if (n < 1 || n > m->max_batch) return fail_m(CG_ERR_ARG, "n must be in [1, max_batch]");
     if (!x || !t) return fail_m(CG_ERR_ARG, "x_dev and t_dev are required");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e = backward_batch(m, x, t, static_cast<int>(n), loss_dev, s);
+    cudaError_t e;
+    if (n <= kTrainRows) {
+        const TrainBatch b{x, t, n, nullptr, static_cast<int>(n)};
+        e = train_prepare(m, b, s);
+        if (e == cudaSuccess) e = train_step(m, b, loss_dev, nullptr, nullptr, s);
+    } else {
+        e = backward_batch(m, x, t, static_cast<int>(n), loss_dev, s);
+    }
     if (e == cudaSuccess && grad_dev)
         e = cudaMemcpyAsync(grad_dev, m->grad, sizeof(float) * m->np, cudaMemcpyDeviceToDevice, s);
     return e == cudaSuccess ? CG_OK : cuda_fail_m(e, "cg_mlp_backward");
@@ -801,7 +743,7 @@ cg_status cg_mlp_adam(cg_mlp_t m, float lr, float b1, float b2, float eps, void*
     if (!m) return fail_m(CG_ERR_ARG, "mlp is NULL");
     if (!(lr >= 0.f) || !(b1 >= 0.f && b1 < 1.f) || !(b2 >= 0.f && b2 < 1.f) || !(eps > 0.f))
         return fail_m(CG_ERR_ARG, "Adam hyper-parameters out of range");
-    cudaError_t e = adam(m, lr, b1, b2, eps, static_cast<cudaStream_t>(stream));
+    cudaError_t e = train_adam(m, next_adam(m, lr, b1, b2, eps), static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? CG_OK : cuda_fail_m(e, "cg_mlp_adam");
 }
 
@@ -815,6 +757,22 @@ cg_status cg_mlp_train_epoch(cg_mlp_t m, const float* x, const float* t, int64_t
     if (!(lr >= 0.f)) return fail_m(CG_ERR_ARG, "lr < 0");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int64_t b = 0;
+    if (batch <= kTrainRows) {
+        // the step on operand images; the next batch's rows are gathered
+        // beside the Adam step of this one
+        auto rows_at = [&](int64_t r0) {
+            return TrainBatch{x, t, n, perm + r0, static_cast<int>(std::min<int64_t>(batch, n - r0))};
+        };
+        cudaError_t e = train_prepare(m, rows_at(0), s);
+        for (int64_t r0 = 0; e == cudaSuccess && r0 < n; r0 += batch, ++b) {
+            const TrainBatch cur = rows_at(r0);
+            const bool more = r0 + batch < n;
+            const TrainBatch nxt = more ? rows_at(r0 + batch) : TrainBatch{};
+            const AdamStep a = next_adam(m, lr, 0.9f, 0.999f, 1e-8f);
+            e = train_step(m, cur, losses ? losses + b : nullptr, &a, more ? &nxt : nullptr, s);
+        }
+        return e == cudaSuccess ? CG_OK : cuda_fail_m(e, "cg_mlp_train_epoch");
+    }
     for (int64_t r0 = 0; r0 < n; r0 += batch, ++b) {
         const int rows = static_cast<int>(std::min<int64_t>(batch, n - r0));
         const int gx = static_cast<int>(std::min<int64_t>((static_cast<int64_t>(rows) * m->n_in + 255) / 256, 2048));
@@ -823,7 +781,7 @@ cg_status cg_mlp_train_epoch(cg_mlp_t m, const float* x, const float* t, int64_t
         gather_rows_kernel<<<gt, 256, 0, s>>>(t, n, perm + r0, rows, m->n_out, m->tb);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = backward_batch(m, m->xb, m->tb, rows, losses ? losses + b : nullptr, s);
-        if (e == cudaSuccess) e = adam(m, lr, 0.9f, 0.999f, 1e-8f, s);
+        if (e == cudaSuccess) e = train_adam(m, next_adam(m, lr, 0.9f, 0.999f, 1e-8f), s);
         if (e != cudaSuccess) return cuda_fail_m(e, "cg_mlp_train_epoch");
     }
     return CG_OK;
