@@ -30,7 +30,12 @@
 // bounded; a block whose wait runs out records it and writes nothing.
 //
 // What bounds it: latency.  A 1,024 x 256 x 256 product is 0.4 GFLOP on 128
-// SMs; its launch, first copy, eight K blocks and epilogue follow one another.
+// SMs; its launch, first copy, eight K blocks and epilogue follow one another
+// (10 us).  So the output tiles are as narrow as fills the SMs (16 columns at
+// 1,024 rows and 256 units; 32 cost 2 us more a product, 64 seven), and eight
+// epilogue warps share a tile.  A step of 1,024 rows, 221 -> 256 -> 256 -> 4:
+// 170 us in 19 launches, 81 in six with four epilogue warps and weights
+// updated element by element, 62 so.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -64,8 +69,10 @@ struct TrainImages {
 namespace {
 
 constexpr int kTile = kGM * 128;                 // one 128-row tile of a K block
-constexpr int kEpiThreads = 128;
-constexpr int kTrThreads = kEpiThreads + 64;     // + the copy warp and the MMA warp
+constexpr int kEpiThreads = 256;                 // warps w and w + 4 share 32 rows, taking every other 8 columns
+constexpr int kCopyWarp = kEpiThreads / 32;
+constexpr int kMmaWarp = kCopyWarp + 1;
+constexpr int kTrThreads = 32 * (kMmaWarp + 1);
 constexpr int kMaxRing = 6;
 constexpr uint32_t kTrPolls = 1u << 22;
 constexpr int kFinThreads = 256;
@@ -162,11 +169,11 @@ __device__ __forceinline__ Ring ring_init(unsigned char* sm, int stages, int bn,
         }
         tc::mbar_init(&r.done[0], 1);
         tc::mbar_init(&r.done[1], 1);
-        tc::mbar_init(&r.done[2], kEpiThreads);
+        tc::mbar_init(&r.done[2], kGM);
         *r.abort_flag = 0;
         tc::fence_mbar_init();
     }
-    if (threadIdx.x >= kEpiThreads + 32) tc::tmem_alloc(r.tmem_slot, tmem_cols);
+    if (threadIdx.x >= 32 * kMmaWarp) tc::tmem_alloc(r.tmem_slot, tmem_cols);
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
@@ -176,7 +183,7 @@ __device__ __forceinline__ void ring_end(const Ring& r, int tmem_cols)
 {
     tc::tc_fence_before();
     __syncthreads();
-    if (threadIdx.x >= kEpiThreads + 32) {
+    if (threadIdx.x >= 32 * kMmaWarp) {
         __syncwarp();
         tc::tc_fence_after();
         tc::tmem_dealloc(*r.tmem_slot, tmem_cols);
@@ -250,50 +257,50 @@ __device__ __forceinline__ bool ring_wait(const Ring& r, uint64_t* done, int* er
     return !failed;
 }
 
-// sixteen values of a row of the batch, columns c0 .. c0 + 15 (nc of them
+// eight values of a row of the batch, columns c0 .. c0 + 7 (nc of them
 // real): images with rows = batch (f) and K = batch (t); zero rows beyond n
-__device__ __forceinline__ void put_images(const Img& f, const Img& t, int row, int n, int c0, int nc, float (&v)[16])
+__device__ __forceinline__ void put_images(const Img& f, const Img& t, int row, int n, int c0, int nc, float (&v)[8])
 {
     if (row >= n)
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = 0.f;
+        for (int i = 0; i < 8; ++i) v[i] = 0.f;
     if (f.p) {
-        if (nc == 16) {
+        if (nc == 8) {
 #pragma unroll
-            for (int i = 0; i < 16; i += 4) put4(f, row, c0 + i, v + i);
+            for (int i = 0; i < 8; i += 4) put4(f, row, c0 + i, v + i);
         } else {
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
+            for (int i = 0; i < 8; ++i)
                 if (i < nc) put(f, row, c0 + i, v[i]);
         }
     }
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
+    for (int i = 0; i < 8; ++i)
         if (i < nc) put(t, c0 + i, row, v[i]);
 }
 // the same values as a row of an FP32 matrix [n][ld]
-__device__ __forceinline__ void put_row(float* m, int ld, int row, int n, int c0, int nc, const float (&v)[16])
+__device__ __forceinline__ void put_row(float* m, int ld, int row, int n, int c0, int nc, const float (&v)[8])
 {
     if (row >= n) return;
     float* d = m + static_cast<int64_t>(row) * ld + c0;
-    if (nc == 16 && (ld & 3) == 0) {
+    if (nc == 8 && (ld & 3) == 0) {
 #pragma unroll
-        for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4*>(d + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+        for (int i = 0; i < 8; i += 4) *reinterpret_cast<float4*>(d + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
     } else {
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
+        for (int i = 0; i < 8; ++i)
             if (i < nc) d[i] = v[i];
     }
 }
-__device__ __forceinline__ void get_row(const float* m, int ld, int row, int n, int c0, int nc, float (&v)[16])
+__device__ __forceinline__ void get_row(const float* m, int ld, int row, int n, int c0, int nc, float (&v)[8])
 {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = 0.f;
+    for (int i = 0; i < 8; ++i) v[i] = 0.f;
     if (row >= n) return;
     const float* d = m + static_cast<int64_t>(row) * ld + c0;
-    if (nc == 16 && (ld & 3) == 0) {
+    if (nc == 8 && (ld & 3) == 0) {
 #pragma unroll
-        for (int i = 0; i < 16; i += 4) {
+        for (int i = 0; i < 8; i += 4) {
             const float4 q = *reinterpret_cast<const float4*>(d + i);
             v[i] = q.x;
             v[i + 1] = q.y;
@@ -302,7 +309,7 @@ __device__ __forceinline__ void get_row(const float* m, int ld, int row, int n, 
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
+        for (int i = 0; i < 8; ++i)
             if (i < nc) v[i] = d[i];
     }
 }
@@ -329,34 +336,34 @@ __global__ void __launch_bounds__(kTrThreads, 1) product_kernel(const __grid_con
     const int ncols = q.N - n0 < q.bn ? q.N - n0 : q.bn, bn = (ncols + 15) & ~15;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t tmem = *r.tmem_slot;
-    if (warp == 4) {
+    if (warp == kCopyWarp) {
         if (lane == 0) ring_copy(r, q.a, m0, q.b, n0, bn, 0, q.nkb);
-    } else if (warp == 5) {
+    } else if (warp == kMmaWarp) {
         if (lane == 0) {
             ring_mma(r, tmem, bn, q.nkb);
             (void)tc::mbar_wait(&r.done[0], 0, kTrPolls);
         }
     } else {
-        const int row = m0 + static_cast<int>(threadIdx.x);
-        float ax[16];
-        if (GRAD) get_row(q.aux, q.N, row, q.n, n0, min(16, ncols), ax);   // the first chunk's, during the products
+        const int row = m0 + 32 * (warp & 3) + lane, c0 = 8 * (warp >> 2);
+        float ax[8];
+        if (GRAD) get_row(q.aux, q.N, row, q.n, n0 + c0, max(0, min(8, ncols - c0)), ax);   // the first, during the products
         if (ring_wait(r, &r.done[0], q.err)) {
-            const uint32_t base = tmem + (static_cast<uint32_t>(warp * 32) << 16);
-            for (int c = 0; c < ncols; c += 16) {
-                const int nc = min(16, ncols - c);
-                float v[16];
-                tc::tmem_ld16(base + c, v);
+            const uint32_t base = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+            for (int c = c0; c < ncols; c += 16) {
+                const int nc = min(8, ncols - c);
+                float v[8];
+                tc::tmem_ld8(base + c, v);
                 if (GRAD) {
-                    if (c > 0) get_row(q.aux, q.N, row, q.n, n0 + c, nc, ax);
+                    if (c > c0) get_row(q.aux, q.N, row, q.n, n0 + c, nc, ax);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] *= gelu_grad_f(ax[i]);
+                    for (int i = 0; i < 8; ++i) v[i] *= gelu_grad_f(ax[i]);
                     put_row(q.fp, q.N, row, q.n, n0 + c, nc, v);
                 } else {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] += i < nc ? q.bias[n0 + c + i] : 0.f;
+                    for (int i = 0; i < 8; ++i) v[i] += i < nc ? q.bias[n0 + c + i] : 0.f;
                     put_row(q.fp, q.N, row, q.n, n0 + c, nc, v);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] = gelu_f(v[i]);
+                    for (int i = 0; i < 8; ++i) v[i] = gelu_f(v[i]);
                 }
                 put_images(q.f, q.t, row, q.n, n0 + c, nc, v);
             }
@@ -396,7 +403,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) mid_kernel(const __grid_constan
         tc::fence_mbar_init();
     }
     __syncthreads();
-    if (warp == 4) {
+    if (warp == kCopyWarp) {
         if (lane == 0) {
             const uint32_t nb = static_cast<uint32_t>(bn) * 128u;
             const unsigned char* pw = q.w3t.p + static_cast<int64_t>(n0) * 128;
@@ -406,7 +413,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) mid_kernel(const __grid_constan
             ring_copy(r, q.a2f, m0, q.w3f, 0, 16, 0, q.nkb);
             (void)tc::mbar_wait(w_full, 0, kTrPolls);
         }
-    } else if (warp == 5) {
+    } else if (warp == kMmaWarp) {
         if (lane == 0) {
             ring_mma(r, tmem, 16, q.nkb);
             // the second product: g_out (written by the epilogue threads) times W3
@@ -421,14 +428,14 @@ __global__ void __launch_bounds__(kTrThreads, 1) mid_kernel(const __grid_constan
             (void)tc::mbar_wait(&r.done[1], 0, kTrPolls);
         }
     } else {
-        const int rl = static_cast<int>(threadIdx.x), row = m0 + rl;
-        const uint32_t base = tmem + (static_cast<uint32_t>(warp * 32) << 16);
-        float ax[16];
-        get_row(q.z2, q.H, row, q.n, n0, min(16, ncols), ax);
+        const int rl = 32 * (warp & 3) + lane, row = m0 + rl, c0 = 8 * (warp >> 2);
+        const uint32_t base = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        float ax[8];
+        get_row(q.z2, q.H, row, q.n, n0 + c0, max(0, min(8, ncols - c0)), ax);
         float tv[16];
 #pragma unroll
         for (int j = 0; j < 16; ++j) tv[j] = 0.f;
-        if (row < q.n) {
+        if (warp < 4 && row < q.n) {
             const int64_t src = q.perm ? q.perm[row] : row;
             if (src >= 0 && src < q.n_src)
 #pragma unroll
@@ -436,34 +443,36 @@ __global__ void __launch_bounds__(kTrThreads, 1) mid_kernel(const __grid_constan
                     if (j < q.no) tv[j] = q.t[src * q.no + j];
         }
         bool ok = ring_wait(r, &r.done[0], q.err);
-        if (ok) {
+        if (warp < 4) {
             float v[16], g[32];
-            tc::tmem_ld16(base, v);
+            if (ok) {
+                tc::tmem_ld16(base, v);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) g[j] = 0.f;
+                for (int j = 0; j < 32; ++j) g[j] = 0.f;
 #pragma unroll
-            for (int j = 0; j < 16; ++j)
-                if (j < q.no) {
-                    v[j] += q.b3[j];
-                    const float d = v[j] - tv[j];
-                    g[j] = row < q.n ? q.scale * d : 0.f;
+                for (int j = 0; j < 16; ++j)
+                    if (j < q.no) {
+                        v[j] += q.b3[j];
+                        const float d = v[j] - tv[j];
+                        g[j] = row < q.n ? q.scale * d : 0.f;
+                    }
+                // the tile of g_out as the MMA reads it: this thread's row of 32 K elements
+#pragma unroll
+                for (int k = 0; k < 32; k += 4) {
+                    float h[4], l[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        h[i] = tf32_rn(g[k + i]);
+                        l[i] = tf32_rn(g[k + i] - h[i]);
+                    }
+                    *reinterpret_cast<float4*>(ga + swz(rl, k)) = make_float4(h[0], h[1], h[2], h[3]);
+                    *reinterpret_cast<float4*>(ga + kTile + swz(rl, k)) = make_float4(l[0], l[1], l[2], l[3]);
                 }
-            // the tile of g_out as the MMA reads it: this thread's row of 32 K elements
-#pragma unroll
-            for (int k = 0; k < 32; k += 4) {
-                float h[4], l[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    h[i] = tf32_rn(g[k + i]);
-                    l[i] = tf32_rn(g[k + i] - h[i]);
-                }
-                *reinterpret_cast<float4*>(ga + swz(rl, k)) = make_float4(h[0], h[1], h[2], h[3]);
-                *reinterpret_cast<float4*>(ga + kTile + swz(rl, k)) = make_float4(l[0], l[1], l[2], l[3]);
+                tc::fence_proxy_async_smem();
+                tc::tc_fence_before();
             }
-            tc::fence_proxy_async_smem();
-            tc::tc_fence_before();
             tc::mbar_arrive(&r.done[2]);
-            if (blockIdx.x == 0) {   // one block of the row tile keeps them
+            if (ok && blockIdx.x == 0) {   // one block of the row tile keeps them
 #pragma unroll
                 for (int j = 0; j < 16; ++j)
                     if (j < q.no) {
@@ -476,18 +485,16 @@ __global__ void __launch_bounds__(kTrThreads, 1) mid_kernel(const __grid_constan
                         }
                     }
             }
-            ok = ring_wait(r, &r.done[1], q.err);
-        } else {
-            tc::mbar_arrive(&r.done[2]);
         }
+        if (ok) ok = ring_wait(r, &r.done[1], q.err);
         if (ok)
-            for (int c = 0; c < ncols; c += 16) {
-                const int nc = min(16, ncols - c);
-                float v[16];
-                tc::tmem_ld16(base + 16 + c, v);
-                if (c > 0) get_row(q.z2, q.H, row, q.n, n0 + c, nc, ax);
+            for (int c = c0; c < ncols; c += 16) {
+                const int nc = min(8, ncols - c);
+                float v[8];
+                tc::tmem_ld8(base + 16 + c, v);
+                if (c > c0) get_row(q.z2, q.H, row, q.n, n0 + c, nc, ax);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] *= gelu_grad_f(ax[i]);
+                for (int i = 0; i < 8; ++i) v[i] *= gelu_grad_f(ax[i]);
                 put_row(q.g_z2, q.H, row, q.n, n0 + c, nc, v);
                 put_images(q.g2f, q.g2t, row, q.n, n0 + c, nc, v);
             }
@@ -523,21 +530,21 @@ __global__ void __launch_bounds__(kTrThreads, 1) dw_kernel(const __grid_constant
     const int ncols = min(q.bn, j.N - n0), bn = (ncols + 15) & ~15;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t tmem = *r.tmem_slot;
-    if (warp == 4) {
+    if (warp == kCopyWarp) {
         if (lane == 0) ring_copy(r, j.a, m0, j.b, n0, bn, kb0, nkb);
-    } else if (warp == 5) {
+    } else if (warp == kMmaWarp) {
         if (lane == 0) {
             ring_mma(r, tmem, bn, nkb);
             (void)tc::mbar_wait(&r.done[0], 0, kTrPolls);
         }
     } else if (ring_wait(r, &r.done[0], q.err)) {
-        const uint32_t base = tmem + (static_cast<uint32_t>(warp * 32) << 16);
-        const int row = m0 + static_cast<int>(threadIdx.x);
+        const uint32_t base = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        const int row = m0 + 32 * (warp & 3) + lane;
         float* ws = j.ws + static_cast<int64_t>(z) * j.M * j.N;
-        for (int c = 0; c < ncols; c += 16) {
-            float v[16];
-            tc::tmem_ld16(base + c, v);
-            put_row(ws, j.N, row, j.M, n0 + c, min(16, ncols - c), v);
+        for (int c = 8 * (warp >> 2); c < ncols; c += 16) {
+            float v[8];
+            tc::tmem_ld8(base + c, v);
+            put_row(ws, j.N, row, j.M, n0 + c, min(8, ncols - c), v);
         }
     }
     ring_end(r, q.tmem_cols);
@@ -597,12 +604,19 @@ struct FinishArgs {
     PrepArgs prep;
 };
 
-__device__ __forceinline__ float finish_param(const FinishArgs& q, int64_t i, float gi)
+struct ParamState {
+    float th, m, v;
+};
+__device__ __forceinline__ ParamState load_param(const FinishArgs& q, int64_t i)
 {
-    float th = q.theta[i];
+    return {q.theta[i], q.adam ? q.m[i] : 0.f, q.adam ? q.v[i] : 0.f};
+}
+__device__ __forceinline__ float finish_param(const FinishArgs& q, int64_t i, float gi, const ParamState& p)
+{
+    float th = p.th;
     if (q.adam) {
-        const float mi = fmaf(q.a.b1, q.m[i], (1.0f - q.a.b1) * gi);
-        const float vi = fmaf(q.a.b2, q.v[i], (1.0f - q.a.b2) * gi * gi);
+        const float mi = fmaf(q.a.b1, p.m, (1.0f - q.a.b1) * gi);
+        const float vi = fmaf(q.a.b2, p.v, (1.0f - q.a.b2) * gi * gi);
         q.m[i] = mi;
         q.v[i] = vi;
         th -= q.a.lr * (mi / q.a.bc1) / (sqrtf(vi / q.a.bc2) + q.a.eps);
@@ -630,7 +644,7 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const __grid_consta
         if (q.ws1) {
             float s = 0.f;
             if (c < cols) {
-#pragma unroll 8
+#pragma unroll 16
                 for (int r = y; r < q.n; r += 32) s += g[static_cast<int64_t>(r) * ld + col];
             }
             buf[y][cx] = s;
@@ -645,7 +659,7 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const __grid_consta
             } else {
                 s = q.grad[i];
             }
-            finish_param(q, i, s);
+            finish_param(q, i, s, load_param(q, i));
         }
         return;
     }
@@ -658,16 +672,25 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const __grid_consta
             const int64_t count = static_cast<int64_t>(q.n) * q.no;
             const int lane = t & 31;
             float* part = &buf[0][0];
-            for (int p = t >> 5; p < kLossBlocks; p += kFinThreads / 32) {
+            part[t] = 0.f;
+            __syncthreads();
+            for (int p = t >> 5; p < kLossBlocks && 256 * p < count; p += kFinThreads / 32) {
                 float s[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    s[k] = 0.f;
-                    for (int64_t e = 256 * p + lane + 32 * k; e < count; e += 256 * kLossBlocks) {
-                        const float d = q.out[e] - q.tb[e];
-                        s[k] = fmaf(d, d, s[k]);
-                    }
+                    const int64_t e = 256 * p + lane + 32 * k;
+                    const float d = e < count ? q.out[e] - q.tb[e] : 0.f;
+                    s[k] = d * d;
                 }
+                for (int64_t e0 = 256 * p + lane + 256 * kLossBlocks; e0 < count; e0 += 256 * kLossBlocks)
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const int64_t e = e0 + 32 * k;
+                        if (e < count) {
+                            const float d = q.out[e] - q.tb[e];
+                            s[k] = fmaf(d, d, s[k]);
+                        }
+                    }
 #pragma unroll
                 for (int w = 4; w > 0; w >>= 1)
 #pragma unroll
@@ -691,36 +714,58 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const __grid_consta
         --b;
     }
     if (b < q.weight_blocks) {
-        int64_t e = static_cast<int64_t>(b) * kFinThreads + t;
-        const int64_t n1 = static_cast<int64_t>(q.H) * q.ni, n2 = static_cast<int64_t>(q.H) * q.H,
-                      n3 = static_cast<int64_t>(q.no) * q.H;
-        if (e >= n1 + n2 + n3) return;
-        const int layer = e < n1 ? 1 : e < n1 + n2 ? 2 : 3;
-        e -= layer == 1 ? 0 : layer == 2 ? n1 : n1 + n2;
-        const int64_t i = (layer == 1 ? q.oW1 : layer == 2 ? q.oW2 : q.oW3) + e;
-        const float* ws = layer == 1 ? q.ws1 : layer == 2 ? q.ws2 : q.ws3;
-        float gi;
-        if (ws) {   // the K ranges in order
-            const int splits = layer == 1 ? q.s1 : layer == 2 ? q.s2 : q.s3;
-            const int64_t mn = layer == 1 ? n1 : layer == 2 ? n2 : n3;
-            gi = ws[e];
-            for (int z = 1; z < splits; ++z) gi += ws[z * mn + e];
-            q.grad[i] = gi;
-        } else {
-            gi = q.grad[i];
+        // a 32 x 32 tile of one weight matrix: gradients, Adam and the image
+        // by rows, the transposed image through shared memory
+        int layer = 1, tiles_k = (q.ni + 31) >> 5, tiles_h = (q.H + 31) >> 5, tile = b;
+        if (tile >= tiles_h * tiles_k) {
+            tile -= tiles_h * tiles_k;
+            layer = 2;
+            tiles_k = tiles_h;
+            if (tile >= tiles_h * tiles_h) {
+                tile -= tiles_h * tiles_h;
+                layer = 3;
+            }
         }
-        const float th = finish_param(q, i, gi);
-        if (q.images) {
-            const int ld = layer == 1 ? q.ni : q.H;
-            const int r = static_cast<int>(e / ld), k = static_cast<int>(e - static_cast<int64_t>(r) * ld);
-            if (layer == 1) {
-                put(q.w1f, r, k, th);
-            } else if (layer == 2) {
-                put(q.w2f, r, k, th);
-                put(q.w2t, k, r, th);
-            } else {
-                put(q.w3f, r, k, th);
-                put(q.w3t, k, r, th);
+        const int rows = layer == 3 ? q.no : q.H, cols = layer == 1 ? q.ni : q.H;
+        const int r0 = (tile / tiles_k) * 32, k0 = (tile % tiles_k) * 32, c = t & 31, y = t >> 5;
+        const int64_t base = layer == 1 ? q.oW1 : layer == 2 ? q.oW2 : q.oW3;
+        const float* ws = layer == 1 ? q.ws1 : layer == 2 ? q.ws2 : q.ws3;
+        const int splits = !ws ? 0 : layer == 1 ? q.s1 : layer == 2 ? q.s2 : q.s3;
+        const int64_t mn = static_cast<int64_t>(rows) * cols;
+        // every load goes out before the first is used; the K ranges are
+        // added in order
+        float part[4][kGMaxSplit];
+        ParamState st[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = r0 + y + 8 * i, k = k0 + c;
+            const bool in = r < rows && k < cols;
+            const int64_t e = in ? static_cast<int64_t>(r) * cols + k : 0;
+            st[i] = load_param(q, base + e);
+#pragma unroll
+            for (int z = 0; z < kGMaxSplit; ++z)
+                part[i][z] = (ws && z < splits) ? ws[z * mn + e] : (z == 0 ? q.grad[base + e] : 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = r0 + y + 8 * i, k = k0 + c;
+            if (r >= rows || k >= cols) continue;
+            float gi = part[i][0];
+#pragma unroll
+            for (int z = 1; z < kGMaxSplit; ++z)
+                if (z < splits) gi += part[i][z];
+            const int64_t p = base + static_cast<int64_t>(r) * cols + k;
+            if (ws) q.grad[p] = gi;
+            const float th = finish_param(q, p, gi, st[i]);
+            buf[y + 8 * i][c] = th;
+            if (q.images) put(layer == 1 ? q.w1f : layer == 2 ? q.w2f : q.w3f, r, k, th);
+        }
+        if (q.images && layer > 1) {
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int k = k0 + y + 8 * i, r = r0 + c;
+                if (r < rows && k < cols) put(layer == 2 ? q.w2t : q.w3t, k, r, buf[c][y + 8 * i]);
             }
         }
         return;
@@ -809,8 +854,8 @@ FinishArgs finish_args(cg_mlp_s* m)
     f.w2t = im.w2t;
     f.w3f = im.w3f;
     f.w3t = im.w3t;
-    const int64_t weights = static_cast<int64_t>(m->H) * (m->n_in + m->H + m->n_out);
-    f.weight_blocks = static_cast<int>((weights + kFinThreads - 1) / kFinThreads);
+    const int th = (m->H + 31) / 32;
+    f.weight_blocks = th * ((m->n_in + 31) / 32 + th + 1);   // 32 x 32 tiles of W1, W2 and W3
     return f;
 }
 
@@ -941,7 +986,7 @@ cudaError_t train_step(cg_mlp_s* m, const TrainBatch& b, float* loss_copy, const
                   {im.g2t, im.a1t, H, H, nkb, r2.kb_per, 0, 0, ws2},
                   {im.g1t, im.xt, H, ni, nkb, r1.kb_per, 0, 0, ws1}}};
         int blocks = 0, longest = 1;
-        for (q.bn = 16; q.bn <= 128; q.bn *= 2) {   // the narrowest tile whose blocks fit the SMs once
+        for (q.bn = 16; q.bn <= 128; q.bn += 16) {   // the narrowest tile whose blocks fit the SMs once
             blocks = 0;
             for (DwJob& j : q.job) {
                 j.tiles_n = (j.N + q.bn - 1) / q.bn;
