@@ -667,6 +667,10 @@ cg_status cg_plan(cg_plan_t* out, double fs, int N, int T, const double* tooth_f
         free_plan(p);
         return fail(CG_ERR_UNSUPPORTED, "n_teeth %d: no fit kernel for the tensor-core readout", T);
     }
+    if ((e = cg::setup_fit8(p)) != cudaSuccess) {
+        free_plan(p);
+        return cuda_fail(e, "standalone fit set-up");
+    }
     if ((e = setup_fast(p, zidx)) != cudaSuccess) {
         free_plan(p);
         return cuda_fail(e, "throughput path set-up");
@@ -788,6 +792,19 @@ static cg_status check_frames_i8(const cg_plan_s* p, const int8_t* frames, int64
                     "8-bit samples are read out by the pruned comb transform only (N = 2200 with every tooth "
                     "bin at +-r mod 10, readout CG_READOUT_FFT)");
     return CG_OK;
+}
+
+// The moment guess (without p0) and fit of spectra, or of magnitudes where y
+// is null.
+static cudaError_t standalone_fit(cg_plan_t p, const float* y, const float* amps, int64_t n, const float* p0,
+                                  float* params, float* rss, int16_t* iters, int16_t* status, cudaStream_t s)
+{
+    if (!p->fit8_ok) return cg::launch_fit(p, y, amps, n, p0, params, rss, iters, status, s);
+    FitOrder order{p, s};
+    cudaError_t e = order.begin();
+    if (e == cudaSuccess) e = cg::launch_fit8(p, y, amps, n, p0, params, rss, iters, status, s);
+    if (e == cudaSuccess) e = order.end();
+    return e;
 }
 
 // The whole path for int16 (sbytes = 2) or int8 (sbytes = 1) frames.
@@ -927,7 +944,7 @@ static cg_status process_impl(cg_plan_t p, const void* frames, int sbytes, int64
         // without y_dev the fit reads the magnitudes and applies the reference itself
         if (e == cudaSuccess)
             e = timed(p, CG_STAGE_FIT, s,
-                      [&] { return cg::launch_fit(p, y, amps, n, nullptr, params, rss, iters, status, s); });
+                      [&] { return standalone_fit(p, y, amps, n, nullptr, params, rss, iters, status, s); });
     }
     if (e != cudaSuccess) return cuda_fail(e, "cg_process launch");
     return CG_OK;
@@ -1006,7 +1023,7 @@ cg_status cg_fit(cg_plan_t p, const float* y, int64_t n, const float* p0, float*
     } else if (fano) {   // the Fano fit makes its own guess; p0 is not read
         e = cg::launch_fit2(p, y, nullptr, n, nullptr, nullptr, params, rss, iters, status, s);
     } else {
-        e = cg::launch_fit(p, y, nullptr, n, p0, params, rss, iters, status, s);
+        e = standalone_fit(p, y, nullptr, n, p0, params, rss, iters, status, s);
     }
     if (e == cudaSuccess && ordered) e = order.end();
     if (e != cudaSuccess) return cuda_fail(e, "cg_fit launch");

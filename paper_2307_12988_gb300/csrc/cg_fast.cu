@@ -232,6 +232,61 @@ __device__ __forceinline__ void moment_finish(Y y, U u, int T, float B0, float u
     if (flag_out) *flag_out = static_cast<int16_t>(flag);
 }
 
+// The same guess as moment_init<8> (cg_fit.cuh) forms it, left on the
+// normalised abscissa: lane l of eight adds up teeth l, l + 8, ... in order and
+// the partial sums are added over lane distances 4, 2, 1; here one lane keeps
+// the eight partial sums.  The largest deviation keeps its first index, and
+// with none (every d undefined) the sign is positive.
+template <class Y, class U>
+__device__ __forceinline__ void moment_finish8(Y y, U u, int T, float B0, float u_mid, float du, float span, float* po)
+{
+    float best = -1.f, dbest = 0.f, wmaxp = 0.f, wmaxn = 0.f;
+    float Wp[8], Up[8], Wn[8], Un[8];
+#pragma unroll
+    for (int l = 0; l < 8; ++l) Wp[l] = Up[l] = Wn[l] = Un[l] = 0.f;
+    for (int k0 = 0; k0 < T; k0 += 8) {
+#pragma unroll
+        for (int l = 0; l < 8; ++l) {
+            const int k = k0 + l;
+            if (k >= T) break;
+            const float d = y(k) - B0;
+            const float dv = fabsf(d);
+            if (dv > best) {
+                best = dv;
+                dbest = d;
+            }
+            const float wp = fmaxf(d, 0.f), wn = fmaxf(-d, 0.f);
+            const float uk = u(k);
+            Wp[l] += wp;
+            Up[l] = fmaf(wp, uk, Up[l]);
+            wmaxp = fmaxf(wmaxp, wp);
+            Wn[l] += wn;
+            Un[l] = fmaf(wn, uk, Un[l]);
+            wmaxn = fmaxf(wmaxn, wn);
+        }
+    }
+    const bool pos = dbest >= 0.f;
+    auto total = [&](const float (&p)[8], const float (&n)[8]) {
+        float v[8];
+#pragma unroll
+        for (int l = 0; l < 8; ++l) v[l] = pos ? p[l] : n[l];
+        return ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+    };
+    const float W = total(Wp, Wn), Wu = total(Up, Un), wmax = pos ? wmaxp : wmaxn;
+    if (!(W > 0.f)) {
+        po[0] = u_mid;
+        po[1] = 0.5f * du;
+        po[2] = 0.f;
+    } else {
+        const float A0 = (pos ? 1.0f : -1.0f) * wmax;
+        const float g0 = W * du / (3.14159265358979f * fabsf(A0));
+        po[0] = Wu / W;
+        po[1] = fminf(fmaxf(g0, 0.5f * du), 0.5f * span);
+        po[2] = A0;
+    }
+    po[3] = B0;
+}
+
 // A warp takes 32 consecutive frames at a time: their normalised spectra
 // (row stride odd, so the lanes' reads of one tooth fall on distinct banks)
 // arrive in shared memory by one bulk copy per 32 rows, double-buffered so the
@@ -241,8 +296,9 @@ __device__ __forceinline__ void moment_finish(Y y, U u, int T, float B0, float u
 // largest deviation, centroid / extreme / area of the one-signed excess.
 // NOUT > 0: the outer set has NOUT teeth (a compile-time count): its median
 // comes from the merge network pruned to the two middle ranks; NOUT = 0 sorts
-// the NPAD wires (a.n_outer real, the rest +infinity) fully
-template <int NPAD, int NOUT>
+// the NPAD wires (a.n_outer real, the rest +infinity) fully.
+// EIGHT: the guess of the fit at eight lanes per frame (moment_finish8)
+template <int NPAD, int NOUT, bool EIGHT = false>
 __global__ void __launch_bounds__(128) init_kernel(InitArgs a)
 {
     extern __shared__ __align__(16) float ism[];
@@ -422,8 +478,32 @@ __global__ void __launch_bounds__(128) init_kernel(InitArgs a)
                 }
                 B0 = 0.5f * (vlo + vhi);
             }
-            moment_finish(yk, [&](int k) { return us[k]; }, T, B0, a.u_mid, a.du, a.span, a.x_mid, a.x_scale,
-                          a.p0_out + fo * 4, a.flag_out ? a.flag_out + fo : nullptr);
+            auto uk = [&](int k) { return us[k]; };
+            if constexpr (EIGHT) {
+                // moment_init ranks by counting: with an undefined value among
+                // the outer teeth the networks give another pair of middle values
+                bool nan = false;
+                for (int i = 0; i < a.n_outer; ++i) nan |= isnan(yk(outer[i]));
+                if (nan) {
+                    const int rlo = (a.n_outer - 1) >> 1, rhi = a.n_outer >> 1;
+                    float vlo = 0.f, vhi = 0.f;
+                    for (int j = 0; j < a.n_outer; ++j) {
+                        const float vj = yk(outer[j]);
+                        int rank = 0;
+                        for (int i = 0; i < a.n_outer; ++i) {
+                            const float vi = yk(outer[i]);
+                            rank += (vi < vj) || (vi == vj && i < j);
+                        }
+                        if (rank == rlo) vlo += vj;
+                        if (rank == rhi) vhi += vj;
+                    }
+                    B0 = 0.5f * (vlo + vhi);
+                }
+                moment_finish8(yk, uk, T, B0, a.u_mid, a.du, a.span, a.p0_out + fo * 4);
+            } else {
+                moment_finish(yk, uk, T, B0, a.u_mid, a.du, a.span, a.x_mid, a.x_scale, a.p0_out + fo * 4,
+                              a.flag_out ? a.flag_out + fo : nullptr);
+            }
         }
     }
     // no copy may land after the block exits
@@ -752,23 +832,25 @@ void* fast_readout_ptr(int Q, int sample_bytes)
 
 // the outer-set sizes of the workload geometries (21, 99, 201 and 221 teeth:
 // the outer fifth with ties kept) have their own pruned median
-void* init_ptr(int npad, int n_outer)
+template <bool EIGHT>
+static void* init_fn(int npad, int n_outer)
 {
     switch (n_outer) {
-    case 6: return reinterpret_cast<void*>(&init_kernel<8, 6>);
-    case 20: return reinterpret_cast<void*>(&init_kernel<32, 20>);
-    case 42: return reinterpret_cast<void*>(&init_kernel<64, 42>);
-    case 46: return reinterpret_cast<void*>(&init_kernel<64, 46>);
+    case 6: return reinterpret_cast<void*>(&init_kernel<8, 6, EIGHT>);
+    case 20: return reinterpret_cast<void*>(&init_kernel<32, 20, EIGHT>);
+    case 42: return reinterpret_cast<void*>(&init_kernel<64, 42, EIGHT>);
+    case 46: return reinterpret_cast<void*>(&init_kernel<64, 46, EIGHT>);
     default: break;
     }
     switch (npad) {
-    case 8: return reinterpret_cast<void*>(&init_kernel<8, 0>);
-    case 16: return reinterpret_cast<void*>(&init_kernel<16, 0>);
-    case 32: return reinterpret_cast<void*>(&init_kernel<32, 0>);
-    case 64: return reinterpret_cast<void*>(&init_kernel<64, 0>);
+    case 8: return reinterpret_cast<void*>(&init_kernel<8, 0, EIGHT>);
+    case 16: return reinterpret_cast<void*>(&init_kernel<16, 0, EIGHT>);
+    case 32: return reinterpret_cast<void*>(&init_kernel<32, 0, EIGHT>);
+    case 64: return reinterpret_cast<void*>(&init_kernel<64, 0, EIGHT>);
     default: return nullptr;
     }
 }
+void* init_ptr(int npad, int n_outer, bool eight) { return eight ? init_fn<true>(npad, n_outer) : init_fn<false>(npad, n_outer); }
 
 template <int G, int PPL, bool EXACT, int MODEL = 0>
 static void* fit2_fn() { return reinterpret_cast<void*>(&fit2_kernel<G, PPL, EXACT, MODEL>); }
@@ -877,7 +959,7 @@ cudaError_t launch_fast_readout_i8(const cg_plan_s* p, const int8_t* frames, int
 
 cudaError_t launch_init(const cg_plan_s* p, const float* y, const float* amps, int64_t n,
                         float* p0_out, int16_t* flag_out, cudaStream_t s, const int* list,
-                        const int* list_n)
+                        const int* list_n, bool eight)
 {
     InitArgs a = p->ia;
     a.n = n;
@@ -892,7 +974,7 @@ cudaError_t launch_init(const cg_plan_s* p, const float* y, const float* amps, i
     const int64_t tasks = (n + 31) / 32;
     const int grid = static_cast<int>(tasks < p->grid_init ? tasks : p->grid_init);
     void* args[] = {&a};
-    return cudaLaunchKernel(init_ptr(p->init_npad, p->n_outer), dim3(grid), dim3(128), args, p->init_smem, s);
+    return cudaLaunchKernel(init_ptr(p->init_npad, p->n_outer, eight), dim3(grid), dim3(128), args, p->init_smem, s);
 }
 
 cudaError_t launch_fit2(const cg_plan_s* p, const float* y, const float* amps, int64_t n,

@@ -1,0 +1,424 @@
+// cg_fit8.cu -- the standalone Levenberg-Marquardt fit at eight lanes per
+// frame (cg_fit, and the fit of CG_PATH_SPLIT), two frames per lane group.
+//
+// Paper ("Data Capture and Processing", fit paragraphs): each normalised
+// spectrum is fit by Levenberg-Marquardt, at most 20 iterations, tolerance
+// 1e-6.  Arithmetic, sums and decisions are those of fit_group<8>
+// (cg_fit.cuh): lane l of a frame's eight adds up teeth l, l + 8, ... in
+// order, the eight partial sums are added over lane distances 4, 2, 1.  What
+// differs is how the work lies on the warp:
+//  * a group of eight lanes evaluates two frames at once, one in each half of
+//    packed FP32x2 operations;
+//  * the 14 sums of the first frame end in its lower four lanes, those of the
+//    second in the upper four (the exchange over distance 4 does both), so one
+//    pass of the 4 x 4 solve and of the decisions serves both frames -- and
+//    eight frames per warp, where every lane of a group repeated one frame's;
+//  * each half pulls its next frame when its own is done; the row arrives
+//    meanwhile by one bulk copy into the half's other slot, so no frame waits
+//    for another's iterations;
+//  * the moment guess runs before, one lane per frame (init_kernel), and
+//    leaves its starting point (normalised abscissa) in params.
+//
+// What bounds it: instruction issue (65 % active; about 970 warp instructions
+// per evaluation of eight frames of 99 teeth, 390 of them in the teeth's loop,
+// where fit_group spent 1,340 on two times four).  10^5 spectra of 99 teeth:
+// 159 us in fit_kernel, which also held every block for its slowest frame;
+// 88 us here and 10 for the guess.
+#include <algorithm>
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "cg_fit.cuh"
+#include "cg_internal.h"
+#include "cg_tc.cuh"
+
+namespace cg {
+
+namespace {
+
+constexpr int kWarps8 = 4;       // warps per block
+constexpr int kSlots8 = 16;      // row slots per warp: two per frame in flight
+
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+struct Fit8Args {
+    int64_t n;
+    int T, RS, task;                // teeth, slot stride (floats), frames per warp task
+    const float* y;                 // [n][T] or null (then amps * inv_ref)
+    const float* amps;
+    const float* inv_ref;
+    const float* u;
+    const float* p0;                // [n][4]: abscissa units, or (guessed) on the normalised abscissa
+    int guessed;
+    unsigned long long* counter;
+    float x_mid, x_scale;
+    int max_iter;
+    float tol, lambda0;
+    float *params, *rss;
+    int16_t *iters, *status;
+    int* err;
+};
+
+// the 14 sums of accum_point for one tooth of two frames
+__device__ __forceinline__ void accum_pair(float u, float2 y, float2 c, float2 g2, float2 nA, float2 nB, float2 (&s)[14])
+{
+    const float2 d = add2(make_float2(u, u), neg2(c));
+    const float2 D = fma2(d, d, g2);
+    const float2 q = make_float2(rcp_fast(D.x), rcp_fast(D.y));
+    const float2 L = mul2(g2, q);
+    const float2 r = fma2(nA, L, add2(y, nB));
+    const float2 t = mul2(L, q);
+    const float2 jc = mul2(t, d);
+    const float2 jg = mul2(jc, d);
+    s[0] = fma2(L, L, s[0]);
+    s[1] = fma2(L, jc, s[1]);
+    s[2] = fma2(L, jg, s[2]);
+    s[3] = add2(s[3], L);
+    s[4] = fma2(jc, jc, s[4]);
+    s[5] = fma2(jc, jg, s[5]);
+    s[6] = add2(s[6], jc);
+    s[7] = fma2(jg, jg, s[7]);
+    s[8] = add2(s[8], jg);
+    s[9] = fma2(L, r, s[9]);
+    s[10] = fma2(jc, r, s[10]);
+    s[11] = fma2(jg, r, s[11]);
+    s[12] = add2(s[12], r);
+    s[13] = fma2(r, r, s[13]);
+}
+
+// sums over the eight lanes, distances 4, 2, 1: the lower four lanes get the
+// first frame's 14 sums, the upper four the second's
+__device__ __forceinline__ void reduce_pair(const float2 (&s)[14], LmSums& S)
+{
+    const int lane = threadIdx.x & 31;
+    const bool hi = (lane & 4) != 0;
+    float a[14];
+#pragma unroll
+    for (int i = 0; i < 14; ++i) {
+        const float send = hi ? s[i].x : s[i].y, keep = hi ? s[i].y : s[i].x;
+        a[i] = keep + __shfl_xor_sync(kFull, send, 4);
+    }
+    // distance 2: each keeps seven; distance 1: four or three of those
+    const bool b2 = (lane & 2) != 0;
+    float b[8];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        const float send = b2 ? a[i] : a[i + 7], keep = b2 ? a[i + 7] : a[i];
+        b[i] = keep + __shfl_xor_sync(kFull, send, 2);
+    }
+    b[7] = 0.f;
+    const bool b1 = (lane & 1) != 0;
+    float c[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float send = b1 ? b[i] : b[i + 4], keep = b1 ? b[i + 4] : b[i];
+        c[i] = keep + __shfl_xor_sync(kFull, send, 1);
+    }
+    const int base = lane & ~3;
+#pragma unroll
+    for (int i = 0; i < 14; ++i) {
+        const int in7 = i % 7, owner = (i / 7) * 2 + in7 / 4;
+        S.v[i] = __shfl_sync(kFull, c[in7 % 4], base + owner);
+    }
+}
+
+template <bool SCALE>
+__global__ void __launch_bounds__(32 * kWarps8, 4) fit8_kernel(Fit8Args a)
+{
+    extern __shared__ __align__(16) float f8sm[];
+    const int T = a.T;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int gl = lane & 7, own = lane & 3, leader = lane & ~3, half = lane >> 2;   // half: 0 .. 7, a frame each
+    float* slots = f8sm + warp * kSlots8 * a.RS;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(f8sm + kWarps8 * kSlots8 * a.RS) + warp * kSlots8;
+    float* us = reinterpret_cast<float*>(reinterpret_cast<uint64_t*>(f8sm + kWarps8 * kSlots8 * a.RS) + kWarps8 * kSlots8);
+    float* iref = us + T;
+    for (int i = threadIdx.x; i < T; i += blockDim.x) {
+        us[i] = a.u[i];
+        iref[i] = SCALE ? a.inv_ref[i] : 1.0f;
+    }
+    // (a half without a frame evaluates whatever its slot holds: finite values)
+    for (int i = threadIdx.x; i < kWarps8 * kSlots8 * a.RS; i += blockDim.x) f8sm[i] = 0.f;
+    if (lane < kSlots8) tc::mbar_init(&bars[lane], 1);
+    tc::fence_mbar_init();
+    tc::fence_proxy_async_smem();
+    __syncthreads();
+
+    const float* src_base = SCALE ? a.amps : a.y;
+    const uintptr_t buf_lo = reinterpret_cast<uintptr_t>(src_base);
+    const uintptr_t buf_hi = buf_lo + static_cast<uintptr_t>(a.n) * T * sizeof(float);
+    const int64_t n = a.n;
+    bool first = true;
+    int64_t next = 0, end = 0;
+    int64_t f = -1, fn = -1;     // frame being fit; next frame (its copy in flight)
+    float pn[4] = {0.f, 1.f, 0.f, 0.f};
+    int cs = 0, oc = 0, on = 0;
+    uint32_t ph = 0;
+    float p[4] = {0.f, 1.f, 0.f, 0.f};
+    float lambda = a.lambda0, chi2 = 0.f;
+    Normal Nm;
+#pragma unroll
+    for (int i = 0; i < 10; ++i) Nm.H[i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) Nm.b[i] = 0.f;
+    int it = 0, st = kMaxIter, flag = 0;
+    bool fresh = false, failed = false;
+
+    while (true) {
+        // ---- a half without a frame starts its next one ----
+        if (f < 0 && fn >= 0) {
+            const int nx = cs ^ 1;
+            const int sl = half + 8 * nx;
+            if (!tc::mbar_wait(&bars[sl], (ph >> nx) & 1u, 1u << 22)) failed = true;
+            ph ^= 1u << nx;
+            cs = nx;
+            f = fn;
+            oc = on;
+            fn = -1;
+            fresh = true;
+            flag = 0;
+            if (a.guessed) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) p[i] = pn[i];
+                flag = pn[2] == 0.f ? kInitFlat : 0;   // (only a flat spectrum's guess has no amplitude)
+            } else {
+                p[0] = (pn[0] - a.x_mid) / a.x_scale;
+                p[1] = pn[1] / a.x_scale;
+                p[2] = pn[2];
+                p[3] = pn[3];
+            }
+            lambda = a.lambda0;
+            it = 0;
+            st = kMaxIter;
+        }
+        if (__any_sync(kFull, failed)) break;
+        // ---- halves without a next frame claim one; its row goes to the free slot ----
+        unsigned need = __ballot_sync(kFull, own == 0 && fn < 0);
+        while (need != 0 && next < n) {
+            if (next >= end) {
+                unsigned long long t = static_cast<unsigned>(warp) * gridDim.x + blockIdx.x;
+                if (!first) {
+                    t = static_cast<unsigned>(kWarps8) * gridDim.x;
+                    if (t * a.task < static_cast<unsigned long long>(n)) {   // (else no task is left to claim)
+                        if (lane == 0) t += atomicAdd(a.counter, 1ULL);
+                        t = __shfl_sync(kFull, t, 0);
+                    }
+                }
+                first = false;
+                next = static_cast<int64_t>(t) * a.task;
+                if (next >= n) {
+                    next = end = n;
+                    break;
+                }
+                end = next + a.task < n ? next + a.task : n;
+            }
+            const int cnt = __popc(need);
+            const int64_t avail = end - next;
+            const int take = static_cast<int>(avail < cnt ? avail : cnt);
+            const int rank = __popc(need & ((1u << leader) - 1u));
+            if (((need >> leader) & 1u) && rank < take) {
+                fn = next + rank;
+                const float* q = a.p0 + fn * 4;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) pn[i] = q[i];
+                const float* src = src_base + fn * T;
+                const uintptr_t ad = reinterpret_cast<uintptr_t>(src);
+                const uintptr_t a16 = ad & ~static_cast<uintptr_t>(15);
+                const uintptr_t e16 = (ad + 4u * T + 15u) & ~static_cast<uintptr_t>(15);
+                on = static_cast<int>((ad - a16) >> 2);
+                const int sl = half + 8 * (cs ^ 1);
+                float* dst = slots + sl * a.RS;
+                if (own == 0) {
+                    if (a16 >= buf_lo && e16 <= buf_hi) {
+                        tc::fence_proxy_async_smem();   // the slot's last reads precede this write
+                        tc::mbar_arrive_expect_tx(&bars[sl], static_cast<uint32_t>(e16 - a16));
+                        tc::bulk_g2s(dst, reinterpret_cast<const void*>(a16), static_cast<uint32_t>(e16 - a16), &bars[sl]);
+                    } else {
+                        // the first or last row of an unaligned buffer: its
+                        // window would leave the buffer
+                        for (int k = 0; k < T; ++k) dst[on + k] = src[k];
+                        tc::mbar_arrive(&bars[sl]);
+                    }
+                }
+            }
+            next += take;
+            need = __ballot_sync(kFull, own == 0 && fn < 0);
+        }
+        if (!__any_sync(kFull, f >= 0 || fn >= 0)) break;
+
+        // ---- trial point of this half's frame ----
+        float pt[4] = {p[0], p[1], p[2], p[3]};
+        bool done = false;
+        if (f >= 0 && !fresh) {
+            float delta[4] = {0.f, 0.f, 0.f, 0.f};
+            if (lm_solve4(Nm, lambda, delta)) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) pt[i] = __fadd_rn(p[i], delta[i]);
+            } else {
+                st = kSingular;
+                done = true;
+            }
+        }
+        // ---- sums of both frames of the group at their trial points ----
+        float2 s[14];
+        {
+            const bool hi = (lane & 4) != 0;
+            auto both = [&](float v) {   // (first frame's, second frame's)
+                const float o = __shfl_xor_sync(kFull, v, 4);
+                return make_float2(hi ? o : v, hi ? v : o);
+            };
+            const float2 c = both(pt[0]), g2 = both(pt[1] * pt[1]), nA = neg2(both(pt[2])), nB = neg2(both(pt[3]));
+            const int mine = (half + 8 * cs) * a.RS + oc, other = __shfl_xor_sync(kFull, mine, 4);
+            const float* ra = slots + (hi ? other : mine);
+            const float* rb = slots + (hi ? mine : other);
+#pragma unroll
+            for (int i = 0; i < 14; ++i) s[i] = make_float2(0.f, 0.f);
+#pragma unroll 2
+            for (int k = gl; k < T; k += 8) {
+                float2 y = make_float2(ra[k], rb[k]);
+                if (SCALE) y = make_float2(__fmul_rn(y.x, iref[k]), __fmul_rn(y.y, iref[k]));
+                accum_pair(us[k], y, c, g2, nA, nB, s);
+            }
+        }
+        LmSums S;
+        reduce_pair(s, S);
+        // ---- decisions (as fit_group) ----
+        if (f >= 0 && !done) {
+            const float chi2t = S.v[13];
+            if (fresh) {
+                chi2 = chi2t;
+                make_normal(S, pt[1], pt[2], T, Nm);
+                if (!(chi2t < INFINITY)) {
+                    st = kNonfinite;
+                    done = true;
+                }
+                if (a.max_iter <= 0) done = true;
+            } else {
+                ++it;
+                if (!(chi2t < INFINITY)) {
+                    lambda *= 10.0f;
+                } else if (chi2_settled(chi2t, chi2, a.tol, p[2], p[3])) {
+                    if (chi2t <= chi2) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) p[i] = pt[i];
+                        chi2 = chi2t;
+                    }
+                    st = kConverged;
+                    done = true;
+                } else if (chi2t < chi2) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) p[i] = pt[i];
+                    chi2 = chi2t;
+                    make_normal(S, pt[1], pt[2], T, Nm);
+                    lambda *= 0.1f;
+                } else {
+                    lambda *= 10.0f;
+                }
+                if (!done && it >= a.max_iter) done = true;
+            }
+        }
+        fresh = false;
+        if (f >= 0 && done) {
+            if (own == 0) {
+                float* po = a.params + f * 4;
+                po[0] = fmaf(a.x_scale, p[0], a.x_mid);
+                po[1] = a.x_scale * fabsf(p[1]);
+                po[2] = p[2];
+                po[3] = p[3];
+                if (a.rss) a.rss[f] = chi2;
+                if (a.iters) a.iters[f] = static_cast<int16_t>(it);
+                if (a.status) a.status[f] = static_cast<int16_t>(st | flag);
+            }
+            f = -1;
+        }
+    }
+    // no copy may land after the block exits (a failed wait only)
+    if (fn >= 0) {
+        const int nx = cs ^ 1;
+        tc::mbar_wait(&bars[half + 8 * nx], (ph >> nx) & 1u, 1u << 22);
+    }
+    if (failed && lane == 0 && a.err) atomicExch(a.err, 4);
+}
+
+int row_window(int T)   // floats of the largest 16-byte window around a row, an odd multiple of 4
+{
+    const int w = (4 * T + 12 + 15) / 16 * 4;
+    return w % 8 == 4 ? w : w + 4;
+}
+int fit8_smem(int T) { return 4 * kWarps8 * kSlots8 * row_window(T) + 8 * kWarps8 * kSlots8 + 8 * T; }
+
+}  // namespace
+
+cudaError_t setup_fit8(cg_plan_s* p)
+{
+    p->fit8_ok = false;
+    if (p->G != 8 || !p->fit_ok) return cudaSuccess;
+    int most = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
+    if (e != cudaSuccess) return e;
+    const int bytes = fit8_smem(p->T);
+    if (bytes > most) return cudaSuccess;
+    int occ[2] = {};
+    for (int i = 0; i < 2; ++i) {
+        void* fn = i ? reinterpret_cast<void*>(&fit8_kernel<true>) : reinterpret_cast<void*>(&fit8_kernel<false>);
+        if ((e = raise_smem_limit(fn, bytes)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[i], fn, 32 * kWarps8, bytes)) != cudaSuccess) return e;
+        if (occ[i] < 1) return cudaSuccess;
+    }
+    if ((e = raise_smem_limit(init_ptr(p->init_npad, p->n_outer, true), p->init_smem)) != cudaSuccess) return e;
+    p->grid_fit8 = p->num_sms * std::min(occ[0], occ[1]);
+    p->fit8_ok = true;
+    return cudaSuccess;
+}
+
+cudaError_t launch_fit8(const cg_plan_s* p, const float* y, const float* amps, int64_t n, const float* p0,
+                        float* params, float* rss, int16_t* iters, int16_t* status, cudaStream_t s)
+{
+    const FitArgs fa = make_fit_args(p);
+    if (!p0) {
+        const cudaError_t e = launch_init(p, y, amps, n, params, nullptr, s, nullptr, nullptr, true);
+        if (e != cudaSuccess) return e;
+    }
+    Fit8Args a{};
+    a.n = n;
+    a.T = p->T;
+    a.RS = row_window(p->T);
+    // frames per task as in launch_fit3: two per frame in flight, fewer where
+    // the schedulers would otherwise have none
+    const int64_t schedulers = 4 * static_cast<int64_t>(p->num_sms);
+    a.task = static_cast<int>(std::min<int64_t>(16, (n + schedulers - 1) / schedulers));
+    a.y = y;
+    a.amps = amps;
+    a.inv_ref = fa.inv_ref;
+    a.u = fa.u;
+    a.p0 = p0 ? p0 : params;
+    a.guessed = p0 ? 0 : 1;
+    a.counter = p->d.fit_counter;
+    a.x_mid = fa.x_mid;
+    a.x_scale = fa.x_scale;
+    a.max_iter = fa.max_iter;
+    a.tol = fa.tol;
+    a.lambda0 = fa.lambda0;
+    a.params = params;
+    a.rss = rss;
+    a.iters = iters;
+    a.status = status;
+    a.err = p->d.err;
+    const int64_t tasks = (n + a.task - 1) / a.task;
+    const int grid = static_cast<int>(tasks < p->grid_fit8 ? tasks : p->grid_fit8);
+    if (tasks > static_cast<int64_t>(grid) * kWarps8) {
+        const cudaError_t e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s);
+        if (e != cudaSuccess) return e;
+    }
+    const int smem = fit8_smem(p->T);
+    if (y)
+        fit8_kernel<false><<<grid, 32 * kWarps8, smem, s>>>(a);
+    else
+        fit8_kernel<true><<<grid, 32 * kWarps8, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace cg

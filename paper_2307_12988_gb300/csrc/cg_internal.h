@@ -302,6 +302,8 @@ struct cg_plan_s {
     int Q = 0;               // L = 10 Q
     bool fit3_ok = false;    // shared-memory LM kernel (cg_fit3.cu) configured
     int fit3_G = 0, fit3_warps = 0, fit3_smem = 0, grid_fit3 = 0;
+    bool fit8_ok = false;    // standalone fit at eight lanes, two frames a group (cg_fit8.cu)
+    int grid_fit8 = 0;
     int G2 = 4;              // LM lanes per frame of the register-resident fit
     int PPL = 0;             // LM points per lane
     bool ppl_exact = false;  // PPL == ceil(T / G2)
@@ -363,7 +365,7 @@ FitArgs make_fit_args(const cg_plan_s* p);
 
 // throughput path (cg_fast.cu)
 void* fast_readout_ptr(int Q, int sample_bytes = 2);
-void* init_ptr(int npad, int n_outer);
+void* init_ptr(int npad, int n_outer, bool eight = false);
 int init_npad(int n_outer);
 void* fit2_ptr(int G, int PPL, bool exact, int model);
 int fit2_ppl(int G, int T, bool* exact, int model);
@@ -386,7 +388,7 @@ struct FitLaunch {
 };
 cudaError_t launch_init(const cg_plan_s* p, const float* y, const float* amps, int64_t n,
                         float* p0_out, int16_t* flag_out, cudaStream_t s, const int* list,
-                        const int* list_n);
+                        const int* list_n, bool eight = false);
 cudaError_t launch_fit2(const cg_plan_s* p, const float* y, const float* amps, int64_t n,
                         const float* p0, const int16_t* flags_in, float* params, float* rss,
                         int16_t* iters, int16_t* status, cudaStream_t s,
@@ -395,6 +397,12 @@ cudaError_t launch_fit2(const cg_plan_s* p, const float* y, const float* amps, i
 // arguments launch_fit2 prepared
 cudaError_t setup_fit3(cg_plan_s* p);
 cudaError_t launch_fit3(const cg_plan_s* p, Fit2Args a, cudaStream_t s);
+
+// standalone fit at eight lanes per frame (cg_fit8.cu); shares the plan's task
+// counter
+cudaError_t setup_fit8(cg_plan_s* p);
+cudaError_t launch_fit8(const cg_plan_s* p, const float* y, const float* amps, int64_t n, const float* p0,
+                        float* params, float* rss, int16_t* iters, int16_t* status, cudaStream_t s);
 
 // learned initial guess (cg_mlp_tc.cu)
 cudaError_t setup_mlp(cg_plan_s* p, const unsigned char* blob, size_t bytes, const char** why);
