@@ -42,6 +42,7 @@ __global__ void __launch_bounds__(128) fast_readout_kernel(FastArgs a)
     // per output (balanced over the block) and the Q-point DFTs read it back
     constexpr bool kSplitFold = Q > 11;
     extern __shared__ __align__(16) unsigned char sm[];
+    tc::pdl_start();
     float2* twL = reinterpret_cast<float2*>(sm + a.sm_twL);
     float2* twN = reinterpret_cast<float2*>(sm + a.sm_twN);
     int* tom = reinterpret_cast<int*>(sm + a.sm_tom);
@@ -302,6 +303,7 @@ template <int NPAD, int NOUT, bool EIGHT = false>
 __global__ void __launch_bounds__(128) init_kernel(InitArgs a)
 {
     extern __shared__ __align__(16) float ism[];
+    tc::pdl_start();
     const int T = a.T, TS = a.row_stride;
     float* us = ism;
     float* iref = us + T;
@@ -324,6 +326,7 @@ __global__ void __launch_bounds__(128) init_kernel(InitArgs a)
     }
     for (int i = threadIdx.x; i < a.n_outer; i += blockDim.x) outer[i] = a.outer_idx[i];
     __syncthreads();
+    tc::pdl_wait();
     constexpr OddEvenNet<NPAD> net{};
     const int64_t nwarps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
     int64_t n = a.n;
@@ -974,7 +977,7 @@ cudaError_t launch_init(const cg_plan_s* p, const float* y, const float* amps, i
     const int64_t tasks = (n + 31) / 32;
     const int grid = static_cast<int>(tasks < p->grid_init ? tasks : p->grid_init);
     void* args[] = {&a};
-    return cudaLaunchKernel(init_ptr(p->init_npad, p->n_outer, eight), dim3(grid), dim3(128), args, p->init_smem, s);
+    return launch_dependent(init_ptr(p->init_npad, p->n_outer, eight), dim3(grid), dim3(128), args, p->init_smem, s);
 }
 
 cudaError_t launch_fit2(const cg_plan_s* p, const float* y, const float* amps, int64_t n,

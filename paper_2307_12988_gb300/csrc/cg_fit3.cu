@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
     for (int i = lane; i < S::kSlots; i += 32) tc::mbar_init(&bars[i], 1);
     tc::fence_mbar_init();
     __syncthreads();
+    tc::pdl_wait();
 
     // the last pair of a lane may hold teeth beyond T: their terms are zeroed
     const int ilast = gl + G * (S::kPPL - 1);
@@ -681,7 +682,7 @@ cudaError_t launch_fit3(const cg_plan_s* p, Fit2Args a, cudaStream_t s)
         if (e != cudaSuccess) return e;
     }
     void* args[] = {&a};
-    return cudaLaunchKernel(fi->fn(), dim3(grid), dim3(32 * p->fit3_warps), args, p->fit3_smem, s);
+    return launch_dependent(fi->fn(), dim3(grid), dim3(32 * p->fit3_warps), args, p->fit3_smem, s);
 }
 
 }  // namespace cg

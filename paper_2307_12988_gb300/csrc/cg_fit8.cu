@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(32 * kWarps8, 4) fit8_kernel(Fit8Args a)
     tc::fence_mbar_init();
     tc::fence_proxy_async_smem();
     __syncthreads();
+    tc::pdl_wait();
 
     const float* src_base = SCALE ? a.amps : a.y;
     const uintptr_t buf_lo = reinterpret_cast<uintptr_t>(src_base);
@@ -413,12 +414,9 @@ cudaError_t launch_fit8(const cg_plan_s* p, const float* y, const float* amps, i
         const cudaError_t e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s);
         if (e != cudaSuccess) return e;
     }
-    const int smem = fit8_smem(p->T);
-    if (y)
-        fit8_kernel<false><<<grid, 32 * kWarps8, smem, s>>>(a);
-    else
-        fit8_kernel<true><<<grid, 32 * kWarps8, smem, s>>>(a);
-    return cudaGetLastError();
+    void* args[] = {&a};
+    void* fn = y ? reinterpret_cast<void*>(&fit8_kernel<false>) : reinterpret_cast<void*>(&fit8_kernel<true>);
+    return launch_dependent(fn, dim3(grid), dim3(32 * kWarps8), args, fit8_smem(p->T), s);
 }
 
 }  // namespace cg

@@ -30,6 +30,7 @@
 #include "cg_fft.cuh"
 #include "cg_internal.h"
 #include "cg_stage.cuh"
+#include "cg_tc.cuh"
 
 namespace cg {
 
@@ -146,6 +147,7 @@ template <bool PAD>
 __global__ void __launch_bounds__(kGenThreads, 6) general_readout_kernel(const __grid_constant__ GenArgs a)
 {
     extern __shared__ __align__(16) unsigned char gsm[];
+    tc::pdl_start();
     float2* tw = reinterpret_cast<float2*>(gsm);
     float2* twn1 = reinterpret_cast<float2*>(gsm + a.sm_n1);   // coset: [L] W_N^(r n1), then [M] W_M^(r n2)
     float2* twb = reinterpret_cast<float2*>(gsm + a.sm_b);     // full: [T] W_N^(b_k)

@@ -322,7 +322,7 @@ struct cg_plan_s {
     // learned initial guess
     bool mlp_ok = false;
     CUtensorMap mlp_map{};
-    int mlp_smem = 0;
+    int mlp_smem = 0, mlp_clusters = 0;
     cg::MlpArgs ma{};
     // device address of the allocation-free reference scratch (set by cg_plan)
     double* noalloc_scratch = nullptr;
@@ -434,5 +434,10 @@ void set_last_error(const char* msg);
 // belongs to the function on the device, so every plan shares it: one plan
 // must not shrink what another plan's launches need.
 cudaError_t raise_smem_limit(const void* fn, int bytes);
+
+// Launches a kernel whose prologue may overlap the end of the kernel before it
+// in the stream (programmatic dependent launch: the kernel calls pdl_wait
+// before it touches anything the others write).
+cudaError_t launch_dependent(const void* fn, dim3 grid, dim3 block, void** args, size_t smem, cudaStream_t s);
 
 }  // namespace cg

@@ -37,6 +37,7 @@
 #include "cg_internal.h"
 #include "cg_net.cuh"
 #include "cg_stage.cuh"
+#include "cg_tc.cuh"
 
 namespace cg {
 
@@ -139,6 +140,7 @@ template <int LPR>
 __global__ void __launch_bounds__(kMedThreads, 4) median_init_kernel(MedianArgs a)
 {
     extern __shared__ __align__(16) unsigned char msm[];
+    tc::pdl_start();
     const int R = a.R, T = a.T, S = a.S;
     const int64_t n = a.n;
     const int W = T + 6;                                               // padded columns
@@ -170,6 +172,7 @@ __global__ void __launch_bounds__(kMedThreads, 4) median_init_kernel(MedianArgs 
         rhi = j1 + 3 < n ? j1 + 3 : n;
     };
     int off = 0;
+    tc::pdl_wait();
     if (static_cast<int64_t>(blockIdx.x) * R < n) {
         int64_t rlo, rhi;
         row_range(blockIdx.x, rlo, rhi);
@@ -425,7 +428,7 @@ cudaError_t launch_median(const cg_plan_s* p, const float* y, const float* amps,
     const int64_t nb = (n + m.R - 1) / m.R;
     const int grid = static_cast<int>(nb < p->grid_median ? nb : p->grid_median);
     void* args[] = {&m};
-    return cudaLaunchKernel(median_fn(m.T), dim3(grid), dim3(kMedThreads), args, m.sm_total, s);
+    return launch_dependent(median_fn(m.T), dim3(grid), dim3(kMedThreads), args, m.sm_total, s);
 }
 
 }  // namespace cg

@@ -6,7 +6,9 @@
 //     p0 = (W3 a2 + b3) * out_scale + out_mean              (FP32 on the CUDA cores)
 // with W1 (K zero-padded to 64 * nkb) and W2 stored as one BF16 matrix
 // [512][256], streamed from L2 by TMA in 128-row x 64-column chunks through an
-// S-stage mbarrier ring.  Persistent blocks, one per SM, with warp roles:
+// S-stage mbarrier ring; two blocks form a cluster, and each loads half of
+// every chunk into both (the 256 KB per tile of 128 spectra otherwise come at
+// the L2's 18 bytes a cycle and SM: 15,000 of a tile's 25,000 cycles).  Persistent blocks, one per SM, with warp roles:
 //   warps 0-7    epilogues: warp w reads TMEM lanes 32 (w % 4).. (rows) and
 //                column half w / 4; layer 1: bias, GELU, BF16 into the a1
 //                tile; layer 2: bias, GELU and the FP32 output layer;
@@ -67,12 +69,21 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, vo
 // for negative z (an absolute tanh error of 2^-11 there shifted the trained
 // network's outputs by 7 % of their scale), the quotient keeps its relative
 // accuracy over the whole range; exp(+large) = inf gives the limit 0.
-__device__ __forceinline__ float gelu_fast(float z)
+// Two at a time: the arithmetic in packed FP32x2 operations (each half rounded
+// as the scalar operation), the exponentials and reciprocals one by one.
+__device__ __forceinline__ float2 gelu_fast2(float2 z)
 {
-    const float v = fmaf(0.044715f * z * z, z, z);
-    float e;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-2.0f * 0.7978845608028654f * 1.4426950408889634f * v));
-    return __fdividef(z, 1.0f + e);
+    const float2 zc = __fmul2_rn(make_float2(0.044715f, 0.044715f), z);
+    const float2 v = __ffma2_rn(__fmul2_rn(zc, z), z, z);
+    constexpr float k = -2.0f * 0.7978845608028654f * 1.4426950408889634f;
+    const float2 x = __fmul2_rn(make_float2(k, k), v);
+    float2 e, r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(x.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(x.y));
+    e = __fadd2_rn(e, make_float2(1.0f, 1.0f));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(e.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(e.y));
+    return __fmul2_rn(z, r);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
@@ -82,9 +93,10 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 }
 
 // GELU of two pre-activations as the BF16 pair the next layer's MMA reads.
-__device__ __forceinline__ uint32_t gelu_bf16x2(float z0, float z1)
+__device__ __forceinline__ uint32_t gelu_bf16x2(float2 z)
 {
-    return pack_bf16(gelu_fast(z0), gelu_fast(z1));
+    const float2 g = gelu_fast2(z);
+    return pack_bf16(g.x, g.y);
 }
 
 // byte offset of BF16 element (row, k) in a swizzled operand tile
@@ -95,7 +107,7 @@ __device__ __forceinline__ uint32_t a_off(int row, int k)
                                  ((kl & 7) << 1));
 }
 
-__global__ void __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_constant__ CUtensorMap tmW, MlpArgs a)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_constant__ CUtensorMap tmW, MlpArgs a)
 {
     extern __shared__ __align__(1024) unsigned char msm_raw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>(
@@ -134,8 +146,11 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t ntiles = (a.n + kMM - 1) / kMM;
-    const int my_tiles =
-        static_cast<int64_t>(blockIdx.x) < ntiles ? static_cast<int>((ntiles - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
+    // both blocks of a cluster take as many tiles (the last may be empty: its
+    // rows are beyond n), since each feeds half of the other's weight ring
+    const int64_t lead = blockIdx.x & ~1u;
+    const int my_tiles = lead < ntiles ? static_cast<int>((ntiles - 1 - lead) / gridDim.x) + 1 : 0;
+    const uint32_t rank = tc::cluster_rank();
     auto tile_f0 = [&](int it) { return (static_cast<int64_t>(blockIdx.x) + static_cast<int64_t>(it) * gridDim.x) * kMM; };
     const int n1 = 2 * nkb;      // layer-1 chunks: column half-major, K blocks within
     const int nch = n1 + 8;      // + layer-2 chunks, per tile
@@ -156,7 +171,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
             tc::mbar_init(&full[s], 1);
-            tc::mbar_init(&empty[s], 1);
+            tc::mbar_init(&empty[s], 2);   // both blocks have read the stage
         }
         tc::mbar_init(a_full, kStageWarps * 32);
         tc::mbar_init(a_empty, 1);
@@ -178,6 +193,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_
     if (warp == kLoadWarp && lane == 0) tc::prefetch_tmap(&tmW);
     tc::tc_fence_before();
     __syncthreads();
+    tc::cluster_sync();   // the other block's barriers exist before anything arrives there
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
@@ -205,12 +221,16 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_
                     }
                     int layer, nh, kb;
                     chunk_geom(c, layer, nh, kb);
+                    // this block's half of the chunk, into both blocks
                     tc::mbar_arrive_expect_tx(&full[s], kChunkBytes);
-                    tc::tma_load_2d(Wst + s * kChunkBytes, &tmW, kb * 64, layer * kHid + nh * kChunkRows, &full[s]);
+                    tc::tma_load_2d_multicast(Wst + s * kChunkBytes + rank * (kChunkBytes / 2), &tmW, kb * 64,
+                                              layer * kHid + nh * kChunkRows + rank * (kChunkRows / 2), &full[s], 3);
                 }
             }
             // the last loads of every stage have landed before the block exits
+            // (and both blocks' reads of them have been reported here)
             for (int q = g - S > 0 ? g - S : 0; q < g; ++q) (void)tc::mbar_wait(&full[q % S], (q / S) & 1u, kPolls);
+            for (int q = g - S > 0 ? g - S : 0; q < g; ++q) (void)tc::mbar_wait(&empty[q % S], (q / S) & 1u, kPolls);
         }
     } else if (warp == kIssueWarp) {
         // ---------------- MMA issue ----------------
@@ -232,7 +252,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_
                     for (int kk = 0; kk < 4; ++kk)
                         tc::mma_f16(d, tc::sdesc_sw128(sa + kk * 32), tc::sdesc_sw128(sb + kk * 32), idesc,
                                     (kb != 0 || kk != 0) ? 1u : 0u);
-                    tc::mma_commit(&empty[s]);
+                    tc::mma_commit_multicast(&empty[s], 3);
                 }
                 return true;
             };
@@ -261,7 +281,22 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_
         const bool scale_in = a.y == nullptr;
         const float* srcbase = scale_in ? a.amps : a.y;
         const int nslices = kMM / kSlice;
-        const int nchunk8 = (T + 7) / 8;
+        // this thread's eight teeth (chunk cc) and its rows rr, rr + 8 of a
+        // slice; their scaling stays in registers (zero beyond T).  Eight rows
+        // by four chunks per warp: with T odd the reads fall on distinct banks,
+        // and so do the 16-byte stores of the swizzled tile
+        const int rr = ls & 7, cc = ls >> 3;
+        float2 ref2[4], mean2[4], scale2[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            float4 t0 = make_float4(0.f, 0.f, 0.f, 0.f), t1 = t0;
+            if (8 * cc + 2 * e < T) t0 = tooth[8 * cc + 2 * e];
+            if (8 * cc + 2 * e + 1 < T) t1 = tooth[8 * cc + 2 * e + 1];
+            ref2[e] = make_float2(t0.x, t1.x);
+            mean2[e] = make_float2(-t0.y, -t1.y);
+            scale2[e] = make_float2(t0.z, t1.z);
+        }
+        const int teeth = T - 8 * cc;   // of this chunk that exist (may be <= 0)
         const uint32_t slice_bytes = static_cast<uint32_t>(kSlice * T * 4);
         // slice q of tile it: rows [f0 + 16 q, +16) clipped to n; a whole,
         // 16-byte-aligned slice goes by bulk copy, anything else by plain loads
@@ -309,30 +344,22 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_
             auto convert = [&](const float* rb) {
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    const int item = ls + 256 * j;            // 16 rows x 32 chunks of 8 teeth
-                    const int r = item & (kSlice - 1), c = item >> 4;
-                    const int row = kSlice * q + r;
+                    const int r = rr + 8 * j, row = kSlice * q + r;
                     uint32_t w[4] = {0u, 0u, 0u, 0u};
-                    if (r < nr && c < nchunk8) {
-                        const float* src = rb + r * T + 8 * c;
+                    if (r < nr && teeth > 0) {
+                        const float* src = rb + r * T + 8 * cc;
+                        float2 x[4];
 #pragma unroll
-                        for (int e = 0; e < 8; e += 2) {
-                            float x2[2];
+                        for (int e = 0; e < 4; ++e)   // (beyond T: anything finite times scale 0)
+                            x[e] = make_float2(2 * e < teeth ? src[2 * e] : 0.f, 2 * e + 1 < teeth ? src[2 * e + 1] : 0.f);
 #pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const int k = 8 * c + e + h;
-                                float x = 0.f;
-                                if (k < T) {
-                                    const float4 tk = tooth[k];
-                                    x = scale_in ? __fmul_rn(src[e + h], tk.x) : src[e + h];
-                                    x = (x - tk.y) * tk.z;
-                                }
-                                x2[h] = x;
-                            }
-                            w[e >> 1] = pack_bf16(x2[0], x2[1]);
+                        for (int e = 0; e < 4; ++e) {
+                            if (scale_in) x[e] = make_float2(__fmul_rn(x[e].x, ref2[e].x), __fmul_rn(x[e].y, ref2[e].y));
+                            x[e] = __fmul2_rn(__fadd2_rn(x[e], mean2[e]), scale2[e]);
+                            w[e] = pack_bf16(x[e].x, x[e].y);
                         }
                     }
-                    *reinterpret_cast<uint4*>(Ain + a_off(row, 8 * c)) = make_uint4(w[0], w[1], w[2], w[3]);
+                    *reinterpret_cast<uint4*>(Ain + a_off(row, 8 * cc)) = make_uint4(w[0], w[1], w[2], w[3]);
                 }
             };
             if (bulk) {
@@ -381,8 +408,8 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_
                         for (int i = 0; i < 8; ++i) {
                             const int c = cb * 16 + 2 * i;
                             const float2 bb = *reinterpret_cast<const float2*>(b1s + c);
-                            w[i] = gelu_bf16x2(__uint_as_float(raw[hh][2 * i]) + bb.x,
-                                               __uint_as_float(raw[hh][2 * i + 1]) + bb.y);
+                            w[i] = gelu_bf16x2(__fadd2_rn(
+                                make_float2(__uint_as_float(raw[hh][2 * i]), __uint_as_float(raw[hh][2 * i + 1])), bb));
                         }
                         unsigned char* base = rbase + (cb >> 2) * (kMM * 128);
                         const int c16 = (cb & 3) * 2;
@@ -399,25 +426,30 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_
             if (!wait_or_abort(acc2_full, ph, abort_flag)) { ok = false; break; }
             __syncwarp();
             tc::tc_fence_after();
-            float o[4] = {0.f, 0.f, 0.f, 0.f};
+            float2 o01 = make_float2(0.f, 0.f), o23 = o01;
             for (int cp = half * 4; cp < half * 4 + 4; ++cp) {
                 uint32_t raw[2][16];
                 tc::tmem_ld16_async(lane_base + kHid + 32 * cp, raw[0]);
                 tc::tmem_ld16_async(lane_base + kHid + 32 * cp + 16, raw[1]);
                 tc::tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 32; ++i) {
+                for (int i = 0; i < 32; i += 2) {
                     const int c = cp * 32 + i;
-                    const float h = gelu_fast(__uint_as_float(raw[i >> 4][i & 15]) + b2s[c]);
-                    const float4 w3 = w3t[c];
-                    o[0] = fmaf(w3.x, h, o[0]);
-                    o[1] = fmaf(w3.y, h, o[1]);
-                    o[2] = fmaf(w3.z, h, o[2]);
-                    o[3] = fmaf(w3.w, h, o[3]);
+                    const float2 bb = *reinterpret_cast<const float2*>(b2s + c);
+                    const float2 h2 = gelu_fast2(__fadd2_rn(
+                        make_float2(__uint_as_float(raw[i >> 4][i & 15]), __uint_as_float(raw[i >> 4][(i & 15) + 1])), bb));
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const float h = q ? h2.y : h2.x;
+                        const float4 w3 = w3t[c + q];
+                        o01 = __ffma2_rn(make_float2(w3.x, w3.y), make_float2(h, h), o01);
+                        o23 = __ffma2_rn(make_float2(w3.z, w3.w), make_float2(h, h), o23);
+                    }
                 }
             }
             tc::tc_fence_before();
             tc::mbar_arrive(acc2_empty);
+            const float o[4] = {o01.x, o01.y, o23.x, o23.y};
             // half 1 hands its partial sums to half 0 through a double buffer
             const int rb = it & 1;
             const uint32_t rph = (it >> 1) & 1u;
@@ -472,6 +504,8 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_
         tc::tc_fence_after();
         tc::tmem_dealloc(tmem, 2 * kHid);
     }
+    // neither block leaves while the other may still write or arrive here
+    tc::cluster_sync();
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder()
@@ -580,7 +614,7 @@ cudaError_t setup_mlp(cg_plan_s* p, const unsigned char* blob, size_t bytes, con
     }
     cuuint64_t gdim[2] = {static_cast<cuuint64_t>(kHid), static_cast<cuuint64_t>(2 * kHid)};
     cuuint64_t gstride[1] = {static_cast<cuuint64_t>(kHid) * 2};
-    cuuint32_t box[2] = {64, static_cast<cuuint32_t>(kChunkRows)};
+    cuuint32_t box[2] = {64, static_cast<cuuint32_t>(kChunkRows / 2)};
     cuuint32_t estride[2] = {1, 1};
     CUresult r = enc(&p->mlp_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p->d.mlp_W, gdim, gstride, box, estride,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -604,6 +638,22 @@ cudaError_t setup_mlp(cg_plan_s* p, const unsigned char* blob, size_t bytes, con
     p->mlp_smem = mlp_smem_bytes(m.stages, p->T);
     if ((e = raise_smem_limit(reinterpret_cast<void*>(&mlp_infer_kernel), p->mlp_smem)) != cudaSuccess)
         return e;
+    // clusters of two blocks that are resident at once
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(2 * (p->num_sms / 2));
+    cfg.blockDim = dim3(kMlpThreads);
+    cfg.dynamicSmemBytes = p->mlp_smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if ((e = cudaOccupancyMaxActiveClusters(&clusters, reinterpret_cast<void*>(&mlp_infer_kernel), &cfg)) != cudaSuccess)
+        return e;
+    p->mlp_clusters = clusters > 0 ? clusters : 1;
     p->mlp_ok = true;
     return cudaSuccess;
 }
@@ -618,7 +668,8 @@ cudaError_t launch_mlp(const cg_plan_s* p, const float* y, const float* amps, in
     m.p0 = p0;
     m.flags = flags;
     const int64_t ntiles = (n + kMM - 1) / kMM;
-    const unsigned grid = static_cast<unsigned>(ntiles < p->num_sms ? ntiles : p->num_sms);
+    const int64_t pairs = (ntiles + 1) / 2, most = p->mlp_clusters;
+    const unsigned grid = 2u * static_cast<unsigned>(pairs < most ? pairs : most);
     void* args[] = {const_cast<CUtensorMap*>(&p->mlp_map), &m};
     return cudaLaunchKernel(reinterpret_cast<void*>(&mlp_infer_kernel), dim3(grid), dim3(kMlpThreads), args, p->mlp_smem, s);
 }

@@ -28,6 +28,7 @@
 
 #include "cg_fft.cuh"
 #include "cg_internal.h"
+#include "cg_tc.cuh"
 
 namespace cg {
 
@@ -69,6 +70,7 @@ __global__ void __launch_bounds__(Pow2Plan<L>::NTH, 512 / Pow2Plan<L>::NTH) pow2
     using P = Pow2Plan<L>;
     constexpr int TPF = P::TPF, FPB = P::FPB, R3 = P::R3, PP = P::PP, N = P::N;
     extern __shared__ __align__(1024) unsigned char sm[];
+    tc::pdl_start();
     const int T = a.T;
     float2* Z = reinterpret_cast<float2*>(sm);                         // [FPB][L]
     // pass twiddles laid out so a warp reads consecutive entries:

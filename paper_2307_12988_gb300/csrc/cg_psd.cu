@@ -28,6 +28,7 @@
 #include "cg_fft.cuh"
 #include "cg_internal.h"
 #include "cg_stage.cuh"
+#include "cg_tc.cuh"
 
 namespace cg {
 constexpr int kWelchThreads = 512;   // threads of a block of the Welch kernel
@@ -649,8 +650,7 @@ __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads
     __shared__ double sp[4];        // parameters at which the sums are taken
     __shared__ int s_ctl;           // 0 continue, 1 stop
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    unsigned rank;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const uint32_t rank = tc::cluster_rank();
     const double* S = a.psd + a.k0;
     const int rows = (a.np + kResRow - 1) / kResRow;
     for (int c = warp; c < rows && c < kResLogRows; c += kResWarps) {
@@ -730,7 +730,7 @@ __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads
             asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there), "d"(sa) : "memory");
             asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there + 8), "d"(sb) : "memory");
         }
-        asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        tc::cluster_sync();
         if (t < 16) {
             double v = 0.0;
             for (int w = 0; w < kResBlocks; ++w) v += red[parity][w][t];

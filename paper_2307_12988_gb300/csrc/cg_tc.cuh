@@ -102,6 +102,21 @@ __device__ __forceinline__ void cp_async_wait_pending(int n)
     }
 }
 
+// ---- programmatic dependent launch -------------------------------------------
+// the next kernel of the stream may begin (it waits before it touches memory)
+__device__ __forceinline__ void pdl_start()
+{
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+// every kernel before this one has ended and its stores are visible, to the
+// bulk copies as well (nothing to wait for in a kernel launched without the
+// attribute)
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("fence.proxy.async;\n" ::: "memory");
+}
+
 // ---- TMA --------------------------------------------------------------------
 __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* map, int x, int y, uint64_t* bar)
 {
@@ -109,6 +124,17 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
         "[%4];\n" ::"r"(smem_u32(smem_dst)),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
+        : "memory");
+}
+// the same into the same place of every block of the cluster in `mask`, each
+// completing on its own barrier at the same place
+__device__ __forceinline__ void tma_load_2d_multicast(void* smem_dst, const CUtensorMap* map, int x, int y, uint64_t* bar,
+                                                      uint16_t mask)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster [%0], "
+        "[%1, {%2, %3}], [%4], %5;\n" ::"r"(smem_u32(smem_dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar)), "h"(mask)
         : "memory");
 }
 // contiguous bytes global -> shared by the bulk copy engine, completing on an
@@ -173,6 +199,29 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                      smem_u32(bar))
                  : "memory");
+}
+
+// the same, arriving at the barrier's place in every block of the cluster in `mask`
+__device__ __forceinline__ void mma_commit_multicast(uint64_t* bar, uint16_t mask)
+{
+    asm volatile(
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n" ::"r"(
+            smem_u32(bar)),
+        "h"(mask)
+        : "memory");
+}
+
+// ---- clusters ---------------------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// barrier of every thread of the cluster's blocks
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;\n" ::: "memory");
 }
 
 // 32 lanes x 16 columns without waiting (complete with tmem_wait_ld before

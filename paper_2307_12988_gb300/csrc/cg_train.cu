@@ -77,17 +77,6 @@ constexpr int kMaxRing = 6;
 constexpr uint32_t kTrPolls = 1u << 22;
 constexpr int kFinThreads = 256;
 
-__device__ __forceinline__ void pdl_start()
-{
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-}
-// (the predecessor's stores also become visible to the bulk copies)
-__device__ __forceinline__ void pdl_wait()
-{
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    asm volatile("fence.proxy.async;\n" ::: "memory");
-}
-
 __device__ __forceinline__ uint32_t swz(int row, int k)
 {
     return static_cast<uint32_t>(row * 128 + (((((k >> 2) & 7) ^ (row & 7))) << 4) + ((k & 3) << 2));
@@ -329,9 +318,9 @@ __global__ void __launch_bounds__(kTrThreads, 1) product_kernel(const __grid_con
 {
     extern __shared__ __align__(1024) unsigned char tsm_raw[];
     unsigned char* const tsm = align1024(tsm_raw);
-    pdl_start();
+    tc::pdl_start();
     const Ring r = ring_init(tsm, q.stages, q.bn, q.tmem_cols);
-    pdl_wait();
+    tc::pdl_wait();
     const int m0 = blockIdx.y * kGM, n0 = blockIdx.x * q.bn;
     const int ncols = q.N - n0 < q.bn ? q.N - n0 : q.bn, bn = (ncols + 15) & ~15;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -387,12 +376,12 @@ __global__ void __launch_bounds__(kTrThreads, 1) mid_kernel(const __grid_constan
 {
     extern __shared__ __align__(1024) unsigned char tsm_raw[];
     unsigned char* const tsm = align1024(tsm_raw);
-    pdl_start();
+    tc::pdl_start();
     const Ring r = ring_init(tsm, q.stages, 16, q.tmem_cols);
     // after the ring: g_out's tile (A of the second product) and the W3 rows (B)
     unsigned char* ga = tsm + ((q.stages * r.bytes + kRingTail + 1023) & ~1023);   // hi, lo
     unsigned char* wb = ga + 2 * kTile;                                            // hi, lo of bn rows
-    pdl_wait();
+    tc::pdl_wait();
     const int m0 = blockIdx.y * kGM, n0 = blockIdx.x * q.bn;
     const int ncols = q.H - n0 < q.bn ? q.H - n0 : q.bn, bn = (ncols + 15) & ~15;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -518,9 +507,9 @@ __global__ void __launch_bounds__(kTrThreads, 1) dw_kernel(const __grid_constant
 {
     extern __shared__ __align__(1024) unsigned char tsm_raw[];
     unsigned char* const tsm = align1024(tsm_raw);
-    pdl_start();
+    tc::pdl_start();
     const Ring r = ring_init(tsm, q.stages, q.bn, q.tmem_cols);
-    pdl_wait();
+    tc::pdl_wait();
     const int bid = static_cast<int>(blockIdx.x);
     const DwJob& j = bid >= q.job[2].first ? q.job[2] : bid >= q.job[1].first ? q.job[1] : q.job[0];
     const int splits = (j.nkb + j.kb_per - 1) / j.kb_per;
@@ -581,8 +570,8 @@ __device__ __forceinline__ void prep_tile(const PrepArgs& q, int tile, float (*b
 __global__ void __launch_bounds__(kFinThreads) prep_kernel(const __grid_constant__ PrepArgs q)
 {
     __shared__ float buf[32][33];
-    pdl_start();
-    pdl_wait();
+    tc::pdl_start();
+    tc::pdl_wait();
     prep_tile(q, static_cast<int>(blockIdx.x), buf);
 }
 
@@ -628,8 +617,8 @@ __device__ __forceinline__ float finish_param(const FinishArgs& q, int64_t i, fl
 __global__ void __launch_bounds__(kFinThreads) finish_kernel(const __grid_constant__ FinishArgs q)
 {
     __shared__ float buf[32][33];
-    pdl_start();
-    pdl_wait();
+    tc::pdl_start();
+    tc::pdl_wait();
     int b = static_cast<int>(blockIdx.x);
     const int t = threadIdx.x;
     if (b < q.bias_blocks) {
@@ -775,19 +764,10 @@ __global__ void __launch_bounds__(kFinThreads) finish_kernel(const __grid_consta
 }
 
 template <class A>
-cudaError_t launch_pdl(void (*fn)(A), dim3 grid, int threads, size_t smem, cudaStream_t s, const A& a)
+cudaError_t launch_pdl(void (*fn)(A), dim3 grid, int threads, size_t smem, cudaStream_t s, A a)
 {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fn, a);
+    void* args[] = {&a};
+    return launch_dependent(reinterpret_cast<void*>(fn), grid, dim3(threads), args, smem, s);
 }
 
 int up(int v, int m) { return (v + m - 1) / m * m; }
