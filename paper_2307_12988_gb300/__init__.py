@@ -73,23 +73,25 @@ class Plan:
 
     def _outputs(self, n, device, want_y=True, want_amps=True):
         import torch
+        empty, f32, i16 = torch.empty, torch.float32, torch.int16
         out = {}
         if want_amps:
-            out["amps"] = torch.empty((n, self.T), dtype=torch.float32, device=device)
-        out["y"] = torch.empty((n, self.T), dtype=torch.float32, device=device) if want_y else None
-        out["params"] = torch.empty((n, 4), dtype=torch.float32, device=device)
-        out["rss"] = torch.empty(n, dtype=torch.float32, device=device)
-        out["iters"] = torch.empty(n, dtype=torch.int16, device=device)
-        out["status"] = torch.empty(n, dtype=torch.int16, device=device)
+            out["amps"] = empty((n, self.T), dtype=f32, device=device)
+        out["y"] = empty((n, self.T), dtype=f32, device=device) if want_y else None
+        out["params"] = empty((n, 4), dtype=f32, device=device)
+        out["rss"] = empty(n, dtype=f32, device=device)
+        out["iters"] = empty(n, dtype=i16, device=device)
+        out["status"] = empty(n, dtype=i16, device=device)
         return out
 
     def process(self, frames, want_y=True, stream=None):
         """Whole path on int16 (or int8) frames [n, N] resident on the device."""
-        n = frames.shape[0]
-        if frames.dim() != 2 or frames.shape[1] != self.N:
-            raise ValueError(f"frames must be [n, {self.N}]")
-        o = self._outputs(n, frames.device, want_y)
         import torch
+        shape = frames.shape
+        if len(shape) != 2 or shape[1] != self.N:
+            raise ValueError(f"frames must be [n, {self.N}]")
+        n = shape[0]
+        o = self._outputs(n, frames.device, want_y)
         fn = cg_process_i8 if frames.dtype == torch.int8 else cg_process
         fn(self.handle, frames, n, o["amps"], o["y"], o["params"], o["rss"], o["iters"], o["status"], stream)
         return o

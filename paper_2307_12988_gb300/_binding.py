@@ -180,24 +180,29 @@ def _ptr(x) -> int | None:
     """Device or host address of a torch tensor / numpy array / int / None."""
     if x is None:
         return None
+    try:
+        return x.data_ptr()          # (a tensor: the common case, found first)
+    except AttributeError:
+        pass
     if isinstance(x, int):
         return x
-    if hasattr(x, "data_ptr"):
-        return x.data_ptr()
     if isinstance(x, np.ndarray):
         return x.ctypes.data
     raise TypeError(f"cannot take the address of {type(x)}")
 
 
 def _stream(stream) -> int | None:
+    """Handle of a stream; None: torch's current stream, or the legacy default
+    stream where torch is absent or has no device."""
     if stream is None:
         try:
             import torch
-            if torch.cuda.is_available():
-                return torch.cuda.current_stream().cuda_stream
-        except Exception:   # torch absent: legacy default stream
+            if torch.cuda.is_initialized():
+                # 0.5 us; torch.cuda.current_stream() builds an object (3 us)
+                return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            return torch.cuda.current_stream().cuda_stream
+        except Exception:
             return None
-        return None
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
