@@ -133,15 +133,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_
     uint64_t* a_full = bars + 0;      // input tile staged (staging threads)
     uint64_t* a_empty = bars + 1;     // layer-1 products done reading it (commit)
     uint64_t* acc1_full = bars + 2;   // layer-1 accumulator complete (commit)
-    uint64_t* a1_full = bars + 3;     // a1 written, layer-1 accumulator read (epilogue threads)
-    uint64_t* acc2_full = bars + 4;   // layer-2 accumulator complete (commit)
-    uint64_t* acc2_empty = bars + 5;  // layer-2 accumulator read (epilogue threads)
-    uint64_t* done = bars + 6;        // every product issued has completed
-    uint64_t* red_full = bars + 7;    // [2] half 1's output partials written (128 threads)
-    uint64_t* red_empty = bars + 9;   // [2] half 0 has read them (128 threads)
-    uint64_t* raw_full = bars + 11;   // [2] a 16-row slice landed (bulk copy)
-    uint64_t* raw_empty = bars + 13;  // [2] the slice was converted (staging threads)
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 15);
+    uint64_t* a1_full = bars + 3;     // [2] half of a1's columns written (epilogue threads)
+    uint64_t* acc2_full = bars + 5;   // layer-2 accumulator complete (commit)
+    uint64_t* acc2_empty = bars + 6;  // layer-2 accumulator read (epilogue threads)
+    uint64_t* done = bars + 7;        // every product issued has completed
+    uint64_t* red_full = bars + 8;    // [2] half 1's output partials written (128 threads)
+    uint64_t* red_empty = bars + 10;  // [2] half 0 has read them (128 threads)
+    uint64_t* raw_full = bars + 12;   // [2] a 16-row slice landed (bulk copy)
+    uint64_t* raw_empty = bars + 14;  // [2] the slice was converted (staging threads)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -152,7 +152,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_
     const int my_tiles = lead < ntiles ? static_cast<int>((ntiles - 1 - lead) / gridDim.x) + 1 : 0;
     const uint32_t rank = tc::cluster_rank();
     auto tile_f0 = [&](int it) { return (static_cast<int64_t>(blockIdx.x) + static_cast<int64_t>(it) * gridDim.x) * kMM; };
-    const int n1 = 2 * nkb;      // layer-1 chunks: column half-major, K blocks within
+    const int n1 = 2 * nkb;      // layer-1 chunks
     const int nch = n1 + 8;      // + layer-2 chunks, per tile
     for (int i = tid; i < kHid; i += blockDim.x) {
         b1s[i] = a.tab[kMlpTabB1 + i];
@@ -176,7 +176,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_
         tc::mbar_init(a_full, kStageWarps * 32);
         tc::mbar_init(a_empty, 1);
         tc::mbar_init(acc1_full, 1);
-        tc::mbar_init(a1_full, kEpiWarps * 32);
+        tc::mbar_init(&a1_full[0], kEpiWarps * 32);
+        tc::mbar_init(&a1_full[1], kEpiWarps * 32);
         tc::mbar_init(acc2_full, 1);
         tc::mbar_init(acc2_empty, kEpiWarps * 32);
         tc::mbar_init(done, 1);
@@ -197,13 +198,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    // chunk c of a tile -> layer, column half and K block
+    // chunk c of a tile -> layer, column half and K block: K blocks in order,
+    // both column halves of each (so layer 2 begins on the first half of a1)
     auto chunk_geom = [&](int c, int& layer, int& nh, int& kb) {
-        const int per = c < n1 ? nkb : 4;
         const int h = c < n1 ? c : c - n1;
         layer = c < n1 ? 0 : 1;
-        nh = h / per;
-        kb = h - nh * per;
+        nh = h & 1;
+        kb = h >> 1;
     };
 
     if (warp == kLoadWarp) {
@@ -263,10 +264,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_
                 if (!run(0, n1, Ain, 0)) { ok = false; break; }
                 tc::mma_commit(a_empty);
                 tc::mma_commit(acc1_full);
-                if (!wait_or_abort(a1_full, ph, abort_flag)) { ok = false; break; }
                 if (it >= 1 && !wait_or_abort(acc2_empty, ph ^ 1u, abort_flag)) { ok = false; break; }
-                tc::tc_fence_after();
-                if (!run(n1, nch, Ah, kHid)) { ok = false; break; }
+                for (int h = 0; ok && h < 2; ++h) {   // K blocks 0, 1, then 2, 3
+                    ok = wait_or_abort(&a1_full[h], ph, abort_flag);
+                    tc::tc_fence_after();
+                    ok = ok && run(n1 + 4 * h, n1 + 4 * h + 4, Ah, kHid);
+                }
+                if (!ok) break;
                 tc::mma_commit(acc2_full);
             }
             if (!ok) *abort_flag = 1;
@@ -395,33 +399,37 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_
             tc::tc_fence_after();
             {
                 unsigned char* rbase = Ah + row * 128;
-                for (int cp = half * 4; cp < half * 4 + 4; ++cp) {
-                    uint32_t raw[2][16];
-                    tc::tmem_ld16_async(lane_base + 32 * cp, raw[0]);
-                    tc::tmem_ld16_async(lane_base + 32 * cp + 16, raw[1]);
-                    tc::tmem_wait_ld();
+                // columns 0-127 by all eight warps, then 128-255: layer 2's
+                // products on the first half run during the second
+                for (int kh = 0; kh < 2; ++kh) {
+                    for (int cp = 4 * kh + 2 * half; cp < 4 * kh + 2 * half + 2; ++cp) {
+                        uint32_t raw[2][16];
+                        tc::tmem_ld16_async(lane_base + 32 * cp, raw[0]);
+                        tc::tmem_ld16_async(lane_base + 32 * cp + 16, raw[1]);
+                        tc::tmem_wait_ld();
 #pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        const int cb = 2 * cp + hh;
-                        uint32_t w[8];
+                        for (int hh = 0; hh < 2; ++hh) {
+                            const int cb = 2 * cp + hh;
+                            uint32_t w[8];
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int c = cb * 16 + 2 * i;
-                            const float2 bb = *reinterpret_cast<const float2*>(b1s + c);
-                            w[i] = gelu_bf16x2(__fadd2_rn(
-                                make_float2(__uint_as_float(raw[hh][2 * i]), __uint_as_float(raw[hh][2 * i + 1])), bb));
+                            for (int i = 0; i < 8; ++i) {
+                                const int c = cb * 16 + 2 * i;
+                                const float2 bb = *reinterpret_cast<const float2*>(b1s + c);
+                                w[i] = gelu_bf16x2(__fadd2_rn(make_float2(__uint_as_float(raw[hh][2 * i]),
+                                                                          __uint_as_float(raw[hh][2 * i + 1])), bb));
+                            }
+                            unsigned char* base = rbase + (cb >> 2) * (kMM * 128);
+                            const int c16 = (cb & 3) * 2;
+                            *reinterpret_cast<uint4*>(base + ((c16 ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                            *reinterpret_cast<uint4*>(base + (((c16 + 1) ^ (row & 7)) << 4)) =
+                                make_uint4(w[4], w[5], w[6], w[7]);
                         }
-                        unsigned char* base = rbase + (cb >> 2) * (kMM * 128);
-                        const int c16 = (cb & 3) * 2;
-                        *reinterpret_cast<uint4*>(base + ((c16 ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-                        *reinterpret_cast<uint4*>(base + (((c16 + 1) ^ (row & 7)) << 4)) =
-                            make_uint4(w[4], w[5], w[6], w[7]);
                     }
+                    tc::tc_fence_before();
+                    tc::fence_proxy_async_smem();
+                    tc::mbar_arrive(&a1_full[kh]);
                 }
             }
-            tc::tc_fence_before();
-            tc::fence_proxy_async_smem();
-            tc::mbar_arrive(a1_full);
             // layer 2 and the FP32 output layer
             if (!wait_or_abort(acc2_full, ph, abort_flag)) { ok = false; break; }
             __syncwarp();
@@ -527,7 +535,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder()
 int mlp_smem_bytes(int stages, int T)
 {
     return 1024 + 2 * kABytes + kRawBytes + stages * kChunkBytes + 4 * (2 * kHid + 4 * kHid + 16 + 4 * T) +
-           2 * 4 * 4 * kMM + 8 * (2 * kStagesMax + 15) + 16;
+           2 * 4 * 4 * kMM + 8 * (2 * kStagesMax + 16) + 16;
 }
 
 // Parses a cg_mlp_save blob, packs the BF16 weight matrix, the FP32 tables and
