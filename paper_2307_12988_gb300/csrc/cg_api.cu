@@ -157,7 +157,7 @@ cudaError_t setup_fast(cg_plan_s* p, const std::vector<int>& zidx)
     const int N = p->N, T = p->T, L = p->L;
     if (p->kind != CG_FFT_COSET || p->M != 10 || L % 10 != 0) return cudaSuccess;
     const int Q = L / 10;
-    if (!cg::fast_readout_ptr(Q)) return cudaSuccess;
+    if (!cg::coset_instantiated(Q, 2)) return cudaSuccess;
     std::vector<int> tom(L, -1);
     for (int k = 0; k < T; ++k) {
         if (tom[zidx[k]] >= 0) return cudaSuccess;   // two teeth on one bin: generic path
@@ -172,64 +172,12 @@ cudaError_t setup_fast(cg_plan_s* p, const std::vector<int>& zidx)
     cudaError_t e;
     if ((e = upload(&p->d.tw_M5, tw5)) != cudaSuccess) return e;
     if ((e = upload(&p->d.tooth_of_m, tom)) != cudaSuccess) return e;
-    // batch size and layout for samples of sb bytes: minimise idle thread
-    // slots of the two transform stages (stage 1: 10 items per frame, cost
-    // ~ 50 Q; stage 2: Q items, cost ~ 200); at most ~52 KiB of shared
-    // memory per block keeps four blocks per SM
-    auto layout = [&](int sb, cg::FastArgs& a, void* fn, int& grid) -> cudaError_t {
-        int bestF = 2;
-        double best = 1e30;
-        for (int F = 2; F <= 32; ++F) {
-            const int bytes = sb * N * F + 32 + 8 * L * F;
-            if (bytes > 52 * 1024) break;
-            const double cost =
-                (std::ceil(10.0 * F / 128.0) * 50.0 * Q + std::ceil(double(Q) * F / 128.0) * 200.0) / F;
-            if (cost < best - 1e-9) { best = cost; bestF = F; }
-        }
-        // frames per block measured best on GB300 for the instantiated
-        // transforms (occupancy and lane use trade against each other, which
-        // the idle-slot model above does not see): 10^6 paper-rate frames
-        // take 0.525 ms at F = 8 vs 0.547 ms at the model's 11; 8-bit
-        // 2200-sample frames 0.996 vs 1.08 ms; wide frames 0.624 vs 0.662 ms
-        struct Measured { int Q, sb, F; };
-        static const Measured kMeasured[] = {{10, 2, 12}, {11, 2, 8}, {22, 1, 8}, {25, 2, 5}};
-        for (const Measured& mf : kMeasured)
-            if (mf.Q == Q && mf.sb == sb && sb * N * mf.F + 32 + 8 * L * mf.F <= 52 * 1024) bestF = mf.F;
-        a.N = N;
-        a.T = T;
-        a.F = bestF;
-        a.pair_isign = (p->r0 & 1) ? -1 : 1;
-        int off = 0;
-        a.sm_twL = off; off = align16(off + 8 * L);
-        a.sm_twN = off; off = align16(off + 8 * L);
-        a.sm_tom = off; off = align16(off + 4 * L);
-        a.sm_iref = off; off = align16(off + 4 * T);
-        a.sm_u = 0;
-        a.sm_raw = off; off = align16(off + sb * N * bestF + 32);
-        a.sm_Y = off; off = align16(off + 8 * L * bestF);
-        a.sm_amps = 0;
-        a.sm_y = 0;
-        a.sm_total = off;
-        a.twL = p->d.tw_L;
-        a.twN = p->d.tw_n1;
-        a.twM = p->d.tw_M5;
-        a.tooth_of_m = p->d.tooth_of_m;
-        a.inv_ref = p->d.inv_ref;
-        a.u = p->d.u;
-        cudaError_t e2 = cg::raise_smem_limit(fn, a.sm_total);
-        if (e2 != cudaSuccess) return e2;
-        int occ = 0;
-        if ((e2 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 128, a.sm_total)) != cudaSuccess) return e2;
-        grid = p->num_sms * occ;
-        return cudaSuccess;
-    };
-    if ((e = layout(2, p->fa, cg::fast_readout_ptr(Q), p->grid_fast)) != cudaSuccess) return e;
+    if ((e = cg::setup_coset(p, Q, 2, p->fa, &p->grid_fast)) != cudaSuccess) return e;
     if (p->grid_fast < 1) return cudaSuccess;
     p->Q = Q;
     p->fast_ok = true;
-    if (void* fr8 = cg::fast_readout_ptr(Q, 1)) {
-        // int8 samples: the staging takes half the bytes, so more frames per block
-        if ((e = layout(1, p->fa8, fr8, p->grid_fast8)) != cudaSuccess) return e;
+    if (cg::coset_instantiated(Q, 1)) {
+        if ((e = cg::setup_coset(p, Q, 1, p->fa8, &p->grid_fast8)) != cudaSuccess) return e;
         p->fast_i8_ok = p->grid_fast8 >= 1;
     }
     return cudaSuccess;

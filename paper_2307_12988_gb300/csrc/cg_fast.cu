@@ -1,18 +1,7 @@
-// cg_fast.cu -- the throughput path for comb geometries whose tooth bins lie in
-// one residue pair +-r mod 10 (every 1 us-frame workload: N = 10 P Q).
+// cg_fast.cu -- the moment initial guess and the register-resident LM of the
+// throughput path.
 //
-// fast_readout_kernel<P, Q, PAIR>: cast + coset transform + tooth readout +
-//   moment initial guess for a batch of frames per thread block:
-//   * the next batch's int16 samples stream into shared memory with cp.async
-//     while the current batch is transformed;
-//   * stage 1 (one thread per frame and residue a < P, or per pair a, a+1):
-//     the radix-10 fold of the samples at n1 = a + P b, using the symmetry
-//     W_10^(r (n2+5)) = -W_10^(r n2) for odd r, times W_N^(r n1), then a Q-point
-//     DFT over b in registers and the twiddle W_L^(u a);
-//   * stage 2 (one thread per frame and u < Q): a P-point DFT over a gives
-//     Z[u + Q v] = X_{10 (u + Q v) + r}; teeth read their |Z|;
-//   * amplitudes leave coalesced; the moment initial guess of each frame is
-//     written as its starting parameters.
+// init_kernel: the guess of each frame, one lane per frame.
 // fit2_kernel<G, PPL>: Levenberg-Marquardt with each lane's PPL points in
 //   registers; the groups of a warp pull frames from the warp's task one by one
 //   as their previous frame finishes, so no group waits for another frame's
@@ -24,7 +13,6 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
-#include "cg_fft.cuh"
 #include "cg_fit.cuh"
 #include "cg_internal.h"
 #include "cg_net.cuh"
@@ -32,150 +20,6 @@
 #include "cg_tc.cuh"
 
 namespace cg {
-
-template <int P, int Q, class S>
-__global__ void __launch_bounds__(128) fast_readout_kernel(FastArgs a)
-{
-    constexpr int L = P * Q;
-    constexpr int MH = 5;                     // M / 2 with M = 10
-    // long Q-point transforms: the fold runs as its own stage with one item
-    // per output (balanced over the block) and the Q-point DFTs read it back
-    constexpr bool kSplitFold = Q > 11;
-    extern __shared__ __align__(16) unsigned char sm[];
-    tc::pdl_start();
-    float2* twL = reinterpret_cast<float2*>(sm + a.sm_twL);
-    float2* twN = reinterpret_cast<float2*>(sm + a.sm_twN);
-    int* tom = reinterpret_cast<int*>(sm + a.sm_tom);
-    float* iref = reinterpret_cast<float*>(sm + a.sm_iref);
-    S* raw = reinterpret_cast<S*>(sm + a.sm_raw);
-    const S* frames = static_cast<const S*>(a.frames);
-    float2* Yb = reinterpret_cast<float2*>(sm + a.sm_Y);
-    const int T = a.T, N = a.N, F = a.F;
-    for (int i = threadIdx.x; i < L; i += blockDim.x) {
-        twL[i] = a.twL[i];
-        twN[i] = a.twN[i];
-        tom[i] = a.tooth_of_m[i];
-    }
-    for (int i = threadIdx.x; i < T; i += blockDim.x) iref[i] = a.inv_ref[i];
-    // fold twiddles w_j = W_10^(r j): with s = (-1)^r, w_{5-j} = s conj(w_j), so
-    // sum_j D_j w_j = D_0 + (E_1 c_1 + E_2 c_2) + i (F_1 s_1 + F_2 s_2) where
-    // D_j = x_j + s x_{j+5}, E_j = D_j + s D_{5-j}, F_j = D_j - s D_{5-j}
-    const float c1 = a.twM[1].x, s1 = a.twM[1].y, c2 = a.twM[2].x, s2 = a.twM[2].y;
-    const int sg = a.pair_isign;
-
-    const int64_t nb = (a.n_frames + F - 1) / F;
-    int64_t b = blockIdx.x;
-    int off = 0;
-    if (b < nb) {
-        const int nf0 = static_cast<int>((a.n_frames - b * F) < F ? (a.n_frames - b * F) : F);
-        off = stage_async(frames, b * F * static_cast<int64_t>(N), static_cast<int64_t>(nf0) * N, raw);
-    }
-    for (; b < nb; b += gridDim.x) {
-        const int64_t f0 = b * F;
-        const int nf = static_cast<int>((a.n_frames - f0) < F ? (a.n_frames - f0) : F);
-        cp_async_wait_all();
-        __syncthreads();
-        int offn = 0;
-        if constexpr (kSplitFold) {
-            // ---------------- stage 0: the fold, one item per output m ------
-            for (int item = threadIdx.x; item < nf * L; item += blockDim.x) {
-                const int f = item / L;
-                const int m = item - f * L;
-                const S* xp = raw + off + f * N + m;
-                int D[MH];
-#pragma unroll
-                for (int j = 0; j < MH; ++j) D[j] = static_cast<int>(xp[L * j]) + sg * static_cast<int>(xp[L * (j + MH)]);
-                const int E1 = D[1] + sg * D[4], F1 = D[1] - sg * D[4];
-                const int E2 = D[2] + sg * D[3], F2 = D[2] - sg * D[3];
-                float2 fz;
-                fz.x = fmaf(static_cast<float>(E2), c2, fmaf(static_cast<float>(E1), c1, static_cast<float>(D[0])));
-                fz.y = fmaf(static_cast<float>(F2), s2, static_cast<float>(F1) * s1);
-                Yb[f * L + m] = cmul(fz, twN[m]);
-            }
-            __syncthreads();
-            // raw is free: start the next batch's samples
-            const int64_t bn = b + gridDim.x;
-            if (bn < nb) {
-                const int nfn = static_cast<int>((a.n_frames - bn * F) < F ? (a.n_frames - bn * F) : F);
-                offn = stage_async(frames, bn * F * static_cast<int64_t>(N), static_cast<int64_t>(nfn) * N, raw);
-            }
-            // ---------------- stage 1: Q-point DFT over b, twiddle (in place) --
-            for (int item = threadIdx.x; item < nf * P; item += blockDim.x) {
-                const int f = item / P;
-                const int a0 = item - f * P;
-                float2* Yf = Yb + f * L + a0;
-                float2 z[Q];
-#pragma unroll
-                for (int bq = 0; bq < Q; ++bq) z[bq] = Yf[P * bq];
-                Dft<Q>::run(z);
-#pragma unroll
-                for (int u = 0; u < Q; ++u) Yf[u * P] = u ? cmul(z[u], twL[u * a0]) : z[u];
-            }
-            __syncthreads();
-        } else {
-            // ---------------- stage 1: fold, Q-point DFT, twiddle ----------------
-            for (int item = threadIdx.x; item < nf * P; item += blockDim.x) {
-                const int f = item / P;
-                const int a0 = item - f * P;
-                const S* xs = raw + off + f * N + a0;
-                float2 z[Q];
-#pragma unroll
-                for (int bq = 0; bq < Q; ++bq) {
-                    const S* xp = xs + P * bq;
-                    int D[MH];
-#pragma unroll
-                    for (int j = 0; j < MH; ++j) D[j] = static_cast<int>(xp[L * j]) + sg * static_cast<int>(xp[L * (j + MH)]);
-                    const int E1 = D[1] + sg * D[4], F1 = D[1] - sg * D[4];
-                    const int E2 = D[2] + sg * D[3], F2 = D[2] - sg * D[3];
-                    float2 fz;
-                    fz.x = fmaf(static_cast<float>(E2), c2, fmaf(static_cast<float>(E1), c1, static_cast<float>(D[0])));
-                    fz.y = fmaf(static_cast<float>(F2), s2, static_cast<float>(F1) * s1);
-                    z[bq] = cmul(fz, twN[a0 + P * bq]);
-                }
-                Dft<Q>::run(z);
-                float2* Yf = Yb + f * L + a0;
-#pragma unroll
-                for (int u = 0; u < Q; ++u) Yf[u * P] = u ? cmul(z[u], twL[u * a0]) : z[u];
-            }
-            __syncthreads();
-            // raw is free: start the next batch's samples
-            const int64_t bn = b + gridDim.x;
-            if (bn < nb) {
-                const int nfn = static_cast<int>((a.n_frames - bn * F) < F ? (a.n_frames - bn * F) : F);
-                offn = stage_async(frames, bn * F * static_cast<int64_t>(N), static_cast<int64_t>(nfn) * N, raw);
-            }
-        }
-        // ---------------- stage 2: P-point DFT over a, tooth magnitudes -------
-        for (int item = threadIdx.x; item < nf * Q; item += blockDim.x) {
-            const int f = item / Q;
-            const int u = item - f * Q;
-            const float2* Yf = Yb + f * L + u * P;
-            float2 z[P];
-#pragma unroll
-            for (int q = 0; q < P; q += 2) {
-                const float4 v = *reinterpret_cast<const float4*>(Yf + q);
-                z[q] = make_float2(v.x, v.y);
-                z[q + 1] = make_float2(v.z, v.w);
-            }
-            Dft<P>::run(z);
-            // straight to global memory: the items of a frame hold runs of
-            // consecutive bins, i.e. runs of consecutive (or reversed) teeth
-            const int64_t orow = (f0 + f) * T;
-#pragma unroll
-            for (int v = 0; v < P; ++v) {
-                const int k = tom[u + Q * v];
-                if (k >= 0) {
-                    const float av = cabs_approx(z[v]);
-                    if (a.amps) a.amps[orow + k] = av;
-                    if (a.y) a.y[orow + k] = __fmul_rn(av, iref[k]);
-                }
-            }
-        }
-        // (the next batch's stages start after the barrier at the loop top)
-        off = offn;
-    }
-    cp_async_wait_all();
-}
 
 // ---------------------------------------------------------------------------
 // moment initial guess, one lane per frame
@@ -816,23 +660,6 @@ __global__ void __launch_bounds__(G == 1 ? 128 : 256, G == 1 ? 3 : 2) fit2_kerne
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-template <int P, int Q, class S>
-static void* fast_fn() { return reinterpret_cast<void*>(&fast_readout_kernel<P, Q, S>); }
-
-// the instantiated coset readouts: L = 10 Q with Q in {10, 11, 22, 25};
-// int16 samples, and int8 samples for the 8-bit 2200-sample frame (Q = 22)
-void* fast_readout_ptr(int Q, int sample_bytes)
-{
-    if (sample_bytes == 1) return Q == 22 ? fast_fn<10, 22, int8_t>() : nullptr;
-    switch (Q) {
-    case 10: return fast_fn<10, 10, int16_t>();
-    case 11: return fast_fn<10, 11, int16_t>();
-    case 22: return fast_fn<10, 22, int16_t>();
-    case 25: return fast_fn<10, 25, int16_t>();
-    default: return nullptr;
-    }
-}
-
 // the outer-set sizes of the workload geometries (21, 99, 201 and 221 teeth:
 // the outer fifth with ties kept) have their own pruned median
 template <bool EIGHT>
@@ -931,33 +758,6 @@ int init_npad(int n_outer)
     for (int np : {8, 16, 32, 64})
         if (n_outer <= np) return np;
     return 0;
-}
-
-static cudaError_t launch_fast(const cg_plan_s* p, const void* frames, int sample_bytes, int64_t n, float* amps,
-                               float* y, cudaStream_t s)
-{
-    FastArgs a = sample_bytes == 1 ? p->fa8 : p->fa;
-    a.frames = frames;
-    a.n_frames = n;
-    a.amps = amps;
-    a.y = y;
-    const int64_t nb = (n + a.F - 1) / a.F;
-    const int gmax = sample_bytes == 1 ? p->grid_fast8 : p->grid_fast;
-    const int grid = static_cast<int>(nb < gmax ? nb : gmax);
-    void* args[] = {&a};
-    return cudaLaunchKernel(fast_readout_ptr(p->Q, sample_bytes), dim3(grid), dim3(128), args, a.sm_total, s);
-}
-
-cudaError_t launch_fast_readout(const cg_plan_s* p, const int16_t* frames, int64_t n, float* amps,
-                                float* y, cudaStream_t s)
-{
-    return launch_fast(p, frames, 2, n, amps, y, s);
-}
-
-cudaError_t launch_fast_readout_i8(const cg_plan_s* p, const int8_t* frames, int64_t n, float* amps, float* y,
-                                   cudaStream_t s)
-{
-    return launch_fast(p, frames, 1, n, amps, y, s);
 }
 
 cudaError_t launch_init(const cg_plan_s* p, const float* y, const float* amps, int64_t n,

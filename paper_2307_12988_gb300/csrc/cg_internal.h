@@ -74,21 +74,20 @@ struct GenArgs {
     int sm_n1, sm_b, sm_pos, sm_iref, sm_raw, sm_z, sm_total;
 };
 
-// Arguments of the fast readout (comb geometries, N = 10 P Q).
-struct FastArgs {
+// Arguments of the comb readout (N = 100 Q).
+struct CosetArgs {
     const void* frames;      // int16 or int8 samples (the kernel's instantiation)
     int64_t n_frames;
-    int N, T, F;
-    int pair_isign;          // (-1)^r: sign pairing x_j with x_{j+5} in the fold
+    int T, F;                // teeth, frames per batch
     const float2* twL;       // [L]  W_L^m
     const float2* twN;       // [L]  W_N^{r n1}
     const float2* twM;       // [5]  W_10^{r j}
     const int* tooth_of_m;   // [L]  tooth reading Z[m], or -1
     const float* inv_ref;    // [T]
-    const float* u;          // [T]
     float* amps;             // [n][T] or null
     float* y;                // [n][T] or null
-    int sm_twL, sm_twN, sm_tom, sm_iref, sm_u, sm_raw, sm_Y, sm_amps, sm_y, sm_total;
+    int* err;                // device error word (a bulk copy that never landed)
+    int sm_twN, sm_twL, sm_twQ, sm_tooth, sm_bar, sm_raw, sm_Y, sm_total;
 };
 
 // Arguments of the lane-per-frame moment initial guess.
@@ -279,7 +278,7 @@ struct cg_plan_s {
     bool fit_ok = false;     // init + fit kernels of the throughput path configured
     bool fast_ok = false;    // geometry admits the fast readout
     bool fast_i8_ok = false; // ... and an int8 instantiation exists for it
-    cg::FastArgs fa8{};      // its batch size and layout
+    cg::CosetArgs fa8{};      // its batch size and layout
     int grid_fast8 = 0;
     // split-precision GEMM readout
     CUtensorMap gemm_map{};
@@ -311,7 +310,7 @@ struct cg_plan_s {
     int init_npad = 0, init_smem = 0;
     cg::InitArgs ia{};
     int64_t chunk = 0;       // frames per pipelined chunk
-    cg::FastArgs fa{};
+    cg::CosetArgs fa{};
     cudaStream_t s_read = nullptr, s_fit = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_read = nullptr, ev_join_r = nullptr, ev_join_f = nullptr;
     // end of the last call's fit and the stream (its unique id) it ran on: the
@@ -364,7 +363,8 @@ cudaError_t bind_noalloc_scratch(cg_plan_s* p);
 FitArgs make_fit_args(const cg_plan_s* p);
 
 // throughput path (cg_fast.cu)
-void* fast_readout_ptr(int Q, int sample_bytes = 2);
+bool coset_instantiated(int Q, int sample_bytes);
+cudaError_t setup_coset(const cg_plan_s* p, int Q, int sample_bytes, CosetArgs& a, int* grid);
 void* init_ptr(int npad, int n_outer, bool eight = false);
 int init_npad(int n_outer);
 void* fit2_ptr(int G, int PPL, bool exact, int model);
