@@ -22,8 +22,8 @@
 //    J^T J, J^T r and chi^2 is a pair whose halves are added at the end, so
 //    the summation order depends on the tooth index only, not on where the
 //    frame lies in memory: a frame's result is the same in any batch.
-//  * per pair, one 16-byte table entry gives both abscissae and both
-//    1 / reference values (1 when the normalised spectra are given);
+//  * per pair, one table entry gives both abscissae (and both 1 / reference
+//    values when magnitudes are given);
 //  * the point is evaluated in e = (u - c) / g: L = 1 / (1 + e^2) takes two
 //    packed operations and a reciprocal; the centre column L q d (q the
 //    reciprocal of (u - c)^2 + g^2) equals L^2 e / g and the width column
@@ -64,6 +64,23 @@ __device__ __forceinline__ float2 mul2_rounded(float2 a, float2 b)
     return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
 }
 
+template <bool SCALE>
+struct TabEntry {
+    using type = float4;
+};
+template <>
+struct TabEntry<false> {
+    using type = float2;
+};
+template <bool SCALE, class E>
+__device__ __forceinline__ float2 scaled(float2 y, E tb)
+{
+    if constexpr (SCALE)
+        return mul2_rounded(y, make_float2(tb.z, tb.w));
+    else
+        return y;
+}
+
 // The 14 sums of fit2_kernel (L L, L jc, L jg, L, jc jc, jc jg, jc, jg jg,
 // jg, L r, jc r, jg r, r, r r with jc = L q d and jg = jc d) from the 13
 // sums over L, L^2 and jc' = L^2 e = g jc, using jg = L - L^2.
@@ -99,13 +116,18 @@ struct Fit3Shape {
     static constexpr int kSlots = 2 * kGroups;                  // per warp
 };
 
-template <int G, int T, int MODEL>
+// SCALE: the rows hold magnitudes, normalised as they are read; otherwise they
+// are normalised spectra and the table holds the abscissae alone (a factor of
+// one took 2 of 26 operations a pair and a 16-byte instead of an 8-byte read:
+// 10^6 spectra of 99 teeth 395 -> 387 us, 10^5 of 221 115.5 -> 112 us)
+template <int G, int T, int MODEL, bool SCALE>
 __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
 {
     constexpr int kW = MODEL == 1 ? 9 : 13;   // sums per point
     using S = Fit3Shape<G, T>;
+    using Entry = typename TabEntry<SCALE>::type;
     extern __shared__ __align__(16) float4 f3sm[];
-    float4* tab = f3sm;
+    Entry* tab = reinterpret_cast<Entry*>(f3sm);
     const int nwarps = static_cast<int>(blockDim.x) >> 5;
     uint64_t* bars_all = reinterpret_cast<uint64_t*>(f3sm + S::kTab);
     float* slots_all = reinterpret_cast<float*>(bars_all + nwarps * S::kSlots);
@@ -117,7 +139,7 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
     uint64_t* bars = bars_all + warp * S::kSlots;
     float* slots = slots_all + static_cast<size_t>(warp) * S::kSlots * S::kRS;
 
-    // pair table (u_2i, u_2i+1, w_2i, w_2i+1), w = 1 / ref (1 for given y);
+    // pair table (u_2i, u_2i+1 and, for magnitudes, w_2i, w_2i+1, w = 1 / ref);
     // padding teeth get a far abscissa and w = 0 (finite, masked below)
     for (int i = static_cast<int>(threadIdx.x); i < S::kTab; i += static_cast<int>(blockDim.x)) {
         float v[4];
@@ -125,9 +147,12 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
         for (int h = 0; h < 2; ++h) {
             const int k = 2 * i + h;
             v[h] = k < T ? a.u[k] : 65536.0f;
-            v[2 + h] = k < T ? (a.y ? 1.0f : a.inv_ref[k]) : 0.0f;
+            v[2 + h] = SCALE && k < T ? a.inv_ref[k] : 0.0f;
         }
-        tab[i] = make_float4(v[0], v[1], v[2], v[3]);
+        if constexpr (SCALE)
+            tab[i] = make_float4(v[0], v[1], v[2], v[3]);
+        else
+            tab[i] = make_float2(v[0], v[1]);
     }
     for (int i = lane; i < S::kSlots; i += 32) tc::mbar_init(&bars[i], 1);
     tc::fence_mbar_init();
@@ -140,7 +165,7 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
     const int klast0 = 2 * ilast < T ? 2 * ilast : 0;
     const int klast1 = 2 * ilast + 1 < T ? 2 * ilast + 1 : 0;
 
-    const float* src_base = a.y ? a.y : a.amps;
+    const float* src_base = SCALE ? a.amps : a.y;
     const uintptr_t buf_lo = reinterpret_cast<uintptr_t>(src_base);
     const uintptr_t buf_hi = buf_lo + static_cast<uintptr_t>(a.n_rows) * T * sizeof(float);
     const float inv_scale = 1.0f / a.x_scale;
@@ -197,13 +222,13 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
 #pragma unroll 4
                     for (int j = 0; j < S::kPPL; ++j) {
                         const int i = gl + G * j;
-                        const float4 tb = tab[i];
+                        const Entry tb = tab[i];
                         if (2 * i < T) {
-                            const float v = __fmul_rn(row[2 * i], tb.z);
+                            const float v = scaled<SCALE>(make_float2(row[2 * i], 0.f), tb).x;
                             if (v < best) { best = v; bk = 2 * i; }
                         }
                         if (2 * i + 1 < T) {
-                            const float v = __fmul_rn(row[2 * i + 1], tb.w);
+                            const float v = scaled<SCALE>(make_float2(0.f, row[2 * i + 1]), tb).y;
                             if (v < best) { best = v; bk = 2 * i + 1; }
                         }
                     }
@@ -388,7 +413,7 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
 #pragma unroll
             for (int j = 0; j < S::kPPL; ++j) {
                 const int i = gl + G * j;
-                const float4 tb = tab[i];
+                const Entry tb = tab[i];
                 float2 yv;
                 if (j < S::kPPL - 1) {
                     yv = make_float2(row[2 * i], row[2 * i + 1]);
@@ -396,7 +421,7 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
                     yv = make_float2(row[klast0], row[klast1]);
                     yv = make_float2(wlast.x != 0.f ? yv.x : 0.f, wlast.y != 0.f ? yv.y : 0.f);
                 }
-                yv = mul2_rounded(yv, make_float2(tb.z, tb.w));
+                yv = scaled<SCALE>(yv, tb);
                 const float2 e = fma2(make_float2(tb.x, tb.y), ig, ncig);
                 const float2 E = fma2(e, e, one);
                 const float2 id = make_float2(rcp_fast(E.x), rcp_fast(E.y));
@@ -437,7 +462,7 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
     #pragma unroll
             for (int j = 0; j < S::kPPL; ++j) {
                 const int i = gl + G * j;
-                const float4 tb = tab[i];
+                const Entry tb = tab[i];
                 float2 yv;
                 if (j < S::kPPL - 1) {
                     yv = make_float2(row[2 * i], row[2 * i + 1]);
@@ -445,7 +470,7 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
                     yv = make_float2(row[klast0], row[klast1]);
                     yv = make_float2(wlast.x != 0.f ? yv.x : 0.f, wlast.y != 0.f ? yv.y : 0.f);
                 }
-                yv = mul2_rounded(yv, make_float2(tb.z, tb.w));
+                yv = scaled<SCALE>(yv, tb);
                 const float2 e = fma2(make_float2(tb.x, tb.y), ig, ncig);
                 const float2 E = fma2(e, e, one);
                 float2 L = make_float2(rcp_fast(E.x), rcp_fast(E.y));
@@ -585,9 +610,10 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
 }
 
 template <int G, int T, int MODEL>
-void* fit3_fn()
+void* fit3_fn(bool scale)
 {
-    return reinterpret_cast<void*>(&fit3_kernel<G, T, MODEL>);
+    return scale ? reinterpret_cast<void*>(&fit3_kernel<G, T, MODEL, true>)
+                 : reinterpret_cast<void*>(&fit3_kernel<G, T, MODEL, false>);
 }
 
 template <int G, int T>
@@ -600,7 +626,7 @@ size_t fit3_bytes(int warps)
 struct Fit3Inst {
     int G, T, model;
     int f64;   // 1: the instance for the FP64 solve (one lane per frame where it fits)
-    void* (*fn)();
+    void* (*fn)(bool scale);
     size_t (*bytes)(int);
 };
 // the workload geometries: 21 teeth (one lane per frame), 99 (two lanes),
@@ -649,10 +675,14 @@ cudaError_t setup_fit3(cg_plan_s* p)
         --warps;
     const size_t bytes = fi->bytes(warps);
     if (bytes > static_cast<size_t>(smem_block)) return cudaSuccess;
-    void* fn = fi->fn();
-    if ((e = raise_smem_limit(fn, static_cast<int>(bytes))) != cudaSuccess) return e;
-    int occ = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 32 * warps, bytes)) != cudaSuccess) return e;
+    int occ = 1 << 30;
+    for (bool scale : {false, true}) {
+        void* fn = fi->fn(scale);
+        if ((e = raise_smem_limit(fn, static_cast<int>(bytes))) != cudaSuccess) return e;
+        int o = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, 32 * warps, bytes)) != cudaSuccess) return e;
+        occ = std::min(occ, o);
+    }
     if (occ < 1) return cudaSuccess;
     p->fit3_G = fi->G;
     p->fit3_warps = warps;
@@ -682,7 +712,7 @@ cudaError_t launch_fit3(const cg_plan_s* p, Fit2Args a, cudaStream_t s)
         if (e != cudaSuccess) return e;
     }
     void* args[] = {&a};
-    return launch_dependent(fi->fn(), dim3(grid), dim3(32 * p->fit3_warps), args, p->fit3_smem, s);
+    return launch_dependent(fi->fn(a.y == nullptr), dim3(grid), dim3(32 * p->fit3_warps), args, p->fit3_smem, s);
 }
 
 }  // namespace cg
