@@ -226,8 +226,9 @@ cudaError_t setup_fit_kernels(cg_plan_s* p)
     ia.x_mid = static_cast<float>(p->x_mid);
     ia.x_scale = static_cast<float>(p->x_scale);
     p->init_npad = npad;
-    // tables, 2 mbarriers and 2 x 32 staged rows per warp (4 warps)
-    p->init_smem = 4 * ((2 * T + p->n_outer + 3) & ~3) + 8 * 2 * 4 + 4 * 4 * 2 * 32 * ia.row_stride;
+    // tables, an mbarrier and 32 staged rows per warp
+    p->init_smem = 4 * ((2 * T + p->n_outer + 3) & ~3) +
+                   (cg::kInitThreads / 32) * (8 + 4 * 32 * ia.row_stride);
     cudaError_t e;
     int occ = 0;
     void* ff = cg::fit2_ptr(G, ppl, exact, model);
@@ -243,7 +244,7 @@ cudaError_t setup_fit_kernels(cg_plan_s* p)
     }
     void* fi = cg::init_ptr(npad, p->n_outer);
     if ((e = cg::raise_smem_limit(fi, p->init_smem)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fi, 128, p->init_smem)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fi, cg::kInitThreads, p->init_smem)) != cudaSuccess) return e;
     if (occ < 1) return cudaSuccess;
     p->grid_init = p->num_sms * occ;
     p->ppl_exact = exact;

@@ -24,6 +24,21 @@ namespace cg {
 // ---------------------------------------------------------------------------
 // moment initial guess, one lane per frame
 // ---------------------------------------------------------------------------
+// Sign of the first of the largest |y - B0|, given the largest deviation to
+// either side (0: none): the larger side, or on a tie of both the side that
+// comes first.  (Without any deviation there is no excess, and no sign either.)
+template <class Y>
+__device__ __forceinline__ bool larger_is_positive(Y y, int T, float B0, float wmaxp, float wmaxn)
+{
+    if (wmaxp != wmaxn) return wmaxp > wmaxn;
+    for (int k = 0; k < T; ++k) {
+        const float d = y(k) - B0;
+        if (d == wmaxp) return true;
+        if (-d == wmaxn) return false;
+    }
+    return true;
+}
+
 // Moment initial guess from the baseline B0 (the median of the outer teeth):
 // d = y - B0, s = sign of the largest |d|, w = max(s d, 0); c0 = centroid of
 // w over the abscissa, A0 = s max w, g0 = area / (pi |A0|) clamped to
@@ -33,29 +48,24 @@ template <class Y, class U>
 __device__ __forceinline__ void moment_finish(Y y, U u, int T, float B0, float u_mid, float du, float span,
                                               float x_mid, float x_scale, float* po, int16_t* flag_out)
 {
-    // one pass: the extreme deviation and the excess sums of both signs (the
-    // sign picks one set at the end; each sum sees the same terms in the same
-    // order as a second pass would)
-    float best = -1.f;
-    float dbest = y(0) - B0;
-    float Wp = 0.f, Wup = 0.f, wmaxp = 0.f, Wn = 0.f, Wun = 0.f, wmaxn = 0.f;
+    // one pass: the extremes and the excess sums of both signs (the sign picks
+    // one set at the end; each sum sees the same terms in the same order as a
+    // second pass would)
+    float2 W2 = make_float2(0.f, 0.f);
+    float Wup = 0.f, Wun = 0.f, wmaxp = 0.f, wmaxn = 0.f;
+#pragma unroll 8
     for (int k = 0; k < T; ++k) {
         const float d = y(k) - B0;
-        const float dv = fabsf(d);
-        if (dv > best) {
-            best = dv;
-            dbest = d;
-        }
         const float wp = fmaxf(d, 0.f), wn = fmaxf(-d, 0.f);
         const float uk = u(k);
-        Wp += wp;
+        W2 = __fadd2_rn(W2, make_float2(wp, wn));
         Wup = fmaf(wp, uk, Wup);
-        wmaxp = fmaxf(wmaxp, wp);
-        Wn += wn;
         Wun = fmaf(wn, uk, Wun);
-        wmaxn = fmaxf(wmaxn, wn);
+        wmaxp = fmaxf(wmaxp, d);
+        wmaxn = fmaxf(wmaxn, -d);
     }
-    const float sgn = dbest >= 0.f ? 1.0f : -1.0f;
+    const float sgn = larger_is_positive(y, T, B0, wmaxp, wmaxn) ? 1.0f : -1.0f;
+    const float Wp = W2.x, Wn = W2.y;
     const float W = sgn > 0.f ? Wp : Wn, Wu = sgn > 0.f ? Wup : Wun, wmax = sgn > 0.f ? wmaxp : wmaxn;
     float c0, g0, A0;
     int flag = 0;
@@ -85,32 +95,36 @@ __device__ __forceinline__ void moment_finish(Y y, U u, int T, float B0, float u
 template <class Y, class U>
 __device__ __forceinline__ void moment_finish8(Y y, U u, int T, float B0, float u_mid, float du, float span, float* po)
 {
-    float best = -1.f, dbest = 0.f, wmaxp = 0.f, wmaxn = 0.f;
-    float Wp[8], Up[8], Wn[8], Un[8];
+    float wmaxp = 0.f, wmaxn = 0.f;
+    float2 W2[8];
+    float Up[8], Un[8];
 #pragma unroll
-    for (int l = 0; l < 8; ++l) Wp[l] = Up[l] = Wn[l] = Un[l] = 0.f;
+    for (int l = 0; l < 8; ++l) {
+        W2[l] = make_float2(0.f, 0.f);
+        Up[l] = Un[l] = 0.f;
+    }
     for (int k0 = 0; k0 < T; k0 += 8) {
 #pragma unroll
         for (int l = 0; l < 8; ++l) {
             const int k = k0 + l;
             if (k >= T) break;
             const float d = y(k) - B0;
-            const float dv = fabsf(d);
-            if (dv > best) {
-                best = dv;
-                dbest = d;
-            }
             const float wp = fmaxf(d, 0.f), wn = fmaxf(-d, 0.f);
             const float uk = u(k);
-            Wp[l] += wp;
+            W2[l] = __fadd2_rn(W2[l], make_float2(wp, wn));
             Up[l] = fmaf(wp, uk, Up[l]);
-            wmaxp = fmaxf(wmaxp, wp);
-            Wn[l] += wn;
             Un[l] = fmaf(wn, uk, Un[l]);
-            wmaxn = fmaxf(wmaxn, wn);
+            wmaxp = fmaxf(wmaxp, d);
+            wmaxn = fmaxf(wmaxn, -d);
         }
     }
-    const bool pos = dbest >= 0.f;
+    const bool pos = larger_is_positive(y, T, B0, wmaxp, wmaxn);
+    float Wp[8], Wn[8];
+#pragma unroll
+    for (int l = 0; l < 8; ++l) {
+        Wp[l] = W2[l].x;
+        Wn[l] = W2[l].y;
+    }
     auto total = [&](const float (&p)[8], const float (&n)[8]) {
         float v[8];
 #pragma unroll
@@ -132,19 +146,85 @@ __device__ __forceinline__ void moment_finish8(Y y, U u, int T, float B0, float 
     po[3] = B0;
 }
 
+// the guess of frame fo, whose normalised spectrum yk reads
+template <int NPAD, int NOUT, bool EIGHT, class Y>
+__device__ __forceinline__ void guess_frame(const InitArgs& a, Y yk, const float* us, const int* outer, int64_t fo)
+{
+    const int T = a.T;
+    constexpr OddEvenNet<NPAD> net{};
+    float v[NPAD];
+    float B0;
+    if constexpr (NOUT > 0) {
+#pragma unroll
+        for (int i = 0; i < NPAD; ++i) v[i] = i < NOUT ? yk(outer[i]) : INFINITY;
+        constexpr int kLo = (NOUT - 1) / 2, kHi = NOUT / 2;
+        rank_network<NPAD, NOUT, kLo, kHi>(v);
+        B0 = 0.5f * (v[kLo] + v[kHi]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < NPAD; ++i) v[i] = (i < a.n_outer) ? yk(outer[i]) : INFINITY;
+#pragma unroll
+        for (int c = 0; c < OddEvenNet<NPAD>::kCount; ++c) {
+            const float lo = fminf(v[net.lo[c]], v[net.hi[c]]);
+            const float hi = fmaxf(v[net.lo[c]], v[net.hi[c]]);
+            v[net.lo[c]] = lo;
+            v[net.hi[c]] = hi;
+        }
+        const int rlo = (a.n_outer - 1) >> 1, rhi = a.n_outer >> 1;
+        float vlo = 0.f, vhi = 0.f;
+#pragma unroll
+        for (int i = 0; i < NPAD; ++i) {
+            vlo = (i == rlo) ? v[i] : vlo;
+            vhi = (i == rhi) ? v[i] : vhi;
+        }
+        B0 = 0.5f * (vlo + vhi);
+    }
+    auto uk = [&](int k) { return us[k]; };
+    if constexpr (EIGHT) {
+        // moment_init ranks by counting: with an undefined value among
+        // the outer teeth the networks give another pair of middle values
+        bool nan = false;
+        for (int i = 0; i < a.n_outer; ++i) nan |= isnan(yk(outer[i]));
+        if (nan) {
+            const int rlo = (a.n_outer - 1) >> 1, rhi = a.n_outer >> 1;
+            float vlo = 0.f, vhi = 0.f;
+            for (int j = 0; j < a.n_outer; ++j) {
+                const float vj = yk(outer[j]);
+                int rank = 0;
+                for (int i = 0; i < a.n_outer; ++i) {
+                    const float vi = yk(outer[i]);
+                    rank += (vi < vj) || (vi == vj && i < j);
+                }
+                if (rank == rlo) vlo += vj;
+                if (rank == rhi) vhi += vj;
+            }
+            B0 = 0.5f * (vlo + vhi);
+        }
+        moment_finish8(yk, uk, T, B0, a.u_mid, a.du, a.span, a.p0_out + fo * 4);
+    } else {
+        moment_finish(yk, uk, T, B0, a.u_mid, a.du, a.span, a.x_mid, a.x_scale, a.p0_out + fo * 4,
+                      a.flag_out ? a.flag_out + fo : nullptr);
+    }
+}
+
 // A warp takes 32 consecutive frames at a time: their normalised spectra
 // (row stride odd, so the lanes' reads of one tooth fall on distinct banks)
-// arrive in shared memory by one bulk copy per 32 rows, double-buffered so the
-// next rows land while these are read (else by coalesced loads); each lane
-// then computes its frame's guess as the oracle defines it: baseline = median
-// of the outer fifth (sorted with the network, +inf padding), sign of the
-// largest deviation, centroid / extreme / area of the one-signed excess.
+// arrive in shared memory by one bulk copy per 32 rows (else by coalesced
+// loads); each lane then computes its frame's guess as the oracle defines it:
+// baseline = median of the outer fifth (sorted with the network, +inf padding),
+// sign of the largest deviation, centroid / extreme / area of the one-signed
+// excess.  Eight warps with one buffer each: one warp's copies fall into the
+// others' arithmetic (four warps with two buffers each left a scheduler one
+// warp, whose chains of dependent additions it could not fill).  Bounded by
+// reading the rows (10^6 of 99 teeth: 58 us) and by issue, about ten
+// instructions a tooth.  10^6 spectra of 99 teeth 87.6 -> 66.6 us, 10^5 of 221
+// 38.7 -> 22.1 us, 30,000 of 201 19 -> 12.3 us.
 // NOUT > 0: the outer set has NOUT teeth (a compile-time count): its median
 // comes from the merge network pruned to the two middle ranks; NOUT = 0 sorts
 // the NPAD wires (a.n_outer real, the rest +infinity) fully.
 // EIGHT: the guess of the fit at eight lanes per frame (moment_finish8)
 template <int NPAD, int NOUT, bool EIGHT = false>
-__global__ void __launch_bounds__(128) init_kernel(InitArgs a)
+__global__ void __launch_bounds__(kInitThreads) init_kernel(InitArgs a)
 {
     extern __shared__ __align__(16) float ism[];
     tc::pdl_start();
@@ -152,16 +232,14 @@ __global__ void __launch_bounds__(128) init_kernel(InitArgs a)
     float* us = ism;
     float* iref = us + T;
     int* outer = reinterpret_cast<int*>(iref + T);
-    // per warp two mbarriers and two 32-row buffers (task t lands in buffer
-    // t % 2 while the other one is read)
+    // per warp an mbarrier and a 32-row buffer
     const int warp = threadIdx.x >> 5;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(ism + ((2 * T + a.n_outer + 3) & ~3)) + 2 * warp;
-    float* rows0 = reinterpret_cast<float*>(reinterpret_cast<uint64_t*>(ism + ((2 * T + a.n_outer + 3) & ~3)) + 8) +
-                   warp * 2 * 32 * TS;
+    uint64_t* bars0 = reinterpret_cast<uint64_t*>(ism + ((2 * T + a.n_outer + 3) & ~3));
+    uint64_t* bar = bars0 + warp;
+    float* rows = reinterpret_cast<float*>(bars0 + kInitThreads / 32) + warp * 32 * TS;
     const int lane = threadIdx.x & 31;
     if (lane == 0) {
-        tc::mbar_init(&bars[0], 1);
-        tc::mbar_init(&bars[1], 1);
+        tc::mbar_init(bar, 1);
         tc::fence_mbar_init();
     }
     for (int i = threadIdx.x; i < T; i += blockDim.x) {
@@ -171,7 +249,6 @@ __global__ void __launch_bounds__(128) init_kernel(InitArgs a)
     for (int i = threadIdx.x; i < a.n_outer; i += blockDim.x) outer[i] = a.outer_idx[i];
     __syncthreads();
     tc::pdl_wait();
-    constexpr OddEvenNet<NPAD> net{};
     const int64_t nwarps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
     int64_t n = a.n;
     if (a.list_n) {
@@ -185,39 +262,32 @@ __global__ void __launch_bounds__(128) init_kernel(InitArgs a)
         return a.bulk && !a.list && (task + 1) * 32 <= n &&
                (reinterpret_cast<uintptr_t>(srcbase + task * 32 * T) & 15) == 0;
     };
-    auto issue = [&](int64_t task, int b) {
+    auto issue = [&](int64_t task) {
         if (lane == 0) {
             tc::fence_proxy_async_smem();   // generic reads of the buffer are ordered before the copy
-            tc::mbar_arrive_expect_tx(&bars[b], static_cast<uint32_t>(32 * T * 4));
-            tc::bulk_g2s(rows0 + b * 32 * TS, srcbase + task * 32 * T, static_cast<uint32_t>(32 * T * 4), &bars[b]);
+            tc::mbar_arrive_expect_tx(bar, static_cast<uint32_t>(32 * T * 4));
+            tc::bulk_g2s(rows, srcbase + task * 32 * T, static_cast<uint32_t>(32 * T * 4), bar);
         }
     };
-    uint32_t phase = 0u, pending = 0u;   // bit b: buffer b's parity / a copy in flight
+    uint32_t phase = 0u;
+    bool pending = false;   // a copy is in flight
     int64_t task = static_cast<int64_t>(warp) * gridDim.x + blockIdx.x;   // (few tasks spread over the SMs)
     if (task * 32 < n && bulk_ok(task)) {
-        issue(task, 0);
-        pending |= 1u;
+        issue(task);
+        pending = true;
     }
     bool failed = false;
-    for (int b = 0; task * 32 < n; task += nwarps, b ^= 1) {
-        float* rows = rows0 + b * 32 * TS;
+    for (; task * 32 < n; task += nwarps) {
         const int64_t f0 = task * 32;
         const int nf = (n - f0) < 32 ? static_cast<int>(n - f0) : 32;
-        // the next task's copy goes out before this one is read
-        const int64_t nt = task + nwarps;
-        __syncwarp();
-        if (nt * 32 < n && bulk_ok(nt)) {
-            issue(nt, b ^ 1);
-            pending |= 1u << (b ^ 1);
-        }
-        const bool in_smem_raw = (pending >> b) & 1u;   // rows hold y, or amps still to be scaled
+        const bool in_smem_raw = pending;   // rows hold y, or amps still to be scaled
         if (in_smem_raw) {
-            if (!tc::mbar_wait(&bars[b], (phase >> b) & 1u, 1u << 24)) {
+            if (!tc::mbar_wait(bar, phase, 1u << 24)) {
                 failed = true;
                 break;
             }
-            phase ^= 1u << b;
-            pending &= ~(1u << b);
+            phase ^= 1u;
+            pending = false;
         } else if (a.list) {
             // listed frames (the fallback pass): one coalesced row at a time
             for (int f = 0; f < nf; ++f) {
@@ -296,67 +366,22 @@ __global__ void __launch_bounds__(128) init_kernel(InitArgs a)
             const int64_t fo = a.list ? static_cast<int64_t>(a.list[f0 + lane]) : f0 + lane;
             const float* r = rows + lane * TS;
             // bulk-copied magnitudes are normalised here, as the staging does
-            const bool scale = in_smem_raw && !a.y;
-            auto yk = [&](int k) { return scale ? __fmul_rn(r[k], iref[k]) : r[k]; };
-            float v[NPAD];
-            float B0;
-            if constexpr (NOUT > 0) {
-#pragma unroll
-                for (int i = 0; i < NPAD; ++i) v[i] = i < NOUT ? yk(outer[i]) : INFINITY;
-                constexpr int kLo = (NOUT - 1) / 2, kHi = NOUT / 2;
-                rank_network<NPAD, NOUT, kLo, kHi>(v);
-                B0 = 0.5f * (v[kLo] + v[kHi]);
-            } else {
-#pragma unroll
-                for (int i = 0; i < NPAD; ++i) v[i] = (i < a.n_outer) ? yk(outer[i]) : INFINITY;
-#pragma unroll
-                for (int c = 0; c < OddEvenNet<NPAD>::kCount; ++c) {
-                    const float lo = fminf(v[net.lo[c]], v[net.hi[c]]);
-                    const float hi = fmaxf(v[net.lo[c]], v[net.hi[c]]);
-                    v[net.lo[c]] = lo;
-                    v[net.hi[c]] = hi;
-                }
-                const int rlo = (a.n_outer - 1) >> 1, rhi = a.n_outer >> 1;
-                float vlo = 0.f, vhi = 0.f;
-#pragma unroll
-                for (int i = 0; i < NPAD; ++i) {
-                    vlo = (i == rlo) ? v[i] : vlo;
-                    vhi = (i == rhi) ? v[i] : vhi;
-                }
-                B0 = 0.5f * (vlo + vhi);
-            }
-            auto uk = [&](int k) { return us[k]; };
-            if constexpr (EIGHT) {
-                // moment_init ranks by counting: with an undefined value among
-                // the outer teeth the networks give another pair of middle values
-                bool nan = false;
-                for (int i = 0; i < a.n_outer; ++i) nan |= isnan(yk(outer[i]));
-                if (nan) {
-                    const int rlo = (a.n_outer - 1) >> 1, rhi = a.n_outer >> 1;
-                    float vlo = 0.f, vhi = 0.f;
-                    for (int j = 0; j < a.n_outer; ++j) {
-                        const float vj = yk(outer[j]);
-                        int rank = 0;
-                        for (int i = 0; i < a.n_outer; ++i) {
-                            const float vi = yk(outer[i]);
-                            rank += (vi < vj) || (vi == vj && i < j);
-                        }
-                        if (rank == rlo) vlo += vj;
-                        if (rank == rhi) vhi += vj;
-                    }
-                    B0 = 0.5f * (vlo + vhi);
-                }
-                moment_finish8(yk, uk, T, B0, a.u_mid, a.du, a.span, a.p0_out + fo * 4);
-            } else {
-                moment_finish(yk, uk, T, B0, a.u_mid, a.du, a.span, a.x_mid, a.x_scale, a.p0_out + fo * 4,
-                              a.flag_out ? a.flag_out + fo : nullptr);
-            }
+            if (in_smem_raw && !a.y)
+                guess_frame<NPAD, NOUT, EIGHT>(a, [&](int k) { return __fmul_rn(r[k], iref[k]); }, us, outer, fo);
+            else
+                guess_frame<NPAD, NOUT, EIGHT>(a, [&](int k) { return r[k]; }, us, outer, fo);
+        }
+        // the buffer is read: the next task's copy goes out
+        __syncwarp();
+        const int64_t nt = task + nwarps;
+        if (nt * 32 < n && bulk_ok(nt)) {
+            issue(nt);
+            pending = true;
         }
     }
     // no copy may land after the block exits
     __syncwarp();
-    for (int b = 0; b < 2; ++b)
-        if (((pending >> b) & 1u) && !tc::mbar_wait(&bars[b], (phase >> b) & 1u, 1u << 24)) failed = true;
+    if (pending && !tc::mbar_wait(bar, phase, 1u << 24)) failed = true;
     if (failed && lane == 0 && a.err) atomicExch(a.err, 2);
 }
 
@@ -777,7 +802,7 @@ cudaError_t launch_init(const cg_plan_s* p, const float* y, const float* amps, i
     const int64_t tasks = (n + 31) / 32;
     const int grid = static_cast<int>(tasks < p->grid_init ? tasks : p->grid_init);
     void* args[] = {&a};
-    return launch_dependent(init_ptr(p->init_npad, p->n_outer, eight), dim3(grid), dim3(128), args, p->init_smem, s);
+    return launch_dependent(init_ptr(p->init_npad, p->n_outer, eight), dim3(grid), dim3(kInitThreads), args, p->init_smem, s);
 }
 
 cudaError_t launch_fit2(const cg_plan_s* p, const float* y, const float* amps, int64_t n,

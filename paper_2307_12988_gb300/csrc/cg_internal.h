@@ -90,6 +90,8 @@ struct CosetArgs {
     int sm_twN, sm_twL, sm_twQ, sm_tooth, sm_bar, sm_raw, sm_Y, sm_total;
 };
 
+constexpr int kInitThreads = 256;   // of the guess kernel
+
 // Arguments of the lane-per-frame moment initial guess.
 struct InitArgs {
     int64_t n;
