@@ -74,7 +74,8 @@ struct Welch {
     static constexpr int kSmemZ = G * L * 8;
     static constexpr int kSmemT = kSmemZ + (15 * 16 + (R3 - 1) * 256) * 8;
     static constexpr int kSmemW = kSmemT + (M / 2 + 4) * 4;
-    static constexpr int kSmem = kSmemW + G * (2 * NT / 32) * 4 + G * 8;
+    static constexpr int kSmemB = kSmemW + G * (2 * NT / 32) * 4 + G * 8;   // two barriers of each group
+    static constexpr int kSmem = kSmemB + G * 16;
 };
 
 struct PsdArgs {
@@ -82,6 +83,7 @@ struct PsdArgs {
     int64_t stride;            // elements between consecutive samples
     int64_t K;                 // segments
     int vec2;                  // sample pairs are 8-byte aligned and contiguous
+    int bulk;                  // so are whole segments, 16-byte aligned
     const float* win;
     const float2* tw;
     const int2* pair0;
@@ -164,9 +166,14 @@ __device__ __forceinline__ void pair_add2(float2& a, float2 b)
 // 10,000 cycles) and the transform's FP32 work.  Before, the sums lived in
 // L2 as FP64 rows and every table but one was read from L2 (0.75 MB per
 // segment), the sums and the mean ran in FP64 on every thread, and each stage
-// took two barriers of 1,024 threads.  Ten minutes of centres (36,620
-// segments of 32,768): 7.99 -> 3.11 ms (27,000 cycles a segment; the shared
-// memory is busy for 54 % of them).
+// took two barriers of 1,024 threads: ten minutes of centres (36,620 segments
+// of 32,768) in 7.99 ms.  In place 3.11 ms (27,000 cycles a segment, the shared
+// memory busy for 54 % of them), of which a segment waited for 8-byte
+// asynchronous copies of the next to begin only when all of it was split;
+// 2.63 ms with bulk copies in two parts, the first under the second half of
+// the split and the sums of the first under the second; 2.53 ms with the last
+// stage's twiddles all requested at once and the split's before its barrier
+// (they come from L2).
 template <int L>
 __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
 {
@@ -185,26 +192,58 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
     const int64_t nslot = static_cast<int64_t>(G) * gridDim.x;
     const uint32_t zt = z + 8 * zsw(t);             // point t, and NT - 1 - t
     const uint32_t zr = z + 8 * zsw(NT - 1 - t);
+    const uint32_t zl = z + 8 * t;                  // point t of the samples
 
+    // The samples of a segment lie in the order of its points (the stages'
+    // places are those of their 16-point block, permuted).  Contiguous ones
+    // come by bulk copies in two parts, as the split of the segment before
+    // leaves the blocks they go to: 0 to 4 and 12 to 15, then 5 to 11.
+    uint64_t* const bars = reinterpret_cast<uint64_t*>(psm + W::kSmemB) + 2 * g;
+    auto stage_part = [&](int64_t s, int part) {   // (one thread)
+        const float* x = a.x + s * static_cast<int64_t>(L);
+        tc::fence_proxy_async_smem();   // the places were read before they are written
+        tc::mbar_arrive_expect_tx(&bars[part], (part ? 7 : 9) * B * 8);
+        auto blocks = [&](int b0, int n) {
+            tc::bulk_g2s(psm + g * L * 8 + b0 * B * 8, x + 2 * b0 * B, n * B * 8, &bars[part]);
+        };
+        if (part) {
+            blocks(5, 7);
+        } else {
+            blocks(0, 5);
+            blocks(12, 4);
+        }
+    };
     auto stage_x = [&](int64_t s) {   // the thread's own 32 points of segment s, asynchronously
         const float* x = a.x + s * static_cast<int64_t>(L) * a.stride;
         if (a.vec2) {
             x += 2 * t;
 #pragma unroll 8
             for (int i = 0; i < 32; ++i)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(zat(zt, NT * i)), "l"(x + 2 * NT * i) : "memory");
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(zl + 8 * NT * i), "l"(x + 2 * NT * i) : "memory");
         } else {
             x += 2 * t * a.stride;
 #pragma unroll 4
             for (int i = 0; i < 32; ++i) {
                 const float* p = x + 2 * NT * i * a.stride;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(zat(zt, NT * i)), "l"(p) : "memory");
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(zat(zt, NT * i) + 4), "l"(p + a.stride) : "memory");
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(zl + 8 * NT * i), "l"(p) : "memory");
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(zl + 8 * NT * i + 4), "l"(p + a.stride) : "memory");
             }
         }
         cp_async_commit();
     };
-    if (slot < a.K) stage_x(slot);
+    if (t == 0) {
+        tc::mbar_init(&bars[0], 1);
+        tc::mbar_init(&bars[1], 1);
+        tc::fence_mbar_init();
+    }
+    if (slot < a.K) {
+        if (!a.bulk) {
+            stage_x(slot);
+        } else if (t == 0) {
+            stage_part(slot, 0);
+            stage_part(slot, 1);
+        }
+    }
     for (int i = threadIdx.x; i < W::kT4; i += kWelchThreads) ts[i] = a.tw[i];
     for (int i = threadIdx.x; i <= M / 2; i += kWelchThreads) win[i] = a.win[i];
     if (t == 0) *half = make_float2(0.f, 0.f);
@@ -215,25 +254,39 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
     __syncthreads();
 
     int since = 0;   // segments since the sums were normalised
-    for (int64_t s = slot; s < a.K; s += nslot) {
+    uint32_t phase = 0;
+    bool landed = true;   // (a copy that never does leaves the sums undefined)
+    for (int64_t s = slot; s < a.K; s += nslot, phase ^= 1u) {
         // the next segment into L2 meanwhile
-        if (s + nslot < a.K && a.stride <= 4) {
+        if (a.bulk) {
+            if (s + nslot < a.K && t == 0) tc::prefetch_l2_bulk(a.x + (s + nslot) * static_cast<int64_t>(L), M * 4);
+        } else if (s + nslot < a.K && a.stride <= 4) {
             const char* nx = reinterpret_cast<const char*>(a.x + (s + nslot) * static_cast<int64_t>(L) * a.stride);
             for (int64_t i = t; i < M * a.stride / 32; i += NT) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(nx + 128 * i));
         }
-        cp_async_wait_all();   // own points only: no barrier
+        if (a.bulk)
+            landed = landed && tc::mbar_wait(&bars[0], phase, 1u << 24);
+        else
+            cp_async_wait_all();   // own points only: no barrier
         // ---- segment mean: FP32 sums of 32 samples per first-stage column ----
+        float sum[2] = {0.f, 0.f};
+        auto column = [&](int r) {
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const float2 v = zld(zl + 8 * NT * (b + 2 * r));
+                sum[b] += v.x + v.y;
+            }
+        };
+#pragma unroll
+        for (int r = 0; r < 5; ++r) column(r);
+        if (a.bulk) landed = landed && tc::mbar_wait(&bars[1], phase, 1u << 24);
+#pragma unroll
+        for (int r = 5; r < 16; ++r) column(r);
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            float sum = 0.0f;
 #pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                const float2 v = zld(zat(zt, NT * (b + 2 * r)));
-                sum += v.x + v.y;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            if (lane == 0) red[w + (NT / 32) * b] = sum;
+            for (int o = 16; o > 0; o >>= 1) sum[b] += __shfl_xor_sync(0xffffffffu, sum[b], o);
+            if (lane == 0) red[w + (NT / 32) * b] = sum[b];
         }
         group_sync<NT>(g);
         // every warp adds the warp sums as FP32 pairs (48 bits) and rounds once
@@ -251,7 +304,7 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
 #pragma unroll
             for (int r = 0; r < 16; ++r) {
                 const int n = j + r * B;
-                v[r] = zld(zat(zj, r * B));
+                v[r] = zld(zl + 8 * (NT * b + r * B));
                 float2 wn;
                 if (r < 8)
                     wn = *reinterpret_cast<const float2*>(win + 2 * n);
@@ -259,6 +312,7 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
                     wn = make_float2(win[M - 2 * n], win[M - 2 * n - 1]);
                 v[r] = make_float2((v[r].x - mean) * wn.x, (v[r].y - mean) * wn.y);
             }
+            __syncwarp();   // (the points' places lie among those the warp has read)
             Dft<16>::run(v);
 #pragma unroll
             for (int r = 0; r < 16; ++r) zst(zat(zj, r * B), v[r]);
@@ -301,7 +355,7 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
         if constexpr (R4 > 1) {
             __syncwarp();
             const float2* t4 = a.tw + W::kT4 + (1024 / R4) * w + lane;
-#pragma unroll 4
+#pragma unroll
             for (int b = 0; b < 32 / R4; ++b) {
                 const uint32_t zb = z + 8 * zsw(1024 * w + R4 * (lane + 32 * b));
                 float2 v[R4];
@@ -314,29 +368,50 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
                 for (int r = 0; r < R4; ++r) zst(zat(zb, r), v[r]);
             }
         }
+        float2 tws[16];   // the split's twiddles, requested ahead of the barriers
+        tws[15] = __ldg(&a.tw[W::kSplit + 15 * NT + t]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) tws[i] = __ldg(&a.tw[W::kSplit + i * NT + t]);
         group_sync<NT>(g);
         // ---- real-FFT split of bins k and L - k, |X|^2 into the sums ----
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
+        const bool more = s + nslot < a.K;
+        auto split = [&](int i) {
             const int k1 = i < 14 ? 1 + (i >> 1) : 8, h = i < 14 ? i & 1 : 0;
             const float2 Zb = zld(i < 15 ? zat(zt, k1 * B + NT * h) : z + 8 * p15.x);
             const float2 Zr = zld(i < 15 ? zat(zr, (16 - k1) * B + NT * (1 - h)) : z + 8 * p15.y);
             const float2 E = make_float2(0.5f * (Zb.x + Zr.x), 0.5f * (Zb.y - Zr.y));
             const float2 Dd = make_float2(0.5f * (Zb.x - Zr.x), 0.5f * (Zb.y + Zr.y));
-            const float2 C = cmul(__ldg(&a.tw[W::kSplit + i * NT + t]), make_float2(Dd.y, -Dd.x));
+            const float2 C = cmul(tws[i], make_float2(Dd.y, -Dd.x));
             // X_k = E + C; X_(L - k) = conj(E - C), since W_M^(L - k) = -conj W_M^k
             const float2 X = cadd(E, C), Y = csub(E, C);
             pair_add(acc[i][0], fmaf(X.x, X.x, X.y * X.y));
             pair_add(acc[i][1], fmaf(Y.x, Y.x, Y.y * Y.y));
-        }
+        };
+        // blocks 0 to 4 and 12 to 15 first: the next segment's samples follow
+        split(15);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) split(i);
+#pragma unroll
+        for (int i = 8; i < 15; ++i) tws[i] = __ldg(&a.tw[W::kSplit + i * NT + t]);
         if (t == 0) {   // bin L / 2 pairs with itself
             constexpr int kPos = R4 > 1 ? R4 / 2 : R3 / 2;   // its last digit is R / 2, the others 0
             const float2 Zh = zld(z + 8 * zsw(kPos));
             const float2 X = cadd(make_float2(Zh.x, 0.f), cmul(__ldg(&a.tw[W::kHalf]), make_float2(Zh.y, -0.f)));
             pair_add2(*half, make_float2(fmaf(X.x, X.x, X.y * X.y), 0.f));
         }
+        if (a.bulk) {
+            group_sync<NT>(g);
+            if (more && t == 0) stage_part(s + nslot, 0);
+        }
+#pragma unroll
+        for (int i = 8; i < 15; ++i) split(i);
         group_sync<NT>(g);
-        if (s + nslot < a.K) stage_x(s + nslot);
+        if (more) {
+            if (!a.bulk)
+                stage_x(s + nslot);
+            else if (t == 0)
+                stage_part(s + nslot, 1);
+        }
         if (++since == 8 || s + nslot >= a.K) {
             since = 0;
 #pragma unroll
@@ -348,12 +423,14 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
     }
     if (slot < a.K) {
         float2* row = a.part + slot * (L + 1);
+        const float undefined = __int_as_float(0x7fffffff);
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
+            if (!landed) acc[i][0] = acc[i][1] = make_float2(undefined, undefined);
             row[(2 * i) * NT + t] = acc[i][0];
             row[(2 * i + 1) * NT + t] = acc[i][1];
         }
-        if (t == 0) row[L] = *half;
+        if (t == 0) row[L] = landed ? *half : make_float2(undefined, undefined);
     }
 }
 
@@ -983,7 +1060,8 @@ cg_status cg_psd_welch(cg_psd_t h, const float* x_dev, int64_t n, int64_t stride
     if (n_segments) *n_segments = K;
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int vec2 = stride == 1 && (reinterpret_cast<uintptr_t>(x_dev) & 7) == 0;
-    PsdArgs a{x_dev, stride, K, vec2, h->win, h->tw, h->pair0, h->part};
+    const int bulk = stride == 1 && (reinterpret_cast<uintptr_t>(x_dev) & 15) == 0;
+    PsdArgs a{x_dev, stride, K, vec2, bulk, h->win, h->tw, h->pair0, h->part};
     WelchInst wi;
     welch_inst(h->L, &wi);
     // one block per SM; the segments go to different SMs before they share one
