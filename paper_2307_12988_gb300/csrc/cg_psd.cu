@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
 {
     using W = Welch<L>;
     constexpr int NT = W::NT, R3 = W::R3, R4 = W::R4, B = W::B, M = W::M, G = W::G;
+    tc::pdl_start();
     extern __shared__ __align__(1024) unsigned char psm[];
     const int g = threadIdx.x / NT, t = threadIdx.x % NT, w = t >> 5, lane = t & 31;
     const uint32_t z = static_cast<uint32_t>(__cvta_generic_to_shared(psm)) + g * L * 8;
@@ -442,6 +443,8 @@ __global__ void __launch_bounds__(256) psd_reduce_kernel(const float2* part, int
                                                          const int* bin, double* psd)
 {
     __shared__ float2 red[8][33];
+    tc::pdl_start();
+    tc::pdl_wait();
     const int i = blockIdx.x * 32 + threadIdx.x;
     float2 s = make_float2(0.f, 0.f);
     if (i <= L) {
@@ -712,7 +715,8 @@ __device__ __forceinline__ bool res_inv_diag(const double* Hu, double (&dg)[4])
 // barrier per step is all that the blocks exchange.  ln S is taken once.  The
 // fit of a 393-bin band: 330 us on one block, 137 on the cluster, 101 with
 // the solve in registers and two divisions per point, 71 with Newton
-// reciprocals, the table logarithm and the solve over four lanes.
+// reciprocals, the table logarithm and the solve over four lanes, 62 with a
+// warp's two sums reduced together and the sums at the result reused.
 __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads)
     resonance_fit_kernel(ResArgs a)
 {
@@ -730,13 +734,14 @@ __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads
     const uint32_t rank = tc::cluster_rank();
     const double* S = a.psd + a.k0;
     const int rows = (a.np + kResRow - 1) / kResRow;
-    for (int c = warp; c < rows && c < kResLogRows; c += kResWarps) {
-        const int i = c * kResRow + static_cast<int>(rank) * 32 + lane;
-        if (i < a.np) logs[c][lane] = log(S[i]);   // read back by this thread only
-    }
     if (t < 128) {
         const double c = static_cast<double>(1.0f / (1.0f + (t + 0.5f) * (1.0f / 128.0f)));
         tab[t] = make_double2(c, -log(c));
+    }
+    tc::pdl_wait();   // (the density may come from the kernel before)
+    for (int c = warp; c < rows && c < kResLogRows; c += kResWarps) {
+        const int i = c * kResRow + static_cast<int>(rank) * 32 + lane;
+        if (i < a.np) logs[c][lane] = log(S[i]);   // read back by this thread only
     }
     // the two sums of this warp: pairs (i, j) of J^T J row by row, then J^T r, r r and the bad points
     const int q0 = 2 * warp;
@@ -795,17 +800,17 @@ __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads
                                            : fma(pts[buf][k][i1][lane], pts[buf][k][j1][lane], sb);
             }
         }
+        // both sums over the lanes, distances 16, 8, 4, 2, 1: after the first
+        // the lower half warp adds up the one, the upper half the other
+        const bool upper = lane >= 16;
+        double sum = (upper ? sb : sa) + __shfl_xor_sync(0xffffffffu, upper ? sa : sb, 16);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sa += __shfl_xor_sync(0xffffffffu, sa, o);
-            sb += __shfl_xor_sync(0xffffffffu, sb, o);
-        }
-        if (lane < kResBlocks) {   // lane b hands this block's two sums to block b
-            const uint32_t own = static_cast<uint32_t>(__cvta_generic_to_shared(&red[parity][rank][q0]));
+        for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if ((lane & 15) < kResBlocks) {   // lanes b and 16 + b hand this block's two sums to block b
+            const uint32_t own = static_cast<uint32_t>(__cvta_generic_to_shared(&red[parity][rank][q0 + (upper ? 1 : 0)]));
             uint32_t there;
-            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(own), "r"(lane));
-            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there), "d"(sa) : "memory");
-            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there + 8), "d"(sb) : "memory");
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(own), "r"(lane & 15));
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there), "d"(sum) : "memory");
         }
         tc::cluster_sync();
         if (t < 16) {
@@ -895,7 +900,7 @@ __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads
     double p = sp[r], chi2 = (tot[15] > 0.0) ? INFINITY : tot[14], lambda = a.lambda0;
     double H[4] = {tot[h0], tot[h1], tot[h2], tot[h3]}, gr = tot[10 + r];
     int it = 0, st = 1;
-    bool stop = false;
+    bool stop = false, here = true;   // here: the sums at hand are those at p
     if (!(chi2 < INFINITY)) {
         st = 3;
         stop = true;
@@ -928,6 +933,7 @@ __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads
             const double c2 = (tot[15] > 0.0) ? INFINITY : tot[14];
             const bool settled = (c2 < INFINITY) && fabs(c2 - chi2) <= a.tol * chi2;
             const bool better = (c2 < INFINITY) && (settled ? c2 <= chi2 : c2 < chi2);
+            here = better;
             if (better) {
                 p = sp[r];
                 chi2 = c2;
@@ -945,14 +951,20 @@ __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads
             }
         }
     }
-    // standard errors from the sums at the result
-    if (warp == 0) {
-        if (lane < 4) sp[r] = p;
-        __syncwarp();
-        constants();
-    }
+    // standard errors from the sums at the result, taken again only where the
+    // last point was refused (every block of the cluster finds the same)
+    __syncthreads();   // (all have read s_ctl)
+    if (warp == 0 && lane == 0) s_ctl = here ? 1 : 0;
     __syncthreads();
-    sums();
+    if (!s_ctl) {
+        if (warp == 0) {
+            if (lane < 4) sp[r] = p;
+            __syncwarp();
+            constants();
+        }
+        __syncthreads();
+        sums();
+    }
     if (t == 0 && rank == 0) {
         double dg[4] = {NAN, NAN, NAN, NAN};
         const bool inv = a.np > 4 && res_inv_diag(tot, dg);
@@ -1072,8 +1084,10 @@ cg_status cg_psd_welch(cg_psd_t h, const float* x_dev, int64_t n, int64_t stride
     cudaError_t e = cudaLaunchKernel(wi.fn, dim3(grid), dim3(wi.threads), args, h->smem, s);
     if (e == cudaSuccess) {
         const double scale = 1.0 / (static_cast<double>(K) * fs * h->sum_w2);
-        psd_reduce_kernel<<<(h->L + 1 + 31) / 32, dim3(32, 8), 0, s>>>(h->part, rows, h->L, scale, h->bin, psd_dev);
-        e = cudaGetLastError();
+        const float2* part = h->part;
+        const int* bin = h->bin;
+        void* rargs[] = {&part, const_cast<int*>(&rows), &h->L, const_cast<double*>(&scale), &bin, &psd_dev};
+        e = launch_dependent(reinterpret_cast<void*>(&psd_reduce_kernel), dim3((h->L + 1 + 31) / 32), dim3(32, 8), rargs, 0, s);
     }
     if (e != cudaSuccess) return psd_cuda_fail(e, "cg_psd_welch");
     return CG_OK;
@@ -1092,9 +1106,8 @@ cg_status cg_resonance_fit(const double* psd_dev, int n_bins, double df, double 
     if (k1 - k0 + 1 < 8) return psd_fail(CG_ERR_ARG, "the band holds fewer than 8 bins");
     ResArgs a{psd_dev, k0, k1 - k0 + 1, df, max_iter, tol, 1e-3, out_dev};
     void* args[] = {&a};
-    cudaError_t e = cudaLaunchKernel(reinterpret_cast<void*>(&resonance_fit_kernel), dim3(kResBlocks),
-                                     dim3(kResThreads),
-                                     args, 0, static_cast<cudaStream_t>(stream));
+    cudaError_t e = launch_dependent(reinterpret_cast<void*>(&resonance_fit_kernel), dim3(kResBlocks),
+                                     dim3(kResThreads), args, 0, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return psd_cuda_fail(e, "cg_resonance_fit");
     return CG_OK;
 }
