@@ -1,5 +1,6 @@
 // cg_fit8.cu -- the standalone Levenberg-Marquardt fit at eight lanes per
-// frame (cg_fit, and the fit of CG_PATH_SPLIT), two frames per lane group.
+// frame (cg_fit, and the fit of CG_PATH_SPLIT), two or four frames per lane
+// group.
 //
 // Paper ("Data Capture and Processing", fit paragraphs): each normalised
 // spectrum is fit by Levenberg-Marquardt, at most 20 iterations, tolerance
@@ -7,23 +8,24 @@
 // (cg_fit.cuh): lane l of a frame's eight adds up teeth l, l + 8, ... in
 // order, the eight partial sums are added over lane distances 4, 2, 1.  What
 // differs is how the work lies on the warp:
-//  * a group of eight lanes evaluates two frames at once, one in each half of
-//    packed FP32x2 operations;
-//  * the 14 sums of the first frame end in its lower four lanes, those of the
-//    second in the upper four (the exchange over distance 4 does both), so one
-//    pass of the 4 x 4 solve and of the decisions serves both frames -- and
-//    eight frames per warp, where every lane of a group repeated one frame's;
-//  * each half pulls its next frame when its own is done; the row arrives
-//    meanwhile by one bulk copy into the half's other slot, so no frame waits
+//  * a group of eight lanes evaluates two (or two pairs of) frames at once, one
+//    in each half of packed FP32x2 operations;
+//  * the exchanges over distances 4 and 2 also sort the 14 sums by frame: they
+//    end in the four (two) lanes that own it, so one pass of the 4 x 4 solve
+//    and of the decisions serves every frame of the group -- eight (sixteen)
+//    per warp, where every lane of a group repeated one frame's;
+//  * each owner pulls its next frame when its own is done; the row arrives
+//    meanwhile by one bulk copy into the owner's other slot, so no frame waits
 //    for another's iterations;
 //  * the moment guess runs before, one lane per frame (init_kernel), and
 //    leaves its starting point (normalised abscissa) in params.
 //
-// What bounds it: instruction issue (65 % active; about 970 warp instructions
-// per evaluation of eight frames of 99 teeth, 390 of them in the teeth's loop,
-// where fit_group spent 1,340 on two times four).  10^5 spectra of 99 teeth:
-// 159 us in fit_kernel, which also held every block for its slowest frame;
-// 88 us here and 10 for the guess.
+// What bounds it: instruction issue (two frames a group: 65 % active; about 970
+// warp instructions per evaluation of eight frames of 99 teeth, 390 of them in
+// the teeth's loop, where fit_group spent 1,340 on two times four; four a
+// group: about 1,350 for sixteen).  10^5 spectra of 99 teeth: 159 us in
+// fit_kernel, which also held every block for its slowest frame; 88 us with
+// two frames a group, 84 with four, and 10 to 17 for the guess.
 #include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -37,7 +39,6 @@ namespace cg {
 namespace {
 
 constexpr int kWarps8 = 4;       // warps per block
-constexpr int kSlots8 = 16;      // row slots per warp: two per frame in flight
 
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
@@ -89,10 +90,11 @@ __device__ __forceinline__ void accum_pair(float u, float2 y, float2 c, float2 g
     s[13] = fma2(r, r, s[13]);
 }
 
-// sums over the eight lanes, distances 4, 2, 1: the lower four lanes get the
-// first frame's 14 sums, the upper four the second's
-__device__ __forceinline__ void reduce_pair(const float2 (&s)[14], LmSums& S)
+// sums over the eight lanes, distances 4, 2, 1.  Two frames: the lower four
+// lanes get the first frame's 14 sums, the upper four the second's
+__device__ __forceinline__ void reduce_frames(const float2 (&s2)[1][14], LmSums& S)
 {
+    const float2 (&s)[14] = s2[0];
     const int lane = threadIdx.x & 31;
     const bool hi = (lane & 4) != 0;
     float a[14];
@@ -125,13 +127,36 @@ __device__ __forceinline__ void reduce_pair(const float2 (&s)[14], LmSums& S)
     }
 }
 
-template <bool SCALE>
-__global__ void __launch_bounds__(32 * kWarps8, 4) fit8_kernel(Fit8Args a)
+// Four frames (the first two in s[0], the others in s[1]): two lanes each
+__device__ __forceinline__ void reduce_frames(const float2 (&s)[2][14], LmSums& S)
 {
+    const int lane = threadIdx.x & 31;
+    const bool b4 = (lane & 4) != 0, b2 = (lane & 2) != 0;
+#pragma unroll
+    for (int i = 0; i < 14; ++i) {
+        const float2 send = b4 ? s[0][i] : s[1][i], keep = b4 ? s[1][i] : s[0][i];
+        const float2 got = make_float2(__shfl_xor_sync(kFull, send.x, 4), __shfl_xor_sync(kFull, send.y, 4));
+        const float2 a = make_float2(keep.x + got.x, keep.y + got.y);
+        const float b = (b2 ? a.y : a.x) + __shfl_xor_sync(kFull, b2 ? a.x : a.y, 2);
+        S.v[i] = b + __shfl_xor_sync(kFull, b, 1);
+    }
+}
+
+// NF: frames of a lane group (2 or 4); 8 / NF lanes own a frame
+template <bool SCALE, int NF>
+__global__ void __launch_bounds__(32 * kWarps8, NF == 2 ? 4 : 3) fit8_kernel(Fit8Args a)
+{
+    constexpr int LP = 8 / NF;               // lanes that own a frame
+    constexpr int kInFlight = 32 / LP;       // frames of a warp
+    constexpr int kSlots8 = 2 * kInFlight;   // its row slots
     extern __shared__ __align__(16) float f8sm[];
     const int T = a.T;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gl = lane & 7, own = lane & 3, leader = lane & ~3, half = lane >> 2;   // half: 0 .. 7, a frame each
+    const int gl = lane & 7, own = lane & (LP - 1), leader = lane & ~(LP - 1), half = lane / LP;   // half: the frame
+    // its slot of either parity: those that the four groups read at a time lie
+    // a quarter of the banks apart (row stride 24 mod 32 for two slots, 8 or 24
+    // for one)
+    const int place = NF == 2 ? half : (half >> 2) + 4 * (half & 3);
     float* slots = f8sm + warp * kSlots8 * a.RS;
     uint64_t* bars = reinterpret_cast<uint64_t*>(f8sm + kWarps8 * kSlots8 * a.RS) + warp * kSlots8;
     float* us = reinterpret_cast<float*>(reinterpret_cast<uint64_t*>(f8sm + kWarps8 * kSlots8 * a.RS) + kWarps8 * kSlots8);
@@ -172,7 +197,7 @@ __global__ void __launch_bounds__(32 * kWarps8, 4) fit8_kernel(Fit8Args a)
         // ---- a half without a frame starts its next one ----
         if (f < 0 && fn >= 0) {
             const int nx = cs ^ 1;
-            const int sl = half + 8 * nx;
+            const int sl = place + kInFlight * nx;
             if (!tc::mbar_wait(&bars[sl], (ph >> nx) & 1u, 1u << 22)) failed = true;
             ph ^= 1u << nx;
             cs = nx;
@@ -230,7 +255,7 @@ __global__ void __launch_bounds__(32 * kWarps8, 4) fit8_kernel(Fit8Args a)
                 const uintptr_t a16 = ad & ~static_cast<uintptr_t>(15);
                 const uintptr_t e16 = (ad + 4u * T + 15u) & ~static_cast<uintptr_t>(15);
                 on = static_cast<int>((ad - a16) >> 2);
-                const int sl = half + 8 * (cs ^ 1);
+                const int sl = place + kInFlight * (cs ^ 1);
                 float* dst = slots + sl * a.RS;
                 if (own == 0) {
                     if (a16 >= buf_lo && e16 <= buf_hi) {
@@ -264,28 +289,46 @@ __global__ void __launch_bounds__(32 * kWarps8, 4) fit8_kernel(Fit8Args a)
             }
         }
         // ---- sums of both frames of the group at their trial points ----
-        float2 s[14];
+        float2 s[NF / 2][14];
         {
-            const bool hi = (lane & 4) != 0;
-            auto both = [&](float v) {   // (first frame's, second frame's)
-                const float o = __shfl_xor_sync(kFull, v, 4);
-                return make_float2(hi ? o : v, hi ? v : o);
-            };
-            const float2 c = both(pt[0]), g2 = both(pt[1] * pt[1]), nA = neg2(both(pt[2])), nB = neg2(both(pt[3]));
-            const int mine = (half + 8 * cs) * a.RS + oc, other = __shfl_xor_sync(kFull, mine, 4);
-            const float* ra = slots + (hi ? other : mine);
-            const float* rb = slots + (hi ? mine : other);
+            // the group's frames: (first, second), (third, fourth)
+            const int base = lane & ~7;
+            auto pairs = [&](float v, float2 (&o)[NF / 2]) {
+                if constexpr (NF == 2) {
+                    const float w = __shfl_xor_sync(kFull, v, 4);
+                    o[0] = (lane & 4) ? make_float2(w, v) : make_float2(v, w);
+                } else {
 #pragma unroll
-            for (int i = 0; i < 14; ++i) s[i] = make_float2(0.f, 0.f);
+                    for (int h = 0; h < NF / 2; ++h)
+                        o[h] = make_float2(__shfl_sync(kFull, v, base + 2 * LP * h), __shfl_sync(kFull, v, base + 2 * LP * h + LP));
+                }
+            };
+            float2 c[NF / 2], g2[NF / 2], nA[NF / 2], nB[NF / 2];
+            pairs(pt[0], c);
+            pairs(pt[1] * pt[1], g2);
+            pairs(-pt[2], nA);
+            pairs(-pt[3], nB);
+            const int mine = (place + kInFlight * cs) * a.RS + oc;
+            const float* row[NF];
+#pragma unroll
+            for (int q = 0; q < NF; ++q) row[q] = slots + __shfl_sync(kFull, mine, base + LP * q);
+#pragma unroll
+            for (int h = 0; h < NF / 2; ++h)
+#pragma unroll
+                for (int i = 0; i < 14; ++i) s[h][i] = make_float2(0.f, 0.f);
 #pragma unroll 2
             for (int k = gl; k < T; k += 8) {
-                float2 y = make_float2(ra[k], rb[k]);
-                if (SCALE) y = make_float2(__fmul_rn(y.x, iref[k]), __fmul_rn(y.y, iref[k]));
-                accum_pair(us[k], y, c, g2, nA, nB, s);
+                const float uk = us[k], ik = SCALE ? iref[k] : 1.f;
+#pragma unroll
+                for (int h = 0; h < NF / 2; ++h) {
+                    float2 y = make_float2(row[2 * h][k], row[2 * h + 1][k]);
+                    if (SCALE) y = make_float2(__fmul_rn(y.x, ik), __fmul_rn(y.y, ik));
+                    accum_pair(uk, y, c[h], g2[h], nA[h], nB[h], s[h]);
+                }
             }
         }
         LmSums S;
-        reduce_pair(s, S);
+        reduce_frames(s, S);
         // ---- decisions (as fit_group) ----
         if (f >= 0 && !done) {
             const float chi2t = S.v[13];
@@ -339,17 +382,26 @@ __global__ void __launch_bounds__(32 * kWarps8, 4) fit8_kernel(Fit8Args a)
     // no copy may land after the block exits (a failed wait only)
     if (fn >= 0) {
         const int nx = cs ^ 1;
-        tc::mbar_wait(&bars[half + 8 * nx], (ph >> nx) & 1u, 1u << 22);
+        tc::mbar_wait(&bars[place + kInFlight * nx], (ph >> nx) & 1u, 1u << 22);
     }
     if (failed && lane == 0 && a.err) atomicExch(a.err, 4);
 }
 
-int row_window(int T)   // floats of the largest 16-byte window around a row, an odd multiple of 4
+// floats of the largest 16-byte window around a row, as a stride: an odd
+// multiple of 4 (two frames a group) or of 8 (four)
+int row_window(int T, int frames)
 {
-    const int w = (4 * T + 12 + 15) / 16 * 4;
-    return w % 8 == 4 ? w : w + 4;
+    const int step = 2 * frames, w = (4 * T + 12 + 15) / 16 * 4;
+    return (w + step - 1) / step * step + ((w + step - 1) / step % 2 ? 0 : step);
 }
-int fit8_smem(int T) { return 4 * kWarps8 * kSlots8 * row_window(T) + 8 * kWarps8 * kSlots8 + 8 * T; }
+int fit8_slots(int frames) { return 2 * 4 * frames; }   // per warp
+int fit8_smem(int T, int frames) { return kWarps8 * fit8_slots(frames) * (4 * row_window(T, frames) + 8) + 8 * T; }
+void* fit8_fn(bool scale, int frames)
+{
+    if (frames == 4)
+        return scale ? reinterpret_cast<void*>(&fit8_kernel<true, 4>) : reinterpret_cast<void*>(&fit8_kernel<false, 4>);
+    return scale ? reinterpret_cast<void*>(&fit8_kernel<true, 2>) : reinterpret_cast<void*>(&fit8_kernel<false, 2>);
+}
 
 }  // namespace
 
@@ -360,17 +412,30 @@ cudaError_t setup_fit8(cg_plan_s* p)
     int most = 0;
     cudaError_t e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
     if (e != cudaSuccess) return e;
-    const int bytes = fit8_smem(p->T);
-    if (bytes > most) return cudaSuccess;
-    int occ[2] = {};
-    for (int i = 0; i < 2; ++i) {
-        void* fn = i ? reinterpret_cast<void*>(&fit8_kernel<true>) : reinterpret_cast<void*>(&fit8_kernel<false>);
-        if ((e = raise_smem_limit(fn, bytes)) != cudaSuccess) return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[i], fn, 32 * kWarps8, bytes)) != cudaSuccess) return e;
-        if (occ[i] < 1) return cudaSuccess;
-    }
+    // blocks per SM with n frames in a lane group (0: they don't fit)
+    auto blocks = [&](int frames, int* occ) -> cudaError_t {
+        const int bytes = fit8_smem(p->T, frames);
+        *occ = 0;
+        if (bytes > most) return cudaSuccess;
+        int o[2] = {};
+        for (int i = 0; i < 2; ++i) {
+            void* fn = fit8_fn(i, frames);
+            cudaError_t r = raise_smem_limit(fn, bytes);
+            if (r == cudaSuccess) r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o[i], fn, 32 * kWarps8, bytes);
+            if (r != cudaSuccess) return r;
+        }
+        *occ = std::min(o[0], o[1]);
+        return cudaSuccess;
+    };
+    int occ = 0;
+    if ((e = blocks(2, &occ)) != cudaSuccess) return e;
+    if (occ < 1) return cudaSuccess;
+    p->grid_fit8 = p->num_sms * occ;
+    // four frames a group where three blocks' rows fit an SM (fewer warps took
+    // longer than two frames a group)
+    if ((e = blocks(4, &occ)) != cudaSuccess) return e;
+    p->grid_fit8_four = occ >= 3 ? p->num_sms * occ : 0;
     if ((e = raise_smem_limit(init_ptr(p->init_npad, p->n_outer, true), p->init_smem)) != cudaSuccess) return e;
-    p->grid_fit8 = p->num_sms * std::min(occ[0], occ[1]);
     p->fit8_ok = true;
     return cudaSuccess;
 }
@@ -383,14 +448,21 @@ cudaError_t launch_fit8(const cg_plan_s* p, const float* y, const float* amps, i
         const cudaError_t e = launch_init(p, y, amps, n, params, nullptr, s, nullptr, nullptr, true);
         if (e != cudaSuccess) return e;
     }
+    // Four frames a group do a third less work per frame but take a third longer
+    // per step of all of them, so they pay where two a group would need a good
+    // part of a second round of frames (99 teeth, two / four: 20,000 spectra 36 / 42 us, 50,000
+    // 70 / 54, 10^5 104 / 99, 400,000 345 / 292; 21 teeth: 20,000 24 / 26,
+    // 50,000 48 / 31, 400,000 217 / 171)
+    const bool four = p->grid_fit8_four > 0 && 4 * n > 5 * static_cast<int64_t>(p->grid_fit8) * kWarps8 * fit8_slots(2) / 2;
+    const int frames = four ? 4 : 2, blocks = four ? p->grid_fit8_four : p->grid_fit8;
     Fit8Args a{};
     a.n = n;
     a.T = p->T;
-    a.RS = row_window(p->T);
+    a.RS = row_window(p->T, frames);
     // frames per task as in launch_fit3: two per frame in flight, fewer where
     // the schedulers would otherwise have none
     const int64_t schedulers = 4 * static_cast<int64_t>(p->num_sms);
-    a.task = static_cast<int>(std::min<int64_t>(16, (n + schedulers - 1) / schedulers));
+    a.task = static_cast<int>(std::min<int64_t>(fit8_slots(frames), (n + schedulers - 1) / schedulers));
     a.y = y;
     a.amps = amps;
     a.inv_ref = fa.inv_ref;
@@ -409,14 +481,13 @@ cudaError_t launch_fit8(const cg_plan_s* p, const float* y, const float* amps, i
     a.status = status;
     a.err = p->d.err;
     const int64_t tasks = (n + a.task - 1) / a.task;
-    const int grid = static_cast<int>(tasks < p->grid_fit8 ? tasks : p->grid_fit8);
+    const int grid = static_cast<int>(tasks < blocks ? tasks : blocks);
     if (tasks > static_cast<int64_t>(grid) * kWarps8) {
         const cudaError_t e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s);
         if (e != cudaSuccess) return e;
     }
     void* args[] = {&a};
-    void* fn = y ? reinterpret_cast<void*>(&fit8_kernel<false>) : reinterpret_cast<void*>(&fit8_kernel<true>);
-    return launch_dependent(fn, dim3(grid), dim3(32 * kWarps8), args, fit8_smem(p->T), s);
+    return launch_dependent(fit8_fn(!y, frames), dim3(grid), dim3(32 * kWarps8), args, fit8_smem(p->T, frames), s);
 }
 
 }  // namespace cg

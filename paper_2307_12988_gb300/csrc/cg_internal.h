@@ -303,8 +303,8 @@ struct cg_plan_s {
     int Q = 0;               // L = 10 Q
     bool fit3_ok = false;    // shared-memory LM kernel (cg_fit3.cu) configured
     int fit3_G = 0, fit3_warps = 0, fit3_smem = 0, grid_fit3 = 0;
-    bool fit8_ok = false;    // standalone fit at eight lanes, two frames a group (cg_fit8.cu)
-    int grid_fit8 = 0;
+    bool fit8_ok = false;    // standalone fit at eight lanes per frame (cg_fit8.cu)
+    int grid_fit8 = 0, grid_fit8_four = 0;   // blocks with two and four frames a lane group
     int G2 = 4;              // LM lanes per frame of the register-resident fit
     int PPL = 0;             // LM points per lane
     bool ppl_exact = false;  // PPL == ceil(T / G2)
