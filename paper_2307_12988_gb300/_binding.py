@@ -198,8 +198,10 @@ def _stream(stream) -> int | None:
         try:
             import torch
             if torch.cuda.is_initialized():
-                # 0.5 us; torch.cuda.current_stream() builds an object (3 us)
-                return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+                try:   # 0.5 us; torch.cuda.current_stream() builds an object (3 us)
+                    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+                except AttributeError:   # a torch without these two
+                    pass
             return torch.cuda.current_stream().cuda_stream
         except Exception:
             return None
