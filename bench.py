@@ -799,9 +799,11 @@ def run_train(args):
                          "cores": int(os.environ.get("OMP_NUM_THREADS", os.cpu_count() or 1)),
                          "kind": "oracle", "sample": f"{rows_cpu} rows: FP64 NumPy minibatch gradients, no Adam"},
         "clocks": clk,
-        # per minibatch: 2 gathers, 8 products, MSE + loss, 3 column sums,
-        # Adam (+ one sum per K-split product, not counted)
-        "gpu_launches": 16 * ((n + B - 1) // B) * args.steps,
+        # per minibatch: 3 products, the middle layer's kernel, the weights'
+        # products, the update; once per epoch the first batch's preparation
+        # (batches beyond 16,384 rows: 2 gathers, 8 products, MSE + loss, 3
+        # column sums, Adam)
+        "gpu_launches": (6 * ((n + B - 1) // B) + 1 if B <= 16384 else 16 * ((n + B - 1) // B)) * args.steps,
     }
     print(json.dumps(line), flush=True)
 
