@@ -10,14 +10,15 @@
 // packed complex values z_n = x_2n + i x_2n+1 are transformed in place in
 // shared memory (radix 16, and one smaller radix); the real-FFT split
 // X_k = E_k + W_M^k O_k gives |X_k|^2 for k = 0..L, which the threads add up
-// over all their segments as FP32 pairs; the groups' rows are summed and
-// scaled by psd_reduce_kernel.
+// in FP64, row by row in the order of the segments; psd_reduce_kernel adds the
+// rows in order and scales them.
 //
 // Resonance: S(f) = A f0^4 / ((f0^2 - f^2)^2 + (f f0 / Q)^2) + B fitted to
 // ln S over the bins of a band by Levenberg-Marquardt in FP64 (one cluster of
 // eight blocks shares the per-point work, each takes the 4x4 solve);
 // initial values from the band (largest bin, smallest bin, half-height
 // width); standard errors from diag(H^-1) chi^2 / (n - 4).
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -37,15 +38,15 @@ constexpr int kWelchThreads = 512;   // threads of a block of the Welch kernel
 struct cg_psd_s {
     int device = 0;
     int L = 0;                 // complex transform length (M / 2)
-    int grid = 0;              // blocks of the Welch kernel at most
-    int groups = 0;            // segments a block transforms at a time
+    int blocks = 0;            // blocks of the Welch kernel at most
+    int rows = 0;              // rows of sums of a block
     size_t smem = 0;
     double sum_w2 = 0.0;       // sum of the squared window
     float* win = nullptr;      // [M / 2 + 1] the window's first half (it is symmetric)
     float2* tw = nullptr;      // the kernel's twiddles (WelchTables)
     int2* pair0 = nullptr;     // [L / 32] buffer places of the last pair of each thread
     int* bin = nullptr;        // [L + 1] PSD bin of each slot of a row of part
-    float2* part = nullptr;    // [grid * groups][L + 1] sums of |X_k|^2 as FP32 pairs
+    double* part = nullptr;    // [blocks * rows][L + 1] sums of |X_k|^2
 };
 
 namespace cg {
@@ -58,6 +59,12 @@ template <int L>
 struct Welch {
     static constexpr int NT = L / 32;                   // threads of a group
     static constexpr int G = kWelchThreads / NT;        // groups of a block
+    // The segments s = r, r + R, r + 2 R, ... of row r (R rows) are added up one
+    // after another; S groups of a block transform S of them at a time, and
+    // each keeps the sums of a 1 / S of the row's bins.
+    static constexpr int ROWS = L == 2048 ? 2 : 1;      // rows of a block
+    static constexpr int S = G / ROWS;                  // groups of a row: 4, 4, 2, 1
+    static constexpr int SL = 32 / S;                   // bins whose sums a thread keeps
     static constexpr int R3 = L == 2048 ? 8 : 16;
     static constexpr int R4 = L / (256 * R3);           // 1, 1, 2, 4
     static constexpr int B = L / 16;                    // points of one first-digit block
@@ -70,11 +77,13 @@ struct Welch {
     static constexpr int kHalf = kSplit + L / 2;        // W_M^(L / 2)
     static constexpr int kTables = kHalf + 1;
     // shared memory: the groups' points, the tables of stages 2 and 3, half
-    // the window, warp sums, the extra bin's sum of each group
+    // the window, |X_k|^2 of the bins that other groups of the row add up,
+    // warp sums, mean and middle bin of each group, two barriers of each
     static constexpr int kSmemZ = G * L * 8;
     static constexpr int kSmemT = kSmemZ + (15 * 16 + (R3 - 1) * 256) * 8;
-    static constexpr int kSmemW = kSmemT + (M / 2 + 4) * 4;
-    static constexpr int kSmemB = kSmemW + G * (2 * NT / 32) * 4 + G * 8;   // two barriers of each group
+    static constexpr int kSmemX = kSmemT + (M / 2 + 4) * 4;
+    static constexpr int kSmemW = kSmemX + G * (S - 1) * SL * NT * 4;
+    static constexpr int kSmemB = kSmemW + G * (2 * NT / 32) * 4 + G * 8;
     static constexpr int kSmem = kSmemB + G * 16;
 };
 
@@ -82,12 +91,13 @@ struct PsdArgs {
     const float* x;
     int64_t stride;            // elements between consecutive samples
     int64_t K;                 // segments
+    int rows;                  // rows of sums
     int vec2;                  // sample pairs are 8-byte aligned and contiguous
     int bulk;                  // so are whole segments, 16-byte aligned
     const float* win;
     const float2* tw;
     const int2* pair0;
-    float2* part;
+    double* part;
 };
 
 // Shared-memory place of point p: its low four bits XORed with the next four.
@@ -118,37 +128,24 @@ __device__ __forceinline__ void group_sync(int g)
     asm volatile("bar.sync %0, %1;\n" ::"r"(g + 1), "n"(NT) : "memory");
 }
 
-// s + e = a + b exactly (Knuth's two-sum)
-__device__ __forceinline__ float two_sum(float a, float b, float& e)
+// the S groups of a row
+template <int NT, int S>
+__device__ __forceinline__ void row_sync(int row, int g)
 {
-    const float s = a + b, bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-    return s;
+    if constexpr (S == 1)
+        group_sync<NT>(g);
+    else
+        asm volatile("bar.sync %0, %1;\n" ::"r"(9 + row), "n"(S * NT) : "memory");
 }
 
-// Sums of |X_k|^2 as unevaluated FP32 pairs (hi, lo).  An FP64 sum costs a
-// conversion and an addition at 2 lanes per cycle and SM (16,384 bins: 16,000
-// cycles of a segment's 61,000); the pair costs 7 FP32 operations at 128 lanes
-// per cycle.  The lost part of each addition is exact; lo, kept below an ulp
-// of hi by a normalisation every eighth segment, rounds it 2^-24 below that.
-__device__ __forceinline__ void pair_add(float2& a, float b)
+// p = |X|^2 as a double.  A normal p by integer operations: the conversion
+// runs on the FP64 pipe, which additions alone keep busy at 1.7 lanes a cycle
+// and SM (with conversions 1.2; converted under a predicate 0.9).
+__device__ __forceinline__ bool is_normal(float p) { return __float_as_uint(p) - 0x00800000u < 0x7f000000u; }
+__device__ __forceinline__ double widen(float p)
 {
-    float e;
-    a.x = two_sum(a.x, b, e);
-    a.y += e;
-}
-// an infinite or undefined sum stays what it is
-__device__ __forceinline__ void pair_norm(float2& a)
-{
-    const float h = a.x + a.y;
-    const bool fin = fabsf(a.x) < INFINITY;
-    a = make_float2(fin ? h : a.x, fin ? a.y - (h - a.x) : 0.f);
-}
-__device__ __forceinline__ void pair_add2(float2& a, float2 b)
-{
-    pair_add(a, b.x);
-    a.y += b.y;
-    pair_norm(a);
+    const uint32_t u = __float_as_uint(p);
+    return __hiloint2double(static_cast<int>((u >> 3) + 0x38000000u), static_cast<int>(u << 29));
 }
 
 // Welch sums.  One segment per group of NT threads, its L packed complex
@@ -156,30 +153,30 @@ __device__ __forceinline__ void pair_add2(float2& a, float2 b)
 // (digit-reversed result): the points of a butterfly go back where they were
 // read, so a thread needs no barrier between its reads and its writes, and
 // after the first stage (stride L / 16) all remaining butterflies of a warp
-// stay inside the warp's own 1,024 points -- two block barriers per
-// transform instead of eight, and 16 live values per thread.  That leaves the
-// registers for the sums of |X_k|^2: the thread that holds bins k and L - k
-// (one split, two bins from the same two points and twiddle) adds them up over
-// all its segments.
+// stay inside the warp's own 1,024 points: 16 live values per thread.  That
+// leaves the registers for the sums of |X_k|^2: the thread that holds bins k
+// and L - k (one split, two bins from the same two points and twiddle) adds
+// them up over all its segments.
 //
-// What bounds it: shared-memory traffic (1.3 MB per 32,768-sample segment,
-// 10,000 cycles) and the transform's FP32 work.  Before, the sums lived in
-// L2 as FP64 rows and every table but one was read from L2 (0.75 MB per
-// segment), the sums and the mean ran in FP64 on every thread, and each stage
-// took two barriers of 1,024 threads: ten minutes of centres (36,620 segments
-// of 32,768) in 7.99 ms.  In place 3.11 ms (27,000 cycles a segment, the shared
-// memory busy for 54 % of them), of which a segment waited for 8-byte
-// asynchronous copies of the next to begin only when all of it was split;
-// 2.63 ms with bulk copies in two parts, the first under the second half of
-// the split and the sums of the first under the second; 2.53 ms with the last
-// stage's twiddles all requested at once and the split's before its barrier
-// (they come from L2).
+// The sums are FP64 and have one order: segment after segment within a row,
+// then row after row.  (The fit of a resonance takes or leaves its last step by
+// the last bit of chi^2, so a density that differs by 1e-15 can move the fitted
+// values by 1e-8.)  Where several groups share a row, each hands |X_k|^2 of the
+// bins that another adds up to it through shared memory.
+//
+// What bounds it: the FP64 additions (16,384 a 32,768-sample segment at 1.7
+// lanes a cycle and SM: 9,700 of its 30,000 cycles) and shared-memory traffic
+// (1.3 MB, 10,000 cycles).  The samples come by bulk copies in two parts, the
+// first under the second half of the split, the second under the additions; the
+// last stage's twiddles are requested at once and the split's before its
+// barrier (they come from L2).  600 million samples in segments of 32,768: 3.53
+// ms, of 16,384 3.74, of 8,192 3.13, of 4,096 3.10 (7.6, 6.3, 5.8 and 4.3 with
+// two barriers a stage, sums in L2 and conversions on the FP64 pipe).
 template <int L>
 __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
 {
     using W = Welch<L>;
-    constexpr int NT = W::NT, R3 = W::R3, R4 = W::R4, B = W::B, M = W::M, G = W::G;
-    tc::pdl_start();
+    constexpr int NT = W::NT, R3 = W::R3, R4 = W::R4, B = W::B, M = W::M, G = W::G, S = W::S, SL = W::SL;
     extern __shared__ __align__(1024) unsigned char psm[];
     const int g = threadIdx.x / NT, t = threadIdx.x % NT, w = t >> 5, lane = t & 31;
     const uint32_t z = static_cast<uint32_t>(__cvta_generic_to_shared(psm)) + g * L * 8;
@@ -187,10 +184,17 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
     const float2* const t2 = ts + W::kT2;
     const float2* const t3 = ts + W::kT3;
     float* const win = reinterpret_cast<float*>(psm + W::kSmemT);
+    float* const xch = reinterpret_cast<float*>(psm + W::kSmemX);   // [G][S - 1][SL][NT]
     float* const red = reinterpret_cast<float*>(psm + W::kSmemW) + g * (2 * NT / 32);
-    float2* const half = reinterpret_cast<float2*>(psm + W::kSmemW + G * (2 * NT / 32) * 4) + g;
-    const int64_t slot = static_cast<int64_t>(g) * gridDim.x + blockIdx.x;   // this group's first segment
-    const int64_t nslot = static_cast<int64_t>(G) * gridDim.x;
+    float* const means = reinterpret_cast<float*>(psm + W::kSmemW + G * (2 * NT / 32) * 4);   // [G]
+    float* const halfs = means + G;                                                          // [G] |X_(L / 2)|^2
+    // group q of the S that share row `row`: its segments are first, first + S R, ...
+    const int rr = g / S, q = g % S;
+    const int64_t R = a.rows;
+    const int64_t row = static_cast<int64_t>(rr) * gridDim.x + blockIdx.x;
+    const int64_t nslot = S * R;
+    const int64_t first = (row < R ? row : a.K) + q * R;
+    // rounds of the row: while its group 0 has a segment
     const uint32_t zt = z + 8 * zsw(t);             // point t, and NT - 1 - t
     const uint32_t zr = z + 8 * zsw(NT - 1 - t);
     const uint32_t zl = z + 8 * t;                  // point t of the samples
@@ -237,145 +241,151 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
         tc::mbar_init(&bars[1], 1);
         tc::fence_mbar_init();
     }
-    if (slot < a.K) {
+    if (first < a.K) {
         if (!a.bulk) {
-            stage_x(slot);
+            stage_x(first);
         } else if (t == 0) {
-            stage_part(slot, 0);
-            stage_part(slot, 1);
+            stage_part(first, 0);
+            stage_part(first, 1);
         }
     }
     for (int i = threadIdx.x; i < W::kT4; i += kWelchThreads) ts[i] = a.tw[i];
     for (int i = threadIdx.x; i <= M / 2; i += kWelchThreads) win[i] = a.win[i];
-    if (t == 0) *half = make_float2(0.f, 0.f);
     const int2 p15 = a.pair0[t];
-    float2 acc[16][2];
+    double acc[SL];   // sums of slots q SL ..; slot 2 i + h is bin h of the thread's pair i
 #pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
+    for (int j = 0; j < SL; ++j) acc[j] = 0.0;
+    double half = 0.0;   // bin L / 2 (thread 0 of group 0 of the row)
     __syncthreads();
 
-    int since = 0;   // segments since the sums were normalised
     uint32_t phase = 0;
     bool landed = true;   // (a copy that never does leaves the sums undefined)
-    for (int64_t s = slot; s < a.K; s += nslot, phase ^= 1u) {
-        // the next segment into L2 meanwhile
-        if (a.bulk) {
-            if (s + nslot < a.K && t == 0) tc::prefetch_l2_bulk(a.x + (s + nslot) * static_cast<int64_t>(L), M * 4);
-        } else if (s + nslot < a.K && a.stride <= 4) {
-            const char* nx = reinterpret_cast<const char*>(a.x + (s + nslot) * static_cast<int64_t>(L) * a.stride);
-            for (int64_t i = t; i < M * a.stride / 32; i += NT) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(nx + 128 * i));
-        }
-        if (a.bulk)
-            landed = landed && tc::mbar_wait(&bars[0], phase, 1u << 24);
-        else
-            cp_async_wait_all();   // own points only: no barrier
-        // ---- segment mean: FP32 sums of 32 samples per first-stage column ----
-        float sum[2] = {0.f, 0.f};
-        auto column = [&](int r) {
+    for (int64_t s = first; s - q * R < a.K; s += nslot, phase ^= 1u) {
+        const bool live = S == 1 || s < a.K;   // (a row's last round may not need all of its groups)
+        float2 tws[16];   // the split's twiddles
+        if (live) {
+            // the next segment into L2 meanwhile
+            if (a.bulk) {
+                if (s + nslot < a.K && t == 0) tc::prefetch_l2_bulk(a.x + (s + nslot) * static_cast<int64_t>(L), M * 4);
+            } else if (s + nslot < a.K && a.stride <= 4) {
+                const char* nx = reinterpret_cast<const char*>(a.x + (s + nslot) * static_cast<int64_t>(L) * a.stride);
+                for (int64_t i = t; i < M * a.stride / 32; i += NT) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(nx + 128 * i));
+            }
+            if (a.bulk)
+                landed = landed && tc::mbar_wait(&bars[0], phase, 1u << 24);
+            else
+                cp_async_wait_all();   // own points only: no barrier
+            // ---- segment mean: FP32 sums of 32 samples per first-stage column ----
+            float sum[2] = {0.f, 0.f};
+            auto column = [&](int r) {
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const float2 v = zld(zl + 8 * NT * (b + 2 * r));
+                    sum[b] += v.x + v.y;
+                }
+            };
+#pragma unroll
+            for (int r = 0; r < 5; ++r) column(r);
+            if (a.bulk) landed = landed && tc::mbar_wait(&bars[1], phase, 1u << 24);
+#pragma unroll
+            for (int r = 5; r < 16; ++r) column(r);
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
-                const float2 v = zld(zl + 8 * NT * (b + 2 * r));
-                sum[b] += v.x + v.y;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sum[b] += __shfl_xor_sync(0xffffffffu, sum[b], o);
+                if (lane == 0) red[w + (NT / 32) * b] = sum[b];
             }
-        };
+            group_sync<NT>(g);
+            if (w == 0) {   // one warp adds the warp sums in FP64
+                double tot = lane < 2 * NT / 32 ? static_cast<double>(red[lane]) : 0.0;
 #pragma unroll
-        for (int r = 0; r < 5; ++r) column(r);
-        if (a.bulk) landed = landed && tc::mbar_wait(&bars[1], phase, 1u << 24);
-#pragma unroll
-        for (int r = 5; r < 16; ++r) column(r);
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sum[b] += __shfl_xor_sync(0xffffffffu, sum[b], o);
-            if (lane == 0) red[w + (NT / 32) * b] = sum[b];
-        }
-        group_sync<NT>(g);
-        // every warp adds the warp sums as FP32 pairs (48 bits) and rounds once
-        float2 tot = make_float2(lane < 2 * NT / 32 ? red[lane] : 0.f, 0.f);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            pair_add2(tot, make_float2(__shfl_xor_sync(0xffffffffu, tot.x, o), __shfl_xor_sync(0xffffffffu, tot.y, o)));
-        const float mean = tot.x * (1.0f / M);
-        // ---- stage 1: subtract the mean, window, 16 points at stride B ----
-#pragma unroll 1
-        for (int b = 0; b < 2; ++b) {
-            const int j = t + NT * b;
-            const uint32_t zj = zat(zt, NT) * b + zt * (1 - b);
-            float2 v[16];
-#pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                const int n = j + r * B;
-                v[r] = zld(zl + 8 * (NT * b + r * B));
-                float2 wn;
-                if (r < 8)
-                    wn = *reinterpret_cast<const float2*>(win + 2 * n);
-                else
-                    wn = make_float2(win[M - 2 * n], win[M - 2 * n - 1]);
-                v[r] = make_float2((v[r].x - mean) * wn.x, (v[r].y - mean) * wn.y);
+                for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+                if (lane == 0) means[g] = static_cast<float>(tot / M);
             }
-            __syncwarp();   // (the points' places lie among those the warp has read)
-            Dft<16>::run(v);
-#pragma unroll
-            for (int r = 0; r < 16; ++r) zst(zat(zj, r * B), v[r]);
-        }
-        group_sync<NT>(g);
-        // ---- stage 2: stride B / 16, inside the warp's 1,024 points from here on ----
+            group_sync<NT>(g);
+            const float mean = landed ? means[g] : __int_as_float(0x7fffffff);
+            // ---- stage 1: subtract the mean, window, 16 points at stride B ----
 #pragma unroll 1
-        for (int b = 0; b < 2; ++b) {
-            const int be = lane + 32 * b;
-            const int base = 1024 * w + (be / (B / 16)) * B + be % (B / 16);
-            const int k1 = base / B;
-            const uint32_t zb = z + 8 * zsw(base);
-            float2 v[16];
+            for (int b = 0; b < 2; ++b) {
+                const int j = t + NT * b;
+                const uint32_t zj = zat(zt, NT) * b + zt * (1 - b);
+                float2 v[16];
 #pragma unroll
-            for (int r = 0; r < 16; ++r) v[r] = zld(zat(zb, r * (B / 16)));
+                for (int r = 0; r < 16; ++r) {
+                    const int n = j + r * B;
+                    v[r] = zld(zl + 8 * (NT * b + r * B));
+                    float2 wn;
+                    if (r < 8)
+                        wn = *reinterpret_cast<const float2*>(win + 2 * n);
+                    else
+                        wn = make_float2(win[M - 2 * n], win[M - 2 * n - 1]);
+                    v[r] = make_float2((v[r].x - mean) * wn.x, (v[r].y - mean) * wn.y);
+                }
+                __syncwarp();   // (the points' places lie among those the warp has read)
+                Dft<16>::run(v);
 #pragma unroll
-            for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], t2[(r - 1) * 16 + k1]);
-            Dft<16>::run(v);
-#pragma unroll
-            for (int r = 0; r < 16; ++r) zst(zat(zb, r * (B / 16)), v[r]);
-        }
-        __syncwarp();
-        // ---- stage 3: stride R4 ----
+                for (int r = 0; r < 16; ++r) zst(zat(zj, r * B), v[r]);
+            }
+            group_sync<NT>(g);
+            // ---- stage 2: stride B / 16, inside the warp's 1,024 points from here on ----
 #pragma unroll 1
-        for (int b = 0; b < 32 / R3; ++b) {
-            const int be = lane + 32 * b;
-            const int base = 1024 * w + (be / R4) * (R3 * R4) + be % R4;
-            const int cg = base / (R3 * R4);
-            const uint32_t zb = z + 8 * zsw(base);
-            float2 v[R3];
+            for (int b = 0; b < 2; ++b) {
+                const int be = lane + 32 * b;
+                const int base = 1024 * w + (be / (B / 16)) * B + be % (B / 16);
+                const int k1 = base / B;
+                const uint32_t zb = z + 8 * zsw(base);
+                float2 v[16];
 #pragma unroll
-            for (int r = 0; r < R3; ++r) v[r] = zld(zat(zb, r * R4));
+                for (int r = 0; r < 16; ++r) v[r] = zld(zat(zb, r * (B / 16)));
 #pragma unroll
-            for (int r = 1; r < R3; ++r) v[r] = cmul(v[r], t3[(r - 1) * 256 + cg]);
-            Dft<R3>::run(v);
+                for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], t2[(r - 1) * 16 + k1]);
+                Dft<16>::run(v);
 #pragma unroll
-            for (int r = 0; r < R3; ++r) zst(zat(zb, r * R4), v[r]);
-        }
-        // ---- stage 4: stride 1 ----
-        if constexpr (R4 > 1) {
+                for (int r = 0; r < 16; ++r) zst(zat(zb, r * (B / 16)), v[r]);
+            }
             __syncwarp();
-            const float2* t4 = a.tw + W::kT4 + (1024 / R4) * w + lane;
+            // ---- stage 3: stride R4 ----
+#pragma unroll 1
+            for (int b = 0; b < 32 / R3; ++b) {
+                const int be = lane + 32 * b;
+                const int base = 1024 * w + (be / R4) * (R3 * R4) + be % R4;
+                const int cg = base / (R3 * R4);
+                const uint32_t zb = z + 8 * zsw(base);
+                float2 v[R3];
 #pragma unroll
-            for (int b = 0; b < 32 / R4; ++b) {
-                const uint32_t zb = z + 8 * zsw(1024 * w + R4 * (lane + 32 * b));
-                float2 v[R4];
+                for (int r = 0; r < R3; ++r) v[r] = zld(zat(zb, r * R4));
 #pragma unroll
-                for (int r = 0; r < R4; ++r) v[r] = zld(zat(zb, r));
+                for (int r = 1; r < R3; ++r) v[r] = cmul(v[r], t3[(r - 1) * 256 + cg]);
+                Dft<R3>::run(v);
 #pragma unroll
-                for (int r = 1; r < R4; ++r) v[r] = cmul(v[r], __ldg(&t4[(r - 1) * (L / R4) + 32 * b]));
-                Dft<R4>::run(v);
-#pragma unroll
-                for (int r = 0; r < R4; ++r) zst(zat(zb, r), v[r]);
+                for (int r = 0; r < R3; ++r) zst(zat(zb, r * R4), v[r]);
             }
-        }
-        float2 tws[16];   // the split's twiddles, requested ahead of the barriers
-        tws[15] = __ldg(&a.tw[W::kSplit + 15 * NT + t]);
+            // ---- stage 4: stride 1 ----
+            if constexpr (R4 > 1) {
+                __syncwarp();
+                const float2* t4 = a.tw + W::kT4 + (1024 / R4) * w + lane;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) tws[i] = __ldg(&a.tw[W::kSplit + i * NT + t]);
-        group_sync<NT>(g);
+                for (int b = 0; b < 32 / R4; ++b) {
+                    const uint32_t zb = z + 8 * zsw(1024 * w + R4 * (lane + 32 * b));
+                    float2 v[R4];
+#pragma unroll
+                    for (int r = 0; r < R4; ++r) v[r] = zld(zat(zb, r));
+#pragma unroll
+                    for (int r = 1; r < R4; ++r) v[r] = cmul(v[r], __ldg(&t4[(r - 1) * (L / R4) + 32 * b]));
+                    Dft<R4>::run(v);
+#pragma unroll
+                    for (int r = 0; r < R4; ++r) zst(zat(zb, r), v[r]);
+                }
+            }
+            // requested ahead of the barrier
+            tws[15] = __ldg(&a.tw[W::kSplit + 15 * NT + t]);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) tws[i] = __ldg(&a.tw[W::kSplit + i * NT + t]);
+        }
+        row_sync<NT, S>(rr, g);   // (and the other groups have read xch)
         // ---- real-FFT split of bins k and L - k, |X|^2 into the sums ----
         const bool more = s + nslot < a.K;
+        float own[SL];   // |X|^2 of the slots that this group adds up
         auto split = [&](int i) {
             const int k1 = i < 14 ? 1 + (i >> 1) : 8, h = i < 14 ? i & 1 : 0;
             const float2 Zb = zld(i < 15 ? zat(zt, k1 * B + NT * h) : z + 8 * p15.x);
@@ -385,82 +395,122 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
             const float2 C = cmul(tws[i], make_float2(Dd.y, -Dd.x));
             // X_k = E + C; X_(L - k) = conj(E - C), since W_M^(L - k) = -conj W_M^k
             const float2 X = cadd(E, C), Y = csub(E, C);
-            pair_add(acc[i][0], fmaf(X.x, X.x, X.y * X.y));
-            pair_add(acc[i][1], fmaf(Y.x, Y.x, Y.y * Y.y));
+            const float v[2] = {fmaf(X.x, X.x, X.y * X.y), fmaf(Y.x, Y.x, Y.y * Y.y)};
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int slot = 2 * i + b, owner = slot / SL;
+                if (S == 1 || owner == q)
+                    own[slot % SL] = v[b];
+                else
+                    xch[((g * (S - 1) + (owner < q ? owner : owner - 1)) * SL + slot % SL) * NT + t] = v[b];
+            }
         };
-        // blocks 0 to 4 and 12 to 15 first: the next segment's samples follow
-        split(15);
+        if (live) {
+            // blocks 0 to 4 and 12 to 15 first: the next segment's samples follow
+            split(15);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) split(i);
+            for (int i = 0; i < 8; ++i) split(i);
 #pragma unroll
-        for (int i = 8; i < 15; ++i) tws[i] = __ldg(&a.tw[W::kSplit + i * NT + t]);
-        if (t == 0) {   // bin L / 2 pairs with itself
-            constexpr int kPos = R4 > 1 ? R4 / 2 : R3 / 2;   // its last digit is R / 2, the others 0
-            const float2 Zh = zld(z + 8 * zsw(kPos));
-            const float2 X = cadd(make_float2(Zh.x, 0.f), cmul(__ldg(&a.tw[W::kHalf]), make_float2(Zh.y, -0.f)));
-            pair_add2(*half, make_float2(fmaf(X.x, X.x, X.y * X.y), 0.f));
+            for (int i = 8; i < 15; ++i) tws[i] = __ldg(&a.tw[W::kSplit + i * NT + t]);
+            if (t == 0) {   // bin L / 2 pairs with itself
+                constexpr int kPos = R4 > 1 ? R4 / 2 : R3 / 2;   // its last digit is R / 2, the others 0
+                const float2 Zh = zld(z + 8 * zsw(kPos));
+                const float2 X = cadd(make_float2(Zh.x, 0.f), cmul(__ldg(&a.tw[W::kHalf]), make_float2(Zh.y, -0.f)));
+                halfs[g] = fmaf(X.x, X.x, X.y * X.y);
+            }
+            if (a.bulk) {
+                group_sync<NT>(g);
+                if (more && t == 0) stage_part(s + nslot, 0);
+            }
+#pragma unroll
+            for (int i = 8; i < 15; ++i) split(i);
         }
-        if (a.bulk) {
-            group_sync<NT>(g);
-            if (more && t == 0) stage_part(s + nslot, 0);
-        }
-#pragma unroll
-        for (int i = 8; i < 15; ++i) split(i);
-        group_sync<NT>(g);
+        row_sync<NT, S>(rr, g);
         if (more) {
             if (!a.bulk)
                 stage_x(s + nslot);
             else if (t == 0)
                 stage_part(s + nslot, 1);
         }
-        if (++since == 8 || s + nslot >= a.K) {
-            since = 0;
+        // ---- the round's segments in order ----
+        int n = 1;   // its segments
+        if constexpr (S > 1) {
+            for (n = 0; n < S && s + (n - q) * R < a.K;) ++n;
+        }
+        float v[S][SL];
+        bool ok = true;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                pair_norm(acc[i][0]);
-                pair_norm(acc[i][1]);
+        for (int u = 0; u < S; ++u) {
+            if (u >= n) break;
+            const float* from = xch + (g - q + u) * (S - 1) * SL * NT + (q < u ? q : q - 1) * SL * NT + t;
+#pragma unroll
+            for (int j = 0; j < SL; ++j) {
+                v[u][j] = S == 1 || u == q ? own[j] : from[j * NT];
+                ok = ok && is_normal(v[u][j]);
             }
         }
-    }
-    if (slot < a.K) {
-        float2* row = a.part + slot * (L + 1);
-        const float undefined = __int_as_float(0x7fffffff);
+        if (ok) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            if (!landed) acc[i][0] = acc[i][1] = make_float2(undefined, undefined);
-            row[(2 * i) * NT + t] = acc[i][0];
-            row[(2 * i + 1) * NT + t] = acc[i][1];
+            for (int u = 0; u < S; ++u)
+                if (u < n)
+#pragma unroll
+                    for (int j = 0; j < SL; ++j) acc[j] += widen(v[u][j]);
+        } else {   // some zero, subnormal, infinite or undefined
+#pragma unroll
+            for (int u = 0; u < S; ++u)
+                if (u < n)
+#pragma unroll
+                    for (int j = 0; j < SL; ++j) acc[j] += static_cast<double>(v[u][j]);
         }
-        if (t == 0) row[L] = landed ? *half : make_float2(undefined, undefined);
+        if (q == 0 && t == 0)
+            for (int u = 0; u < n; ++u) half += static_cast<double>(halfs[g + u]);
+    }
+    if (row < R) {
+        double* sums = a.part + row * (L + 1);
+#pragma unroll
+        for (int j = 0; j < SL; ++j) sums[(q * SL + j) * NT + t] = acc[j];
+        if (q == 0 && t == 0) sums[L] = half;
     }
 }
 
-// psd[bin[i]] = scale * sum over the rows of part: 32 slots per block, eight
-// threads per slot over rows y, y + 8, ..., then in order of y (fixed order).
-// The rows are summed as FP32 pairs too: 152 rows of 16,385 bins took 22 us as
-// FP64 additions on 65 blocks, 8 us so (60 rows: 10.9 and 5.6 us).
-__global__ void __launch_bounds__(256) psd_reduce_kernel(const float2* part, int rows, int L, double scale,
-                                                         const int* bin, double* psd)
+// psd[bin[i]] = scale * the sum of the rows of part in order, one thread per
+// slot.  A warp's FP64 addition takes its scheduler 64 cycles, so the blocks are
+// one warp each, spread over all schedulers, and the next 16 rows are requested
+// before the 16 at hand are added.
+__global__ void __launch_bounds__(32) psd_reduce_kernel(const double* part, int rows, int L, double scale,
+                                                        const int* bin, double* psd)
 {
-    __shared__ float2 red[8][33];
+    constexpr int kAhead = 16;
     tc::pdl_start();
-    tc::pdl_wait();
     const int i = blockIdx.x * 32 + threadIdx.x;
-    float2 s = make_float2(0.f, 0.f);
-    if (i <= L) {
-#pragma unroll 4
-        for (int b = threadIdx.y; b < rows; b += 8) {
-            const float2 v = part[static_cast<int64_t>(b) * (L + 1) + i];
-            pair_add2(s, v);
+    if (i > L) return;
+    const double* p = part + i;
+    const int64_t ld = L + 1;
+    double s = 0.0, v[kAhead];
+    int b = 0;
+    if (rows >= kAhead) {
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) v[u] = p[u * ld];
+        for (b = kAhead; b + kAhead <= rows; b += kAhead) {
+            double w[kAhead];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) w[u] = p[(b + u) * ld];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                s += v[u];
+                v[u] = w[u];
+            }
         }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) s += v[u];
     }
-    red[threadIdx.y][threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.y == 0 && i <= L) {
-        for (int y = 1; y < 8; ++y) pair_add2(s, red[y][threadIdx.x]);
-        const int k = bin[i];
-        psd[k] = (static_cast<double>(s.x) + static_cast<double>(s.y)) * scale * ((k == 0 || k == L) ? 1.0 : 2.0);
-    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) v[u] = b + u < rows ? p[(b + u) * ld] : 0.0;
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+        if (b + u < rows) s += v[u];
+    const int k = bin[i];
+    psd[k] = s * scale * ((k == 0 || k == L) ? 1.0 : 2.0);
 }
 
 // position of bin k (< L) after the in-place stages, and the tables
@@ -508,13 +558,13 @@ struct WelchTables {
 
 struct WelchInst {
     void* fn;
-    int threads, groups, smem;
+    int threads, rows, smem;
     void (*fill)(std::vector<float2>&, std::vector<int2>&, std::vector<int>&);
 };
 template <int L>
 WelchInst welch_of()
 {
-    return {reinterpret_cast<void*>(&psd_welch_kernel<L>), kWelchThreads, Welch<L>::G, Welch<L>::kSmem,
+    return {reinterpret_cast<void*>(&psd_welch_kernel<L>), kWelchThreads, Welch<L>::ROWS, Welch<L>::kSmem,
             &WelchTables<L>::fill};
 }
 bool welch_inst(int L, WelchInst* w)
@@ -1027,8 +1077,8 @@ cg_status cg_psd_create(int seg_len, cg_psd_t* out)
     int sms = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     h->smem = wi.smem;
-    h->groups = wi.groups;
-    h->grid = sms;
+    h->rows = wi.rows;
+    h->blocks = sms;
     auto upload = [&](auto** dst, const auto& src) {
         const size_t bytes = sizeof(src[0]) * src.size();
         if (e == cudaSuccess) e = cudaMalloc(dst, bytes);
@@ -1040,7 +1090,7 @@ cg_status cg_psd_create(int seg_len, cg_psd_t* out)
     upload(&h->pair0, pair0);
     upload(&h->bin, bin);
     if (e == cudaSuccess)
-        e = cudaMalloc(&h->part, sizeof(float2) * (L + 1) * static_cast<size_t>(h->grid) * h->groups);
+        e = cudaMalloc(&h->part, sizeof(double) * (L + 1) * static_cast<size_t>(h->blocks) * h->rows);
     if (e != cudaSuccess) {
         cg_psd_destroy(h);
         return psd_cuda_fail(e, "cg_psd_create");
@@ -1073,21 +1123,22 @@ cg_status cg_psd_welch(cg_psd_t h, const float* x_dev, int64_t n, int64_t stride
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int vec2 = stride == 1 && (reinterpret_cast<uintptr_t>(x_dev) & 7) == 0;
     const int bulk = stride == 1 && (reinterpret_cast<uintptr_t>(x_dev) & 15) == 0;
-    PsdArgs a{x_dev, stride, K, vec2, bulk, h->win, h->tw, h->pair0, h->part};
+    // the rows go to different SMs before they share one
+    const int rows = static_cast<int>(std::min<int64_t>(K, static_cast<int64_t>(h->blocks) * h->rows));
+    const int grid = std::min(rows, h->blocks);
+    PsdArgs a{x_dev, stride, K, rows, vec2, bulk, h->win, h->tw, h->pair0, h->part};
     WelchInst wi;
     welch_inst(h->L, &wi);
-    // one block per SM; the segments go to different SMs before they share one
-    const int grid = static_cast<int>(K < h->grid ? K : h->grid);
-    const int64_t slots = static_cast<int64_t>(grid) * h->groups;
-    const int rows = static_cast<int>(K < slots ? K : slots);
     void* args[] = {&a};
     cudaError_t e = cudaLaunchKernel(wi.fn, dim3(grid), dim3(wi.threads), args, h->smem, s);
     if (e == cudaSuccess) {
         const double scale = 1.0 / (static_cast<double>(K) * fs * h->sum_w2);
-        const float2* part = h->part;
+        const double* part = h->part;
         const int* bin = h->bin;
         void* rargs[] = {&part, const_cast<int*>(&rows), &h->L, const_cast<double*>(&scale), &bin, &psd_dev};
-        e = launch_dependent(reinterpret_cast<void*>(&psd_reduce_kernel), dim3((h->L + 1 + 31) / 32), dim3(32, 8), rargs, 0, s);
+        // (not as a dependent launch: started beside the Welch blocks, the
+        // small blocks would crowd on few SMs)
+        e = cudaLaunchKernel(reinterpret_cast<void*>(&psd_reduce_kernel), dim3((h->L + 1 + 31) / 32), dim3(32), rargs, 0, s);
     }
     if (e != cudaSuccess) return psd_cuda_fail(e, "cg_psd_welch");
     return CG_OK;
