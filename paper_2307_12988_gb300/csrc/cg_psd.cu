@@ -788,6 +788,7 @@ __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads
         const double c = static_cast<double>(1.0f / (1.0f + (t + 0.5f) * (1.0f / 128.0f)));
         tab[t] = make_double2(c, -log(c));
     }
+    tc::cluster_sync();   // every block runs before another stores into its shared memory
     tc::pdl_wait();   // (the density may come from the kernel before)
     for (int c = warp; c < rows && c < kResLogRows; c += kResWarps) {
         const int i = c * kResRow + static_cast<int>(rank) * 32 + lane;
