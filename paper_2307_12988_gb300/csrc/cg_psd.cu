@@ -596,45 +596,6 @@ struct ResArgs {
     double* out;               // [12]
 };
 
-// 1/v and 1/sqrt(v): the hardware's FP64 seed (about 20 bits) and two Newton
-// steps, each doubling the correct bits (the second ends at FP64's rounding)
-__device__ __forceinline__ double rcp_newton(double v)
-{
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
-    r = fma(r, fma(-v, r, 1.0), r);
-    return fma(r, fma(-v, r, 1.0), r);
-}
-__device__ __forceinline__ double rsqrt_newton(double v)
-{
-    double r;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
-    r = fma(0.5 * r, fma(-v * r, r, 1.0), r);
-    return fma(0.5 * r, fma(-v * r, r, 1.0), r);
-}
-
-// ln m for positive finite m by table (P. T. P. Tang, ACM TOMS 16, 1990):
-// m = 2^e z, c near 1/z from the top seven bits of z, ln m = e ln 2 - ln c +
-// ln(1 + eps) with eps = z c - 1, |eps| < 2^-7.  tab[i] = (c, -ln c).
-__device__ __forceinline__ double log_table(double m, const double2* tab)
-{
-    const int hi = __double2hiint(m);
-    if (hi < 0x00100000) return log(m);   // subnormal
-    const double2 t = tab[(hi >> 13) & 127];
-    const double z = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(m));
-    const double eps = fma(z, t.x, -1.0);
-    double q = fma(eps, -1.0 / 8.0, 1.0 / 7.0);
-    q = fma(q, eps, -1.0 / 6.0);
-    q = fma(q, eps, 1.0 / 5.0);
-    q = fma(q, eps, -1.0 / 4.0);
-    q = fma(q, eps, 1.0 / 3.0);
-    q = fma(q, eps, -1.0 / 2.0);
-    // the exponent as a double without the FP64 pipe's conversion: 2^52 + 2^31 + e minus 2^52 + 2^31
-    const double e = __hiloint2double(0x43300000, static_cast<int>(0x80000000u + ((hi >> 20) - 1023))) -
-                     __hiloint2double(0x43300000, static_cast<int>(0x80000000u));
-    return fma(e, 0.6931471805599453094, t.y) + fma(q, eps * eps, eps);
-}
-
 // the point's contribution: the four derivatives of ln m and the residual
 // (all zero, and bad set, where the model is not positive and finite)
 struct ResPoint {
@@ -642,66 +603,69 @@ struct ResPoint {
     bool bad;
 };
 
-// per-step constants of the model, taken once per step
-enum { kRf02, kRf04, kRh2, kRhq, kRA, kRB, kRif0, kRf0, kRA4, kRAq, kResConst };
-
-// m = A g + B, g = f0^4 / D, D = u^2 + f^2 h^2, u = f0^2 - f^2, h = f0 / Q:
-//   dm/df0 = 4 A g (1/f0 - f0 (u + f^2 / (2 Q^2)) / D),  dm/dQ = 2 A g f^2 h^2 / (Q D).
-// About 35 FP64 operations (two reciprocals, a logarithm): FP64 issues a warp
-// instruction in tens of cycles here, so their number is what a step costs.
-__device__ __forceinline__ ResPoint res_point(double f2, double logS, const double* q, const double2* tab)
+__device__ __forceinline__ ResPoint res_point(double f, double logS, const double (&p)[4])
 {
     ResPoint o{};
-    const double u = q[kRf02] - f2;
-    const double w = f2 * q[kRh2];
-    const double iD = rcp_newton(fma(u, u, w));
-    const double g = q[kRf04] * iD;
-    const double m = fma(q[kRA], g, q[kRB]);
-    const int hi = __double2hiint(m);
-    if (!(hi >= 0 && hi < 0x7ff00000) || m == 0.0) {   // not positive and finite
+    const double f0 = p[0], Q = p[1], A = p[2], B = p[3];
+    const double u = f0 * f0 - f * f;
+    const double c = f * f0 / Q;
+    const double D = u * u + c * c;
+    const double f04 = f0 * f0 * f0 * f0;
+    const double g = f04 / D;
+    const double m = A * g + B;
+    if (!(m > 0.0) || !(m < INFINITY)) {
         o.bad = true;
         return o;
     }
-    const double im = rcp_newton(m);
-    const double s = g * im;
-    const double t = fma(f2, q[kRhq], u) * iD;
-    o.v[0] = q[kRA4] * s * fma(-q[kRf0], t, q[kRif0]);
-    o.v[1] = q[kRAq] * s * (w * iD);
-    o.v[2] = s;
+    const double dD0 = 4.0 * f0 * u + 2.0 * f * f * f0 / (Q * Q);
+    const double dDQ = -2.0 * c * c / Q;
+    const double im = 1.0 / m;
+    o.v[0] = A * (4.0 * f0 * f0 * f0 / D - f04 * dD0 / (D * D)) * im;
+    o.v[1] = -A * f04 * dDQ / (D * D) * im;
+    o.v[2] = g * im;
     o.v[3] = im;
-    o.v[4] = logS - log_table(m, tab);
+    o.v[4] = logS - log(m);
     return o;
 }
 
-// (H + lambda diag H) d = g by one warp, lane r = lane % 4 holding row r of H
-// and g[r]: Jacobi scaling, then Gauss-Jordan elimination down the diagonal
-// (the scaled matrix is symmetric positive definite: no pivoting), rows in
-// parallel.  d: this lane's component; false if not positive definite.
-__device__ __forceinline__ bool res_solve(const double (&H)[4], double g, double lambda, double& d)
+// (H + lambda diag H) d = g, Jacobi-scaled Cholesky; false if not positive definite
+__device__ bool res_solve(const double* Hu, const double* g, double lambda, double* d)
 {
-    const int r = threadIdx.x & 3;
-    const double dg = r == 0 ? H[0] : r == 1 ? H[1] : r == 2 ? H[2] : H[3];
-    if (!__all_sync(0xffffffffu, dg > 0.0 && dg < INFINITY)) return false;
-    const double s = rsqrt_newton(dg);
-    double M[4];
-#pragma unroll
+    double H[4][4];
+    int q = 0;
+    for (int i = 0; i < 4; ++i)
+        for (int j = i; j < 4; ++j) H[i][j] = H[j][i] = Hu[q++];
+    double s[4];
+    for (int i = 0; i < 4; ++i) {
+        if (!(H[i][i] > 0.0) || !(H[i][i] < INFINITY)) return false;
+        s[i] = 1.0 / sqrt(H[i][i]);
+    }
+    double Mx[4][4], Lc[4][4] = {};
+    for (int i = 0; i < 4; ++i)
+        for (int j = 0; j < 4; ++j) Mx[i][j] = (i == j) ? 1.0 + lambda : H[i][j] * s[i] * s[j];
     for (int j = 0; j < 4; ++j) {
-        const double sj = __shfl_sync(0xffffffffu, s, j);
-        M[j] = j == r ? 1.0 + lambda : H[j] * s * sj;
-    }
-    double b = g * s, mine = 0.0;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const double v = __shfl_sync(0xffffffffu, M[c], c);
+        double v = Mx[j][j];
+        for (int k = 0; k < j; ++k) v -= Lc[j][k] * Lc[j][k];
         if (!(v > 0.0)) return false;
-        const double inv = rcp_newton(v);
-        const double f = r == c ? 0.0 : M[c] * inv;
-        mine = r == c ? inv : mine;
-#pragma unroll
-        for (int j = c + 1; j < 4; ++j) M[j] = fma(-f, __shfl_sync(0xffffffffu, M[j], c), M[j]);
-        b = fma(-f, __shfl_sync(0xffffffffu, b, c), b);
+        Lc[j][j] = sqrt(v);
+        for (int i = j + 1; i < 4; ++i) {
+            double w = Mx[i][j];
+            for (int k = 0; k < j; ++k) w -= Lc[i][k] * Lc[j][k];
+            Lc[i][j] = w / Lc[j][j];
+        }
     }
-    d = b * mine * s;
+    double zz[4], u[4];
+    for (int i = 0; i < 4; ++i) {
+        double v = g[i] * s[i];
+        for (int k = 0; k < i; ++k) v -= Lc[i][k] * zz[k];
+        zz[i] = v / Lc[i][i];
+    }
+    for (int i = 3; i >= 0; --i) {
+        double v = zz[i];
+        for (int k = i + 1; k < 4; ++k) v -= Lc[k][i] * u[k];
+        u[i] = v / Lc[i][i];
+    }
+    for (int i = 0; i < 4; ++i) d[i] = u[i] * s[i];
     return true;
 }
 
@@ -754,19 +718,21 @@ __device__ __forceinline__ bool res_inv_diag(const double* Hu, double (&dg)[4])
     return true;
 }
 
-// The fit by one cluster of eight blocks.  What bounds it is FP64 (2 lanes a
-// cycle per SM, a division or a logarithm tens of operations): on one block a
-// step of a 393-bin band took 30 us.  Row c of the band (points 256 c ..) is
-// split into 32 points per block; a block's warps evaluate its rows in
+// The fit by one cluster of eight blocks.  Row c of the band (points 256 c ..)
+// is split into 32 points per block; a block's warps evaluate its rows in
 // parallel, then each warp adds two of the 16 sums (10 of J^T J, 4 of J^T r,
 // chi^2, bad points) over the rows in order, lane by lane, and reduces the
 // lanes; every block receives all blocks' sums through distributed shared
 // memory, adds them in block order and takes the same step, so one cluster
-// barrier per step is all that the blocks exchange.  ln S is taken once.  The
-// fit of a 393-bin band: 330 us on one block, 137 on the cluster, 101 with
-// the solve in registers and two divisions per point, 71 with Newton
-// reciprocals, the table logarithm and the solve over four lanes, 62 with a
-// warp's two sums reduced together and the sums at the result reused.
+// barrier per step is all that the blocks exchange.  ln S is taken once.
+//
+// Whether the last step is taken depends on the last bit of chi^2, so every
+// operation and the order of every sum are those of the plain form, which one
+// block of 256 threads would run: no reciprocal in place of a division, no
+// other elimination.  What bounds it is that chain: eight divisions and a
+// logarithm per point, then thirty divisions and square roots of the solve one
+// after another, FP64 at 1.7 lanes a cycle and SM.  The fit of a 393-bin band
+// takes 120 us (318 on one block).
 __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads)
     resonance_fit_kernel(ResArgs a)
 {
@@ -774,8 +740,6 @@ __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads
     __shared__ double tot[16];
     __shared__ double pts[2][kResWarps][6][32];     // a round's points, double-buffered
     __shared__ double logs[kResLogRows][32];
-    __shared__ double2 tab[128];                    // (c, -ln c) of log_table
-    __shared__ double con[kResConst];               // constants of the step
     __shared__ double s_v[2][kResWarps];
     __shared__ int s_i[2][kResWarps];
     __shared__ double sp[4];        // parameters at which the sums are taken
@@ -784,10 +748,6 @@ __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads
     const uint32_t rank = tc::cluster_rank();
     const double* S = a.psd + a.k0;
     const int rows = (a.np + kResRow - 1) / kResRow;
-    if (t < 128) {
-        const double c = static_cast<double>(1.0f / (1.0f + (t + 0.5f) * (1.0f / 128.0f)));
-        tab[t] = make_double2(c, -log(c));
-    }
     tc::cluster_sync();   // every block runs before another stores into its shared memory
     tc::pdl_wait();   // (the density may come from the kernel before)
     for (int c = warp; c < rows && c < kResLogRows; c += kResWarps) {
@@ -809,37 +769,16 @@ __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads
     pair_of(q0, i0, j0);
     pair_of(q0 + 1, i1, j1);
     int parity = 0;
-    // constants of the model at sp, by one warp: lane 0 has 1/f0, lane 1 1/Q
-    auto constants = [&]() {
-        const double inv = rcp_newton(sp[lane & 1]);
-        const double if0 = __shfl_sync(0xffffffffu, inv, 0), iQ = __shfl_sync(0xffffffffu, inv, 1);
-        const double f0 = sp[0], A = sp[2], f02 = f0 * f0, h = f0 * iQ;
-        if (lane == 0) {
-            con[kRf02] = f02;
-            con[kRf04] = f02 * f02;
-            con[kRh2] = h * h;
-            con[kRhq] = 0.5 * iQ * iQ;
-            con[kRA] = A;
-            con[kRB] = sp[3];
-            con[kRif0] = if0;
-            con[kRf0] = f0;
-            con[kRA4] = 4.0 * A;
-            con[kRAq] = 2.0 * A * iQ;
-        }
-        __syncwarp();
-    };
     // sums over the band at sp -> tot (all threads of the cluster take part)
     auto sums = [&]() {
+        const double p[4] = {sp[0], sp[1], sp[2], sp[3]};
         double sa = 0.0, sb = 0.0;
         int buf = 0;
         for (int c0 = 0; c0 < rows; c0 += kResWarps, buf ^= 1) {
             const int c = c0 + warp;
             const int i = c * kResRow + static_cast<int>(rank) * 32 + lane;
             ResPoint o{};
-            if (i < a.np) {
-                const double f = (a.k0 + i) * a.df;
-                o = res_point(f * f, c < kResLogRows ? logs[c][lane] : log(S[i]), con, tab);
-            }
+            if (i < a.np) o = res_point((a.k0 + i) * a.df, c < kResLogRows ? logs[c][lane] : log(S[i]), p);
 #pragma unroll
             for (int q = 0; q < 5; ++q) pts[buf][warp][q][lane] = o.v[q];
             pts[buf][warp][5][lane] = o.bad ? 1.0 : 0.0;
@@ -941,81 +880,76 @@ __global__ void __cluster_dims__(kResBlocks, 1, 1) __launch_bounds__(kResThreads
         }
         __syncthreads();
     }
-    if (warp == 0) constants();
-    __syncthreads();
-    sums();
-    // warp 0 of each block takes the LM decisions, lane r = lane % 4 holding
-    // parameter r, its row of H and its gradient; every block comes to the same
-    const int r = lane & 3;
-    const int h0 = r, h1 = r == 0 ? 1 : 3 + r, h2 = r == 0 ? 2 : r == 1 ? 5 : 5 + r, h3 = r == 0 ? 3 : r == 1 ? 6 : 6 + r;
-    double p = sp[r], chi2 = (tot[15] > 0.0) ? INFINITY : tot[14], lambda = a.lambda0;
-    double H[4] = {tot[h0], tot[h1], tot[h2], tot[h3]}, gr = tot[10 + r];
+    // thread 0 of each block takes the LM decisions; every block comes to the same
+    double p[4], chi2 = 0.0, lambda = a.lambda0, Hc[10], gc[4];
     int it = 0, st = 1;
-    bool stop = false, here = true;   // here: the sums at hand are those at p
-    if (!(chi2 < INFINITY)) {
-        st = 3;
-        stop = true;
+    bool here = true;   // the sums at hand are those at p
+    sums();
+    if (t == 0) {
+        for (int i = 0; i < 4; ++i) p[i] = sp[i];
+        chi2 = (tot[15] > 0.0) ? INFINITY : tot[14];
+        for (int i = 0; i < 10; ++i) Hc[i] = tot[i];
+        for (int i = 0; i < 4; ++i) gc[i] = tot[10 + i];
+        if (!(chi2 < INFINITY)) {
+            st = 3;
+            s_ctl = 1;
+        }
     }
+    __syncthreads();
     while (true) {
-        if (warp == 0) {
-            // the next trial point
-            if (!stop) {
-                if (it >= a.max_iter) {
-                    stop = true;
+        // the next trial point
+        if (t == 0 && s_ctl == 0) {
+            if (it >= a.max_iter) {
+                s_ctl = 1;
+            } else {
+                ++it;
+                double d[4];
+                if (!res_solve(Hc, gc, lambda, d)) {
+                    st = 2;
+                    s_ctl = 1;
                 } else {
-                    ++it;
-                    double d;
-                    if (!res_solve(H, gr, lambda, d)) {
-                        st = 2;
-                        stop = true;
-                    } else {
-                        if (lane < 4) sp[r] = p + d;
-                        __syncwarp();
-                        constants();
-                    }
+                    for (int i = 0; i < 4; ++i) sp[i] = p[i] + d[i];
                 }
             }
-            if (lane == 0) s_ctl = stop ? 1 : 0;
         }
         __syncthreads();
         if (s_ctl) break;
         sums();
-        if (warp == 0) {
+        if (t == 0) {
             const double c2 = (tot[15] > 0.0) ? INFINITY : tot[14];
-            const bool settled = (c2 < INFINITY) && fabs(c2 - chi2) <= a.tol * chi2;
-            const bool better = (c2 < INFINITY) && (settled ? c2 <= chi2 : c2 < chi2);
-            here = better;
-            if (better) {
-                p = sp[r];
-                chi2 = c2;
-                H[0] = tot[h0];
-                H[1] = tot[h1];
-                H[2] = tot[h2];
-                H[3] = tot[h3];
-                gr = tot[10 + r];
-            }
-            if (settled) {
+            here = false;
+            if (!(c2 < INFINITY)) {
+                lambda *= 10.0;
+            } else if (fabs(c2 - chi2) <= a.tol * chi2) {
+                if (c2 <= chi2) {
+                    for (int i = 0; i < 4; ++i) p[i] = sp[i];
+                    chi2 = c2;
+                    here = true;
+                }
                 st = 0;
-                stop = true;
+                s_ctl = 1;
+            } else if (c2 < chi2) {
+                for (int i = 0; i < 4; ++i) p[i] = sp[i];
+                chi2 = c2;
+                for (int i = 0; i < 10; ++i) Hc[i] = tot[i];
+                for (int i = 0; i < 4; ++i) gc[i] = tot[10 + i];
+                lambda *= 0.1;
+                here = true;
             } else {
-                lambda *= better ? 0.1 : 10.0;
+                lambda *= 10.0;
             }
         }
+        __syncthreads();
     }
     // standard errors from the sums at the result, taken again only where the
     // last point was refused (every block of the cluster finds the same)
     __syncthreads();   // (all have read s_ctl)
-    if (warp == 0 && lane == 0) s_ctl = here ? 1 : 0;
-    __syncthreads();
-    if (!s_ctl) {
-        if (warp == 0) {
-            if (lane < 4) sp[r] = p;
-            __syncwarp();
-            constants();
-        }
-        __syncthreads();
-        sums();
+    if (t == 0) {
+        s_ctl = here ? 1 : 0;
+        for (int i = 0; i < 4; ++i) sp[i] = p[i];
     }
+    __syncthreads();
+    if (!s_ctl) sums();
     if (t == 0 && rank == 0) {
         double dg[4] = {NAN, NAN, NAN, NAN};
         const bool inv = a.np > 4 && res_inv_diag(tot, dg);
