@@ -323,7 +323,7 @@ struct cg_plan_s {
     // learned initial guess
     bool mlp_ok = false;
     CUtensorMap mlp_map{};
-    int mlp_smem = 0, mlp_clusters = 0;
+    int mlp_smem = 0;
     cg::MlpArgs ma{};
     // device address of the allocation-free reference scratch (set by cg_plan)
     double* noalloc_scratch = nullptr;

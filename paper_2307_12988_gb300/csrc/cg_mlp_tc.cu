@@ -6,9 +6,7 @@
 //     p0 = (W3 a2 + b3) * out_scale + out_mean              (FP32 on the CUDA cores)
 // with W1 (K zero-padded to 64 * nkb) and W2 stored as one BF16 matrix
 // [512][256], streamed from L2 by TMA in 128-row x 64-column chunks through an
-// S-stage mbarrier ring; two blocks form a cluster, and each loads half of
-// every chunk into both (the 256 KB per tile of 128 spectra otherwise come at
-// the L2's 18 bytes a cycle and SM: 15,000 of a tile's 25,000 cycles).  Persistent blocks, one per SM, with warp roles:
+// S-stage mbarrier ring.  Persistent blocks, one per SM, with warp roles:
 //   warps 0-7    epilogues: warp w reads TMEM lanes 32 (w % 4).. (rows) and
 //                column half w / 4; layer 1: bias, GELU, BF16 into the a1
 //                tile; layer 2: bias, GELU and the FP32 output layer;
@@ -107,7 +105,7 @@ __device__ __forceinline__ uint32_t a_off(int row, int k)
                                  ((kl & 7) << 1));
 }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_constant__ CUtensorMap tmW, MlpArgs a)
+__global__ void __launch_bounds__(kMlpThreads, 1) mlp_infer_kernel(const __grid_constant__ CUtensorMap tmW, MlpArgs a)
 {
     extern __shared__ __align__(1024) unsigned char msm_raw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>(
@@ -146,11 +144,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t ntiles = (a.n + kMM - 1) / kMM;
-    // both blocks of a cluster take as many tiles (the last may be empty: its
-    // rows are beyond n), since each feeds half of the other's weight ring
-    const int64_t lead = blockIdx.x & ~1u;
-    const int my_tiles = lead < ntiles ? static_cast<int>((ntiles - 1 - lead) / gridDim.x) + 1 : 0;
-    const uint32_t rank = tc::cluster_rank();
+    const int my_tiles =
+        static_cast<int64_t>(blockIdx.x) < ntiles ? static_cast<int>((ntiles - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
     auto tile_f0 = [&](int it) { return (static_cast<int64_t>(blockIdx.x) + static_cast<int64_t>(it) * gridDim.x) * kMM; };
     const int n1 = 2 * nkb;      // layer-1 chunks
     const int nch = n1 + 8;      // + layer-2 chunks, per tile
@@ -171,7 +166,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
             tc::mbar_init(&full[s], 1);
-            tc::mbar_init(&empty[s], 2);   // both blocks have read the stage
+            tc::mbar_init(&empty[s], 1);
         }
         tc::mbar_init(a_full, kStageWarps * 32);
         tc::mbar_init(a_empty, 1);
@@ -194,7 +189,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_
     if (warp == kLoadWarp && lane == 0) tc::prefetch_tmap(&tmW);
     tc::tc_fence_before();
     __syncthreads();
-    tc::cluster_sync();   // the other block's barriers exist before anything arrives there
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
@@ -222,16 +216,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_
                     }
                     int layer, nh, kb;
                     chunk_geom(c, layer, nh, kb);
-                    // this block's half of the chunk, into both blocks
                     tc::mbar_arrive_expect_tx(&full[s], kChunkBytes);
-                    tc::tma_load_2d_multicast(Wst + s * kChunkBytes + rank * (kChunkBytes / 2), &tmW, kb * 64,
-                                              layer * kHid + nh * kChunkRows + rank * (kChunkRows / 2), &full[s], 3);
+                    tc::tma_load_2d(Wst + s * kChunkBytes, &tmW, kb * 64, layer * kHid + nh * kChunkRows, &full[s]);
                 }
             }
             // the last loads of every stage have landed before the block exits
-            // (and both blocks' reads of them have been reported here)
             for (int q = g - S > 0 ? g - S : 0; q < g; ++q) (void)tc::mbar_wait(&full[q % S], (q / S) & 1u, kPolls);
-            for (int q = g - S > 0 ? g - S : 0; q < g; ++q) (void)tc::mbar_wait(&empty[q % S], (q / S) & 1u, kPolls);
         }
     } else if (warp == kIssueWarp) {
         // ---------------- MMA issue ----------------
@@ -253,7 +243,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_
                     for (int kk = 0; kk < 4; ++kk)
                         tc::mma_f16(d, tc::sdesc_sw128(sa + kk * 32), tc::sdesc_sw128(sb + kk * 32), idesc,
                                     (kb != 0 || kk != 0) ? 1u : 0u);
-                    tc::mma_commit_multicast(&empty[s], 3);
+                    tc::mma_commit(&empty[s]);
                 }
                 return true;
             };
@@ -512,8 +502,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1) mlp_
         tc::tc_fence_after();
         tc::tmem_dealloc(tmem, 2 * kHid);
     }
-    // neither block leaves while the other may still write or arrive here
-    tc::cluster_sync();
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder()
@@ -622,7 +610,7 @@ cudaError_t setup_mlp(cg_plan_s* p, const unsigned char* blob, size_t bytes, con
     }
     cuuint64_t gdim[2] = {static_cast<cuuint64_t>(kHid), static_cast<cuuint64_t>(2 * kHid)};
     cuuint64_t gstride[1] = {static_cast<cuuint64_t>(kHid) * 2};
-    cuuint32_t box[2] = {64, static_cast<cuuint32_t>(kChunkRows / 2)};
+    cuuint32_t box[2] = {64, static_cast<cuuint32_t>(kChunkRows)};
     cuuint32_t estride[2] = {1, 1};
     CUresult r = enc(&p->mlp_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p->d.mlp_W, gdim, gstride, box, estride,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -646,22 +634,6 @@ cudaError_t setup_mlp(cg_plan_s* p, const unsigned char* blob, size_t bytes, con
     p->mlp_smem = mlp_smem_bytes(m.stages, p->T);
     if ((e = raise_smem_limit(reinterpret_cast<void*>(&mlp_infer_kernel), p->mlp_smem)) != cudaSuccess)
         return e;
-    // clusters of two blocks that are resident at once
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(2 * (p->num_sms / 2));
-    cfg.blockDim = dim3(kMlpThreads);
-    cfg.dynamicSmemBytes = p->mlp_smem;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int clusters = 0;
-    if ((e = cudaOccupancyMaxActiveClusters(&clusters, reinterpret_cast<void*>(&mlp_infer_kernel), &cfg)) != cudaSuccess)
-        return e;
-    p->mlp_clusters = clusters > 0 ? clusters : 1;
     p->mlp_ok = true;
     return cudaSuccess;
 }
@@ -676,8 +648,7 @@ cudaError_t launch_mlp(const cg_plan_s* p, const float* y, const float* amps, in
     m.p0 = p0;
     m.flags = flags;
     const int64_t ntiles = (n + kMM - 1) / kMM;
-    const int64_t pairs = (ntiles + 1) / 2, most = p->mlp_clusters;
-    const unsigned grid = 2u * static_cast<unsigned>(pairs < most ? pairs : most);
+    const unsigned grid = static_cast<unsigned>(ntiles < p->num_sms ? ntiles : p->num_sms);
     void* args[] = {const_cast<CUtensorMap*>(&p->mlp_map), &m};
     return cudaLaunchKernel(reinterpret_cast<void*>(&mlp_infer_kernel), dim3(grid), dim3(kMlpThreads), args, p->mlp_smem, s);
 }
