@@ -205,7 +205,10 @@ cg_status cg_set_reference(cg_plan_t plan, const double* ref_spectrum);
  *   rss_dev      float [n_frames] or NULL: sum of squared residuals of y
  *   iters_dev    int16 [n_frames] or NULL: LM trial steps taken
  *   status_dev   int16 [n_frames] or NULL: CG_FIT_* outcome | flags
- * n_frames == 0 is a no-op.  Asynchronous on cuda_stream.
+ * n_frames == 0 is a no-op.  Asynchronous on cuda_stream.  A captured call
+ * shares nothing with other calls and may be replayed beside them, except
+ * with CG_INIT_MLP: its fallback list belongs to the plan, so calls of one
+ * capture are ordered, and a replay must not overlap other calls of the plan.
  */
 cg_status cg_process(cg_plan_t plan, const int16_t* frames_dev, int64_t n_frames,
                      float* amps_dev, float* y_dev, float* params_dev, float* rss_dev,

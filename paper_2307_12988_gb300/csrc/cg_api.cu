@@ -325,22 +325,29 @@ cudaError_t timed(cg_plan_s* p, int stage, cudaStream_t s, F&& launch)
     return e;
 }
 
+cudaError_t is_capturing(cudaStream_t s, bool* yes)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(s, &st);
+    *yes = st != cudaStreamCaptureStatusNone;
+    return e;
+}
+
 // The fits of a plan's calls share its task counter and fallback list, so they
 // run one after another whatever streams the calls are on: begin() makes the
 // stream wait for the fit of a call on another stream, end() marks this one's
-// end.  (Captured calls are ordered by their graph alone.)
+// end.  A captured call may be replayed beside any other: it has no counter.
 struct FitOrder {
     cg_plan_s* p;
     cudaStream_t s;
+    unsigned long long* counter = nullptr;   // of the call's fit kernels, or null (a fixed stride of tasks)
     unsigned long long id = 0;
     bool captured = false;
     cudaError_t begin()
     {
-        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-        cudaError_t e = cudaStreamIsCapturing(s, &st);
-        if (e != cudaSuccess) return e;
-        captured = st != cudaStreamCaptureStatusNone;
-        if (captured) return cudaSuccess;
+        cudaError_t e = is_capturing(s, &captured);
+        if (e != cudaSuccess || captured) return e;
+        counter = p->d.fit_counter;
         if ((e = cudaStreamGetId(s, &id)) != cudaSuccess) return e;
         return p->fit_recorded && p->fit_stream_id != id ? cudaStreamWaitEvent(s, p->ev_fit, 0) : cudaSuccess;
     }
@@ -766,7 +773,7 @@ static cudaError_t standalone_fit(cg_plan_t p, const float* y, const float* amps
     if (!p->fit8_ok) return cg::launch_fit(p, y, amps, n, p0, params, rss, iters, status, s);
     FitOrder order{p, s};
     cudaError_t e = order.begin();
-    if (e == cudaSuccess) e = cg::launch_fit8(p, y, amps, n, p0, params, rss, iters, status, s);
+    if (e == cudaSuccess) e = cg::launch_fit8(p, y, amps, n, p0, params, rss, iters, status, order.counter, s);
     if (e == cudaSuccess) e = order.end();
     return e;
 }
@@ -816,8 +823,12 @@ static cg_status process_impl(cg_plan_t p, const void* frames, int sbytes, int64
         // Several: fork onto the plan's two streams; chunk c
         // is read out (and its initial guess made) on s_read while chunk c-1
         // is fitted on s_fit.  The guess goes to params and its flag to
-        // status, where the fit reads them.
-        const bool fork = n > chunk;
+        // status, where the fit reads them.  A captured call that uses the
+        // plan's fallback list forks as well, so that the plan's streams order
+        // it with other calls of the same capture.
+        bool captured = false;
+        if (mlp && (e = is_capturing(s, &captured)) != cudaSuccess) return cuda_fail(e, "capture status");
+        const bool fork = n > chunk || captured;
         const cudaStream_t sr = fork ? p->s_read : s, sf = fork ? p->s_fit : s;
         e = cudaSuccess;
         if (fork) {
@@ -864,6 +875,7 @@ static cg_status process_impl(cg_plan_t p, const void* frames, int sbytes, int64
                 // converge are listed and refit by the full LM from the moment
                 // guess
                 cg::FitLaunch pol;
+                pol.counter = order.counter;
                 pol.max_iter = p->opts.polish_iter < p->opts.max_iter ? p->opts.polish_iter : p->opts.max_iter;
                 pol.fb_list = p->d.fb_list;
                 pol.fb_count = p->d.fb_count;
@@ -877,6 +889,7 @@ static cg_status process_impl(cg_plan_t p, const void* frames, int sbytes, int64
                         return cg::launch_init(p, yc, ac, m, pc, sc, sf, p->d.fb_list, p->d.fb_count);
                     });
                 cg::FitLaunch fb;
+                fb.counter = order.counter;
                 fb.list = p->d.fb_list;
                 fb.list_n = p->d.fb_count;
                 fb.iters_base = pol.max_iter;
@@ -889,8 +902,10 @@ static cg_status process_impl(cg_plan_t p, const void* frames, int sbytes, int64
                 // the Fano fit reads a given centre only from the median filter
                 const float* p0 = (fano && !median) ? nullptr : pc;
                 const int16_t* fl = fano ? nullptr : sc;
+                cg::FitLaunch fit;
+                fit.counter = order.counter;
                 e = timed(p, CG_STAGE_FIT, sf,
-                          [&] { return cg::launch_fit2(p, yc, ac, m, p0, fl, pc, rc, ic, sc, sf); });
+                          [&] { return cg::launch_fit2(p, yc, ac, m, p0, fl, pc, rc, ic, sc, sf, fit); });
             }
         }
         if (e == cudaSuccess) e = order.end();
@@ -978,14 +993,16 @@ cg_status cg_fit(cg_plan_t p, const float* y, int64_t n, const float* p0, float*
     const bool ordered = (p->opts.init == CG_INIT_MEDIAN && !p0) || fano;
     if (ordered) e = order.begin();
     if (e != cudaSuccess) return cuda_fail(e, "cg_fit launch");
+    cg::FitLaunch fit;
+    fit.counter = order.counter;
     if (p->opts.init == CG_INIT_MEDIAN && !p0) {
         // guess in params (Lorentzian: moments, then the filtered centre), then the fit from it
         if (!fano) e = cg::launch_init(p, y, nullptr, n, params, status, s, nullptr, nullptr);
         if (e == cudaSuccess) e = cg::launch_median(p, y, nullptr, n, params, s);
         if (e == cudaSuccess)
-            e = cg::launch_fit2(p, y, nullptr, n, params, fano ? nullptr : status, params, rss, iters, status, s);
+            e = cg::launch_fit2(p, y, nullptr, n, params, fano ? nullptr : status, params, rss, iters, status, s, fit);
     } else if (fano) {   // the Fano fit makes its own guess; p0 is not read
-        e = cg::launch_fit2(p, y, nullptr, n, nullptr, nullptr, params, rss, iters, status, s);
+        e = cg::launch_fit2(p, y, nullptr, n, nullptr, nullptr, params, rss, iters, status, s, fit);
     } else {
         e = standalone_fit(p, y, nullptr, n, p0, params, rss, iters, status, s);
     }

@@ -412,7 +412,10 @@ __global__ void __launch_bounds__(G == 1 ? 128 : 256, G == 1 ? 3 : 2) fit2_kerne
     const int gl = lane & (G - 1);
     const int leader_lane = lane & ~(G - 1);
     const float inv_scale = 1.0f / a.x_scale;
-    int64_t next = 0, end = 0;   // current task [next, end); tasks come from a.counter
+    // the warp's tasks, the current one [next, end)
+    const unsigned warps = (blockDim.x >> 5) * gridDim.x;
+    unsigned turn = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    int64_t next = 0, end = 0;
     int64_t n = a.n;
     if (a.list_n) {
         const int64_t c = *a.list_n;
@@ -440,10 +443,7 @@ __global__ void __launch_bounds__(G == 1 ? 128 : 256, G == 1 ? 3 : 2) fit2_kerne
         unsigned need = __ballot_sync(kFull, gl == 0 && (kPrefetch ? fn < 0 : f < 0));
         while (need != 0 && next < n) {
             if (next >= end) {
-                unsigned long long t = 0;
-                if (lane == 0) t = atomicAdd(a.counter, 1ULL);
-                t = __shfl_sync(kFull, t, 0);
-                next = static_cast<int64_t>(t) * a.task;
+                next = next_task(a.counter, turn, warps, a.task, n);
                 if (next >= n) {
                     next = end = n;
                     break;
@@ -849,7 +849,7 @@ cudaError_t launch_fit2(const cg_plan_s* p, const float* y, const float* amps, i
         a.fano_Bhi = static_cast<float>(std::max(B0 * (1.0 - bx), B0 * (1.0 + bx)));
     }
     a.row_stride = p->T | 1;
-    a.counter = p->d.fit_counter;
+    a.counter = fl.counter;
     a.solve_f64 = p->solve_f64;
     a.n_rows = n;
     a.err = p->d.err;
@@ -865,8 +865,10 @@ cudaError_t launch_fit2(const cg_plan_s* p, const float* y, const float* amps, i
     const int64_t tasks = (n + a.task - 1) / a.task;
     const int64_t blocks = (tasks + wpb - 1) / wpb;
     const int grid = static_cast<int>(blocks < p->grid_fit2 ? blocks : p->grid_fit2);
-    cudaError_t e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
+    if (a.counter && tasks > static_cast<int64_t>(grid) * wpb) {
+        const cudaError_t e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s);
+        if (e != cudaSuccess) return e;
+    }
     void* args[] = {&a};
     return cudaLaunchKernel(fit2_ptr(p->G2, p->PPL, p->ppl_exact, p->opts.model), dim3(grid), dim3(threads), args,
                             fit2_smem(p->G2, p->T, p->opts.model), s);

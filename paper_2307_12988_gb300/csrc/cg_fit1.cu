@@ -55,6 +55,8 @@ __global__ void __launch_bounds__(128) fit1_kernel(Fit2Args a)
         const int64_t c = *a.list_n;
         n = c < n ? c : n;
     }
+    const unsigned warps = nw * gridDim.x;
+    unsigned turn = warp * gridDim.x + blockIdx.x;
     int64_t next = 0, end = 0;      // the warp's current task [next, end)
     int64_t cur = -1, nxt = -1;     // task being fit / claimed task in flight
     int64_t cur_f = -1, nxt_f = -1; // their frame indices (list[task] for a frame list)
@@ -80,10 +82,7 @@ __global__ void __launch_bounds__(128) fit1_kernel(Fit2Args a)
             const unsigned need = __ballot_sync(kFull, nxt < 0);
             if (need != 0 && next < n) {
                 if (next >= end) {
-                    unsigned long long t = 0;
-                    if (lane == 0) t = atomicAdd(a.counter, 1ULL);
-                    t = __shfl_sync(kFull, t, 0);
-                    next = static_cast<int64_t>(t) * a.task;
+                    next = next_task(a.counter, turn, warps, a.task, n);
                     if (next >= n) next = n;
                     end = next + a.task < n ? next + a.task : n;
                 }

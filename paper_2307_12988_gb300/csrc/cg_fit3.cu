@@ -174,10 +174,10 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
         const int64_t c = *a.list_n;
         n = c < n ? c : n;
     }
-    // the warp's current task [next, end): its first one by its place (warp w
-    // of block b takes task b + w gridDim.x, so few tasks spread over the SMs),
-    // the others from the counter
-    bool first = true;
+    // the warp's tasks, the current one [next, end): warp w of block b begins
+    // with task b + w gridDim.x, so few tasks spread over the SMs
+    const unsigned warps = static_cast<unsigned>(nwarps) * gridDim.x;
+    unsigned turn = static_cast<unsigned>(warp) * gridDim.x + blockIdx.x;
     int64_t next = 0, end = 0;
     int64_t f = -1, fr = -1;     // task index and row of the frame being fit
     int64_t fn = -1, frn = -1;   // the group's next frame (its copy in flight)
@@ -266,16 +266,7 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
         unsigned need = __ballot_sync(kFull, gl == 0 && fn < 0);
         while (need != 0 && next < n) {
             if (next >= end) {
-                unsigned long long t = static_cast<unsigned>(warp) * gridDim.x + blockIdx.x;
-                if (!first) {
-                    t = static_cast<unsigned>(nwarps) * gridDim.x;
-                    if (t * a.task < static_cast<unsigned long long>(n)) {   // (else no task is left to claim)
-                        if (lane == 0) t += atomicAdd(a.counter, 1ULL);
-                        t = __shfl_sync(kFull, t, 0);
-                    }
-                }
-                first = false;
-                next = static_cast<int64_t>(t) * a.task;
+                next = next_task(a.counter, turn, warps, a.task, n);
                 if (next >= n) {
                     next = end = n;
                     break;
@@ -707,7 +698,7 @@ cudaError_t launch_fit3(const cg_plan_s* p, Fit2Args a, cudaStream_t s)
     const int64_t tasks = (a.n + a.task - 1) / a.task;
     const int grid = static_cast<int>(tasks < p->grid_fit3 ? tasks : p->grid_fit3);
     // tasks beyond one per warp are claimed from the counter
-    if (tasks > static_cast<int64_t>(grid) * p->fit3_warps) {
+    if (a.counter && tasks > static_cast<int64_t>(grid) * p->fit3_warps) {
         cudaError_t e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s);
         if (e != cudaSuccess) return e;
     }

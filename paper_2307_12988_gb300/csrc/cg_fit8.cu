@@ -54,7 +54,7 @@ struct Fit8Args {
     const float* u;
     const float* p0;                // [n][4]: abscissa units, or (guessed) on the normalised abscissa
     int guessed;
-    unsigned long long* counter;
+    unsigned long long* counter;    // see next_task
     float x_mid, x_scale;
     int max_iter;
     float tol, lambda0;
@@ -177,7 +177,9 @@ __global__ void __launch_bounds__(32 * kWarps8, NF == 2 ? 4 : 3) fit8_kernel(Fit
     const uintptr_t buf_lo = reinterpret_cast<uintptr_t>(src_base);
     const uintptr_t buf_hi = buf_lo + static_cast<uintptr_t>(a.n) * T * sizeof(float);
     const int64_t n = a.n;
-    bool first = true;
+    // the warp's tasks, the current one [next, end)
+    const unsigned warps = static_cast<unsigned>(kWarps8) * gridDim.x;
+    unsigned turn = static_cast<unsigned>(warp) * gridDim.x + blockIdx.x;
     int64_t next = 0, end = 0;
     int64_t f = -1, fn = -1;     // frame being fit; next frame (its copy in flight)
     float pn[4] = {0.f, 1.f, 0.f, 0.f};
@@ -225,16 +227,7 @@ __global__ void __launch_bounds__(32 * kWarps8, NF == 2 ? 4 : 3) fit8_kernel(Fit
         unsigned need = __ballot_sync(kFull, own == 0 && fn < 0);
         while (need != 0 && next < n) {
             if (next >= end) {
-                unsigned long long t = static_cast<unsigned>(warp) * gridDim.x + blockIdx.x;
-                if (!first) {
-                    t = static_cast<unsigned>(kWarps8) * gridDim.x;
-                    if (t * a.task < static_cast<unsigned long long>(n)) {   // (else no task is left to claim)
-                        if (lane == 0) t += atomicAdd(a.counter, 1ULL);
-                        t = __shfl_sync(kFull, t, 0);
-                    }
-                }
-                first = false;
-                next = static_cast<int64_t>(t) * a.task;
+                next = next_task(a.counter, turn, warps, a.task, n);
                 if (next >= n) {
                     next = end = n;
                     break;
@@ -441,7 +434,8 @@ cudaError_t setup_fit8(cg_plan_s* p)
 }
 
 cudaError_t launch_fit8(const cg_plan_s* p, const float* y, const float* amps, int64_t n, const float* p0,
-                        float* params, float* rss, int16_t* iters, int16_t* status, cudaStream_t s)
+                        float* params, float* rss, int16_t* iters, int16_t* status, unsigned long long* counter,
+                        cudaStream_t s)
 {
     const FitArgs fa = make_fit_args(p);
     if (!p0) {
@@ -469,7 +463,7 @@ cudaError_t launch_fit8(const cg_plan_s* p, const float* y, const float* amps, i
     a.u = fa.u;
     a.p0 = p0 ? p0 : params;
     a.guessed = p0 ? 0 : 1;
-    a.counter = p->d.fit_counter;
+    a.counter = counter;
     a.x_mid = fa.x_mid;
     a.x_scale = fa.x_scale;
     a.max_iter = fa.max_iter;
@@ -482,7 +476,7 @@ cudaError_t launch_fit8(const cg_plan_s* p, const float* y, const float* amps, i
     a.err = p->d.err;
     const int64_t tasks = (n + a.task - 1) / a.task;
     const int grid = static_cast<int>(tasks < blocks ? tasks : blocks);
-    if (tasks > static_cast<int64_t>(grid) * kWarps8) {
+    if (counter && tasks > static_cast<int64_t>(grid) * kWarps8) {
         const cudaError_t e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s);
         if (e != cudaSuccess) return e;
     }

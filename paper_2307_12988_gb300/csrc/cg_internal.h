@@ -119,7 +119,7 @@ struct Fit2Args {
     int task;                // frames per warp task
     int row_stride;          // odd stride of the lane-per-frame spectrum slots
     int solve_f64;           // 1: the 4x4 normal equations are solved in FP64
-    unsigned long long* counter;  // next task (zeroed before the launch)
+    unsigned long long* counter;  // tasks claimed (zeroed before the launch), or null: a fixed stride
     const float* y;          // [n][T] normalised, or null
     const float* amps;       // [n][T] magnitudes when y is null
     const float* inv_ref;    // [T]
@@ -387,24 +387,24 @@ struct FitLaunch {
     int* fb_count = nullptr;
     int iters_base = 0;
     int status_or = 0;
+    unsigned long long* counter = nullptr;   // task counter that no other fit in flight uses, or null
 };
 cudaError_t launch_init(const cg_plan_s* p, const float* y, const float* amps, int64_t n,
                         float* p0_out, int16_t* flag_out, cudaStream_t s, const int* list,
                         const int* list_n, bool eight = false);
 cudaError_t launch_fit2(const cg_plan_s* p, const float* y, const float* amps, int64_t n,
                         const float* p0, const int16_t* flags_in, float* params, float* rss,
-                        int16_t* iters, int16_t* status, cudaStream_t s,
-                        const FitLaunch& fl = FitLaunch());
+                        int16_t* iters, int16_t* status, cudaStream_t s, const FitLaunch& fl);
 // the shared-memory LM kernel: set-up at plan creation, launch with the
 // arguments launch_fit2 prepared
 cudaError_t setup_fit3(cg_plan_s* p);
 cudaError_t launch_fit3(const cg_plan_s* p, Fit2Args a, cudaStream_t s);
 
-// standalone fit at eight lanes per frame (cg_fit8.cu); shares the plan's task
-// counter
+// standalone fit at eight lanes per frame (cg_fit8.cu); counter as in FitLaunch
 cudaError_t setup_fit8(cg_plan_s* p);
 cudaError_t launch_fit8(const cg_plan_s* p, const float* y, const float* amps, int64_t n, const float* p0,
-                        float* params, float* rss, int16_t* iters, int16_t* status, cudaStream_t s);
+                        float* params, float* rss, int16_t* iters, int16_t* status,
+                        unsigned long long* counter, cudaStream_t s);
 
 // learned initial guess (cg_mlp_tc.cu)
 cudaError_t setup_mlp(cg_plan_s* p, const unsigned char* blob, size_t bytes, const char** why);
