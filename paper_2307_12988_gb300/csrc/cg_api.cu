@@ -138,8 +138,10 @@ void free_plan(cg_plan_s* p)
     free_tables(p->d);
     if (p->s_read) cudaStreamDestroy(p->s_read);
     if (p->s_fit) cudaStreamDestroy(p->s_fit);
-    for (cudaEvent_t e : {p->ev_fork, p->ev_read, p->ev_join_r, p->ev_join_f, p->ev_fit})
+    for (cudaEvent_t e : {p->ev_fork, p->ev_read, p->ev_join_r, p->ev_join_f})
         if (e) cudaEventDestroy(e);
+    for (const auto& slot : p->fit_slots)
+        if (slot.ev) cudaEventDestroy(slot.ev);
     for (const auto& t : p->timed) {
         cudaEventDestroy(t.a);
         cudaEventDestroy(t.b);
@@ -235,7 +237,7 @@ cudaError_t setup_fit_kernels(cg_plan_s* p)
     const size_t fsm = cg::fit2_smem(G, T, model);
     if ((e = cg::raise_smem_limit(ff, static_cast<int>(fsm))) != cudaSuccess) return e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ff, cg::fit2_threads(G), fsm)) != cudaSuccess) return e;
-    if ((e = cudaMalloc(&p->d.fit_counter, sizeof(unsigned long long))) != cudaSuccess) return e;
+    if ((e = cudaMalloc(&p->d.fit_counter, sizeof(unsigned long long) * (cg::kFitSlots + 1))) != cudaSuccess) return e;
     if (occ < 1) return cudaSuccess;
     p->grid_fit2 = p->num_sms * occ;
     if (!p->d.err) {
@@ -250,8 +252,10 @@ cudaError_t setup_fit_kernels(cg_plan_s* p)
     p->ppl_exact = exact;
     if ((e = cudaStreamCreateWithFlags(&p->s_read, cudaStreamNonBlocking)) != cudaSuccess) return e;
     if ((e = cudaStreamCreateWithFlags(&p->s_fit, cudaStreamNonBlocking)) != cudaSuccess) return e;
-    for (cudaEvent_t* ev : {&p->ev_fork, &p->ev_read, &p->ev_join_r, &p->ev_join_f, &p->ev_fit})
+    for (cudaEvent_t* ev : {&p->ev_fork, &p->ev_read, &p->ev_join_r, &p->ev_join_f})
         if ((e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess) return e;
+    for (auto& slot : p->fit_slots)
+        if ((e = cudaEventCreateWithFlags(&slot.ev, cudaEventDisableTiming)) != cudaSuccess) return e;
     p->G2 = G;
     p->PPL = ppl;
     // lanes per frame left to the library: the shared-memory kernel where it
@@ -333,30 +337,51 @@ cudaError_t is_capturing(cudaStream_t s, bool* yes)
     return e;
 }
 
-// The fits of a plan's calls share its task counter and fallback list, so they
-// run one after another whatever streams the calls are on: begin() makes the
-// stream wait for the fit of a call on another stream, end() marks this one's
-// end.  A captured call may be replayed beside any other: it has no counter.
+// A call's fits take one of the plan's task counters.  A stream keeps its own
+// while no more than kFitSlots streams are in use, so calls on different streams
+// run side by side; a counter that changes streams is waited for.  Calls with the
+// learned guess share the fallback list: they take the last counter and run one
+// after another.  A captured call may be replayed beside any other: it has none.
+// begin() to end() (or the end of the object) enqueue the fits under a lock, so
+// several threads may use a plan.
 struct FitOrder {
     cg_plan_s* p;
     cudaStream_t s;
+    bool list;                               // the call uses the fallback list
     unsigned long long* counter = nullptr;   // of the call's fit kernels, or null (a fixed stride of tasks)
-    unsigned long long id = 0;
-    bool captured = false;
+    cg_plan_s::FitSlot* slot = nullptr;
+    std::unique_lock<std::mutex> lock;
+    FitOrder(cg_plan_s* plan, cudaStream_t stream, bool uses_list) : p(plan), s(stream), list(uses_list) {}
+    ~FitOrder() { (void)end(); }
     cudaError_t begin()
     {
+        bool captured = false;
+        unsigned long long id = 0;
         cudaError_t e = is_capturing(s, &captured);
         if (e != cudaSuccess || captured) return e;
-        counter = p->d.fit_counter;
         if ((e = cudaStreamGetId(s, &id)) != cudaSuccess) return e;
-        return p->fit_recorded && p->fit_stream_id != id ? cudaStreamWaitEvent(s, p->ev_fit, 0) : cudaSuccess;
+        lock = std::unique_lock<std::mutex>(p->fit_mutex);
+        int k = cg::kFitSlots;
+        if (!list) {
+            for (k = 0; k < cg::kFitSlots; ++k)
+                if (p->fit_slots[k].used && p->fit_slots[k].stream_id == id) break;
+            if (k == cg::kFitSlots) {
+                k = p->fit_next;
+                p->fit_next = (k + 1) % cg::kFitSlots;
+            }
+        }
+        slot = &p->fit_slots[k];
+        if (slot->used && slot->stream_id != id && (e = cudaStreamWaitEvent(s, slot->ev, 0)) != cudaSuccess) return e;
+        slot->stream_id = id;
+        counter = p->d.fit_counter + k;
+        return cudaSuccess;
     }
     cudaError_t end()
     {
-        if (captured) return cudaSuccess;
-        const cudaError_t e = cudaEventRecord(p->ev_fit, s);
-        p->fit_recorded = p->fit_recorded || e == cudaSuccess;
-        p->fit_stream_id = id;
+        if (!lock.owns_lock()) return cudaSuccess;
+        const cudaError_t e = cudaEventRecord(slot->ev, s);
+        slot->used = true;
+        lock.unlock();
         return e;
     }
 };
@@ -771,7 +796,7 @@ static cudaError_t standalone_fit(cg_plan_t p, const float* y, const float* amps
                                   float* params, float* rss, int16_t* iters, int16_t* status, cudaStream_t s)
 {
     if (!p->fit8_ok) return cg::launch_fit(p, y, amps, n, p0, params, rss, iters, status, s);
-    FitOrder order{p, s};
+    FitOrder order(p, s, false);
     cudaError_t e = order.begin();
     if (e == cudaSuccess) e = cg::launch_fit8(p, y, amps, n, p0, params, rss, iters, status, order.counter, s);
     if (e == cudaSuccess) e = order.end();
@@ -836,7 +861,7 @@ static cg_status process_impl(cg_plan_t p, const void* frames, int sbytes, int64
             if (e == cudaSuccess) e = cudaStreamWaitEvent(sr, p->ev_fork, 0);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(sf, p->ev_fork, 0);
         }
-        FitOrder order{p, sf};
+        FitOrder order(p, sf, mlp);
         for (int64_t c0 = 0; c0 < n && e == cudaSuccess; c0 += chunk) {
             const int64_t m = (n - c0) < chunk ? (n - c0) : chunk;
             const int64_t T = p->T;
@@ -989,9 +1014,8 @@ cg_status cg_fit(cg_plan_t p, const float* y, int64_t n, const float* p0, float*
     cudaError_t e = cudaSuccess;
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     const bool fano = p->opts.model == CG_MODEL_FANO;
-    FitOrder order{p, s};
-    const bool ordered = (p->opts.init == CG_INIT_MEDIAN && !p0) || fano;
-    if (ordered) e = order.begin();
+    FitOrder order(p, s, false);
+    if ((p->opts.init == CG_INIT_MEDIAN && !p0) || fano) e = order.begin();
     if (e != cudaSuccess) return cuda_fail(e, "cg_fit launch");
     cg::FitLaunch fit;
     fit.counter = order.counter;
@@ -1006,7 +1030,7 @@ cg_status cg_fit(cg_plan_t p, const float* y, int64_t n, const float* p0, float*
     } else {
         e = standalone_fit(p, y, nullptr, n, p0, params, rss, iters, status, s);
     }
-    if (e == cudaSuccess && ordered) e = order.end();
+    if (e == cudaSuccess) e = order.end();
     if (e != cudaSuccess) return cuda_fail(e, "cg_fit launch");
     return CG_OK;
 }

@@ -2,6 +2,7 @@
 // library's translation units (not part of the public ABI).
 #pragma once
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 #include <cuda.h>
@@ -18,6 +19,7 @@ constexpr int kMaxN = 16384;
 constexpr int kMinT = 5;
 constexpr int kMaxT = 1024;
 constexpr int kThreads = 256;
+constexpr int kFitSlots = 8;   // fits of a plan that run side by side
 
 // Arguments of the readout kernels (cast -> shared-memory FFT -> tooth read).
 struct ReadoutArgs {
@@ -244,7 +246,7 @@ struct DevTables {
     double* ref_part = nullptr;   // [ref_part_rows][T]
     double* ref_out = nullptr;    // [T]
     int ref_part_rows = 0;
-    unsigned long long* fit_counter = nullptr;   // dynamic task counter of the fit kernels
+    unsigned long long* fit_counter = nullptr;   // [kFitSlots + 1] task counters of the fit kernels
     void* mlp_W = nullptr;        // [512][256] BF16 weights of the learned guess
     float* mlp_tab = nullptr;     // its FP32 tables
     int* fb_list = nullptr;       // [fb_cap] frames left by the polish
@@ -315,11 +317,16 @@ struct cg_plan_s {
     cg::CosetArgs fa{};
     cudaStream_t s_read = nullptr, s_fit = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_read = nullptr, ev_join_r = nullptr, ev_join_f = nullptr;
-    // end of the last call's fit and the stream (its unique id) it ran on: the
-    // fits of a plan share its task counter and fallback list
-    cudaEvent_t ev_fit = nullptr;
-    unsigned long long fit_stream_id = 0;
-    bool fit_recorded = false;
+    // the task counters: end of the last fit that used each, and the stream (its
+    // unique id) it ran on.  The last one goes with the fallback list.
+    struct FitSlot {
+        cudaEvent_t ev = nullptr;
+        unsigned long long stream_id = 0;
+        bool used = false;
+    };
+    FitSlot fit_slots[cg::kFitSlots + 1];
+    int fit_next = 0;
+    std::mutex fit_mutex;
     // learned initial guess
     bool mlp_ok = false;
     CUtensorMap mlp_map{};
