@@ -413,8 +413,7 @@ __global__ void __launch_bounds__(G == 1 ? 128 : 256, G == 1 ? 3 : 2) fit2_kerne
     const int leader_lane = lane & ~(G - 1);
     const float inv_scale = 1.0f / a.x_scale;
     // the warp's tasks, the current one [next, end)
-    const unsigned warps = (blockDim.x >> 5) * gridDim.x;
-    unsigned turn = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    bool first = true;
     int64_t next = 0, end = 0;
     int64_t n = a.n;
     if (a.list_n) {
@@ -443,7 +442,8 @@ __global__ void __launch_bounds__(G == 1 ? 128 : 256, G == 1 ? 3 : 2) fit2_kerne
         unsigned need = __ballot_sync(kFull, gl == 0 && (kPrefetch ? fn < 0 : f < 0));
         while (need != 0 && next < n) {
             if (next >= end) {
-                next = next_task(a.counter, turn, warps, a.task, n);
+                next = next_task(a.counter, first, (threadIdx.x >> 5) * gridDim.x + blockIdx.x,
+                                 (blockDim.x >> 5) * gridDim.x, a.task, end, n);
                 if (next >= n) {
                     next = end = n;
                     break;

@@ -28,20 +28,21 @@ constexpr unsigned kFull = 0xffffffffu;
 // The counter evens out what the warps' frames cost (process calls of 10^6
 // frames of 99 teeth 902 us, at a stride 920; fits of 400,000 spectra of 221
 // teeth 663 and 690 us), but must be this launch's alone; a captured call, which
-// may be replayed beside any other, has none.  turn: the warp's place before its
-// first task.
-__device__ __forceinline__ int64_t next_task(unsigned long long* counter, unsigned& turn, unsigned warps, int task,
-                                             int64_t n)
+// may be replayed beside any other, has none.  place: the warp among the grid's
+// `warps`; end: where its last task ended.
+__device__ __forceinline__ int64_t next_task(unsigned long long* counter, bool& first, unsigned place, unsigned warps,
+                                             int task, int64_t end, int64_t n)
 {
-    unsigned long long t = turn;
-    if (counter && turn >= warps) {
+    if (!first && !counter) return end + static_cast<int64_t>(warps - 1) * task;   // (beyond n after a short last task)
+    unsigned long long t = place;
+    if (!first) {
         t = warps;
         if (t * task < static_cast<unsigned long long>(n)) {   // (else no task is left to claim)
             if ((threadIdx.x & 31) == 0) t += atomicAdd(counter, 1ULL);
             t = __shfl_sync(kFull, t, 0);
         }
     }
-    turn += warps;
+    first = false;
     return static_cast<int64_t>(t) * task;
 }
 

@@ -55,8 +55,7 @@ __global__ void __launch_bounds__(128) fit1_kernel(Fit2Args a)
         const int64_t c = *a.list_n;
         n = c < n ? c : n;
     }
-    const unsigned warps = nw * gridDim.x;
-    unsigned turn = warp * gridDim.x + blockIdx.x;
+    bool placed = true;             // (its first task is the one of its place)
     int64_t next = 0, end = 0;      // the warp's current task [next, end)
     int64_t cur = -1, nxt = -1;     // task being fit / claimed task in flight
     int64_t cur_f = -1, nxt_f = -1; // their frame indices (list[task] for a frame list)
@@ -82,7 +81,7 @@ __global__ void __launch_bounds__(128) fit1_kernel(Fit2Args a)
             const unsigned need = __ballot_sync(kFull, nxt < 0);
             if (need != 0 && next < n) {
                 if (next >= end) {
-                    next = next_task(a.counter, turn, warps, a.task, n);
+                    next = next_task(a.counter, placed, warp * gridDim.x + blockIdx.x, nw * gridDim.x, a.task, end, n);
                     if (next >= n) next = n;
                     end = next + a.task < n ? next + a.task : n;
                 }

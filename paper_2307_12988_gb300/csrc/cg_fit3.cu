@@ -176,8 +176,7 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
     }
     // the warp's tasks, the current one [next, end): warp w of block b begins
     // with task b + w gridDim.x, so few tasks spread over the SMs
-    const unsigned warps = static_cast<unsigned>(nwarps) * gridDim.x;
-    unsigned turn = static_cast<unsigned>(warp) * gridDim.x + blockIdx.x;
+    bool first = true;
     int64_t next = 0, end = 0;
     int64_t f = -1, fr = -1;     // task index and row of the frame being fit
     int64_t fn = -1, frn = -1;   // the group's next frame (its copy in flight)
@@ -266,7 +265,7 @@ __global__ void __launch_bounds__(256, 2) fit3_kernel(Fit2Args a)
         unsigned need = __ballot_sync(kFull, gl == 0 && fn < 0);
         while (need != 0 && next < n) {
             if (next >= end) {
-                next = next_task(a.counter, turn, warps, a.task, n);
+                next = next_task(a.counter, first, warp * gridDim.x + blockIdx.x, nwarps * gridDim.x, a.task, end, n);
                 if (next >= n) {
                     next = end = n;
                     break;

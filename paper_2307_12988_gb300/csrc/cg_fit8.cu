@@ -178,8 +178,7 @@ __global__ void __launch_bounds__(32 * kWarps8, NF == 2 ? 4 : 3) fit8_kernel(Fit
     const uintptr_t buf_hi = buf_lo + static_cast<uintptr_t>(a.n) * T * sizeof(float);
     const int64_t n = a.n;
     // the warp's tasks, the current one [next, end)
-    const unsigned warps = static_cast<unsigned>(kWarps8) * gridDim.x;
-    unsigned turn = static_cast<unsigned>(warp) * gridDim.x + blockIdx.x;
+    bool first = true;
     int64_t next = 0, end = 0;
     int64_t f = -1, fn = -1;     // frame being fit; next frame (its copy in flight)
     float pn[4] = {0.f, 1.f, 0.f, 0.f};
@@ -227,7 +226,7 @@ __global__ void __launch_bounds__(32 * kWarps8, NF == 2 ? 4 : 3) fit8_kernel(Fit
         unsigned need = __ballot_sync(kFull, own == 0 && fn < 0);
         while (need != 0 && next < n) {
             if (next >= end) {
-                next = next_task(a.counter, turn, warps, a.task, n);
+                next = next_task(a.counter, first, warp * gridDim.x + blockIdx.x, kWarps8 * gridDim.x, a.task, end, n);
                 if (next >= n) {
                     next = end = n;
                     break;
