@@ -358,6 +358,12 @@ int64_t cg_mlp_param_count(int n_in, int n_hidden, int n_out);
  * 1 <= n_in, n_hidden <= 1024; 1 <= n_out <= 16; 1 <= max_batch <= 1<<20.
  * Weights are drawn uniformly from +-1/sqrt(fan_in) by a counter-based hash
  * (SplitMix64) of (seed, parameter index); biases are zero; Adam state zero.
+ * Device memory: the parameters, their gradient, Adam state and images, and
+ * 6 n_hidden + n_in + 3 n_out floats per row of max_batch.  The first backward
+ * or training call (not one under capture) with batches up to 16,384 rows adds
+ * operand images of about 14 n_hidden + 4 n_in + 256 floats per row of
+ * min(max_batch, 16384); without room for them the steps run on slower
+ * products, with the same result.
  */
 cg_status cg_mlp_create(cg_mlp_t* mlp, int n_in, int n_hidden, int n_out, int max_batch,
                         uint64_t seed);

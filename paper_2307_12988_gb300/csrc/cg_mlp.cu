@@ -725,8 +725,10 @@ cg_status cg_mlp_backward(cg_mlp_t m, const float* x, const float* t, int64_t n,
     if (n < 1 || n > m->max_batch) return fail_m(CG_ERR_ARG, "n must be in [1, max_batch]");
     if (!x || !t) return fail_m(CG_ERR_ARG, "x_dev and t_dev are required");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e;
-    if (n <= kTrainRows) {
+    bool images = false;
+    cudaError_t e = train_ready(m, static_cast<int>(n), s, &images);
+    if (e != cudaSuccess) return cuda_fail_m(e, "cg_mlp_backward");
+    if (images) {
         const TrainBatch b{x, t, n, nullptr, static_cast<int>(n)};
         e = train_prepare(m, b, s);
         if (e == cudaSuccess) e = train_step(m, b, loss_dev, nullptr, nullptr, s);
@@ -757,7 +759,9 @@ cg_status cg_mlp_train_epoch(cg_mlp_t m, const float* x, const float* t, int64_t
     if (!(lr >= 0.f)) return fail_m(CG_ERR_ARG, "lr < 0");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int64_t b = 0;
-    if (batch <= kTrainRows) {
+    bool images = false;
+    if (cudaError_t e = train_ready(m, batch, s, &images); e != cudaSuccess) return cuda_fail_m(e, "cg_mlp_train_epoch");
+    if (images) {
         // the step on operand images; the next batch's rows are gathered
         // beside the Adam step of this one
         auto rows_at = [&](int64_t r0) {

@@ -82,8 +82,11 @@ struct SplitRule {
 };
 SplitRule split_rule(int M, int N, int K, bool can_split);
 
-// the training step on operand images (cg_train.cu)
+// the training step on operand images (cg_train.cu); create: the weights' images
 cudaError_t train_create(cg_mlp_s* m);
+// *ready: batches of `rows` take the step on images (the first such call on a
+// stream that is not capturing allocates the batch images)
+cudaError_t train_ready(cg_mlp_s* m, int rows, cudaStream_t s, bool* ready);
 void train_destroy(cg_mlp_s* m);
 // weight images from the parameters (after the parameters were set)
 cudaError_t train_refresh(cg_mlp_s* m, cudaStream_t s);

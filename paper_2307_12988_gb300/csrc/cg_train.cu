@@ -26,7 +26,11 @@
 // Consecutive kernels of a step overlap their prologues (programmatic
 // dependent launch): each waits for its predecessor before it touches memory.
 // Rows beyond the batch and columns beyond an operand are zeros in the images,
-// so no product needs a bounds check.  Every sum has a fixed order.  Waits are
+// so no product needs a bounds check.  The weights' images live with the object
+// and follow every change of the parameters; those of the batch (nine operands
+// of up to kTrainRows rows) are allocated by the first step that wants them, so
+// an object that only runs forward does without.  A first step under capture,
+// or where they do not fit, takes the generic products (same sums).  Every sum has a fixed order.  Waits are
 // bounded; a block whose wait runs out records it and writes nothing.
 //
 // What bounds it: latency.  A 1,024 x 256 x 256 product is 0.4 GFLOP on 128
@@ -59,12 +63,13 @@ struct Img {
 };
 
 struct TrainImages {
-    int cap = 0;         // batch rows (a multiple of 128)
     int num_sms = 0;
+    bool ready = false;          // the batch images are allocated
+    bool refused = false;        // they did not fit: the generic products serve
     Img xf, xt, a1f, a1t, a2f, a2t, g3t, g2f, g2t, g1t;   // of the batch
     Img w1f, w2f, w2t, w3f, w3t;                          // of the parameters
     float* ws = nullptr;         // K ranges of dW3, dW2, dW1
-    unsigned char* pool = nullptr;
+    unsigned char *weights = nullptr, *batch = nullptr;   // the images' memory
 };
 
 namespace {
@@ -842,36 +847,53 @@ FinishArgs finish_args(cg_mlp_s* m)
 
 }  // namespace
 
+namespace {
+
+struct ImgShape {
+    Img* im;
+    int rows, k;
+};
+// zeroed memory for some images (padding stays zero)
+template <int N>
+cudaError_t alloc_images(const ImgShape (&all)[N], unsigned char** pool, cudaStream_t s)
+{
+    int64_t bytes = 0;
+    for (const ImgShape& a : all) {
+        a.im->rows = up(a.rows, kGM);
+        a.im->lo = static_cast<int64_t>(kblocks(a.k)) * a.im->rows * 128;
+        bytes += 2 * a.im->lo;
+    }
+    cudaError_t e = cudaMalloc(pool, bytes);
+    if (e == cudaSuccess) e = cudaMemsetAsync(*pool, 0, bytes, s);
+    if (e != cudaSuccess) return e;
+    unsigned char* p = *pool;
+    for (const ImgShape& a : all) {
+        a.im->p = p;
+        p += 2 * a.im->lo;
+    }
+    return cudaSuccess;
+}
+
+void free_batch_images(TrainImages* im)
+{
+    if (im->batch) cudaFree(im->batch);
+    if (im->ws) cudaFree(im->ws);
+    im->batch = nullptr;
+    im->ws = nullptr;
+}
+
+}  // namespace
+
 cudaError_t train_create(cg_mlp_s* m)
 {
     TrainImages* im = new (std::nothrow) TrainImages;
     if (!im) return cudaErrorMemoryAllocation;
     m->img = im;
-    im->cap = up(std::min(m->max_batch, kTrainRows), kGM);
     cudaError_t e = cudaDeviceGetAttribute(&im->num_sms, cudaDevAttrMultiProcessorCount, m->device);
     if (e != cudaSuccess) return e;
-    const int ni = m->n_in, H = m->H, no = m->n_out, B = im->cap;
-    struct {
-        Img* im;
-        int rows, k;
-    } all[] = {{&im->xf, B, ni},  {&im->xt, ni, B},  {&im->a1f, B, H}, {&im->a1t, H, B}, {&im->a2f, B, H},
-               {&im->a2t, H, B},  {&im->g3t, no, B}, {&im->g2f, B, H}, {&im->g2t, H, B}, {&im->g1t, H, B},
-               {&im->w1f, H, ni}, {&im->w2f, H, H},  {&im->w2t, H, H}, {&im->w3f, no, H}, {&im->w3t, H, no}};
-    int64_t bytes = 0;
-    for (auto& a : all) {
-        a.im->rows = up(a.rows, kGM);
-        a.im->lo = static_cast<int64_t>(kblocks(a.k)) * a.im->rows * 128;
-        bytes += 2 * a.im->lo;
-    }
-    if ((e = cudaMalloc(&im->pool, bytes)) != cudaSuccess) return e;
-    if ((e = cudaMemset(im->pool, 0, bytes)) != cudaSuccess) return e;   // padding stays zero
-    unsigned char* p = im->pool;
-    for (auto& a : all) {
-        a.im->p = p;
-        p += 2 * a.im->lo;
-    }
-    if ((e = cudaMalloc(&im->ws, sizeof(float) * kGMaxSplit * H * (static_cast<int64_t>(ni) + H + no))) != cudaSuccess)
-        return e;
+    const int ni = m->n_in, H = m->H, no = m->n_out;
+    const ImgShape all[] = {{&im->w1f, H, ni}, {&im->w2f, H, H}, {&im->w2t, H, H}, {&im->w3f, no, H}, {&im->w3t, H, no}};
+    if ((e = alloc_images(all, &im->weights, nullptr)) != cudaSuccess) return e;
     const int most = 227 * 1024;
     for (void* fn : {reinterpret_cast<void*>(&product_kernel<false>), reinterpret_cast<void*>(&product_kernel<true>),
                      reinterpret_cast<void*>(&mid_kernel), reinterpret_cast<void*>(&dw_kernel)})
@@ -879,11 +901,39 @@ cudaError_t train_create(cg_mlp_s* m)
     return train_refresh(m, nullptr);
 }
 
+cudaError_t train_ready(cg_mlp_s* m, int rows, cudaStream_t s, bool* ready)
+{
+    TrainImages* im = m->img;
+    *ready = im->ready && rows <= kTrainRows;
+    if (im->ready || im->refused || rows > kTrainRows) return cudaSuccess;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &st);
+    if (e != cudaSuccess || st != cudaStreamCaptureStatusNone) return e;
+    // (allocation does not disturb another thread's capture in relaxed mode)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if ((e = cudaThreadExchangeStreamCaptureMode(&mode)) != cudaSuccess) return e;
+    const int ni = m->n_in, H = m->H, no = m->n_out, B = up(std::min(m->max_batch, kTrainRows), kGM);
+    const ImgShape all[] = {{&im->xf, B, ni}, {&im->xt, ni, B}, {&im->a1f, B, H}, {&im->a1t, H, B}, {&im->a2f, B, H},
+                            {&im->a2t, H, B}, {&im->g3t, no, B}, {&im->g2f, B, H}, {&im->g2t, H, B}, {&im->g1t, H, B}};
+    e = cudaMalloc(&im->ws, sizeof(float) * kGMaxSplit * H * (static_cast<int64_t>(ni) + H + no));
+    if (e == cudaSuccess) e = alloc_images(all, &im->batch, s);
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();
+        free_batch_images(im);
+        im->refused = true;
+        e = cudaSuccess;
+    } else if (e == cudaSuccess) {
+        *ready = im->ready = true;
+    }
+    (void)cudaThreadExchangeStreamCaptureMode(&mode);
+    return e;
+}
+
 void train_destroy(cg_mlp_s* m)
 {
     if (!m->img) return;
-    if (m->img->pool) cudaFree(m->img->pool);
-    if (m->img->ws) cudaFree(m->img->ws);
+    free_batch_images(m->img);
+    if (m->img->weights) cudaFree(m->img->weights);
     delete m->img;
     m->img = nullptr;
 }
