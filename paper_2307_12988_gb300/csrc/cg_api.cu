@@ -791,11 +791,17 @@ static cg_status check_frames_i8(const cg_plan_s* p, const int8_t* frames, int64
 }
 
 // The moment guess (without p0) and fit of spectra, or of magnitudes where y
-// is null.
+// is null.  As many spectra as the groups of fit_kernel take at once (14,592 up
+// to 221 teeth) go to it: guess and fit are one launch, a step one frame's.
+// Beyond that it holds every block for its slowest frame, round by round.
+// fit_kernel / fit8_kernel, us: 21 teeth, 1,000 spectra 8.9 / 13.1, 9,609 10.4 /
+// 20.3, 16,999 17 / 22, 40,000 33 / 28; 99 teeth 15 / 19, 19 / 28, 31 / 32, 62 /
+// 51; 221 teeth 55 / 61, 62 / 75, 94 / 82, 160 / 128.
 static cudaError_t standalone_fit(cg_plan_t p, const float* y, const float* amps, int64_t n, const float* p0,
                                   float* params, float* rss, int16_t* iters, int16_t* status, cudaStream_t s)
 {
-    if (!p->fit8_ok) return cg::launch_fit(p, y, amps, n, p0, params, rss, iters, status, s);
+    const int64_t at_once = static_cast<int64_t>(p->grid_fit) * (cg::kThreads / p->G);
+    if (!p->fit8_ok || n <= at_once) return cg::launch_fit(p, y, amps, n, p0, params, rss, iters, status, s);
     FitOrder order(p, s, false);
     cudaError_t e = order.begin();
     if (e == cudaSuccess) e = cg::launch_fit8(p, y, amps, n, p0, params, rss, iters, status, order.counter, s);
