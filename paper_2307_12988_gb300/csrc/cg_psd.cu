@@ -177,6 +177,7 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
 {
     using W = Welch<L>;
     constexpr int NT = W::NT, R3 = W::R3, R4 = W::R4, B = W::B, M = W::M, G = W::G, S = W::S, SL = W::SL;
+    tc::pdl_start();
     extern __shared__ __align__(1024) unsigned char psm[];
     const int g = threadIdx.x / NT, t = threadIdx.x % NT, w = t >> 5, lane = t & 31;
     const uint32_t z = static_cast<uint32_t>(__cvta_generic_to_shared(psm)) + g * L * 8;
@@ -473,6 +474,11 @@ __global__ void __launch_bounds__(kWelchThreads, 1) psd_welch_kernel(PsdArgs a)
     }
 }
 
+// Shared memory that a block of the reduction asks for and does not use: the
+// blocks wait for the Welch kernel's end (dependent launch) beside its blocks,
+// and without it dozens of them would crowd on one SM; so four, one a scheduler.
+constexpr int kReduceSmem = 50 * 1024;
+
 // psd[bin[i]] = scale * the sum of the rows of part in order, one thread per
 // slot.  A warp's FP64 addition takes its scheduler 64 cycles, so the blocks are
 // one warp each, spread over all schedulers, and the next 16 rows are requested
@@ -482,6 +488,7 @@ __global__ void __launch_bounds__(32) psd_reduce_kernel(const double* part, int 
 {
     constexpr int kAhead = 16;
     tc::pdl_start();
+    tc::pdl_wait();
     const int i = blockIdx.x * 32 + threadIdx.x;
     if (i > L) return;
     const double* p = part + i;
@@ -1020,6 +1027,7 @@ cg_status cg_psd_create(int seg_len, cg_psd_t* out)
         if (e == cudaSuccess) e = cudaMemcpy(*dst, src.data(), bytes, cudaMemcpyHostToDevice);
     };
     if (e == cudaSuccess) e = cg::raise_smem_limit(wi.fn, wi.smem);
+    if (e == cudaSuccess) e = cg::raise_smem_limit(reinterpret_cast<void*>(&psd_reduce_kernel), kReduceSmem);
     upload(&h->win, w);
     upload(&h->tw, tw);
     upload(&h->pair0, pair0);
@@ -1071,9 +1079,8 @@ cg_status cg_psd_welch(cg_psd_t h, const float* x_dev, int64_t n, int64_t stride
         const double* part = h->part;
         const int* bin = h->bin;
         void* rargs[] = {&part, const_cast<int*>(&rows), &h->L, const_cast<double*>(&scale), &bin, &psd_dev};
-        // (not as a dependent launch: started beside the Welch blocks, the
-        // small blocks would crowd on few SMs)
-        e = cudaLaunchKernel(reinterpret_cast<void*>(&psd_reduce_kernel), dim3((h->L + 1 + 31) / 32), dim3(32), rargs, 0, s);
+        e = launch_dependent(reinterpret_cast<void*>(&psd_reduce_kernel), dim3((h->L + 1 + 31) / 32), dim3(32), rargs,
+                             kReduceSmem, s);
     }
     if (e != cudaSuccess) return psd_cuda_fail(e, "cg_psd_welch");
     return CG_OK;
