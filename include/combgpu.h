@@ -103,8 +103,10 @@ enum {
     CG_PATH_PIPELINE = 3   /* readout kernel (the pruned comb transform when the
                               geometry admits it and the frames are 4-byte
                               aligned, else the general transform), then the
-                              initial-guess and fit kernels, over chunks on two
-                              plan-owned streams */
+                              initial-guess and fit kernels: one after another
+                              on cuda_stream where the call is one chunk, over
+                              chunks on two plan-owned streams where it is
+                              several */
 };
 
 /* Options of a plan.  Fill with cg_opts_default() and change what you need. */

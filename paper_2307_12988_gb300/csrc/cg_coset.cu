@@ -22,11 +22,12 @@
 //    A, 5 R1 in B, Q in C), and a value keeps its place between the stages;
 //  * a batch's samples arrive by one bulk copy, issued when stage A has read
 //    the batch before; tooth number and 1 / reference share one table entry.
-// Measured against single transforms fed by 16-bit loads, integer folds and
-// 16-byte cp.async: 10^6 frames of 1,100 samples 566 -> 439 us (the bytes take
-// 441 at the measured copy rate), 10^5 of 2,500 samples 165 -> 111 us (100),
-// 250,000 of 2,200 8-bit samples 256 -> 207 us (111; 560 warp instructions and
-// 150 shared-memory wavefronts per frame, 16 warps per SM).
+// 10^6 frames of 1,100 samples take 439 us, 10^5 of 2,500 samples 111, 250,000 of
+// 2,200 8-bit samples 207 (560 warp instructions and 150 shared-memory
+// wavefronts per frame, 16 warps per SM); single transforms fed by 16-bit loads,
+// integer folds and 16-byte cp.async took 566, 165 and 256.  At the rate of a
+// copy, half of whose bytes are writes, their bytes would take 441, 100 and 111:
+// no upper bound for these kernels, three quarters of whose bytes are reads.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>

@@ -1,6 +1,6 @@
 // cg_fit8.cu -- the standalone Levenberg-Marquardt fit at eight lanes per
-// frame (cg_fit, and the fit of CG_PATH_SPLIT), two or four frames per lane
-// group.
+// frame (cg_fit, and the fit of CG_PATH_SPLIT) of more spectra than the groups
+// of fit_kernel hold at once, two or four frames per lane group.
 //
 // Paper ("Data Capture and Processing", fit paragraphs): each normalised
 // spectrum is fit by Levenberg-Marquardt, at most 20 iterations, tolerance
